@@ -248,7 +248,7 @@ class State:
             self.v_out = torch.empty(shape, dtype=torch.bfloat16, device=device)
             # what the path produces: the index lists and the compacted cache
             self.results = [self.idx, self.cnt, self.k_out, self.v_out]
-        # kernels of the library per step: two scoring passes + merge; keep set: reduce + cluster select;
+        # kernels of the library per step: two scoring passes; keep set: reduce + cluster select;
         # else the selection (sample floor + sweep + finish; one kernel for up to 592 units of up to 16384
         # positions, and for a budget above a sixth of the sequence) and the gather
         max_len = w.len_hi if w.n_seq > 1 else w.n_in
@@ -256,7 +256,7 @@ class State:
         self.select_kernels = ("sample_floor + stream_sweep + stream_finish" if w.c_max * 6 <= max_len and
                                (max_len + 3 > 16384 + (3 if w.n_seq == 1 else 0) or n_units > 592) else
                                "unit_select" if w.c_max * 6 <= max_len else "cluster_select")
-        self.launches_per_step = 3 + ((3 if w.paper_specpc else 2) if self.specpc else
+        self.launches_per_step = 2 + ((3 if w.paper_specpc else 2) if self.specpc else
                                       (3 if self.select_kernels.startswith("sample") else 1) + 1)
 
     def step(self, events=None, v_src=None):
@@ -475,7 +475,7 @@ def main(argv=None):
     # denominator of `frac`; both fractions are always in the line.
     capped = clocks is not None and "sw_power_cap" in clocks.get("reasons", [])
     peak_tf = peaks["bf16_tflops_sustained"] if capped else peaks["bf16_tflops"]
-    roofline = {"bound": "tensor", "kernel": "spec_score: score_kernel<1> + merge + score_kernel<2>",
+    roofline = {"bound": "tensor", "kernel": "spec_score: score_kernel<1> + score_kernel<2>",
                 "achieved": tf, "peak": peak_tf, "unit": "TFLOP/s", "frac": tf / peak_tf,
                 "peak_source": peak_src + (" (sustained cuBLAS bf16: sw_power_cap seen in the timed region)" if capped
                                            else " (burst cuBLAS bf16)"),

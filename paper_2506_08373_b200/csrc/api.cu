@@ -87,9 +87,6 @@ WorkspacePlan plan_workspace(const spec_problem* p) {
   w.partial_off = off;
   w.partial_bytes = (size_t)(n_units + ctas) * 4 * (size_t)M * 2 * sizeof(float);   // four epilogue warpgroups
   off = align_up(off + w.partial_bytes, 256);
-  w.rowc_off = off;
-  w.rowc_bytes = (size_t)p->n_seq * p->n_layers * p->n_q_heads * (size_t)R * sizeof(float);
-  off = align_up(off + w.rowc_bytes, 256);
   w.token_off = off;
   w.token_bytes = 2 * (size_t)(p->total_tokens > 0 ? p->total_tokens : 1) * sizeof(float);   // token scores, and their average pool
   off = align_up(off + w.token_bytes, 256);

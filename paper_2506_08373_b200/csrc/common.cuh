@@ -32,7 +32,6 @@ SPEC_HIDDEN inline bool aligned16(const void* ptr) { return (reinterpret_cast<ui
 struct WorkspacePlan {
   int score_ctas;          // persistent grid of the scoring kernels
   size_t partial_off, partial_bytes;   // per-segment row statistics (pass 1)
-  size_t rowc_off, rowc_bytes;         // per-row softmax constants
   size_t token_off, token_bytes;       // SpecPC token scores (two vectors of total_tokens floats)
   size_t sel_head_off, sel_head_bytes; // streaming selection: sel_head_words words per (sequence, layer, KV head) unit
   int sel_head_words;                  // four words, then one candidate count per chunk
@@ -54,6 +53,25 @@ constexpr int kSelCandSlack = 2 * kSelChunkMax;
     if (e__ != cudaSuccess)                                                             \
       return ::spec::fail(SPEC_ERR_CUDA, "%s: %s", #expr, cudaGetErrorString(e__));     \
   } while (0)
+
+// Launches a kernel that may start before the kernel in front of it on the stream has ended (and then
+// waits for it with griddepcontrol.wait before it touches memory): the launch's own latency and the
+// kernel's set-up overlap the tail of the one before.
+template <class... Params, class... Args>
+SPEC_HIDDEN inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                                                const Args&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 // Token range of sequence s.
 __device__ __forceinline__ void seq_range(const int32_t* cu, int n_in, int s, int& begin, int& n) {

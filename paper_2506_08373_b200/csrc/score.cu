@@ -4,9 +4,8 @@
 // KV head.  The M x n probability matrix never leaves the SM:
 //   pass 1   S = Q K^T per 128-key tile (query rows on TMEM lanes): running row max and
 //            sum-exp, kept per thread, written per (CTA, unit) segment;
-//   merge    combines the segments' statistics into one constant per row,
-//            c_i = log2e*scale*max_i + log2 Z_i - log2 w_i;
-//   pass 2   S^T = K Q^T per tile (keys on TMEM lanes, query rows on columns):
+//   pass 2   first combines the segments' statistics into one constant per row,
+//            c_i = log2e*scale*max_i + log2 Z_i - log2 w_i; then S^T = K Q^T per tile (keys on TMEM lanes, query rows on columns):
 //            p = exp2(scale*log2e*S - c_i), reduced over columns thread-locally, one reduction per key
 //            and warpgroup.
 // Both passes are persistent, warp-specialised kernels: warp 0 feeds K tiles (and the unit's Q)
@@ -69,13 +68,13 @@ struct ScoreParams {
   const int32_t* cu;
   const float* row_weight;
   float* partial;       // [n_units + n_ctas][4 warpgroups][M][2]  (max in log2 domain, sum-exp)
-  float* rowc;          // [n_seq*L*Hq*R]  minus the per-row constant
   float* scores;        // [L, Hkv, T]
   int32_t* status;
   long long T;
   int n_in, n_seq, L, Hq, Hkv, G, R, M, M_pad, d;   // M, M_pad: the query rows of this launch, rows [row0, row0 + M) of every unit
   int row0;
   int causal, n_window;  // causal != 0: window row r sees keys up to position n - n_window + r only
+  int merge_slots;       // threads that share the merging of a unit's statistics when there are fewer rows than threads (0: none do)
   int n_stages, n_chunks, cw_last;   // pass 2: chunks of 128 query rows, the last of cw_last (64 or 128)
   int reduce;
   float a;              // softmax_scale * log2(e)
@@ -174,6 +173,10 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr) : "memory");
 }
 
+// Programmatic dependent launch: the next kernel on the stream may start; wait for the one before.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -206,7 +209,7 @@ struct Seg {
 };
 
 struct SegIter {
-  long long g, g_end;
+  long long g, g_end, per_cta;
   int TT;
 };
 
@@ -227,6 +230,7 @@ __device__ __forceinline__ SegIter seg_begin(const ScoreParams& p, const int* tp
   it.TT = tp[p.n_seq];
   const long long N = (long long)p.L * p.Hkv * it.TT;
   const long long P = (N + n_ctas - 1) / n_ctas;
+  it.per_cta = P;
   it.g = P * cta;
   it.g_end = it.g + P < N ? it.g + P : N;
   return it;
@@ -354,6 +358,73 @@ __device__ __forceinline__ void prob_accumulate_causal(const uint32_t (&r)[32], 
   }
 }
 
+// Combines the statistics that pass 1 left for a unit (one partial per warpgroup and CTA that worked
+// on it, `n` of them from `part`, M rows each) into minus the softmax constant of every row, in
+// shared memory.  Called by all epilogue threads.  Every CTA of pass 2 does this for each of its
+// segments: a unit's partials are read from L2 by the few CTAs that share the unit, which takes
+// about a microsecond, where a kernel of its own between the passes took 4 to 22 (one layer of 64K:
+// 80 partials per row in a serial loop) plus two launch gaps.  When there are fewer rows than half
+// the threads, several threads take a share of a row's partials each and meet in shared memory.
+__device__ __forceinline__ void fold_stats(float& m, float& z, float pm, float pz) {
+  const float mn = fmaxf(m, pm);
+  if (mn > -INFINITY) z = z * exp2f(m - mn) + pz * exp2f(pm - mn);
+  m = mn;
+}
+
+__device__ __forceinline__ void row_constants(const ScoreParams& p, const float2* __restrict__ part, int n, int et, float* c_sm, float2* merge_sm) {
+  const int Mr = (p.M + 31) & ~31;
+  const int slices = p.merge_slots > 0 ? p.merge_slots / Mr : 1;
+  for (int i0 = 0; i0 < p.M_pad; i0 += kEpilogueThreads) {
+    const int sl = slices > 1 ? et / Mr : 0;
+    const int i = slices > 1 ? et - sl * Mr : i0 + et;
+    float m = -INFINITY, z = 0.f;
+    if (i < p.M && sl < slices) {
+      int c = sl;
+      for (; c + 7 * slices < n; c += 8 * slices) {           // eight loads in flight
+        float2 v[8];
+        float mx = m;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldcg(part + (size_t)(c + u * slices) * p.M + i);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mx = fmaxf(mx, v[u].x);
+        if (mx > -INFINITY) {
+          z *= exp2f(m - mx);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) z += v[u].y * exp2f(v[u].x - mx);
+        }
+        m = mx;
+      }
+      for (; c < n; c += slices) {
+        const float2 v = __ldcg(part + (size_t)c * p.M + i);
+        fold_stats(m, z, v.x, v.y);
+      }
+    }
+    if (slices > 1) {
+      if (sl < slices) merge_sm[et] = make_float2(m, z);
+      asm volatile("bar.sync 1, 512;" ::: "memory");
+      if (et < p.M) {
+        for (int s = 1; s < slices; ++s) {
+          const float2 v = merge_sm[s * Mr + et];
+          fold_stats(m, z, v.x, v.y);
+        }
+      }
+    }
+    if (sl == 0 && i < p.M_pad) {
+      float c = -INFINITY;                                     // rows that pad the last tile weigh nothing
+      if (i < p.M) {
+        c = m + log2f(z);
+        if (p.row_weight) c -= log2f(p.row_weight[(p.row0 + i) % p.R]);
+        c = -c;
+      }
+      c_sm[i] = c;
+    }
+    if (slices > 1) {                                          // the padding rows beyond the slices' reach
+      for (int j = Mr + et; j < p.M_pad; j += kEpilogueThreads) c_sm[j] = -INFINITY;
+      break;
+    }
+  }
+}
+
 // ------------------------------------------------------------------ the kernel --------
 
 template <int PASS, bool MAXRED>
@@ -366,7 +437,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   uint8_t* k_sm = smem;
   uint8_t* q_sm = smem + (size_t)p.n_stages * p.stage_bytes;
   float* c_sm = reinterpret_cast<float*>(q_sm + p.q_bytes);
-  int* tp = reinterpret_cast<int*>(c_sm + p.M_pad);
+  float2* merge_sm = reinterpret_cast<float2*>(c_sm + p.M_pad);            // pass 2, units of few rows: see row_constants
+  int* tp = reinterpret_cast<int*>(merge_sm + p.merge_slots);
   uint64_t* bars = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(tp + p.n_seq + 1) + 7) & ~(uintptr_t)7);
   uint64_t* k_full = bars;
   uint64_t* k_empty = bars + kMaxStages;
@@ -380,6 +452,12 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   if ((smem_u32(smem) & 1023u) != 0) {      // the swizzled tiles need 1024-byte alignment
     if (tid == 0) report(p.status, SPEC_ERR_ALIGNMENT);
     return;
+  }
+  // Pass 1 may be launched while whatever fills its inputs still runs; pass 2 while pass 1 still does, but
+  // every CTA of pass 1 is past its wait by then, so that only what pass 1 writes has to be waited for (below).
+  if (PASS == 1) {
+    wait_for_previous_grid();
+    launch_dependents();
   }
   if (tid == 0) {
     *abort_flag = 0;
@@ -519,9 +597,23 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     const uint32_t my_taddr = lane_base + wg * BUFCOLS;
     if (PASS == 1) {
       // Work item = 128 query rows (on lanes) x the 128 keys of a tile, all of it mine.
+      // The scores are zeroed here, tile by tile, for pass 2 to add into: tokens of a sequence by the CTA that has
+      // their tile, tokens that no sequence covers by whole rows in turn.
+      const bool clears = p.row0 == 0;
+      if (clears) {
+        const long long lo = p.cu ? p.cu[0] : 0, hi = p.cu ? p.cu[p.n_seq] : p.n_in;
+        if (lo > 0 || hi < p.T) {
+          for (int r = blockIdx.x; r < p.L * p.Hkv; r += gridDim.x) {
+            float* row = p.scores + (long long)r * p.T;
+            for (long long j = et; j < lo; j += kEpilogueThreads) row[j] = 0.f;
+            for (long long j = hi + et; j < p.T; j += kEpilogueThreads) row[j] = 0.f;
+          }
+        }
+      }
       const int n_mt = p.M_pad / 128;
       float mrun[kMaxMTiles], zrun[kMaxMTiles];
       while (ok && seg_next(it, p, tp, sg)) {
+        float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
 #pragma unroll
         for (int i = 0; i < kMaxMTiles; ++i) { mrun[i] = -INFINITY; zrun[i] = 0.f; }
         for (int t = pair; t < sg.nt && ok; t += 2) {
@@ -529,6 +621,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const int nv = min(kTileKeys, sg.n - key0);                              // valid keys of the tile
           const bool in_window = p.causal && key0 + kTileKeys > sg.n - p.n_window;    // warp-uniform
           const bool plain = nv >= kTileKeys && !in_window;
+          if (clears && half == 0 && row_in_tile < nv) out[key0 + row_in_tile] = 0.f;
           for (int mt = ((t >> 1) + half) & 1; mt < n_mt && ok; mt += 2) {
             ok = mbar_wait(&t_full[wg], used & 1, abort_flag);
             if (!ok) break;
@@ -581,12 +674,21 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       // Work item = one key tile (keys on lanes) x one chunk of 128 query rows, all of it mine; the
       // chunks of a tile alternate between the two warpgroups of the pair.
       const float2 a2 = splat2(p.a);
-      // Every epilogue thread passes the two barriers of every segment, also after a wait has
+      const long long per_cta = it.per_cta;
+      wait_for_previous_grid();                                 // pass 1: statistics and zeroed scores
+      launch_dependents();
+      // Every epilogue thread passes the barriers of every segment, also after a wait has
       // given up, so that no warp is left waiting at them.
       while (seg_next(it, p, tp, sg)) {
-        const int qrow0 = ((sg.s * p.L + sg.l) * p.Hq + sg.h * p.G) * p.R;
         asm volatile("bar.sync 1, 512;" ::: "memory");          // previous unit's constants no longer read
-        for (int i = et; i < p.M_pad; i += kEpilogueThreads) c_sm[i] = i < p.M ? p.rowc[qrow0 + p.row0 + i] : -INFINITY;
+        {
+          // the CTAs of pass 1 that worked on this unit: its tiles are u0 .. u0 + n_tiles - 1 of the global tile space
+          const long long u0 = (long long)(sg.l * p.Hkv + sg.h) * it.TT + tp[sg.s];
+          const int n_tiles = tp[sg.s + 1] - tp[sg.s];
+          const int b0 = (int)(u0 / per_cta), b1 = (int)((u0 + n_tiles - 1) / per_cta);
+          row_constants(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
+                        (b1 - b0 + 1) * kEpilogueWarpgroups, et, c_sm, merge_sm);
+        }
         asm volatile("bar.sync 1, 512;" ::: "memory");
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
         for (int t = pair; t < sg.nt && ok; t += 2) {
@@ -645,51 +747,6 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   }
 }
 
-// Combines the per-segment statistics of every query row into its softmax constant.
-__global__ void __launch_bounds__(128) merge_kernel(const ScoreParams p, int n_ctas) {
-  __shared__ int sh_before, sh_total;
-  const int unit = blockIdx.x;
-  const int lh = unit / p.n_seq, s = unit % p.n_seq;
-  if (threadIdx.x == 0) { sh_before = 0; sh_total = 0; }
-  __syncthreads();
-  int before = 0, total = 0;
-  for (int i = threadIdx.x; i < p.n_seq; i += blockDim.x) {
-    int b, n;
-    seq_range(p.cu, p.n_in, i, b, n);
-    const int tiles = (n + kTileKeys - 1) / kTileKeys;
-    total += tiles;
-    if (i < s) before += tiles;
-  }
-  atomicAdd(&sh_before, before);
-  atomicAdd(&sh_total, total);
-  __syncthreads();
-  int b, n;
-  seq_range(p.cu, p.n_in, s, b, n);
-  const int tiles = (n + kTileKeys - 1) / kTileKeys;
-  if (tiles == 0) return;
-  const long long TT = sh_total;
-  const long long N = (long long)p.L * p.Hkv * TT;
-  const long long P = (N + n_ctas - 1) / n_ctas;
-  const long long u0 = (long long)lh * TT + sh_before;
-  const int b0 = (int)(u0 / P), b1 = (int)((u0 + tiles - 1) / P);
-  const int l = lh / p.Hkv, h = lh % p.Hkv;
-  const int qrow0 = ((s * p.L + l) * p.Hq + h * p.G) * p.R;
-  for (int i = threadIdx.x; i < p.M; i += blockDim.x) {
-    float m = -INFINITY;
-    const int s0 = (unit + b0) * kEpilogueWarpgroups, s1 = (unit + b1) * kEpilogueWarpgroups + kEpilogueWarpgroups - 1;   // one partial per warpgroup and CTA
-    for (int c = s0; c <= s1; ++c) m = fmaxf(m, p.partial[((size_t)c * p.M + i) * 2]);
-    float z = 0.f;
-    for (int c = s0; c <= s1; ++c) {
-      const float pm = p.partial[((size_t)c * p.M + i) * 2];
-      const float pz = p.partial[((size_t)c * p.M + i) * 2 + 1];
-      if (pm > -INFINITY) z += pz * exp2f(pm - m);
-    }
-    float c = m + log2f(z);
-    if (p.row_weight) c -= log2f(p.row_weight[(p.row0 + i) % p.R]);
-    p.rowc[qrow0 + p.row0 + i] = -c;
-  }
-}
-
 // ------------------------------------------------------------------ host side ---------
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -739,11 +796,12 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   rc = check_device();
   if (rc != SPEC_OK) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // the whole output is overwritten: tokens that no sequence covers read as 0, and pass 2 adds into it
-  const size_t out_bytes = (size_t)pr->n_layers * pr->n_kv_heads * (size_t)pr->total_tokens * sizeof(float);
-  if (out_bytes) SPEC_CUDA_OK(cudaMemsetAsync(scores_out, 0, out_bytes, st));
   const int64_t tokens = pr->cu_seqlens ? pr->total_tokens : pr->n_in;
-  if (tokens == 0) return SPEC_OK;
+  if (tokens == 0) {                                       // nothing to score: the whole output reads as 0
+    const size_t out_bytes = (size_t)pr->n_layers * pr->n_kv_heads * (size_t)pr->total_tokens * sizeof(float);
+    if (out_bytes) SPEC_CUDA_OK(cudaMemsetAsync(scores_out, 0, out_bytes, st));
+    return SPEC_OK;
+  }
 
   EncodeTiledFn encode = encode_fn();
   if (!encode) return fail(SPEC_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
@@ -775,7 +833,6 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   p.row_weight = row_weight;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   p.partial = reinterpret_cast<float*>(ws + wp.partial_off);
-  p.rowc = reinterpret_cast<float*>(ws + wp.rowc_off);
   p.scores = scores_out;
   p.status = status_word;
   p.T = pr->total_tokens;
@@ -788,7 +845,6 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   p.stage_bytes = (uint32_t)kTileKeys * d * 2;
 
   const int n_ctas = wp.score_ctas;
-  const unsigned n_units = (unsigned)(pr->n_seq * pr->n_layers * pr->n_kv_heads);
   auto pass1 = score_kernel<1, false>;
   auto pass2 = reduce == SPEC_REDUCE_MAX ? score_kernel<2, true> : score_kernel<2, false>;
   // The kernels may use all of an SM's shared memory; the attribute is set once per device (it is per
@@ -813,7 +869,9 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     p.n_chunks = (M64 + 127) / 128;
     p.cw_last = M64 - (p.n_chunks - 1) * 128;
     p.q_bytes = (uint32_t)p.M_pad * d * 2;
-    const int small = p.M_pad * 4 + (pr->n_seq + 1) * 4 + 8 + kNumBars * 8 + 16;
+    const int Mr = (p.M + 31) & ~31;
+    p.merge_slots = 2 * Mr <= kEpilogueThreads ? kEpilogueThreads / Mr * Mr : 0;
+    const int small = p.M_pad * 4 + p.merge_slots * 8 + (pr->n_seq + 1) * 4 + 8 + kNumBars * 8 + 16;
     const int smem_max = 227 * 1024;
     int stages = (smem_max - (int)p.q_bytes - small) / (int)p.stage_bytes;
     if (stages > kMaxStages) stages = kMaxStages;
@@ -821,12 +879,8 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     p.n_stages = stages;
     int smem = stages * (int)p.stage_bytes + (int)p.q_bytes + small;
     if (smem < 120 * 1024) smem = 120 * 1024;             // one CTA per SM: each CTA owns the whole TMEM
-    pass1<<<n_ctas, kThreads, smem, st>>>(tm_q, tm_k, p);
-    SPEC_CUDA_OK(cudaGetLastError());
-    merge_kernel<<<n_units, 128, 0, st>>>(p, n_ctas);
-    SPEC_CUDA_OK(cudaGetLastError());
-    pass2<<<n_ctas, kThreads, smem, st>>>(tm_q, tm_k, p);
-    SPEC_CUDA_OK(cudaGetLastError());
+    SPEC_CUDA_OK(launch_dependent(pass1, dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
+    SPEC_CUDA_OK(launch_dependent(pass2, dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
   }
   return SPEC_OK;
 }
