@@ -2,26 +2,27 @@
 //
 // score[j] = reduce_i softmax_j(scale * q_i . k_j) over the M = G*R query rows that share a
 // KV head.  The M x n probability matrix never leaves the SM:
-//   pass 1   S = Q K^T per 128-key tile (query rows on TMEM lanes): running row max and
-//            sum-exp, kept per thread, written per (CTA, unit) segment;
+//   pass 1   S = Q K^T per 128-key tile (query rows on TMEM lanes): sum-exp over a
+//            reference per row, kept per thread, written per (CTA, unit) segment;
 //   pass 2   first combines the segments' statistics into one constant per row,
-//            c_i = log2e*scale*max_i + log2 Z_i - log2 w_i; then S^T = K Q^T per tile (keys on TMEM lanes, query rows on columns):
-//            p = exp2(scale*log2e*S - c_i), reduced over columns thread-locally, one reduction per key
-//            and warpgroup.
+//            c_i = log2e*scale*m_i + log2 Z_i - log2 w_i; then S^T = K Q^T per tile (keys on TMEM lanes,
+//            query rows on columns): p = exp2(scale*log2e*S - c_i), reduced over columns
+//            thread-locally, one reduction per key and warpgroup.
 // Both passes are persistent, warp-specialised kernels: warp 0 feeds K tiles (and the unit's Q)
-// with TMA into a shared-memory ring, two threads issue tcgen05.mma into TMEM, and four epilogue
+// with TMA into a shared-memory ring, two warps issue tcgen05.mma into TMEM, and four epilogue
 // warpgroups (16 warps, four per SM sub-partition) drain the accumulators with tcgen05.ld and
 // do the exponentials.  Every warpgroup owns one 128-column TMEM buffer.  A work item is
 // 128 x 128 logits: 128 query rows x the 128 keys of a tile in pass 1, the 128 keys of a tile x
 // a chunk of 128 query rows in pass 2.  Key tiles alternate between the two pairs of
-// warpgroups (each pair has its own issuing thread); within a pair the items of a tile
+// warpgroups (each pair has its own issuing warp); within a pair the items of a tile
 // alternate between its two warpgroups, which start alternately from tile to tile.  A
-// warpgroup drains an item whole, four 32-column loads with the arithmetic in between, and
-// hands the buffer back after the last load, so the four warps that share an SM
-// sub-partition run out of step with one another.
+// warpgroup drains an item whole, four 32-column loads with the arithmetic in between (two
+// blocks in registers: the other roles give up registers for that), and hands the buffer back
+// after the last load, so the four warps that share an SM sub-partition run out of step with one
+// another.
 // The exponential is the scarce resource (16 MUFU results per clock per SM against 32 logits per
 // clock from the tensor cores), so a fixed share of the elements is evaluated on the FMA pipes
-// instead (range reduction + cubic polynomial, relative error 7.5e-5), and the surrounding
+// instead (range reduction + quartic polynomial, relative error 2.6e-6), and the surrounding
 // arithmetic uses the packed two-lane fp32 instructions to halve its issue slots.  Warpgroups
 // never synchronise inside a unit: pass 1 writes their statistics as separate partials; in
 // pass 2 a key tile belongs to one pair, whose two warpgroups add their per-key sums (over the
@@ -43,17 +44,20 @@ namespace spec {
 
 constexpr int kEpilogueWarpgroups = 4;
 constexpr int kEpilogueThreads = kEpilogueWarpgroups * 128;
-constexpr int kMmaWarpB = 2 + kEpilogueThreads / 32;    // second MMA-issuing warp, after the epilogue warps
-constexpr int kThreads = 64 + kEpilogueThreads + 32;
-#ifndef SPEC_POLY_PAIRS_1
-#define SPEC_POLY_PAIRS_1 4
+constexpr int kThreads = 128 + kEpilogueThreads;        // one more warpgroup: TMA producer, two MMA issuers, an idle warp
+// Registers per thread: at launch (the most that five warps per SM sub-partition leave), and after the
+// warpgroups have divided them; the epilogue needs two blocks of 32 accumulator columns at a time.
+constexpr int kLaunchRegs = 96, kIssueRegs = 64, kEpilogueRegs = 104;
+static_assert(128 * kIssueRegs + kEpilogueThreads * kEpilogueRegs <= kThreads * kLaunchRegs, "the warpgroups' shares must fit what the block is launched with");
+// Of the 16 element pairs in a 32-element block, evaluated on the FMA pipes.  Sustained time of 8 layers at 128K
+// (640 rows) for 3, 4, 5, 6 pairs: 3.083, 3.061, 3.057, 3.128 ms.
+#ifndef SPEC_POLY_PAIRS
+#define SPEC_POLY_PAIRS 5
 #endif
-#ifndef SPEC_POLY_PAIRS_2
-#define SPEC_POLY_PAIRS_2 4
-#endif
-// of the 16 element pairs in a 32-element block, evaluated on the FMA pipes (pass 1, pass 2)
-constexpr int kPolyPairs1 = SPEC_POLY_PAIRS_1, kPolyPairs2 = SPEC_POLY_PAIRS_2;
-constexpr int kBufCols = 128;                 // TMEM columns of a pass-2 accumulator buffer (pass 1 uses two of 256)
+constexpr int kPolyPairs = SPEC_POLY_PAIRS;
+// minimax quartic of 2^f on [-1/2, 1/2], from the lowest coefficient
+constexpr float kExpC0 = 0.9999992614f, kExpC1 = 0.6931218147f, kExpC2 = 0.2402474482f, kExpC3 = 0.0559178603f, kExpC4 = 0.0095701019f;
+constexpr int kBufCols = 128;                 // TMEM columns of an accumulator buffer, one per epilogue warpgroup
 constexpr int kTileKeys = 128;
 constexpr int kMaxStages = 8;
 constexpr int kMaxMTiles = 10;
@@ -136,6 +140,19 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return mbar_wait_slow(bar, parity, abort_flag);
 }
 
+// The same for a whole warp: every lane gets the same answer, and the branches that depend on it do not
+// diverge as far as the compiler can see.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+// True in exactly one lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e != 0;
+}
+__device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
@@ -159,18 +176,26 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
-// 32 consecutive fp32 columns of this thread's TMEM lane, complete on return (the load and
-// the wait for it are one statement, so no use of the registers can be scheduled in between).
+// 32 consecutive fp32 columns of this thread's TMEM lane; not to be read before tmem_wait.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-      "tcgen05.wait::ld.sync.aligned;"
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
         "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr) : "memory");
+}
+// Waits for this thread's TMEM loads.  The registers of the load go through the statement, so that
+// no use of them can be scheduled before it.
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+        "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+        "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+        "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+      :: "memory");
 }
 
 // Programmatic dependent launch: the next kernel on the stream may start; wait for the one before.
@@ -272,71 +297,90 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 __device__ __forceinline__ float2 ex2_mufu2(float2 x) {
   return make_float2(ex2(x.x), ex2(x.y));
 }
-// 2^x for both lanes without the MUFU unit: x = n + f with n = round(x), |f| <= 1/2 (adding
-// 1.5 * 2^23 leaves n in the low mantissa bits), 2^f by a cubic with relative error 7.5e-5,
-// then n is added into the exponent field.  x is clamped at -125 so the exponent cannot wrap.
-__device__ __forceinline__ float2 ex2_poly2(float2 x) {
-  x = make_float2(fmaxf(x.x, -125.f), fmaxf(x.y, -125.f));
-  const float2 xr = __fadd2_rn(x, splat2(12582912.f));
-  const float2 n = __fadd2_rn(xr, splat2(-12582912.f));
-  const float2 f = __ffma2_rn(n, splat2(-1.f), x);
-  float2 q = __ffma2_rn(f, splat2(0.0551713221f), splat2(0.2426105440f));
-  q = __ffma2_rn(q, f, splat2(0.6932609677f));
-  q = __ffma2_rn(q, f, splat2(0.9999281168f));
-  return make_float2(__uint_as_float(__float_as_uint(q.x) + (__float_as_uint(xr.x) << 23)),
-                     __uint_as_float(__float_as_uint(q.y) + (__float_as_uint(xr.y) << 23)));
+// 2^x for both lanes without the MUFU unit, x = s*a + c held in [-B, 128 - B]: in units of 128,
+// y = (x + B) / 128 is one multiply-add that saturates to [0, 1] for nothing, so that neither end of the
+// range needs a clamp of its own.  Adding 1.5 * 2^16 rounds y to a multiple of 1/128 and leaves
+// n = round(128 y) in the low mantissa bits; 2^f of the rest, |f| <= 1/2, is a quartic (relative
+// error 2.6e-6), and n goes into the exponent field.  a128 = a / 128, c128 = (c + B) / 128.
+template <int B>
+__device__ __forceinline__ float2 ex2_poly2(float s0, float s1, float a128, float2 c128) {
+  constexpr float k = B == 64 ? 5.421010862427522e-20f : 2.350988701644575e-38f;   // 2^-B
+  static_assert(B == 64 || B == 125, "the scale of the coefficients");
+  const float2 y = make_float2(__saturatef(fmaf(s0, a128, c128.x)), __saturatef(fmaf(s1, a128, c128.y)));
+  const float2 yr = __fadd2_rn(y, splat2(98304.f));
+  const float2 n = __fadd2_rn(yr, splat2(-98304.f));
+  const float2 f = __fadd2_rn(y, make_float2(-n.x, -n.y));
+  float2 q = __ffma2_rn(f, splat2(k * 268435456.f * kExpC4), splat2(k * 2097152.f * kExpC3));
+  q = __ffma2_rn(q, f, splat2(k * 16384.f * kExpC2));
+  q = __ffma2_rn(q, f, splat2(k * 128.f * kExpC1));
+  q = __ffma2_rn(q, f, splat2(k * kExpC0));
+  return make_float2(__uint_as_float(__float_as_uint(q.x) + (__float_as_uint(yr.x) << 23)),
+                     __uint_as_float(__float_as_uint(q.y) + (__float_as_uint(yr.y) << 23)));
 }
 // Pair i (0..15) of a 32-element block: NP of them, evenly spread, avoid the MUFU unit.
 template <int NP>
-__device__ __forceinline__ float2 ex2_pair(float2 x, int i) {
-  return (i * NP) / 16 != ((i + 1) * NP) / 16 ? ex2_poly2(x) : ex2_mufu2(x);
-}
+__host__ __device__ constexpr bool is_poly(int i) { return (i * NP) / 16 != ((i + 1) * NP) / 16; }
 
-// Pass 1: fold 32 logits of one row into the running (max, sum-exp), log2 domain.  At least one
-// of the 32 logits is valid.
-template <bool MASKED>
-__device__ __forceinline__ void stats_update(const uint32_t (&r)[32], int valid, float a, float& m, float& z) {
-  float v[32];
+// Pass 1: fold logits of one row into the running statistics (m, z): z sums 2^(a*s - m).  m is not the
+// running maximum but a reference, the maximum of the first block the row saw: fp32 holds sums of
+// terms up to 2^62 above it and loses nothing below it that a sum of at least 1 would show, so
+// the maximum (a third of an instruction per logit, and a chain in front of every exponential) is
+// only taken again by the rare row whose block exceeds the reference by 2^62.
+// The general form: only the first `valid` logits count, the reference becomes the maximum so far.
+__device__ __forceinline__ void stats_general(const uint32_t (&r)[32], int valid, float a, float& m, float& z) {
+  float g = -INFINITY;
 #pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    v[i] = __uint_as_float(r[i]);
-    if (MASKED && i >= valid) v[i] = -INFINITY;
-  }
-  float g[11];
+  for (int i = 0; i < 32; ++i)
+    if (i < valid) g = fmaxf(g, __uint_as_float(r[i]));
+  const float mn = fmaxf(m, g * a);                        // a > 0
+  if (!(mn > -INFINITY)) return;
+  float s = 0.f;
 #pragma unroll
-  for (int i = 0; i < 10; ++i) g[i] = max3(v[3 * i], v[3 * i + 1], v[3 * i + 2]);
-  g[10] = fmaxf(v[30], v[31]);
-  const float g0 = max3(g[0], g[1], g[2]), g1 = max3(g[3], g[4], g[5]), g2 = max3(g[6], g[7], g[8]);
-  const float gm = max3(max3(g0, g1, g2), g[9], g[10]);
-  const float mn = fmaxf(m, gm * a);                       // a > 0
-  z *= ex2(m - mn);                                        // first block: 0 * 2^-inf = 0
+  for (int i = 0; i < 32; ++i)
+    if (i < valid) s += ex2(fmaf(__uint_as_float(r[i]), a, -mn));
+  z = z * ex2(m - mn) + s;                                 // first block: 0 * 2^-inf = 0
   m = mn;
-  const float2 a2 = splat2(a), neg2 = splat2(-mn);
+}
+// 32 logits that all count.
+__device__ __forceinline__ void stats_update(const uint32_t (&r)[32], float a, float& m, float& z) {
+  const float2 a2 = splat2(a), neg2 = splat2(-m);
+  const float a128 = a * (1.f / 128.f);
+  const float2 c128 = splat2(fmaf(m, -1.f / 128.f, 0.5f));
   float2 s0 = splat2(0.f), s1 = splat2(0.f);
 #pragma unroll
-  for (int i = 0; i < 16; i += 2) {
-    s0 = __fadd2_rn(s0, ex2_pair<kPolyPairs1>(__ffma2_rn(make_float2(v[2 * i], v[2 * i + 1]), a2, neg2), i));
-    s1 = __fadd2_rn(s1, ex2_pair<kPolyPairs1>(__ffma2_rn(make_float2(v[2 * i + 2], v[2 * i + 3]), a2, neg2), i + 1));
+  for (int i = 0; i < 16; ++i) {
+    const float x0 = __uint_as_float(r[2 * i]), x1 = __uint_as_float(r[2 * i + 1]);
+    const float2 e = is_poly<kPolyPairs>(i) ? ex2_poly2<64>(x0, x1, a128, c128) : ex2_mufu2(__ffma2_rn(make_float2(x0, x1), a2, neg2));
+    if (i & 1) s1 = __fadd2_rn(s1, e); else s0 = __fadd2_rn(s0, e);
   }
-  z += (s0.x + s0.y) + (s1.x + s1.y);
+  const float s = (s0.x + s0.y) + (s1.x + s1.y);
+  if (s < 4.6e18f) z += s;                                 // 2^62; also false for the row's first block (m = -inf: infinite terms)
+  else stats_general(r, 32, a, m, z);
 }
 
 // Pass 2: probabilities of 32 query rows for this thread's key, reduced into acc (two packed
-// partial sums, or two packed maxima).
+// partial sums, or two packed maxima).  The row constants come in the form that each column's
+// exponential wants.
+__device__ __forceinline__ float row_const(int row, float negc) {
+  return is_poly<kPolyPairs>((row & 31) >> 1) ? (negc + 125.f) * (1.f / 128.f) : negc;
+}
 template <bool MAXRED>
-__device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const float* __restrict__ negc, float2 a2, float2 (&acc)[2]) {
-  const float4* c4 = reinterpret_cast<const float4*>(negc);
+__device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const float* __restrict__ rowc, float2 a2, float a128, float2 (&acc)[2]) {
+  const float4* c4 = reinterpret_cast<const float4*>(rowc);
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const float4 c = c4[i];
-    const float2 p0 = ex2_pair<kPolyPairs2>(__ffma2_rn(make_float2(__uint_as_float(r[4 * i + 0]), __uint_as_float(r[4 * i + 1])), a2, make_float2(c.x, c.y)), 2 * i);
-    const float2 p1 = ex2_pair<kPolyPairs2>(__ffma2_rn(make_float2(__uint_as_float(r[4 * i + 2]), __uint_as_float(r[4 * i + 3])), a2, make_float2(c.z, c.w)), 2 * i + 1);
-    if (MAXRED) {
-      acc[0].x = max3(acc[0].x, p0.x, p0.y);               // one maximum per chain: the four are merged at the end
-      acc[1].x = max3(acc[1].x, p1.x, p1.y);
-    } else {
-      acc[0] = __fadd2_rn(acc[0], p0);
-      acc[1] = __fadd2_rn(acc[1], p1);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const float x0 = __uint_as_float(r[4 * i + 2 * u]), x1 = __uint_as_float(r[4 * i + 2 * u + 1]);
+      const float2 cc = u == 0 ? make_float2(c.x, c.y) : make_float2(c.z, c.w);
+      const float2 e = is_poly<kPolyPairs>(2 * i + u) ? ex2_poly2<125>(x0, x1, a128, cc) : ex2_mufu2(__ffma2_rn(make_float2(x0, x1), a2, cc));
+      if (MAXRED) {
+        if (u == 0) acc[0].x = max3(acc[0].x, e.x, e.y);   // one maximum per chain: they are merged at the end
+        else acc[1].x = max3(acc[1].x, e.x, e.y);
+      } else {
+        acc[u] = __fadd2_rn(acc[u], e);
+      }
     }
   }
 }
@@ -346,12 +390,13 @@ __device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const f
 // is window row r < n_window and the key lies after the row's own position n - n_window + r.
 // Plain scalar code: only the last tile or two of a sequence come here.
 template <bool MAXRED>
-__device__ __forceinline__ void prob_accumulate_causal(const uint32_t (&r)[32], const float* __restrict__ negc, float a,
+__device__ __forceinline__ void prob_accumulate_causal(const uint32_t (&r)[32], const float* __restrict__ rowc, float a,
                                                        float2 (&acc)[2], int row0, int R, int n_window, int n, int key) {
   int rr = row0 % R;
 #pragma unroll
   for (int i = 0; i < 32; ++i) {
-    float pr = ex2(fmaf(__uint_as_float(r[i]), a, negc[i]));
+    const float negc = is_poly<kPolyPairs>(i >> 1) ? fmaf(rowc[i], 128.f, -125.f) : rowc[i];
+    float pr = ex2(fmaf(__uint_as_float(r[i]), a, negc));
     if (rr < n_window && key > max(n - n_window + rr, 0)) pr = 0.f;
     if (MAXRED) acc[0].x = fmaxf(acc[0].x, pr); else acc[0].x += pr;
     if (++rr == R) rr = 0;
@@ -371,7 +416,7 @@ __device__ __forceinline__ void fold_stats(float& m, float& z, float pm, float p
   m = mn;
 }
 
-__device__ __forceinline__ void row_constants(const ScoreParams& p, const float2* __restrict__ part, int n, int et, float* c_sm, float2* merge_sm) {
+__device__ __forceinline__ void row_constants(const ScoreParams& p, const float2* __restrict__ part, int n, int et, float scale_log2, float* c_sm, float2* merge_sm) {
   const int Mr = (p.M + 31) & ~31;
   const int slices = p.merge_slots > 0 ? p.merge_slots / Mr : 1;
   for (int i0 = 0; i0 < p.M_pad; i0 += kEpilogueThreads) {
@@ -413,10 +458,10 @@ __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2
       float c = -INFINITY;                                     // rows that pad the last tile weigh nothing
       if (i < p.M) {
         c = m + log2f(z);
-        if (p.row_weight) c -= log2f(p.row_weight[(p.row0 + i) % p.R]);
+        if (p.row_weight) c -= log2f(p.row_weight[(p.row0 + i) % p.R]) - scale_log2;
         c = -c;
       }
-      c_sm[i] = c;
+      c_sm[i] = row_const(i, c);
     }
     if (slices > 1) {                                          // the padding rows beyond the slices' reach
       for (int j = Mr + et; j < p.M_pad; j += kEpilogueThreads) c_sm[j] = -INFINITY;
@@ -433,7 +478,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int BUFCOLS = kBufCols;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   uint8_t* k_sm = smem;
   uint8_t* q_sm = smem + (size_t)p.n_stages * p.stage_bytes;
   float* c_sm = reinterpret_cast<float*>(q_sm + p.q_bytes);
@@ -448,6 +493,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   uint64_t* t_empty = t_full + 4;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kNumBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  float* scale_sm = reinterpret_cast<float*>(tmem_slot + 2);
 
   if ((smem_u32(smem) & 1023u) != 0) {      // the swizzled tiles need 1024-byte alignment
     if (tid == 0) report(p.status, SPEC_ERR_ALIGNMENT);
@@ -466,8 +512,6 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
   }
   if (tid == 32) {
-    // pass 1: one MMA thread, every buffer drained by all 16 epilogue warps;
-    // pass 2: two MMA threads release a stage, a buffer is drained by the 8 warps of one pair
     for (int i = 0; i < kMaxStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 2); }
     mbar_init(q_full, 1);
     mbar_init(q_empty, 2);
@@ -481,54 +525,59 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = (uint32_t)uniform((int)*tmem_slot);
   const int n_kh = p.d / 64;                               // 64-element halves of the contraction
   const uint32_t q_half_bytes = (uint32_t)p.M_pad * 128u;
   // K ring: [64-element half of the contraction][stage][128 keys x 128 bytes]
   const uint32_t k_half_bytes = (uint32_t)p.n_stages * (128u * 128u);
 
-  if (warp == 0) {
-    // ------------------------------------------------ TMA producer ----
-    if (lane == 0) {
-      SegIter it = seg_begin(p, tp, gridDim.x, blockIdx.x);
-      Seg sg;
-      uint32_t kit = 0, nseg = 0;
-      bool ok = true;
-      while (ok && seg_next(it, p, tp, sg)) {
-        if (nseg > 0) ok = mbar_wait(q_empty, (nseg - 1) & 1, abort_flag);   // previous unit's MMAs retired
-        if (!ok) break;
-        ++nseg;
-        mbar_expect_tx(q_full, p.q_bytes);
-        const int qrow0 = ((sg.s * p.L + sg.l) * p.Hq + sg.h * p.G) * p.R;
-        for (int kh = 0; kh < n_kh; ++kh)
-          for (int rb = 0; rb < p.M_pad / 128; ++rb)
-            tma_load_2d(q_sm + kh * q_half_bytes + rb * (128 * 128), &tm_q, kh * 64, qrow0 + p.row0 + rb * 128, q_full);
-        for (int t = 0; t < sg.nt; ++t, ++kit) {
-          const int stage = kit % p.n_stages;
-          const uint32_t par = (kit / p.n_stages) & 1;
-          ok = mbar_wait(&k_empty[stage], par ^ 1, abort_flag);
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIssueRegs));
+    if (warp == 0) {
+      // ------------------------------------------------ TMA producer ----
+      if (lane == 0) {
+        SegIter it = seg_begin(p, tp, gridDim.x, blockIdx.x);
+        Seg sg;
+        uint32_t kit = 0, nseg = 0;
+        bool ok = true;
+        while (ok && seg_next(it, p, tp, sg)) {
+          if (nseg > 0) ok = mbar_wait(q_empty, (nseg - 1) & 1, abort_flag);   // previous unit's MMAs retired
           if (!ok) break;
-          mbar_expect_tx(&k_full[stage], p.stage_bytes);
-          uint8_t* dst = k_sm + (size_t)stage * (128 * 128);
-          const int row = sg.begin + (sg.t0 + t) * kTileKeys;
+          ++nseg;
+          mbar_expect_tx(q_full, p.q_bytes);
+          const int qrow0 = ((sg.s * p.L + sg.l) * p.Hq + sg.h * p.G) * p.R;
           for (int kh = 0; kh < n_kh; ++kh)
-            tma_load_4d(dst + kh * k_half_bytes, &tm_k, kh * 64, row, sg.h, sg.l, &k_full[stage]);
+            for (int rb = 0; rb < p.M_pad / 128; ++rb)
+              tma_load_2d(q_sm + kh * q_half_bytes + rb * (128 * 128), &tm_q, kh * 64, qrow0 + p.row0 + rb * 128, q_full);
+          for (int t = 0; t < sg.nt; ++t, ++kit) {
+            const int stage = kit % p.n_stages;
+            const uint32_t par = (kit / p.n_stages) & 1;
+            ok = mbar_wait(&k_empty[stage], par ^ 1, abort_flag);
+            if (!ok) break;
+            mbar_expect_tx(&k_full[stage], p.stage_bytes);
+            uint8_t* dst = k_sm + (size_t)stage * (128 * 128);
+            const int row = sg.begin + (sg.t0 + t) * kTileKeys;
+            for (int kh = 0; kh < n_kh; ++kh)
+              tma_load_4d(dst + kh * k_half_bytes, &tm_k, kh * 64, row, sg.h, sg.l, &k_full[stage]);
+          }
         }
       }
-    }
-  } else if (warp == 1 || warp == kMmaWarpB) {
-    // ------------------------------------------------ MMA issuers -----
-    // Two issuing threads, one per warpgroup pair.  An issuing thread is a serial chain of
-    // barrier waits and tcgen05.mma instructions (each holds the thread for about 60 cycles),
-    // so one thread alone leaves the tensor pipe idle for more than half of the time.  Thread s
-    // feeds pair s only: the buffers 2s and 2s + 1 of that pair's two warpgroups.  Both threads
-    // wait for every key tile and commit to its "empty" barrier, whether or not they used it,
-    // so that every phase of those barriers sees exactly two arrivals.
-    if (lane == 0) {
-      const int strm = warp == 1 ? 0 : 1;
+    } else if (warp <= 2) {
+      // ------------------------------------------------ MMA issuers -----
+      // Two issuing warps, one per warpgroup pair: warp s feeds the buffers of that pair's two
+      // warpgroups.  Both wait for every key tile and commit to its "empty" barrier, whether or not
+      // they used it, so that every phase of those barriers sees exactly two arrivals.
+      // The whole warp runs the loops, and one elected lane issues: in converged code the descriptors stay in
+      // the uniform registers that tcgen05.mma reads them from.  Issued from a branch that one lane had
+      // taken, the eight instructions of an item took 1400 cycles among the epilogue warps (512 on the
+      // tensor pipe), and the epilogue waited for them; this form takes 1000 with the pipe shared by two.  A
+      // single issuing warp for all four buffers was slower (32 layers at 16K: 1.02 against 0.98 ms).
+      const int strm = warp - 1;
       SegIter it = seg_begin(p, tp, gridDim.x, blockIdx.x);
       Seg sg;
-      uint32_t kit = 0, nseg = 0;
+      uint32_t nseg = 0, uses0 = 0, uses1 = 0;                 // segments; items issued into each of my pair's two buffers
+      int stage = 0;
+      uint32_t k_par = 0;
       bool ok = true;
       const uint32_t idesc_full = make_idesc(128);
       const uint32_t idesc_last = make_idesc(PASS == 1 ? 128 : p.cw_last);
@@ -536,18 +585,19 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       const uint32_t q_lo0 = desc_lo(smem_u32(q_sm)), k_lo0 = desc_lo(smem_u32(k_sm));
       const uint32_t q_half16 = q_half_bytes >> 4;
       const uint32_t k_half16 = k_half_bytes >> 4;
-      uint32_t uses[2] = {0u, 0u};                            // items issued into each of my pair's two buffers
-      while (ok && seg_next(it, p, tp, sg)) {
-        ok = mbar_wait(q_full, nseg & 1, abort_flag);
+      while (ok) {
+        const bool more = seg_next(it, p, tp, sg);
+        const int nt = uniform(more ? sg.nt : 0);
+        if (nt == 0) break;
+        ok = mbar_wait_warp(q_full, nseg & 1, abort_flag);
         if (!ok) break;
         ++nseg;
         tc_fence_after();
         // A key tile belongs to the pair with the parity of its index in the segment; within the
         // pair, sub-item `sub` (a block of 128 query rows) of the pair's k-th tile goes to the
         // warpgroup (sub + k) & 1, whose private 128-column buffer receives it.
-        for (int t = 0; t < sg.nt && ok; ++t, ++kit) {
-          const int stage = kit % p.n_stages;
-          ok = mbar_wait(&k_full[stage], (kit / p.n_stages) & 1, abort_flag);
+        for (int t = 0; t < nt && ok; ++t) {
+          ok = mbar_wait_warp(&k_full[stage], k_par, abort_flag);
           if (!ok) break;
           tc_fence_after();
           const uint32_t k_lo = k_lo0 + stage * ((128 * 128) >> 4);
@@ -555,44 +605,51 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             for (int sub = 0; sub < n_sub; ++sub) {
               const int h = (sub + (t >> 1)) & 1;
               const int buf = strm * 2 + h;
-              ok = mbar_wait(&t_empty[buf], (uses[h] & 1) ^ 1, abort_flag);
+              ok = mbar_wait_warp(&t_empty[buf], ((h ? uses1 : uses0) & 1) ^ 1, abort_flag);
               if (!ok) break;
-              ++uses[h];
+              if (h) ++uses1; else ++uses0;
               tc_fence_after();
               const uint32_t d_tmem = tmem_base + buf * BUFCOLS;
               const uint32_t q_lo = q_lo0 + sub * ((128 * 128) >> 4);
               const uint32_t idesc = (PASS == 2 && sub == n_sub - 1) ? idesc_last : idesc_full;
+              if (elect_one()) {
 #pragma unroll
-              for (int kh = 0; kh < 2; ++kh) {
-                if (kh < n_kh) {
+                for (int kh = 0; kh < 2; ++kh) {
+                  if (kh < n_kh) {
 #pragma unroll
-                  for (int ks = 0; ks < 4; ++ks) {
-                    if (PASS == 1) tc_mma(d_tmem, desc_at(q_lo + kh * q_half16 + ks * 2), desc_at(k_lo + kh * k_half16 + ks * 2), idesc, (kh | ks) != 0);
-                    else tc_mma(d_tmem, desc_at(k_lo + kh * k_half16 + ks * 2), desc_at(q_lo + kh * q_half16 + ks * 2), idesc, (kh | ks) != 0);
+                    for (int ks = 0; ks < 4; ++ks) {
+                      if (PASS == 1) tc_mma(d_tmem, desc_at(q_lo + kh * q_half16 + ks * 2), desc_at(k_lo + kh * k_half16 + ks * 2), idesc, (kh | ks) != 0);
+                      else tc_mma(d_tmem, desc_at(k_lo + kh * k_half16 + ks * 2), desc_at(q_lo + kh * q_half16 + ks * 2), idesc, (kh | ks) != 0);
+                    }
                   }
                 }
+                tc_commit(&t_full[buf]);
               }
-              tc_commit(&t_full[buf]);
+              __syncwarp();
             }
           }
-          if (ok) tc_commit(&k_empty[stage]);      // arrives once my MMAs on this stage (if any) retire
+          if (ok && elect_one()) tc_commit(&k_empty[stage]);      // arrives once my MMAs on this stage (if any) retire
+          __syncwarp();
+          if (++stage == p.n_stages) { stage = 0; k_par ^= 1; }
         }
-        if (ok) tc_commit(q_empty);
+        if (ok && elect_one()) tc_commit(q_empty);
+        __syncwarp();
       }
     }
-  } else if (warp < kMmaWarpB) {
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpilogueRegs));
     // ------------------------------------------------ epilogue --------
-    const int wg = (warp - 2) >> 2;                        // warpgroup 0..3
+    const int wg = (warp - 4) >> 2;                        // warpgroup 0..3
     const int pair = wg >> 1;                              // pairs take alternate key tiles
     const int half = wg & 1;                               // column half of the pair's buffer
     const int quarter = warp & 3;                          // TMEM lane quarter this warp may read
     const int row_in_tile = quarter * 32 + lane;
-    const int et = tid - 64;                               // 0..511 among epilogue threads
+    const int et = tid - 128;                              // 0..511 among epilogue threads
     const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
     SegIter it = seg_begin(p, tp, gridDim.x, blockIdx.x);
     Seg sg;
     bool ok = true;
-    uint32_t ra[32];
+    uint32_t ra[32], rb[32];
     uint32_t used = 0;                                       // items drained from my warpgroup's buffer
     const uint32_t my_taddr = lane_base + wg * BUFCOLS;
     if (PASS == 1) {
@@ -629,17 +686,23 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             tc_fence_after();
             float m = mrun[mt], z = zrun[mt];
             if (plain) {
-              // every row sees all 128 keys: no masks, no per-row arithmetic
+              // Every row sees all 128 keys: no masks, no per-row arithmetic.  The next block of columns is on its way
+              // while one is worked on; the last two are both in registers when the buffer is given
+              // back, whose refill takes about as long as their arithmetic.
               tmem_ld32(my_taddr, ra);
-              stats_update<false>(ra, 32, p.a, m, z);
-              tmem_ld32(my_taddr + 32, ra);
-              stats_update<false>(ra, 32, p.a, m, z);
+              tmem_wait(ra);
+              tmem_ld32(my_taddr + 32, rb);
+              stats_update(ra, p.a, m, z);
+              tmem_wait(rb);
               tmem_ld32(my_taddr + 64, ra);
-              stats_update<false>(ra, 32, p.a, m, z);
-              tmem_ld32(my_taddr + 96, ra);
+              stats_update(rb, p.a, m, z);
+              tmem_ld32(my_taddr + 96, rb);
+              tmem_wait(ra);
+              tmem_wait(rb);
               tc_fence_before();
-              arrive_lane0(&t_empty[wg], lane);               // all reads done: the buffer can be refilled
-              stats_update<false>(ra, 32, p.a, m, z);
+              arrive_lane0(&t_empty[wg], lane);
+              stats_update(ra, p.a, m, z);
+              stats_update(rb, p.a, m, z);
             } else {
               int vis = nv;                                    // keys of the tile that this thread's row may see
               if (in_window) {
@@ -650,7 +713,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               for (int c = 0; c < 4; ++c) {
                 if (c * 32 >= nv) break;                                    // warp-uniform
                 tmem_ld32(my_taddr + c * 32, ra);
-                if (vis - c * 32 > 0) stats_update<true>(ra, min(vis - c * 32, 32), p.a, m, z);
+                tmem_wait(ra);
+                if (vis - c * 32 > 0) stats_general(ra, min(vis - c * 32, 32), p.a, m, z);
               }
               tc_fence_before();
               arrive_lane0(&t_empty[wg], lane);
@@ -674,7 +738,19 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       // Work item = one key tile (keys on lanes) x one chunk of 128 query rows, all of it mine; the
       // chunks of a tile alternate between the two warpgroups of the pair.
       const float2 a2 = splat2(p.a);
+      const float a128 = p.a * (1.f / 128.f);
       const long long per_cta = it.per_cta;
+      // Weighted probabilities above 8 would leave the range of the polynomial exponential: with larger weights
+      // everything is scaled down by a power of two, and the scores up again as they are written.
+      float scale_log2 = 0.f;
+      if (p.row_weight) {
+        float w = 0.f;
+        for (int i = lane; i < p.R; i += 32) w = fmaxf(w, __ldg(p.row_weight + i));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) w = fmaxf(w, __shfl_xor_sync(0xffffffffu, w, o));
+        scale_log2 = fminf(fmaxf(floorf(log2f(w)) - 1.f, 0.f), 126.f);
+      }
+      if (et == 0) *scale_sm = exp2f(scale_log2);               // read after the barriers below
       wait_for_previous_grid();                                 // pass 1: statistics and zeroed scores
       launch_dependents();
       // Every epilogue thread passes the barriers of every segment, also after a wait has
@@ -687,7 +763,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const int n_tiles = tp[sg.s + 1] - tp[sg.s];
           const int b0 = (int)(u0 / per_cta), b1 = (int)((u0 + n_tiles - 1) / per_cta);
           row_constants(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
-                        (b1 - b0 + 1) * kEpilogueWarpgroups, et, c_sm, merge_sm);
+                        (b1 - b0 + 1) * kEpilogueWarpgroups, et, scale_log2, c_sm, merge_sm);
         }
         asm volatile("bar.sync 1, 512;" ::: "memory");
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
@@ -703,29 +779,48 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             any = true;
             tc_fence_after();
             const int cw = ch == p.n_chunks - 1 ? p.cw_last : 128;            // my columns: 64 or 128
-            const float* negc = c_sm + ch * 128;
+            const float* rowc = c_sm + ch * 128;
             const int row0 = p.row0 + ch * 128;                 // query row of my first column
-            const int nb = cw >> 5;                             // blocks of 32 columns: 2 or 4
+            if (in_window) {
 #pragma unroll 1
-            for (int c = 0; c < nb; ++c) {
-              tmem_ld32(my_taddr + c * 32, ra);
-              if (c == nb - 1) {
-                tc_fence_before();
-                arrive_lane0(&t_empty[wg], lane);
+              for (int c = 0; c < cw; c += 32) {
+                tmem_ld32(my_taddr + c, ra);
+                tmem_wait(ra);
+                prob_accumulate_causal<MAXRED>(ra, rowc + c, p.a, acc, row0 + c, p.R, p.n_window, sg.n, key);
               }
-              if (!in_window) prob_accumulate<MAXRED>(ra, negc + c * 32, a2, acc);
-              else prob_accumulate_causal<MAXRED>(ra, negc + c * 32, p.a, acc, row0 + c * 32, p.R, p.n_window, sg.n, key);
+              tc_fence_before();
+              arrive_lane0(&t_empty[wg], lane);
+              continue;
             }
+            tmem_ld32(my_taddr, ra);                            // look-ahead as in pass 1
+            if (cw == 128) {
+              tmem_wait(ra);
+              tmem_ld32(my_taddr + 32, rb);
+              prob_accumulate<MAXRED>(ra, rowc, a2, a128, acc);
+              tmem_wait(rb);
+              tmem_ld32(my_taddr + 64, ra);
+              prob_accumulate<MAXRED>(rb, rowc + 32, a2, a128, acc);
+              rowc += 64;
+              tmem_ld32(my_taddr + 96, rb);
+            } else {
+              tmem_ld32(my_taddr + 32, rb);
+            }
+            tmem_wait(ra);
+            tmem_wait(rb);
+            tc_fence_before();
+            arrive_lane0(&t_empty[wg], lane);
+            prob_accumulate<MAXRED>(ra, rowc, a2, a128, acc);
+            prob_accumulate<MAXRED>(rb, rowc + 32, a2, a128, acc);
           }
           if (!ok) break;
           if (any && key < sg.n) {
             // The output was zero-filled; the two warpgroups of the pair contribute once per key.
             const float v0 = acc[0].x, v1 = acc[0].y, v2 = acc[1].x, v3 = acc[1].y;
             if (MAXRED) {
-              const float v = fmaxf(fmaxf(v0, v1), fmaxf(v2, v3));
+              const float v = fmaxf(fmaxf(v0, v1), fmaxf(v2, v3)) * *scale_sm;
               asm volatile("red.global.max.u32 [%0], %1;" ::"l"(out + key), "r"(__float_as_uint(v)) : "memory");
             } else {
-              const float v = (v0 + v1) + (v2 + v3);
+              const float v = ((v0 + v1) + (v2 + v3)) * *scale_sm;
               asm volatile("red.global.add.f32 [%0], %1;" ::"l"(out + key), "f"(v) : "memory");
             }
           }
@@ -858,6 +953,14 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
       SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
       SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
       SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+      // The warpgroups divide the registers that the block was launched with: a build that launches with fewer
+      // would wait for registers that do not exist.
+      const void* fns[3] = {(const void*)score_kernel<1, false>, (const void*)score_kernel<2, false>, (const void*)score_kernel<2, true>};
+      for (const void* f : fns) {
+        cudaFuncAttributes at;
+        SPEC_CUDA_OK(cudaFuncGetAttributes(&at, f));
+        if (at.numRegs < kLaunchRegs) return fail(SPEC_ERR_UNSUPPORTED, "the scoring kernel was built with %d registers per thread, %d needed", at.numRegs, kLaunchRegs);
+      }
       __atomic_store_n(&set[dev], 1, __ATOMIC_RELEASE);
     }
   }

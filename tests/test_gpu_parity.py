@@ -115,6 +115,28 @@ def test_score_max_reduce_and_row_weights(B, W, oracle):
         assert_scores_close(got, ref, g.cu)
 
 
+@pytest.mark.parametrize("reduce", [0, 1])
+@pytest.mark.parametrize("case", ["large_weights", "rising_logits", "falling_logits", "steep_logits"])
+def test_score_range_of_the_exponentials(B, W, oracle, case, reduce):
+    """Row weights beyond the range of the polynomial exponential, and rows whose later logits lie far above or
+    below the reference that the first block of keys gave (beyond 2^62 for the rising and the steep ones)."""
+    w = small(W, n_in=1500, zipf_bias=False, planted="singletons", n_planted=0)
+    g = Gpu(B, W, w, [0])
+    rw = None
+    if case == "large_weights":
+        rw = torch.logspace(-3, 4, w.rows)
+    else:
+        # the last feature as a bias on the natural-log logits: -80 .. 80 over the sequence, or jumps of 120
+        bias = {"rising_logits": torch.linspace(-80, 80, w.n_in), "falling_logits": torch.linspace(80, -80, w.n_in),
+                "steep_logits": torch.where(torch.arange(w.n_in) % 700 > 690, 120.0, 0.0)}[case]
+        g.q[..., -1] = w.head_dim ** 0.5
+        g.k[..., -1] = bias.to(g.k)
+    got = g.score(reduce=reduce, row_weight=None if rw is None else rw.cuda()).cpu().numpy()
+    ref = oracle.spec_score(bits(g.q), bits(g.k), g.cu, w.n_lookahead, w.n_window, w.scale, mode=reduce,
+                            row_weight=None if rw is None else rw.double().numpy())
+    assert_scores_close(got, ref, g.cu)
+
+
 def test_score_causal_window(B, W, oracle):
     """Window row r sees keys up to its own prompt position only (the model's causal mask)."""
     cases = [small(W, n_in=600), small(W, n_in=257, n_window=40, n_lookahead=3),
