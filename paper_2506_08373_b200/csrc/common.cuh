@@ -73,6 +73,10 @@ SPEC_HIDDEN inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// Programmatic dependent launch: the next kernel on the stream may start; wait for the one before.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Token range of sequence s.
 __device__ __forceinline__ void seq_range(const int32_t* cu, int n_in, int s, int& begin, int& n) {
   if (cu) {

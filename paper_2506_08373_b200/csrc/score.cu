@@ -198,10 +198,6 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&r)[32]) {
       :: "memory");
 }
 
-// Programmatic dependent launch: the next kernel on the stream may start; wait for the one before.
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
