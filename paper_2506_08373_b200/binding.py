@@ -75,11 +75,18 @@ def lib() -> ctypes.CDLL:
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# The current stream's handle as a number: torch.cuda.current_stream() builds a Stream object around it, which took
+# 3.3 us of the 10 to 16 us of host time of a call (0.3 us this way).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
 
 
 def _check(rc: int):
@@ -125,20 +132,20 @@ def spec_last_error() -> str:
 def spec_score(problem, q, k, scores_out, workspace, row_weight=None, reduce=REDUCE_SUM, causal_window=0,
                status_word=None):
     _check(lib().spec_score(ctypes.byref(problem), _ptr(q), _ptr(k), _ptr(row_weight), reduce, causal_window,
-                            _ptr(scores_out), _ptr(workspace), workspace.numel() * workspace.element_size(),
+                            _ptr(scores_out), _ptr(workspace), workspace.nbytes,
                             _ptr(status_word), _stream()))
 
 
 def spec_pool_topk(problem, scores, pool, pool_k, c_max, n_forced_tail, idx_out, count_out=None,
                    workspace=None, status_word=None):
-    wsb = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    wsb = 0 if workspace is None else workspace.nbytes
     _check(lib().spec_pool_topk(ctypes.byref(problem), _ptr(scores), pool, pool_k, c_max, n_forced_tail,
                                 _ptr(idx_out), _ptr(count_out), _ptr(workspace), wsb, _ptr(status_word), _stream()))
 
 
 def spec_pool_topk_vert(problem, scores, pool, pool_k, c_max, n_forced_tail, idx_out, count_out, n_vert,
                         vert_idx_out, vert_count_out=None, workspace=None, status_word=None):
-    wsb = 0 if workspace is None else workspace.numel() * workspace.element_size()
+    wsb = 0 if workspace is None else workspace.nbytes
     _check(lib().spec_pool_topk_vert(ctypes.byref(problem), _ptr(scores), pool, pool_k, c_max, n_forced_tail,
                                      _ptr(idx_out), _ptr(count_out), n_vert, _ptr(vert_idx_out), _ptr(vert_count_out),
                                      _ptr(workspace), wsb, _ptr(status_word), _stream()))
@@ -154,7 +161,7 @@ def specpc_token_select(problem, scores, layer_head_reduce, pool, pool_k, c_max,
                         keep_out, keep_capacity, n_keep_out, workspace, status_word=None):
     _check(lib().specpc_token_select(ctypes.byref(problem), _ptr(scores), layer_head_reduce, pool, pool_k, c_max,
                                      n_neighbor, n_forced_tail, _ptr(keep_out), keep_capacity, _ptr(n_keep_out),
-                                     _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                     _ptr(workspace), workspace.nbytes,
                                      _ptr(status_word), _stream()))
 
 

@@ -110,8 +110,6 @@ __global__ void __launch_bounds__(kBulkThreads) compact_bulk_kernel(CompactParam
   const int h = unit % p.H;
   const int l = (unit / p.H) % p.L;
   const int s = unit / (p.H * p.L);
-  int begin, n;
-  seq_range(p.cu, p.n_in, s, begin, n);
   const int tid = threadIdx.x;
   const int c0 = rb * kBulkRows;
   const int n_rows = min(kBulkRows, p.c_max - c0);
@@ -121,6 +119,10 @@ __global__ void __launch_bounds__(kBulkThreads) compact_bulk_kernel(CompactParam
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
+  wait_for_previous_grid();                                // the index lists; whatever fills or reads the caches
+  launch_dependents();
+  int begin, n;
+  seq_range(p.cu, p.n_in, s, begin, n);
   uint8_t* k_sm = rows_sm;
   uint8_t* v_sm = rows_sm + (size_t)kBulkRows * row_bytes;
   int64_t page_dst = -1;                                   // paged: element offset of my row in the pools
@@ -332,8 +334,8 @@ SPEC_EXPORT int32_t spec_compact_kv(const spec_problem* pr, const void* k, const
         __atomic_store_n(&set[dev], 1, __ATOMIC_RELEASE);
       }
     }
-    if (v) compact_bulk_kernel<true><<<(unsigned)bulk_blocks, kBulkThreads, smem, st>>>(p, row_bytes);
-    else   compact_bulk_kernel<false><<<(unsigned)bulk_blocks, kBulkThreads, smem, st>>>(p, row_bytes);
+    if (v) SPEC_CUDA_OK(launch_dependent(compact_bulk_kernel<true>, dim3((unsigned)bulk_blocks), kBulkThreads, smem, st, p, row_bytes));
+    else   SPEC_CUDA_OK(launch_dependent(compact_bulk_kernel<false>, dim3((unsigned)bulk_blocks), kBulkThreads, smem, st, p, row_bytes));
   } else if (v) {
     if (d128) compact_kernel<16, true><<<(unsigned)blocks, kCompactThreads, 0, st>>>(p);
     else      compact_kernel<8, true><<<(unsigned)blocks, kCompactThreads, 0, st>>>(p);

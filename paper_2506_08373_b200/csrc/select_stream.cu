@@ -389,52 +389,37 @@ __device__ __forceinline__ WarpCandidates find_candidates(const UnitGeom& g, con
 }
 
 // Calls put(rank, key, position) for every candidate of the warp, rank in position order from `base` on.
+// Every lane walks its own nibbles, most lanes none and few more than one, and reads the twelve scores
+// around each again from L2: a step-by-step walk of the whole warp over its registers (18 shuffles a step)
+// was three times the instructions.
 template <class Put>
 __device__ __forceinline__ void pool_candidates(const UnitGeom& g, const WarpScores& w, const WarpCandidates& c, int base, int lane, Put put) {
-  if (c.total == 0) return;                                // warp-uniform
-#pragma unroll
-  for (int k = 0; k < kWarpSteps; ++k) {
-    const int in_step = (int)(((k & 1 ? c.tot_odd : c.tot_even) >> (8 * (k >> 1))) & 255u);
-    if (in_step == 0) continue;                            // warp-uniform
-    const float4 v = w.v[k];
-    float x[10];
-    x[0] = __shfl_up_sync(0xffffffffu, v.y, 1);
-    x[1] = __shfl_up_sync(0xffffffffu, v.z, 1);
-    x[2] = __shfl_up_sync(0xffffffffu, v.w, 1);
-    x[3] = v.x; x[4] = v.y; x[5] = v.z; x[6] = v.w;
-    x[7] = __shfl_down_sync(0xffffffffu, v.x, 1);
-    x[8] = __shfl_down_sync(0xffffffffu, v.y, 1);
-    x[9] = __shfl_down_sync(0xffffffffu, v.z, 1);
-    float b0, b1, b2, a0 = __shfl_sync(0xffffffffu, w.after, 0), a1 = __shfl_sync(0xffffffffu, w.after, 1), a2 = __shfl_sync(0xffffffffu, w.after, 2);
-    if (k > 0) {
-      b0 = __shfl_sync(0xffffffffu, w.v[k > 0 ? k - 1 : 0].y, 31);
-      b1 = __shfl_sync(0xffffffffu, w.v[k > 0 ? k - 1 : 0].z, 31);
-      b2 = __shfl_sync(0xffffffffu, w.v[k > 0 ? k - 1 : 0].w, 31);
+  uint32_t left = c.mask;
+  while (left) {
+    const int k = (__ffs((int)left) - 1) >> 2;
+    const uint32_t nib = (left >> (4 * k)) & 15u;
+    left &= ~(15u << (4 * k));
+    const int x0 = w.x0 + k * 128 + lane * 4;
+    float4 pv, cv, nv;
+    if (x0 - 4 >= g.mis && x0 + 8 <= g.X) {
+      const float4* at = reinterpret_cast<const float4*>(g.src + (x0 - g.mis));
+      pv = __ldcg(at - 1); cv = __ldcg(at); nv = __ldcg(at + 1);
     } else {
-      b0 = __shfl_sync(0xffffffffu, w.before, 0);
-      b1 = __shfl_sync(0xffffffffu, w.before, 1);
-      b2 = __shfl_sync(0xffffffffu, w.before, 2);
+      pv = make_float4(0.f, score_at(g, x0 - 3), score_at(g, x0 - 2), score_at(g, x0 - 1));
+      cv = make_float4(score_at(g, x0), score_at(g, x0 + 1), score_at(g, x0 + 2), score_at(g, x0 + 3));
+      nv = make_float4(score_at(g, x0 + 4), score_at(g, x0 + 5), score_at(g, x0 + 6), 0.f);
     }
-    if (k + 1 < w.n_steps) {
-      const float4 nx = w.v[k + 1 < kWarpSteps ? k + 1 : k];
-      a0 = __shfl_sync(0xffffffffu, nx.x, 0);
-      a1 = __shfl_sync(0xffffffffu, nx.y, 0);
-      a2 = __shfl_sync(0xffffffffu, nx.z, 0);
-    }
-    if (lane == 0) { x[0] = b0; x[1] = b1; x[2] = b2; }
-    if (lane == 31) { x[7] = a0; x[8] = a1; x[9] = a2; }
-    const uint32_t nib = (c.mask >> (4 * k)) & 15u;
-    if (nib) {
-      // the four windows share x[3..6]; neighbouring windows share a pair on either side
-      const float mid = fmax3(x[3], x[4], fmaxf(x[5], x[6])), l12 = fmaxf(x[1], x[2]), r78 = fmaxf(x[7], x[8]);
-      const float v4[4] = {fmax3(mid, x[0], l12), fmax3(mid, l12, x[7]), fmax3(mid, x[2], r78), fmax3(mid, r78, x[9])};
-      int at = base + (int)(((k & 1 ? c.pre_odd : c.pre_even) >> (8 * (k >> 1))) & 255u);
-      const int j0 = w.x0 + k * 128 + lane * 4 - g.mis;
+    // candidates of earlier steps (even steps below k: (k + 1) / 2 of them, odd ones: k / 2), of lower lanes in this one
+    const uint32_t in_even = (uint32_t)((1ull << (8 * ((k + 1) >> 1))) - 1ull), in_odd = (uint32_t)((1ull << (8 * (k >> 1))) - 1ull);
+    int at = base + (int)__dp4a(c.tot_even & in_even, 0x01010101u, __dp4a(c.tot_odd & in_odd, 0x01010101u, 0u)) +
+             (int)(((k & 1 ? c.pre_odd : c.pre_even) >> (8 * (k >> 1))) & 255u);
+    // the four windows share the middle four; neighbouring windows share a pair on either side
+    const float mid = fmax3(cv.x, cv.y, fmaxf(cv.z, cv.w)), l12 = fmaxf(pv.z, pv.w), r78 = fmaxf(nv.x, nv.y);
+    const float v4[4] = {fmax3(mid, pv.y, l12), fmax3(mid, l12, nv.x), fmax3(mid, pv.w, r78), fmax3(mid, r78, nv.z)};
+    const int j0 = x0 - g.mis;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (nib & (1u << u)) { put(at, to_key(v4[u]), j0 + u); ++at; }
-    }
-    base += in_step;
+    for (int u = 0; u < 4; ++u)
+      if (nib & (1u << u)) { put(at, to_key(v4[u]), j0 + u); ++at; }
   }
 }
 
@@ -495,7 +480,7 @@ __global__ void __launch_bounds__(kSelThreads) sample_floor_kernel(const StreamP
 // ---------------------------------------------------------------- 2. the sweep -------
 
 #ifndef SPEC_SWEEP_CTAS
-#define SPEC_SWEEP_CTAS 6
+#define SPEC_SWEEP_CTAS 8
 #endif
 constexpr int kSweepThreads = 128;
 constexpr int kSweepWarps = kSweepThreads / 32;
