@@ -412,6 +412,8 @@ __device__ __forceinline__ void fold_stats(float& m, float& z, float pm, float p
   m = mn;
 }
 
+constexpr int kMergeLoads = 16;       // in flight per thread; with 8, one layer of 12K (72 partials per row) spent 8 us here
+
 __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2* __restrict__ part, int n, int et, float scale_log2, float* c_sm, float2* merge_sm) {
   const int Mr = (p.M + 31) & ~31;
   const int slices = p.merge_slots > 0 ? p.merge_slots / Mr : 1;
@@ -420,24 +422,22 @@ __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2
     const int i = slices > 1 ? et - sl * Mr : i0 + et;
     float m = -INFINITY, z = 0.f;
     if (i < p.M && sl < slices) {
-      int c = sl;
-      for (; c + 7 * slices < n; c += 8 * slices) {           // eight loads in flight
-        float2 v[8];
+      for (int c0 = sl; c0 < n; c0 += kMergeLoads * slices) {
+        float2 v[kMergeLoads];
         float mx = m;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = __ldcg(part + (size_t)(c + u * slices) * p.M + i);
+        for (int u = 0; u < kMergeLoads; ++u) {
+          const int c = c0 + u * slices;
+          v[u] = c < n ? __ldcg(part + (size_t)c * p.M + i) : make_float2(-INFINITY, 0.f);
+        }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) mx = fmaxf(mx, v[u].x);
+        for (int u = 0; u < kMergeLoads; ++u) mx = fmaxf(mx, v[u].x);
         if (mx > -INFINITY) {
           z *= exp2f(m - mx);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) z += v[u].y * exp2f(v[u].x - mx);
+          for (int u = 0; u < kMergeLoads; ++u) z += v[u].y * exp2f(v[u].x - mx);
         }
         m = mx;
-      }
-      for (; c < n; c += slices) {
-        const float2 v = __ldcg(part + (size_t)c * p.M + i);
-        fold_stats(m, z, v.x, v.y);
       }
     }
     if (slices > 1) {
@@ -495,15 +495,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     if (tid == 0) report(p.status, SPEC_ERR_ALIGNMENT);
     return;
   }
-  // Pass 1 may be launched while whatever fills its inputs still runs; pass 2 while pass 1 still does, but
-  // every CTA of pass 1 is past its wait by then, so that only what pass 1 writes has to be waited for (below).
-  if (PASS == 1) {
-    wait_for_previous_grid();
-    launch_dependents();
-  }
   if (tid == 0) {
     *abort_flag = 0;
-    build_tile_prefix(p, tp);
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_q) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
   }
@@ -518,6 +511,13 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  // Pass 1 may be launched while whatever fills its inputs still runs; pass 2 while pass 1 still does, but
+  // every CTA of pass 1 is past its wait by then, so that only what pass 1 writes has to be waited for (below).
+  if (PASS == 1) {
+    wait_for_previous_grid();
+    launch_dependents();
+  }
+  if (tid == 0) build_tile_prefix(p, tp);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
