@@ -60,6 +60,7 @@ constexpr float kExpC0 = 0.9999992614f, kExpC1 = 0.6931218147f, kExpC2 = 0.24024
 constexpr int kBufCols = 128;                 // TMEM columns of an accumulator buffer, one per epilogue warpgroup
 constexpr int kTileKeys = 128;
 constexpr int kMaxStages = 8;
+constexpr int kRemMinTiles = 16;              // key tiles per CTA from which remaining rows are scored on columns
 constexpr int kMaxMTiles = 10;
 constexpr int kNumBars = 2 * kMaxStages + 2 + 8;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
@@ -79,7 +80,8 @@ struct ScoreParams {
   int row0;
   int causal, n_window;  // causal != 0: window row r sees keys up to position n - n_window + r only
   int merge_slots;       // threads that share the merging of a unit's statistics when there are fewer rows than threads (0: none do)
-  int n_stages, n_chunks, cw_last;   // pass 2: chunks of 128 query rows, the last of cw_last (64 or 128)
+  int n_stages, n_chunks, cw_last;   // pass 2: chunks of 128 query rows, the last of cw_last (a multiple of 16)
+  int n_full, rem_cols;  // pass 1: blocks of 128 query rows on lanes, and 16..48 remaining rows on columns (0: none)
   int reduce;
   float a;              // softmax_scale * log2(e)
   uint32_t q_bytes, stage_bytes;
@@ -176,7 +178,7 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
-// 32 consecutive fp32 columns of this thread's TMEM lane; not to be read before tmem_wait.
+// 32 (16) consecutive fp32 columns of this thread's TMEM lane; not to be read before tmem_wait.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -185,6 +187,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
         "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 }
 // Waits for this thread's TMEM loads.  The registers of the load go through the statement, so that
@@ -354,17 +363,98 @@ __device__ __forceinline__ void stats_update(const uint32_t (&r)[32], float a, f
   else stats_general(r, 32, a, m, z);
 }
 
-// Pass 2: probabilities of 32 query rows for this thread's key, reduced into acc (two packed
+// Pass 1, the rows that remain behind the last full block of 128: up to 48 of them would leave most lanes of
+// a block idle, so they are scored the other way round, keys on lanes and rows on columns, and the
+// sums over the lanes are taken by a butterfly that halves the columns at every step: lane l ends up
+// with column l of a 32-column block (of 16 columns: l & 15).  With the butterfly a block of 32 costs
+// about 0.4 of a block of 128 lanes, one of 16 about 0.2.
+template <int COLS, bool MAX>
+__device__ __forceinline__ float reduce_lanes(float (&e)[COLS], int lane) {
+#pragma unroll
+  for (int o = COLS / 2; o >= 1; o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float got = __shfl_xor_sync(0xffffffffu, up ? e[i] : e[i + o], o);
+      const float kept = up ? e[i + o] : e[i];
+      e[i] = MAX ? fmaxf(kept, got) : kept + got;
+    }
+  }
+  if (COLS == 16) {
+    const float got = __shfl_xor_sync(0xffffffffu, e[0], 16);
+    e[0] = MAX ? fmaxf(e[0], got) : e[0] + got;
+  }
+  return e[0];
+}
+// One block of a warp's remaining rows: z belongs to this lane's column, ref holds the references of the
+// block's columns in the form that each column's exponential wants.  False, with nothing changed, when a sum
+// is 2^62 above its reference or more (stats_update).
+template <int COLS>
+__device__ __forceinline__ bool rem_update(const uint32_t (&r)[32], float a, int lane, const float* ref, float& z) {
+  const float a128 = a * (1.f / 128.f);
+  const float2 a2 = splat2(a);
+  const float4* c4 = reinterpret_cast<const float4*>(ref);
+  float e[COLS];
+#pragma unroll
+  for (int i = 0; i < COLS / 2; ++i) {
+    const float4 c = c4[i >> 1];
+    const float2 cc = i & 1 ? make_float2(c.z, c.w) : make_float2(c.x, c.y);
+    const float x0 = __uint_as_float(r[2 * i]), x1 = __uint_as_float(r[2 * i + 1]);
+    const float2 v = is_poly<kPolyPairs>(i) ? ex2_poly2<64>(x0, x1, a128, cc) : ex2_mufu2(__ffma2_rn(make_float2(x0, x1), a2, cc));
+    e[2 * i] = v.x;
+    e[2 * i + 1] = v.y;
+  }
+  const float s = reduce_lanes<COLS, false>(e, lane);
+  if (__any_sync(0xffffffffu, !(s < 4.6e18f))) return false;
+  z += s;
+  return true;
+}
+// The same for a block with keys that not every row sees, or rows without a reference: the columns of
+// `visible` see this lane's key.  References become the maxima so far.
+template <int COLS>
+__device__ __noinline__ void rem_general(uint32_t taddr, uint32_t visible, float a, int lane, float* ref, float& m, float& z) {
+  uint32_t r[32];
+  if (COLS == 32) tmem_ld32(taddr, r); else tmem_ld16(taddr, r);
+  tmem_wait(r);
+  float v[COLS];
+#pragma unroll
+  for (int i = 0; i < COLS; ++i) v[i] = (visible >> i) & 1u ? __uint_as_float(r[i]) * a : -INFINITY;
+  const float mn = fmaxf(m, reduce_lanes<COLS, true>(v, lane));
+  if (mn > -INFINITY) z *= ex2(m - mn);
+  m = mn;
+  __syncwarp();                                            // the references are no longer read
+  if (lane < COLS) ref[lane] = !(mn > -INFINITY) ? 0.f : is_poly<kPolyPairs>(lane >> 1) ? fmaf(mn, -1.f / 128.f, 0.5f) : -mn;
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < COLS; ++i) {
+    const float mi = __shfl_sync(0xffffffffu, mn, i);
+    v[i] = (visible >> i) & 1u ? ex2(fmaf(__uint_as_float(r[i]), a, -mi)) : 0.f;
+  }
+  const float s = reduce_lanes<COLS, false>(v, lane);
+  if (mn > -INFINITY) z += s;
+}
+template <int COLS>
+__device__ __forceinline__ void rem_block(uint32_t taddr, bool general, uint32_t visible, float a, int lane, float* ref, float& m, float& z) {
+  if (!general) {
+    uint32_t r[32];
+    if (COLS == 32) tmem_ld32(taddr, r); else tmem_ld16(taddr, r);
+    tmem_wait(r);
+    if (rem_update<COLS>(r, a, lane, ref, z)) return;
+  }
+  rem_general<COLS>(taddr, visible, a, lane, ref, m, z);
+}
+
+// Pass 2: probabilities of COLS (16 or 32) query rows for this thread's key, reduced into acc (two packed
 // partial sums, or two packed maxima).  The row constants come in the form that each column's
 // exponential wants.
 __device__ __forceinline__ float row_const(int row, float negc) {
   return is_poly<kPolyPairs>((row & 31) >> 1) ? (negc + 125.f) * (1.f / 128.f) : negc;
 }
-template <bool MAXRED>
+template <bool MAXRED, int COLS>
 __device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const float* __restrict__ rowc, float2 a2, float a128, float2 (&acc)[2]) {
   const float4* c4 = reinterpret_cast<const float4*>(rowc);
 #pragma unroll
-  for (int i = 0; i < 8; ++i) {
+  for (int i = 0; i < COLS / 4; ++i) {
     const float4 c = c4[i];
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -387,13 +477,13 @@ __device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const f
 // Plain scalar code: only the last tile or two of a sequence come here.
 template <bool MAXRED>
 __device__ __forceinline__ void prob_accumulate_causal(const uint32_t (&r)[32], const float* __restrict__ rowc, float a,
-                                                       float2 (&acc)[2], int row0, int R, int n_window, int n, int key) {
+                                                       float2 (&acc)[2], int row0, int cols, int R, int n_window, int n, int key) {
   int rr = row0 % R;
 #pragma unroll
   for (int i = 0; i < 32; ++i) {
     const float negc = is_poly<kPolyPairs>(i >> 1) ? fmaf(rowc[i], 128.f, -125.f) : rowc[i];
     float pr = ex2(fmaf(__uint_as_float(r[i]), a, negc));
-    if (rr < n_window && key > max(n - n_window + rr, 0)) pr = 0.f;
+    if (i >= cols || (rr < n_window && key > max(n - n_window + rr, 0))) pr = 0.f;
     if (MAXRED) acc[0].x = fmaxf(acc[0].x, pr); else acc[0].x += pr;
     if (++rr == R) rr = 0;
   }
@@ -468,18 +558,22 @@ __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2
 
 // ------------------------------------------------------------------ the kernel --------
 
-template <int PASS, bool MAXRED>
+// FLAG: pass 1, whether remaining rows are scored on columns (a variant of its own: the registers that it needs
+// slowed the other one down by 4 to 20 %); pass 2, whether the reduction is the maximum.
+template <int PASS, bool FLAG>
 __global__ void __launch_bounds__(kThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int BUFCOLS = kBufCols;
+  constexpr bool REM = PASS == 1 && FLAG, MAXRED = PASS == 2 && FLAG;
 
   const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   uint8_t* k_sm = smem;
   uint8_t* q_sm = smem + (size_t)p.n_stages * p.stage_bytes;
   float* c_sm = reinterpret_cast<float*>(q_sm + p.q_bytes);
   float2* merge_sm = reinterpret_cast<float2*>(c_sm + p.M_pad);            // pass 2, units of few rows: see row_constants
-  int* tp = reinterpret_cast<int*>(merge_sm + p.merge_slots);
+  float* rem_sm = reinterpret_cast<float*>(merge_sm + p.merge_slots);      // pass 1: [16 warps][rem_cols] references, then as many sums
+  int* tp = reinterpret_cast<int*>(rem_sm + (REM ? 2 * 16 * p.rem_cols : 0));
   uint64_t* bars = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(tp + p.n_seq + 1) + 7) & ~(uintptr_t)7);
   uint64_t* k_full = bars;
   uint64_t* k_empty = bars + kMaxStages;
@@ -576,8 +670,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       uint32_t k_par = 0;
       bool ok = true;
       const uint32_t idesc_full = make_idesc(128);
-      const uint32_t idesc_last = make_idesc(PASS == 1 ? 128 : p.cw_last);
-      const int n_sub = PASS == 1 ? p.M_pad / 128 : p.n_chunks;
+      const uint32_t idesc_last = make_idesc(PASS == 2 ? p.cw_last : REM ? p.rem_cols : 128);
+      const int n_sub = PASS == 1 ? p.n_full + REM : p.n_chunks;
       const uint32_t q_lo0 = desc_lo(smem_u32(q_sm)), k_lo0 = desc_lo(smem_u32(k_sm));
       const uint32_t q_half16 = q_half_bytes >> 4;
       const uint32_t k_half16 = k_half_bytes >> 4;
@@ -607,15 +701,17 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               tc_fence_after();
               const uint32_t d_tmem = tmem_base + buf * BUFCOLS;
               const uint32_t q_lo = q_lo0 + sub * ((128 * 128) >> 4);
-              const uint32_t idesc = (PASS == 2 && sub == n_sub - 1) ? idesc_last : idesc_full;
+              const uint32_t idesc = (PASS == 2 || REM) && sub == n_sub - 1 ? idesc_last : idesc_full;
+              const bool rows_on_lanes = PASS == 1 && (!REM || sub < p.n_full);
+              const uint32_t a_lo = rows_on_lanes ? q_lo : k_lo, a_half16 = rows_on_lanes ? q_half16 : k_half16;
+              const uint32_t b_lo = rows_on_lanes ? k_lo : q_lo, b_half16 = rows_on_lanes ? k_half16 : q_half16;
               if (elect_one()) {
 #pragma unroll
                 for (int kh = 0; kh < 2; ++kh) {
                   if (kh < n_kh) {
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks) {
-                      if (PASS == 1) tc_mma(d_tmem, desc_at(q_lo + kh * q_half16 + ks * 2), desc_at(k_lo + kh * k_half16 + ks * 2), idesc, (kh | ks) != 0);
-                      else tc_mma(d_tmem, desc_at(k_lo + kh * k_half16 + ks * 2), desc_at(q_lo + kh * q_half16 + ks * 2), idesc, (kh | ks) != 0);
+                      tc_mma(d_tmem, desc_at(a_lo + kh * a_half16 + ks * 2), desc_at(b_lo + kh * b_half16 + ks * 2), idesc, (kh | ks) != 0);
                     }
                   }
                 }
@@ -663,9 +759,12 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           }
         }
       }
-      const int n_mt = p.M_pad / 128;
+      const int n_full = p.n_full, n_sub = n_full + REM;
       float mrun[kMaxMTiles], zrun[kMaxMTiles];
-      while (ok && seg_next(it, p, tp, sg)) {
+      float* my_ref = rem_sm + (warp - 4) * p.rem_cols;
+      // Every epilogue thread passes the barriers of every segment, also after a wait has given up.
+      while (seg_next(it, p, tp, sg)) {
+        float rem_m[2] = {-INFINITY, -INFINITY}, rem_z[2] = {0.f, 0.f};
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
 #pragma unroll
         for (int i = 0; i < kMaxMTiles; ++i) { mrun[i] = -INFINITY; zrun[i] = 0.f; }
@@ -675,11 +774,34 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const bool in_window = p.causal && key0 + kTileKeys > sg.n - p.n_window;    // warp-uniform
           const bool plain = nv >= kTileKeys && !in_window;
           if (clears && half == 0 && row_in_tile < nv) out[key0 + row_in_tile] = 0.f;
-          for (int mt = ((t >> 1) + half) & 1; mt < n_mt && ok; mt += 2) {
+          for (int mt = ((t >> 1) + half) & 1; mt < n_sub && ok; mt += 2) {
             ok = mbar_wait(&t_full[wg], used & 1, abort_flag);
             if (!ok) break;
             ++used;
             tc_fence_after();
+            if (REM && mt == n_full) {
+              // the remaining rows, on columns; this lane's key is key0 + row_in_tile
+              const int cols = p.rem_cols;
+              // warp-uniform: not every key is seen by every row, or a row has not seen any key yet
+              const bool general = !plain || !__all_sync(0xffffffffu, rem_m[0] > -INFINITY && (cols <= 32 || rem_m[1] > -INFINITY));
+              uint32_t seen = row_in_tile < nv ? 0xffffffffu : 0u, seen1 = seen;
+              if (in_window) {
+                int rr = (p.row0 + n_full * 128) % p.R;
+#pragma unroll 1
+                for (int i = 0; i < cols; ++i) {
+                  if (rr < p.n_window && key0 + row_in_tile > max(sg.n - p.n_window + rr, 0)) {
+                    if (i < 32) seen &= ~(1u << i); else seen1 &= ~(1u << (i - 32));
+                  }
+                  if (++rr == p.R) rr = 0;
+                }
+              }
+              if (cols >= 32) rem_block<32>(my_taddr, general, seen, p.a, lane, my_ref, rem_m[0], rem_z[0]);
+              else rem_block<16>(my_taddr, general, seen, p.a, lane, my_ref, rem_m[0], rem_z[0]);
+              if (cols > 32) rem_block<16>(my_taddr + 32, general, seen1, p.a, lane, my_ref + 32, rem_m[1], rem_z[1]);
+              tc_fence_before();
+              arrive_lane0(&t_empty[wg], lane);
+              continue;
+            }
             float m = mrun[mt], z = zrun[mt];
             if (plain) {
               // Every row sees all 128 keys: no masks, no per-row arithmetic.  The next block of columns is on its way
@@ -721,13 +843,33 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         }
         if (ok) {
           float* dst = p.partial + ((size_t)(sg.unit + blockIdx.x) * kEpilogueWarpgroups + wg) * p.M * 2;
-          for (int mt = 0; mt < n_mt; ++mt) {
+          for (int mt = 0; mt < n_full; ++mt) {
             const int row = mt * 128 + row_in_tile;
             if (row < p.M) {
               dst[row * 2 + 0] = mrun[mt];
               dst[row * 2 + 1] = zrun[mt];
             }
           }
+        }
+        if (REM) {
+          // the four warps of the warpgroup saw different keys: their (reference, sum) meet in shared memory
+          float* sums = rem_sm + 16 * p.rem_cols;
+          const int b1 = p.rem_cols - 32;                       // columns of the second block, if positive
+          if (lane < min(p.rem_cols, 32)) { my_ref[lane] = rem_m[0]; sums[(warp - 4) * p.rem_cols + lane] = rem_z[0]; }
+          if (lane < b1) { my_ref[32 + lane] = rem_m[1]; sums[(warp - 4) * p.rem_cols + 32 + lane] = rem_z[1]; }
+          asm volatile("bar.sync %0, 128;" ::"r"(2 + wg) : "memory");
+          const int row = n_full * 128 + row_in_tile;
+          if (row_in_tile < p.rem_cols && row < p.M && ok) {
+            float m = -INFINITY, z = 0.f;
+            for (int w = 0; w < 4; ++w) {
+              const int o = (wg * 4 + w) * p.rem_cols + row_in_tile;
+              fold_stats(m, z, rem_sm[o], sums[o]);
+            }
+            float* dst = p.partial + (((size_t)(sg.unit + blockIdx.x) * kEpilogueWarpgroups + wg) * p.M + row) * 2;
+            dst[0] = m;
+            dst[1] = z;
+          }
+          asm volatile("bar.sync %0, 128;" ::"r"(2 + wg) : "memory");
         }
       }
     } else {
@@ -774,7 +916,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             ++used;
             any = true;
             tc_fence_after();
-            const int cw = ch == p.n_chunks - 1 ? p.cw_last : 128;            // my columns: 64 or 128
+            const int cw = ch == p.n_chunks - 1 ? p.cw_last : 128;            // my columns
             const float* rowc = c_sm + ch * 128;
             const int row0 = p.row0 + ch * 128;                 // query row of my first column
             if (in_window) {
@@ -782,31 +924,44 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               for (int c = 0; c < cw; c += 32) {
                 tmem_ld32(my_taddr + c, ra);
                 tmem_wait(ra);
-                prob_accumulate_causal<MAXRED>(ra, rowc + c, p.a, acc, row0 + c, p.R, p.n_window, sg.n, key);
+                prob_accumulate_causal<MAXRED>(ra, rowc + c, p.a, acc, row0 + c, cw - c, p.R, p.n_window, sg.n, key);
               }
               tc_fence_before();
               arrive_lane0(&t_empty[wg], lane);
               continue;
             }
-            tmem_ld32(my_taddr, ra);                            // look-ahead as in pass 1
-            if (cw == 128) {
+            if (cw == 128) {                                    // look-ahead as in pass 1
+              tmem_ld32(my_taddr, ra);
               tmem_wait(ra);
               tmem_ld32(my_taddr + 32, rb);
-              prob_accumulate<MAXRED>(ra, rowc, a2, a128, acc);
+              prob_accumulate<MAXRED, 32>(ra, rowc, a2, a128, acc);
               tmem_wait(rb);
               tmem_ld32(my_taddr + 64, ra);
-              prob_accumulate<MAXRED>(rb, rowc + 32, a2, a128, acc);
-              rowc += 64;
+              prob_accumulate<MAXRED, 32>(rb, rowc + 32, a2, a128, acc);
               tmem_ld32(my_taddr + 96, rb);
+              tmem_wait(ra);
+              tmem_wait(rb);
+              tc_fence_before();
+              arrive_lane0(&t_empty[wg], lane);
+              prob_accumulate<MAXRED, 32>(ra, rowc + 64, a2, a128, acc);
+              prob_accumulate<MAXRED, 32>(rb, rowc + 96, a2, a128, acc);
             } else {
-              tmem_ld32(my_taddr + 32, rb);
+              // a last chunk of 16 to 112 rows, the odd half block first
+              const int n32 = cw >> 5;
+              if (cw & 16) {
+                tmem_ld16(my_taddr + n32 * 32, rb);
+                tmem_wait(rb);
+                if (n32 == 0) { tc_fence_before(); arrive_lane0(&t_empty[wg], lane); }
+                prob_accumulate<MAXRED, 16>(rb, rowc + n32 * 32, a2, a128, acc);
+              }
+#pragma unroll 1
+              for (int c = 0; c < n32; ++c) {
+                tmem_ld32(my_taddr + c * 32, ra);
+                tmem_wait(ra);
+                if (c == n32 - 1) { tc_fence_before(); arrive_lane0(&t_empty[wg], lane); }
+                prob_accumulate<MAXRED, 32>(ra, rowc + c * 32, a2, a128, acc);
+              }
             }
-            tmem_wait(ra);
-            tmem_wait(rb);
-            tc_fence_before();
-            arrive_lane0(&t_empty[wg], lane);
-            prob_accumulate<MAXRED>(ra, rowc, a2, a128, acc);
-            prob_accumulate<MAXRED>(rb, rowc + 32, a2, a128, acc);
           }
           if (!ok) break;
           if (any && key < sg.n) {
@@ -936,7 +1091,6 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   p.stage_bytes = (uint32_t)kTileKeys * d * 2;
 
   const int n_ctas = wp.score_ctas;
-  auto pass1 = score_kernel<1, false>;
   auto pass2 = reduce == SPEC_REDUCE_MAX ? score_kernel<2, true> : score_kernel<2, false>;
   // The kernels may use all of an SM's shared memory; the attribute is set once per device (it is per
   // function and context, so setting it per call would race between host threads).
@@ -947,11 +1101,12 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     if (dev < 0 || dev >= 64) return fail(SPEC_ERR_UNSUPPORTED, "device ordinal %d is not supported", dev);
     if (!__atomic_load_n(&set[dev], __ATOMIC_ACQUIRE)) {
       SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+      SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
       SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
       SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
       // The warpgroups divide the registers that the block was launched with: a build that launches with fewer
       // would wait for registers that do not exist.
-      const void* fns[3] = {(const void*)score_kernel<1, false>, (const void*)score_kernel<2, false>, (const void*)score_kernel<2, true>};
+      const void* fns[4] = {(const void*)score_kernel<1, false>, (const void*)score_kernel<1, true>, (const void*)score_kernel<2, false>, (const void*)score_kernel<2, true>};
       for (const void* f : fns) {
         cudaFuncAttributes at;
         SPEC_CUDA_OK(cudaFuncGetAttributes(&at, f));
@@ -964,21 +1119,38 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     p.row0 = g * rows_group;
     p.M = std::min(rows_group, M - p.row0);
     p.M_pad = (p.M + 127) / 128 * 128;
-    const int M64 = (p.M + 63) / 64 * 64;                  // pass 2 splits each chunk's columns in two halves of 32 or 64
-    p.n_chunks = (M64 + 127) / 128;
-    p.cw_last = M64 - (p.n_chunks - 1) * 128;
+    p.n_chunks = (p.M + 127) / 128;
+    p.cw_last = (p.M - (p.n_chunks - 1) * 128 + 15) / 16 * 16;
     p.q_bytes = (uint32_t)p.M_pad * d * 2;
     const int Mr = (p.M + 31) & ~31;
     p.merge_slots = 2 * Mr <= kEpilogueThreads ? kEpilogueThreads / Mr * Mr : 0;
     const int small = p.M_pad * 4 + p.merge_slots * 8 + (pr->n_seq + 1) * 4 + 8 + kNumBars * 8 + 16;
     const int smem_max = 227 * 1024;
-    int stages = (smem_max - (int)p.q_bytes - small) / (int)p.stage_bytes;
-    if (stages > kMaxStages) stages = kMaxStages;
+    int stages = std::min((smem_max - (int)p.q_bytes - small) / (int)p.stage_bytes, kMaxStages);
+    // Up to 48 rows behind the last full block are scored on columns: head_dim 64, 128 units of 32768, 260 rows 0.657 ->
+    // 0.580 ms, 132 rows 0.447 -> 0.350.  Not where CTAs have only a few tiles each (the first tile of a segment, which
+    // sets the references, takes the general form: 148 rows, 16 units of 9000, 8 tiles per CTA, 0.023 -> 0.028 ms), nor
+    // where the memory for it would leave fewer than three key stages.
+    p.n_full = p.M_pad / 128;
+    p.rem_cols = 0;
+    int rem_bytes = 0;
+    const int rem_cols = (p.M % 128 + 15) / 16 * 16;
+    const int64_t tiles = (int64_t)pr->n_layers * pr->n_kv_heads * ((tokens + kTileKeys - 1) / kTileKeys);
+    if (rem_cols >= 16 && rem_cols <= 48 && tiles >= (int64_t)kRemMinTiles * n_ctas) {
+      const int bytes = 2 * 16 * rem_cols * 4;
+      const int left = std::min((smem_max - (int)p.q_bytes - small - bytes) / (int)p.stage_bytes, kMaxStages);
+      if (left >= std::min(stages, 3)) {
+        stages = left;
+        rem_bytes = bytes;
+        p.n_full = p.M / 128;
+        p.rem_cols = rem_cols;
+      }
+    }
     if (stages < 2) return fail(SPEC_ERR_UNSUPPORTED, "not enough shared memory for two key stages (%d rows, head_dim=%d)", p.M, d);
     p.n_stages = stages;
-    int smem = stages * (int)p.stage_bytes + (int)p.q_bytes + small;
+    int smem = stages * (int)p.stage_bytes + (int)p.q_bytes + small + rem_bytes;
     if (smem < 120 * 1024) smem = 120 * 1024;             // one CTA per SM: each CTA owns the whole TMEM
-    SPEC_CUDA_OK(launch_dependent(pass1, dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
+    SPEC_CUDA_OK(launch_dependent(p.rem_cols ? score_kernel<1, true> : score_kernel<1, false>, dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
     SPEC_CUDA_OK(launch_dependent(pass2, dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
   }
   return SPEC_OK;

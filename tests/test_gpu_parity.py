@@ -115,6 +115,35 @@ def test_score_max_reduce_and_row_weights(B, W, oracle):
         assert_scores_close(got, ref, g.cu)
 
 
+@pytest.mark.parametrize("rows", [1, 16, 17, 31, 33, 40, 48, 49])
+@pytest.mark.parametrize("d", [64, 128])
+def test_score_rows_behind_the_last_full_block(B, W, oracle, rows, d):
+    """Row counts whose remainder behind full blocks of 128 is scored on columns (up to 48, given 16 key tiles per CTA) or not
+    (49), alone and behind a full block, with tiles that end inside a segment, a causal window that hides the last
+    keys, and several sequences.  The first, a middle and the last head of many are compared."""
+    L, H = 16, 24                                     # 384 units of 7 tiles on up to 148 CTAs
+    for lookahead, lens in ((rows, [860]), (128 + rows, [129, 3, 700])):
+        window = min(lookahead, 13)
+        gen = torch.Generator().manual_seed(rows)
+        n_seq, T = len(lens), sum(lens)
+        q = torch.randn(n_seq, L, H, lookahead, d, generator=gen).to(torch.bfloat16).cuda()
+        k = torch.randn(L, H, T, d, generator=gen).to(torch.bfloat16).cuda()
+        cu = [0] + list(np.cumsum(lens))
+        cu_t = torch.tensor(cu, dtype=torch.int32, device="cuda") if n_seq > 1 else None
+        pr = B.make_problem(n_layers=L, n_q_heads=H, n_kv_heads=H, head_dim=d, n_lookahead=lookahead - window, n_window=window,
+                            softmax_scale=d ** -0.5, total_tokens=T, n_in=max(lens), n_seq=n_seq, cu_seqlens=cu_t, k=k)
+        ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        for causal in (0, 1):
+            got = torch.full((L, H, T), float("nan"), device="cuda")
+            B.spec_score(pr, q, k, got, ws, causal_window=causal, status_word=status)
+            assert status.item() == 0
+            for l, h in ((0, 0), (7, 11), (L - 1, H - 1)):
+                ref = oracle.spec_score(bits(q[:, l:l + 1, h:h + 1]), bits(k[l:l + 1, h:h + 1]), cu, lookahead - window, window,
+                                        d ** -0.5, causal_window=bool(causal))
+                assert_scores_close(got[l:l + 1, h:h + 1].cpu().numpy(), ref, cu)
+
+
 @pytest.mark.parametrize("reduce", [0, 1])
 @pytest.mark.parametrize("case", ["large_weights", "rising_logits", "falling_logits", "steep_logits"])
 def test_score_range_of_the_exponentials(B, W, oracle, case, reduce):
