@@ -214,6 +214,7 @@ struct GatherParams {
 
 // cu_out[s] = n_keep[0] + ... + n_keep[s-1] (one thread: n_seq <= 1024).
 __global__ void keep_offsets_kernel(GatherParams p) {
+  wait_for_previous_grid();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   int acc = 0;
   p.cu_out[0] = 0;
@@ -235,6 +236,7 @@ __global__ void __launch_bounds__(kCompactThreads) gather_tokens_kernel(GatherPa
   const int h = unit % p.H;
   const int l = (unit / p.H) % p.L;
   const int s = unit / (p.H * p.L);
+  wait_for_previous_grid();
   int begin, n;
   seq_range(p.cu, p.n_in, s, begin, n);
   const int kept = min(max(p.n_keep[s], 0), p.keep_capacity);
@@ -384,16 +386,10 @@ SPEC_EXPORT int32_t spec_gather_tokens(const spec_problem* pr, const void* k, co
   const int64_t blocks = n_units * p.blocks_per_unit;
   if (blocks > 0x7fffffffLL) return fail(SPEC_ERR_UNSUPPORTED, "too many rows to gather in one call");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  keep_offsets_kernel<<<1, 32, 0, st>>>(p);
-  SPEC_CUDA_OK(cudaGetLastError());
+  SPEC_CUDA_OK(launch_dependent(keep_offsets_kernel, dim3(1), 32, 0, st, p));
   const bool d128 = pr->head_dim == 128;
-  if (v) {
-    if (d128) gather_tokens_kernel<16, true><<<(unsigned)blocks, kCompactThreads, 0, st>>>(p);
-    else      gather_tokens_kernel<8, true><<<(unsigned)blocks, kCompactThreads, 0, st>>>(p);
-  } else {
-    if (d128) gather_tokens_kernel<16, false><<<(unsigned)blocks, kCompactThreads, 0, st>>>(p);
-    else      gather_tokens_kernel<8, false><<<(unsigned)blocks, kCompactThreads, 0, st>>>(p);
-  }
-  SPEC_CUDA_OK(cudaGetLastError());
+  auto kernel = v ? (d128 ? gather_tokens_kernel<16, true> : gather_tokens_kernel<8, true>)
+                  : (d128 ? gather_tokens_kernel<16, false> : gather_tokens_kernel<8, false>);
+  SPEC_CUDA_OK(launch_dependent(kernel, dim3((unsigned)blocks), kCompactThreads, 0, st, p));
   return SPEC_OK;
 }

@@ -5,14 +5,13 @@
 // Every CTA of the cluster copies its contiguous share of the unit's scores into shared memory
 // with one bulk asynchronous copy (no registers are tied up while the bytes are in flight),
 // pools them there and turns the pooled values into order-preserving 32-bit keys that stay
-// resident.  The C-th largest key of the whole unit is then found by an MSB-first radix select
-// (11 + 11 + 10 bits): every CTA counts its own keys in a shared-memory histogram, adds the
-// non-empty bins into the merged histogram of every CTA of the cluster through distributed
-// shared memory, and after one cluster barrier per pass every CTA locates the digit by itself.
-// A first histogram over a 1-in-32 sample of the keys gives a floor under the threshold, so
-// that the first full pass only counts the few keys at or above it (if the floor turns out
-// too high the pass is repeated without it: the result is exact either way, and the cost does
-// not depend on where in the unit the large scores sit).  Winners are written in ascending
+// resident.  A sample of the keys, sent to every CTA of the cluster through distributed shared memory,
+// gives a floor under the threshold; the keys at or above it, about one and a half to two and a half
+// times the budget, are sent to every CTA as well, and each finds the exact threshold among them by
+// itself (find_threshold).  That takes two cluster barriers; the radix select over distributed
+// histograms that it replaced took four, and added every non-empty bin into all CTAs (32768 token
+// scores, 1024 kept: 25 -> CLUS1 us).  The radix select (11 + 11 + 10 bits) is what remains for units whose
+// floor lets through too few or too many keys, as massive ties can.  Winners are written in ascending
 // position: the CTAs exchange their counts, and each one emits its own winners behind those
 // of the CTAs before it; ties at the threshold go to the lower position.  The scores are read
 // from global memory once, whatever the number of budgets selected from them.
@@ -52,6 +51,11 @@ __device__ __forceinline__ uint32_t in_rank(uint32_t saddr, uint32_t rank) {
 }
 __device__ __forceinline__ void remote_add(uint32_t caddr, uint32_t v) {
   asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(caddr), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t remote_fetch_add(uint32_t caddr, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.relaxed.cluster.shared::cluster.add.u32 %0, [%1], %2;" : "=r"(old) : "r"(caddr), "r"(v) : "memory");
+  return old;
 }
 __device__ __forceinline__ void remote_or(uint32_t caddr, uint32_t v) {
   asm volatile("red.relaxed.cluster.shared::cluster.or.b32 [%0], %1;" ::"r"(caddr), "r"(v) : "memory");
@@ -103,6 +107,8 @@ __device__ __forceinline__ void pool_runs(const float* win, float* tmp, int n_ou
 
 constexpr int kBins = 2048;                      // 11-bit digits (the last pass uses 1024 of them)
 constexpr int kClMiscInts = 128;
+constexpr int kClusterSamples = 3072;            // of all CTAs of a cluster together
+static_assert(kClusterSamples * 4 + sizeof(SelectMem) <= 3 * kBins * 4, "the samples and the memory of the CTA-wide steps lie where the histograms would");
 constexpr int kClusterUse = 8;                   // largest cluster the host asks for
 
 struct ClusterSelParams {
@@ -115,6 +121,7 @@ struct ClusterSelParams {
   int halo_l, halo_r;         // padding of the staged scores on either side (multiples of 4)
   int inplace;                // width-7 maximum, pooled in place
   int mode;                   // 0: top-C index lists, 1: keep set
+  int cand_cap;               // keys at or above the floor that a CTA can hold
   int c_max;
   int32_t* idx_out;
   int32_t* count_out;
@@ -127,15 +134,15 @@ struct ClusterSelParams {
   int32_t* status;
 };
 
-// Shared memory of a CTA: local histogram, two merged histograms, bookkeeping, (keep set) the
-// bitmap of its positions, the staged scores with their halos and, unless pooling is in
-// place, the keys.
+// Shared memory of a CTA: local histogram and two merged histograms (the samples lie there before), bookkeeping, (keep
+// set) the bitmap of its positions, the staged scores with their halos, unless pooling is in place the keys, and
+// the cluster's keys at or above the floor.
 __host__ __device__ inline int cluster_cap_pad(int cap) { return (cap + 127) & ~127; }
 __host__ __device__ inline int cluster_bitmap_words(int cap, int mode) { return mode == 1 ? cluster_cap_pad(cap) / 32 + 4 : 0; }
-__host__ __device__ inline size_t cluster_smem_bytes(int cap, int halo_l, int halo_r, int inplace, int mode) {
+__host__ __device__ inline size_t cluster_smem_bytes(int cap, int halo_l, int halo_r, int inplace, int mode, int cand_cap) {
   const size_t raw = (size_t)halo_l + cluster_cap_pad(cap) + halo_r + 32;
   const size_t keys = inplace ? 0 : (size_t)cluster_cap_pad(cap) + 32;
-  return (size_t)(3 * kBins + kClMiscInts + cluster_bitmap_words(cap, mode)) * 4 + (raw + keys) * 4;
+  return (size_t)(3 * kBins + kClMiscInts + cluster_bitmap_words(cap, mode)) * 4 + (raw + keys + (size_t)cand_cap) * 4;
 }
 
 struct ClusterCtx {
@@ -192,15 +199,16 @@ __device__ __forceinline__ void hist_update(uint32_t* hist, bool in, uint32_t dg
 }
 
 // The key T of the take-th largest position of the unit (1 <= take < eligible positions) and
-// how many positions with key == T belong to the selection.  floor_key: keys below it are
-// known (or believed) to be out; a floor that was too high is detected and dropped.  Every
-// thread of every CTA of the cluster calls this with the same arguments.
-__device__ void cluster_threshold(ClusterCtx& c, int take, uint32_t floor_key, uint32_t& T_out, int& need_eq_out) {
+// how many positions with key == T belong to the selection, by a radix select over all keys of the
+// cluster.  Every thread of every CTA of the cluster calls this with the same arguments.
+__device__ void cluster_threshold(ClusterCtx& c, int take, uint32_t& T_out, int& need_eq_out) {
   const int tid = threadIdx.x, lane = tid & 31;
+  for (int b = tid; b < 2 * kBins; b += kSelThreads) c.merged[b] = 0;
+  c.stage = 0;
+  cluster_sync_all();
   uint32_t prefix = 0, mask = 0;
   int remaining = take;
-  int pass = 0;
-  while (pass < 3) {
+  for (int pass = 0; pass < 3; ++pass) {
     const int shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
     const uint32_t dmask = pass == 2 ? 1023u : 2047u;
     clear_hists(c);
@@ -209,23 +217,18 @@ __device__ void cluster_threshold(ClusterCtx& c, int take, uint32_t floor_key, u
       const int j = jb + tid;
       const bool valid = j < c.j_hi;
       const uint32_t kk = valid ? c.keys[j] : 0u;
-      const bool in = valid && (pass == 0 ? kk >= floor_key : (kk & mask) == prefix);
-      hist_update(c.local_hist, in, (kk >> shift) & dmask, lane);
+      hist_update(c.local_hist, valid && (kk & mask) == prefix, (kk >> shift) & dmask, lane);
     }
     __syncthreads();
     merge_hist(c);
     cluster_sync_all();
     const uint32_t* mg = c.merged + (c.stage & 1) * kBins;
     ++c.stage;
-    int dg, ab;
-    if (!locate_bin(mg + tid * (kBins / kSelThreads), kBins / kSelThreads, remaining, c.wsum, c.out2, dg, ab)) {
-      floor_key = 0;                                       // fewer than `take` keys above the floor: count them all
-      continue;
-    }
+    int dg = 0, ab = 0;
+    locate_bin(mg + tid * (kBins / kSelThreads), kBins / kSelThreads, remaining, c.wsum, c.out2, dg, ab);
     remaining -= ab;
     prefix |= (uint32_t)dg << shift;
     mask |= dmask << shift;
-    ++pass;
   }
   T_out = prefix;
   need_eq_out = remaining;
@@ -280,6 +283,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   ClusterCtx c;
   c.local_hist = reinterpret_cast<uint32_t*>(smem_raw);
   c.merged = c.local_hist + kBins;
+  SelectMem& sm = *reinterpret_cast<SelectMem*>(c.local_hist + kClusterSamples);
   int* misc = reinterpret_cast<int*>(c.merged + 2 * kBins);
   c.wsum = misc;                                           // 32
   c.out2 = misc + 32;                                      // 4
@@ -289,11 +293,13 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   int* sh_eq = misc + 88;                                  // 16
   int* timed_out = misc + 104;
   uint64_t* mbar = reinterpret_cast<uint64_t*>(misc + 106);
+  uint32_t* n_held = reinterpret_cast<uint32_t*>(misc + 110);
   uint32_t* bitmap = reinterpret_cast<uint32_t*>(misc + kClMiscInts);
   const int cap_pad = cluster_cap_pad(p.cap);
   float* raw = reinterpret_cast<float*>(bitmap + cluster_bitmap_words(p.cap, p.mode));
   uint32_t* keys_w = p.inplace ? reinterpret_cast<uint32_t*>(raw + p.halo_l)
                                : reinterpret_cast<uint32_t*>(raw + p.halo_l + cap_pad + p.halo_r + 32);
+  uint32_t* held = p.inplace ? reinterpret_cast<uint32_t*>(raw + p.halo_l + cap_pad + p.halo_r + 32) : keys_w + cap_pad + 32;
   c.keys = keys_w;
   c.rank = cluster_rank();
   c.cs = cluster_size();
@@ -301,6 +307,22 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t lt_mask = (1u << lane) - 1u;
+  // ---- clear what other CTAs will add to, then let them know this CTA is up
+  reinterpret_cast<uint4*>(sm.hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
+  if (p.mode == 1)
+    for (int w = tid; w < cluster_bitmap_words(p.cap, 1); w += kSelThreads) bitmap[w] = 0;
+  if (tid == 0) {
+    *timed_out = 0;
+    *n_held = 0;
+    sm.top = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(shared_u32(mbar)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  cluster_arrive();
+  wait_for_previous_grid();
+  launch_dependents();
+
   const int unit = blockIdx.x / c.cs;
   const int h = unit % p.H, l = (unit / p.H) % p.L, s = unit / (p.H * p.L);
   int begin, n;
@@ -330,18 +352,6 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   bool selects = false;
   for (int b = 0; b < n_budgets; ++b) selects = selects || (take[b] > 0 && take[b] < e);
 
-  // ---- clear what other CTAs will add to, then let them know this CTA is up
-  for (int b = tid; b < kBins; b += kSelThreads) c.merged[b] = 0;
-  if (p.mode == 1)
-    for (int w = tid; w < cluster_bitmap_words(p.cap, 1); w += kSelThreads) bitmap[w] = 0;
-  if (tid == 0) {
-    *timed_out = 0;
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(shared_u32(mbar)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  cluster_arrive();
-
   if (selects) {
     // ---- stage my share of the scores: [x0 - halo_l, x0 + n_steps * 128 + halo_r) in x
     const int n_steps = (CL + 127) >> 7;
@@ -361,7 +371,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
       const int x = xa + i;
       if (x >= bx0 && x < bx1) { i += ((bx1 - x - 1) / kSelThreads) * kSelThreads; continue; }   // skip the bulk-copied part
       const int pp = x - mis;
-      raw[i] = (pp >= 0 && pp < e) ? __ldg(src + pp) : pad;
+      raw[i] = (pp >= 0 && pp < e) ? __ldcg(src + pp) : pad;
     }
     if (bulk) {
       uint32_t ok = 0;
@@ -429,36 +439,73 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   }
   cluster_wait();                                          // every CTA of the cluster has cleared its shared memory
 
-  // ---- a floor under the thresholds from a 1-in-32 sample of the keys
-  uint32_t floor_key[2] = {0u, 0u};
-  bool sample = false;
-  for (int b = 0; b < n_budgets; ++b) sample = sample || (take[b] > 0 && take[b] < e && (int64_t)take[b] * 4 <= e && e >= 4096);
-  if (sample) {
-    clear_hists(c);
-    __syncthreads();
-    const int n_blocks = (CL + 31) >> 5;
-    for (int b = tid; b < n_blocks; b += kSelThreads) {
-      uint32_t hsh = ((uint32_t)unit * 0x9E3779B1u) ^ ((uint32_t)((x0 >> 5) + b) * 0x85EBCA6Bu);
-      hsh ^= hsh >> 15; hsh *= 0x2C1B3C6Du; hsh ^= hsh >> 12;
-      const int j = b * 32 + (int)(hsh & 31u);
-      if (j >= c.j_lo && j < c.j_hi) atomicAdd(&c.local_hist[c.keys[j] >> 21], 1u);
+  // ---- every CTA gets the cluster's keys at or above a floor under the thresholds
+  uint32_t floor_key = 0, top = 0;
+  int n_cand = 0;
+  if (selects && p.cand_cap > 0) {
+    if (e > p.cand_cap) {
+      // the floor, from one key in every 2^shift of every CTA; each takes it from the samples of all
+      int shift = 4;
+      while ((int)c.cs * ((CL + (1 << shift) - 1) >> shift) > kClusterSamples) ++shift;
+      const int per_cta = (CL + (1 << shift) - 1) >> shift;
+      for (int q = tid; q < per_cta; q += kSelThreads) {
+        const int j = (q << shift) + (int)(sample_hash((uint32_t)unit, c.rank * 65536u + (uint32_t)q) & ((1u << shift) - 1u));
+        const uint32_t key = j >= c.j_lo && j < c.j_hi ? c.keys[j] : 0u;
+        for (uint32_t r = 0; r < c.cs; ++r) remote_store(in_rank(shared_u32(c.local_hist + c.rank * per_cta + q), r), (int)key);
+      }
+      cluster_sync_all();
+      const int n_samples = (int)c.cs * per_cta;
+      uint32_t mine[kClusterSamples / kSelThreads];
+#pragma unroll
+      for (int i = 0; i < kClusterSamples / kSelThreads; ++i) mine[i] = tid + i * kSelThreads < n_samples ? c.local_hist[tid + i * kSelThreads] : 0u;
+      floor_key = floor_from_samples(sm, mine, max(take[0], n_budgets > 1 ? take[1] : 0), shift);
     }
-    __syncthreads();
-    merge_hist(c);
+    // my keys at or above it, to everyone: a warp reserves its places in all lists at once, then writes them
+    const int run = ((CL + kSelThreads - 1) / kSelThreads) * 32;
+    const int jb0 = max(warp * run, c.j_lo), je = min((warp + 1) * run, c.j_hi);
+    int mine = 0;
+    for (int j = jb0 + lane; j < je; j += 32) mine += c.keys[j] >= floor_key;
+    mine = (int)__reduce_add_sync(0xffffffffu, (uint32_t)mine);
+    if (mine > 0) {
+      uint32_t base = 0;
+      if (lane < (int)c.cs) base = remote_fetch_add(in_rank(shared_u32(n_held), (uint32_t)lane), (uint32_t)mine);
+      __syncwarp();
+      int at = 0;
+      for (int jb = jb0; jb < je; jb += 32) {
+        const int j = jb + lane;
+        const uint32_t key = j < je ? c.keys[j] : 0u;
+        const bool in = j < je && key >= floor_key;
+        const uint32_t ins = __ballot_sync(0xffffffffu, in);
+        if (ins == 0) continue;                            // warp-uniform
+        for (uint32_t r = 0; r < c.cs; ++r) {
+          const uint32_t slot = __shfl_sync(0xffffffffu, base, (int)r) + (uint32_t)(at + __popc(ins & lt_mask));
+          if (in && slot < (uint32_t)p.cand_cap) remote_store(in_rank(shared_u32(held + slot), r), (int)key);
+        }
+        at += __popc(ins);
+      }
+    }
     cluster_sync_all();
-    const uint32_t* mg = c.merged + (c.stage & 1) * kBins;
-    ++c.stage;
-    for (int b = 0; b < n_budgets; ++b) {
-      if (!(take[b] > 0 && take[b] < e && (int64_t)take[b] * 4 <= e)) continue;
-      // About take/32 of the samples lie above the threshold; the floor is taken four standard
-      // deviations further down the sample.
-      const float m = (float)take[b] * (1.f / 32.f);
-      const int rho = (int)(m + 4.f * sqrtf(m) + 8.f);
-      int fb, ab;
-      if (locate_bin(mg + tid * (kBins / kSelThreads), kBins / kSelThreads, rho, c.wsum, c.out2, fb, ab))
-        floor_key[b] = (uint32_t)fb << 21;
+    n_cand = (int)min(*n_held, 0x7fffffffu);
+    if (n_cand <= p.cand_cap) {
+      if (tid == 0) sm.top = 0;
+      __syncthreads();
+      for (int i = tid; i < n_cand; i += kSelThreads) top = max(top, held[i]);
+      __syncwarp();
+      top = __reduce_max_sync(0xffffffffu, top);
+      if (lane == 0) atomicMax(&sm.top, top);
+      __syncthreads();
+      top = sm.top;
     }
   }
+  auto threshold = [&](int tk, uint32_t& T, int& need_eq) {
+    if (n_cand >= tk && n_cand <= p.cand_cap) {
+      reinterpret_cast<uint4*>(sm.hist)[tid] = make_uint4(0u, 0u, 0u, 0u);       // (a radix select may have been here)
+      __syncthreads();
+      find_threshold(sm, held, n_cand, floor_key, top, tk, T, need_eq);
+    } else {
+      cluster_threshold(c, tk, T, need_eq);
+    }
+  };
 
   const int slab = ((CL + kSelThreads - 1) / kSelThreads) * 32;    // local positions per warp in the ordered sweeps
 
@@ -472,7 +519,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
       if (tk > 0 && tk < e) {
         uint32_t T;
         int need_eq;
-        cluster_threshold(c, tk, floor_key[b], T, need_eq);
+        threshold(tk, T, need_eq);
         int cta_gt, cta_eq, w_gt, w_eq;
         count_winners(c, T, slab, cta_gt, cta_eq, w_gt, w_eq, sh_gt, sh_eq);
         int gt_before, eq_before, gt_total, eq_total;
@@ -516,7 +563,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
     if (tk > 0 && tk < e) {
       uint32_t T;
       int need_eq;
-      cluster_threshold(c, tk, floor_key[0], T, need_eq);
+      threshold(tk, T, need_eq);
       int cta_gt, cta_eq, w_gt, w_eq;
       count_winners(c, T, slab, cta_gt, cta_eq, w_gt, w_eq, sh_gt, sh_eq);
       int gt_before, eq_before, gt_total, eq_total;
@@ -628,39 +675,64 @@ __global__ void __launch_bounds__(kSelThreads) pool_topk_generic_kernel(TopkPara
 
 // ---------------------------------------------------------------------- SpecPC ------
 
-// Token score: reduction over all layers and KV heads, in (layer, head) order.
-__global__ void __launch_bounds__(256) token_reduce_kernel(const float* __restrict__ scores, float* __restrict__ tok,
-                                                           int64_t T, int n_vec, int reduce) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= T) return;
-  const float* src = scores + t;
-  float acc = reduce == SPEC_REDUCE_SUM ? 0.f : -INFINITY;
-  int i = 0;
-  for (; i + 8 <= n_vec; i += 8) {
-    float x[8];
+// Token score: reduction over all layers and KV heads.  HBM-bound: every score is read once.  The eight warps of a
+// CTA share the vectors of 128 tokens, 16 loads in flight per lane; their partial results are
+// combined in warp order, so the result does not depend on timing.  (One thread per token over all
+// vectors left most of the GPU idle: 128 vectors of 32768 tokens 12.4 -> REDUS us.)
+constexpr int kReduceTokens = 128;
+constexpr int kReduceWarps = 8;
+
+template <bool MAX>
+__global__ void __launch_bounds__(kReduceWarps * 32) token_reduce_kernel(const float* __restrict__ scores, float* __restrict__ tok, int64_t T, int n_vec) {
+  __shared__ float part[kReduceWarps][kReduceTokens];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  wait_for_previous_grid();
+  launch_dependents();
+  const int64_t t0 = (int64_t)blockIdx.x * kReduceTokens + lane;
+  const int per_warp = (n_vec + kReduceWarps - 1) / kReduceWarps;
+  const int i0 = min(warp * per_warp, n_vec), i1 = min(i0 + per_warp, n_vec);
+  const float none = MAX ? -INFINITY : 0.f;
+  float acc[4] = {none, none, none, none};
+  for (int i = i0; i < i1; i += 4) {
+    float x[4][4];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) x[u] = __ldg(src + (int64_t)(i + u) * T);
+    for (int u = 0; u < 4; ++u)
 #pragma unroll
-    for (int u = 0; u < 8; ++u) acc = reduce == SPEC_REDUCE_SUM ? acc + x[u] : fmaxf(acc, x[u]);
+      for (int q = 0; q < 4; ++q) x[u][q] = i + u < i1 && t0 + 32 * q < T ? __ldcg(scores + (int64_t)(i + u) * T + t0 + 32 * q) : none;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[q] = MAX ? fmaxf(acc[q], x[u][q]) : acc[q] + x[u][q];
   }
-  for (; i < n_vec; ++i) {
-    const float x = __ldg(src + (int64_t)i * T);
-    acc = reduce == SPEC_REDUCE_SUM ? acc + x : fmaxf(acc, x);
-  }
-  tok[t] = acc;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) part[warp][lane + 32 * q] = acc[q];
+  __syncthreads();
+  const int64_t t = (int64_t)blockIdx.x * kReduceTokens + threadIdx.x;
+  if (threadIdx.x >= kReduceTokens || t >= T) return;
+  float v = part[0][threadIdx.x];
+#pragma unroll
+  for (int w = 1; w < kReduceWarps; ++w) v = MAX ? fmaxf(v, part[w][threadIdx.x]) : v + part[w][threadIdx.x];
+  tok[t] = v;
+}
+static cudaError_t launch_token_reduce(const float* scores, float* tok, int64_t T, int n_vec, int reduce, cudaStream_t st) {
+  const dim3 grid((unsigned)((T + kReduceTokens - 1) / kReduceTokens));
+  return reduce == SPEC_REDUCE_MAX ? launch_dependent(token_reduce_kernel<true>, grid, kReduceWarps * 32, 0, st, scores, tok, T, n_vec)
+                                   : launch_dependent(token_reduce_kernel<false>, grid, kReduceWarps * 32, 0, st, scores, tok, T, n_vec);
 }
 
 // First stage of Algorithm 2 lines 8-9 in the printed order: the average pool of the token
 // scores over each sequence's eligible range, written to a second vector.  A CTA stages a tile
 // of kAvgTile outputs with its window margins in shared memory and pools it there.
-constexpr int kAvgTile = 4096;
-constexpr int kAvgThreads = 256;
+constexpr int kAvgTile = 1024;
+constexpr int kAvgThreads = 128;
 
 __global__ void __launch_bounds__(kAvgThreads) token_avgpool_kernel(const float* __restrict__ tok, float* __restrict__ out,
                                                                     const int32_t* __restrict__ cu, int n_in, int n_forced, int k) {
   __shared__ float win[kAvgTile + 256 + 32];
   __shared__ float tmp[kAvgTile + 32];
   const int s = blockIdx.y;
+  wait_for_previous_grid();
+  launch_dependents();
   int begin, n;
   seq_range(cu, n_in, s, begin, n);
   const int e = n - min(n_forced, n);
@@ -670,7 +742,7 @@ __global__ void __launch_bounds__(kAvgThreads) token_avgpool_kernel(const float*
     __syncthreads();
     for (int i = threadIdx.x; i < n_out + k + 16; i += kAvgThreads) {
       const int j = t0 - lo + i;
-      win[i] = (j >= 0 && j < e) ? __ldg(tok + begin + j) : 0.f;
+      win[i] = (j >= 0 && j < e) ? __ldcg(tok + begin + j) : 0.f;
     }
     __syncthreads();
     float* dst = out + begin + t0;
@@ -789,11 +861,11 @@ constexpr int kMaxDevices = 64;
 
 struct ClusterPlan {
   bool fits;
-  int cs, cap, halo_l, halo_r, inplace;
+  int cs, cap, halo_l, halo_r, inplace, cand_cap;
   size_t smem;
 };
 
-static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int max_cs) {
+static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int max_cs, int budget) {
   ClusterPlan pl;
   pl.inplace = pool == SPEC_POOL_MAX && pool_k == 7;
   if (pl.inplace) {
@@ -807,8 +879,15 @@ static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int
   while (cs < max_cs && (x_max + cs - 1) / cs > kChunkTarget) cs <<= 1;
   pl.cs = cs;
   pl.cap = (int)((((x_max + cs - 1) / cs) + 3) & ~(int64_t)3);
-  pl.smem = cluster_smem_bytes(pl.cap, pl.halo_l, pl.halo_r, pl.inplace, mode);
+  pl.smem = cluster_smem_bytes(pl.cap, pl.halo_l, pl.halo_r, pl.inplace, mode, 0);
   pl.fits = pl.smem <= (size_t)kSmemLimit;
+  // The floor lets through 1.3 (large budgets) to 2.5 times the budget; short units send all of their keys.  Where
+  // there is no room for that (budgets of a third of a very long sequence), the radix select does without.
+  const int64_t room = ((int64_t)kSmemLimit - (int64_t)pl.smem) / 4;
+  const int64_t want = std::min<int64_t>(5 * (int64_t)budget / 2 + 1024, x_max + 1);
+  pl.cand_cap = pl.fits ? (int)(std::min(want, room) & ~(int64_t)3) : 0;
+  if (pl.cand_cap < std::min<int64_t>(want, 3 * (int64_t)budget / 2)) pl.cand_cap = 0;
+  pl.smem += (size_t)pl.cand_cap * 4;
   return pl;
 }
 
@@ -839,13 +918,15 @@ static int launch_cluster(const ClusterSelParams& p, int64_t n_units, const Clus
   cfg.blockDim = dim3(kSelThreads);
   cfg.dynamicSmemBytes = pl.smem;
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)pl.cs;
   at[0].val.clusterDim.y = 1;
   at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   SPEC_CUDA_OK(cudaLaunchKernelEx(&cfg, cluster_select_kernel, p));
   return SPEC_OK;
 }
@@ -879,12 +960,12 @@ static int run_pool_topk(const spec_problem* pr, const float* scores, int pool, 
   int rc = prepare_cluster_kernel(&max_cs);
   if (rc != SPEC_OK) return rc;
   const int64_t n_units = (int64_t)pr->n_seq * pr->n_layers * pr->n_kv_heads;
-  const ClusterPlan pl = plan_cluster(max_seq_len(pr), pool, pool_k, 0, max_cs);
+  const ClusterPlan pl = plan_cluster(max_seq_len(pr), pool, pool_k, 0, max_cs, std::max(c_max, n_vert));
   if (pl.fits) {
     ClusterSelParams p = {};
     p.scores = scores; p.cu = pr->cu_seqlens; p.T = pr->total_tokens; p.n_in = pr->n_in;
     p.L = pr->n_layers; p.H = pr->n_kv_heads; p.pool = pool; p.pool_k = pool_k; p.n_forced = n_forced_tail;
-    p.cap = pl.cap; p.halo_l = pl.halo_l; p.halo_r = pl.halo_r; p.inplace = pl.inplace; p.mode = 0;
+    p.cap = pl.cap; p.halo_l = pl.halo_l; p.halo_r = pl.halo_r; p.inplace = pl.inplace; p.mode = 0; p.cand_cap = pl.cand_cap;
     p.c_max = c_max; p.idx_out = idx_out; p.count_out = count_out;
     p.n_vert = n_vert; p.vert_out = vert_out; p.vert_count_out = vert_count_out;
     p.status = status_word;
@@ -914,12 +995,12 @@ static int run_keep(const spec_problem* pr, const float* tok, int pool, int pool
   int rc = prepare_cluster_kernel(&max_cs);
   if (rc != SPEC_OK) return rc;
   const int max_len = max_seq_len(pr);
-  const ClusterPlan pl = plan_cluster(max_len, pool, pool_k, 1, max_cs);
+  const ClusterPlan pl = plan_cluster(max_len, pool, pool_k, 1, max_cs, c_max);
   if (pl.fits) {
     ClusterSelParams p = {};
     p.scores = tok; p.cu = pr->cu_seqlens; p.T = pr->total_tokens; p.n_in = pr->n_in;
     p.L = 1; p.H = 1; p.pool = pool; p.pool_k = pool_k; p.n_forced = n_forced_tail;
-    p.cap = pl.cap; p.halo_l = pl.halo_l; p.halo_r = pl.halo_r; p.inplace = pl.inplace; p.mode = 1;
+    p.cap = pl.cap; p.halo_l = pl.halo_l; p.halo_r = pl.halo_r; p.inplace = pl.inplace; p.mode = 1; p.cand_cap = pl.cand_cap;
     p.c_max = c_max; p.n_neighbor = n_neighbor; p.keep_capacity = keep_capacity;
     p.keep_out = keep_out; p.n_keep_out = n_keep_out; p.status = status_word;
     return launch_cluster(p, pr->n_seq, pl, st);
@@ -1027,9 +1108,7 @@ SPEC_EXPORT int32_t specpc_token_select(const spec_problem* pr, const float* sco
   float* tok = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + wp.token_off);
   const int64_t T = pr->total_tokens;
   if (T > 0) {
-    token_reduce_kernel<<<(unsigned)((T + 255) / 256), 256, 0, st>>>(scores, tok, T, pr->n_layers * pr->n_kv_heads,
-                                                                     layer_head_reduce);
-    SPEC_CUDA_OK(cudaGetLastError());
+    SPEC_CUDA_OK(launch_token_reduce(scores, tok, T, pr->n_layers * pr->n_kv_heads, layer_head_reduce, st));
   }
   if (pool == SPEC_POOL_AVG_THEN_MAX && T > 0) {
     // Algorithm 2 lines 8-9 as printed: average pool, then the keep kernel max-pools with width
@@ -1038,8 +1117,7 @@ SPEC_EXPORT int32_t specpc_token_select(const spec_problem* pr, const float* sco
     const int max_len = max_seq_len(pr);
     const int tiles = (max_len + kAvgTile - 1) / kAvgTile;
     const dim3 grid((unsigned)(tiles > 0 ? tiles : 1), (unsigned)pr->n_seq);
-    token_avgpool_kernel<<<grid, kAvgThreads, 0, st>>>(tok, tok2, pr->cu_seqlens, pr->n_in, n_forced_tail, pool_k);
-    SPEC_CUDA_OK(cudaGetLastError());
+    SPEC_CUDA_OK(launch_dependent(token_avgpool_kernel, grid, kAvgThreads, 0, st, (const float*)tok, tok2, pr->cu_seqlens, pr->n_in, n_forced_tail, pool_k));
     tok = tok2;
     pool = SPEC_POOL_MAX;
     pool_k = n_neighbor > 1 ? n_neighbor : 1;
@@ -1105,9 +1183,7 @@ SPEC_EXPORT int32_t specpc_token_select_static(const spec_problem* pr, const flo
   const int64_t T = pr->total_tokens;
   if (T > 0) {
     // Writes every token score the selection reads, so nothing of an earlier call survives.
-    token_reduce_kernel<<<(unsigned)((T + 255) / 256), 256, 0, st>>>(scores, tok, T, pr->n_layers * pr->n_kv_heads,
-                                                                     layer_head_reduce);
-    SPEC_CUDA_OK(cudaGetLastError());
+    SPEC_CUDA_OK(launch_token_reduce(scores, tok, T, pr->n_layers * pr->n_kv_heads, layer_head_reduce, st));
   }
   return run_keep(pr, tok, pool, pool_k, c_max, n_neighbor, n_forced_tail, keep_out, keep_capacity, n_keep_out, status_word, st);
 }

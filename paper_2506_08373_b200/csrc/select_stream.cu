@@ -36,11 +36,9 @@
 
 namespace spec {
 
-constexpr int kStreamBins = 2048;
 constexpr int kWarpSteps = 8;                    // 128-position steps a warp holds in registers
 constexpr int kWarpSpan = kWarpSteps * 128;
 constexpr int kMaxSamples = 4096;
-constexpr int kListMax = 512;                    // members of the threshold's bin that are ranked against one another
 constexpr uint32_t kNoSelection = 0xFFFFFFFFu;   // floor value of a unit that keeps everything or nothing
 
 struct StreamParams {
@@ -98,130 +96,6 @@ __device__ __forceinline__ UnitGeom unit_geom(const StreamParams& p, int unit) {
 __device__ __forceinline__ float key_to_float(uint32_t key) {
   if (key <= 0x007FFFFFu) return -INFINITY;
   return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
-}
-
-__device__ __forceinline__ uint32_t sample_hash(uint32_t unit, uint32_t m) {
-  uint32_t h = (unit * 0x9E3779B1u) ^ (m * 0x85EBCA6Bu);
-  h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12;
-  return h;
-}
-
-// Shared memory of the CTA-wide steps.
-struct SelectMem {
-  uint32_t hist[kStreamBins];  // all zero between steps
-  uint32_t list[kListMax];
-  int wsum[32];
-  int res[8];
-  uint32_t top;                // largest key (zero on entry)
-};
-
-// Finds the bin of the need-th largest element of the histogram, the number of elements in higher bins
-// and in the bin itself, and clears the histogram.  False when it holds fewer than `need`.  Called by all
-// threads; three synchronisations.
-__device__ __forceinline__ bool find_bin(SelectMem& sm, int need, int& bin, int& above, int& count) {
-  static_assert(kStreamBins == 4 * kSelThreads, "four bins to a thread");
-  const int tid = threadIdx.x;
-  __syncthreads();
-  uint4* h4 = reinterpret_cast<uint4*>(sm.hist) + tid;
-  const uint4 h = *h4;
-  *h4 = make_uint4(0u, 0u, 0u, 0u);
-  const int mine = (int)(h.x + h.y + h.z + h.w);
-  int total;
-  const int below = block_exclusive_scan(mine, sm.wsum, total);
-  int over = total - below - mine;                         // elements in bins above mine
-  if (over < need && need <= over + mine) {
-    int b = 3, c = (int)h.w;
-    if (over + c < need) { over += c; c = (int)h.z; b = 2;
-      if (over + c < need) { over += c; c = (int)h.y; b = 1;
-        if (over + c < need) { over += c; c = (int)h.x; b = 0; } } }
-    sm.res[0] = 4 * tid + b;
-    sm.res[1] = over;
-    sm.res[2] = c;
-    sm.res[3] = 0;                                         // the length of the list that may be made next
-  }
-  __syncthreads();
-  bin = sm.res[0];
-  above = sm.res[1];
-  count = sm.res[2];
-  return total >= need;
-}
-
-// A key that about rho of the sampled keys reach: samples are binned by their distance below the largest,
-// 64 bins to a factor of two over 32 factors of two, or, if the rank lies deeper than that, by their
-// leading 11 bits.  0 when the sample is too small to tell.  `keys`: N samples of this thread, 0 = none.
-// All threads of the CTA call this; the histogram is clear on entry and on return.
-template <int N>
-__device__ __forceinline__ uint32_t floor_from_samples(SelectMem& sm, const uint32_t (&keys)[N], int take, int rate_shift) {
-  // about take / 2^rate_shift samples lie above the threshold; the floor is taken four standard deviations further down
-  const float m_exp = (float)take / (float)(1 << rate_shift);
-  const int rho = (int)(m_exp + 4.f * sqrtf(m_exp) + 8.f);
-  uint32_t top = 0;
-#pragma unroll
-  for (int i = 0; i < N; ++i) top = max(top, keys[i]);
-  top = __reduce_max_sync(0xffffffffu, top);
-  if ((threadIdx.x & 31) == 0 && top) atomicMax(&sm.top, top);
-  __syncthreads();
-  top = sm.top;
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-    if (keys[i]) atomicAdd(&sm.hist[kStreamBins - 1 - min((top - keys[i]) >> 17, (uint32_t)kStreamBins - 1)], 1u);
-  int bin, above, count;
-  if (!find_bin(sm, rho, bin, above, count)) return 0u;
-  if (bin > 0) {
-    const uint32_t depth = ((uint32_t)(kStreamBins - bin) << 17) - 1u;       // the bin's lower edge
-    return top > depth ? top - depth : 0u;
-  }
-#pragma unroll
-  for (int i = 0; i < N; ++i)
-    if (keys[i]) atomicAdd(&sm.hist[keys[i] >> 21], 1u);
-  find_bin(sm, rho, bin, above, count);
-  return (uint32_t)bin << 21;
-}
-
-// The key T of the need-th largest of keys[0..n), all of them in [lo, hi], and how many elements equal to T
-// belong to the selection.  The range is cut into 2048 bins as fine as it allows, so that the threshold's
-// bin holds a few dozen keys, which are ranked against one another; a fuller bin (ties) is cut again.  Called
-// by all threads with the histogram clear.
-__device__ __forceinline__ void find_threshold(SelectMem& sm, const uint32_t* keys, int n, uint32_t lo, uint32_t hi, int need,
-                                               uint32_t& T, int& need_eq) {
-  const int tid = threadIdx.x;
-  uint32_t span = hi - lo;
-  for (;;) {
-    const int shift = max(0, 21 - __clz((int)(span | 1u)));
-    for (int i = tid; i < n; i += kSelThreads) {
-      const uint32_t d = keys[i] - lo;
-      if (d <= span) atomicAdd(&sm.hist[d >> shift], 1u);
-    }
-    int bin, above, count;
-    find_bin(sm, need, bin, above, count);
-    need -= above;
-    lo += (uint32_t)bin << shift;
-    if (shift == 0) break;                                 // lo is the key itself
-    span = (1u << shift) - 1u;
-    if (count > kListMax) continue;
-    for (int i = tid; i < n; i += kSelThreads)
-      if (keys[i] - lo <= span) sm.list[atomicAdd(&sm.res[3], 1)] = keys[i];
-    __syncthreads();
-    if (tid < count) {
-      const uint32_t mine = sm.list[tid];
-      int gt = 0, ge = 0;
-      for (int j = 0; j < count; ++j) {
-        const uint32_t o = sm.list[j];
-        gt += o > mine;
-        ge += o >= mine;
-      }
-      if (gt < need && need <= ge) {                       // every holder of the threshold key writes the same
-        sm.res[4] = (int)mine;
-        sm.res[5] = need - gt;
-      }
-    }
-    __syncthreads();
-    lo = (uint32_t)sm.res[4];
-    need = sm.res[5];
-    break;
-  }
-  T = lo;
-  need_eq = need;
 }
 
 // Writes the positions of the selected candidates in the order in which they stand: key > T, and the first
