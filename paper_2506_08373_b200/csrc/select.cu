@@ -179,25 +179,6 @@ __device__ __forceinline__ void clear_hists(const ClusterCtx& c) {
   }
 }
 
-// Counts digit dg of the warp's keys that are `in`; neighbouring lanes with equal digits (the
-// runs that pooling produces) are merged into one update.
-__device__ __forceinline__ void hist_update(uint32_t* hist, bool in, uint32_t dg, int lane) {
-  const uint32_t ins = __ballot_sync(0xffffffffu, in);
-  if (ins == 0) return;                                    // warp-uniform
-  if (__popc(ins) <= 4) {
-    if (in) atomicAdd(&hist[dg], 1u);
-    return;
-  }
-  const uint32_t lt_mask = (1u << lane) - 1u;
-  const uint32_t dg_prev = __shfl_up_sync(0xffffffffu, dg, 1);
-  const bool head = in && (lane == 0 || !((ins >> (lane - 1)) & 1u) || dg_prev != dg);
-  const uint32_t heads = __ballot_sync(0xffffffffu, head);
-  if (head) {
-    const uint32_t stop = (heads | ~ins) & ~(lt_mask | (1u << lane));   // next run, or a lane that is out
-    atomicAdd(&hist[dg], (uint32_t)((stop ? __ffs(stop) - 1 : 32) - lane));
-  }
-}
-
 // The key T of the take-th largest position of the unit (1 <= take < eligible positions) and
 // how many positions with key == T belong to the selection, by a radix select over all keys of the
 // cluster.  Every thread of every CTA of the cluster calls this with the same arguments.
@@ -501,7 +482,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
     if (n_cand >= tk && n_cand <= p.cand_cap) {
       reinterpret_cast<uint4*>(sm.hist)[tid] = make_uint4(0u, 0u, 0u, 0u);       // (a radix select may have been here)
       __syncthreads();
-      find_threshold(sm, held, n_cand, floor_key, top, tk, T, need_eq);
+      find_threshold<true>(sm, held, n_cand, floor_key, top, tk, T, need_eq);
     } else {
       cluster_threshold(c, tk, T, need_eq);
     }
@@ -586,33 +567,34 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
       }
     }
     cluster_sync_all();                                    // all marks have landed
-    // ---- ordered extraction: every thread owns a run of consecutive bitmap words
+    // ---- ordered extraction: every warp owns a run of consecutive bitmap words and writes a word at a time
     const int n_words = (CL + 31) >> 5;
-    const int wpt = (n_words + kSelThreads - 1) / kSelThreads;
-    const int w0 = tid * wpt, w1 = min(w0 + wpt, n_words);
+    const int wpw = (n_words + kSelWarps - 1) / kSelWarps;
+    const int w0 = min(warp * wpw, n_words), w1 = min(w0 + wpw, n_words);
     int mine = 0;
-    for (int w = w0; w < w1; ++w) mine += __popc(bitmap[w]);
-    int cta_total;
-    const int before = block_exclusive_scan(mine, c.wsum, cta_total);
+    for (int w = w0 + lane; w < w1; w += 32) mine += __popc(bitmap[w]);
+    mine = (int)__reduce_add_sync(0xffffffffu, (uint32_t)mine);
+    if (lane == 0) c.wsum[warp] = mine;
+    __syncthreads();
+    const int of_warp = lane < kSelWarps ? c.wsum[lane] : 0;
+    const int cta_total = (int)__reduce_add_sync(0xffffffffu, (uint32_t)of_warp);
+    const int before = (int)__reduce_add_sync(0xffffffffu, (uint32_t)(lane < warp ? of_warp : 0));
     int tot_before, dummy_b, total, dummy_t;
     exchange_counts(c, cta_total, 0, tot_before, dummy_b, total, dummy_t);
     int32_t* keep = p.keep_out + (int64_t)s * p.keep_capacity;
     int pos = tot_before + before;
     for (int w = w0; w < w1; ++w) {
-      uint32_t bits = bitmap[w];
-      while (bits) {
-        const int b = __ffs(bits) - 1;
-        bits &= bits - 1;
-        if (pos < p.keep_capacity) keep[pos] = x0 + (w << 5) + b - mis;
-        ++pos;
-      }
+      const uint32_t bits = bitmap[w];
+      const int at = pos + __popc(bits & lt_mask);
+      if (((bits >> lane) & 1u) && at < p.keep_capacity) keep[at] = x0 + (w << 5) + lane - mis;
+      pos += __popc(bits);
     }
+    const int kept = min(total + forced, p.keep_capacity);
+    for (int q = kept + (int)c.rank * kSelThreads + tid; q < p.keep_capacity; q += (int)c.cs * kSelThreads) keep[q] = -1;
     if (c.rank == 0) {
       // the forced tail (the always-kept window) follows the selected positions
       for (int q = tid; q < forced; q += kSelThreads)
         if (total + q < p.keep_capacity) keep[total + q] = e + q;
-      const int kept = min(total + forced, p.keep_capacity);
-      for (int q = kept + tid; q < p.keep_capacity; q += kSelThreads) keep[q] = -1;
       if (tid == 0) {
         if (total + forced > p.keep_capacity) report(p.status, SPEC_ERR_BAD_ARG);
         p.n_keep_out[s] = kept;
@@ -856,7 +838,7 @@ __global__ void __launch_bounds__(kSelThreads) specpc_keep_generic_kernel(KeepPa
 
 // ------------------------------------------------------------------ host side ---------
 
-constexpr int kChunkTarget = 8192;               // positions per CTA the cluster size is chosen for
+constexpr int kChunkMin = 512;                   // positions per CTA below which no larger cluster is taken
 constexpr int kMaxDevices = 64;
 
 struct ClusterPlan {
@@ -865,7 +847,7 @@ struct ClusterPlan {
   size_t smem;
 };
 
-static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int max_cs, int budget) {
+static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int max_cs, int budget, int64_t n_units) {
   ClusterPlan pl;
   pl.inplace = pool == SPEC_POOL_MAX && pool_k == 7;
   if (pl.inplace) {
@@ -875,12 +857,26 @@ static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int
     pl.halo_r = ((pool_k - 1 - (pool_k >> 1)) + kPoolRun + 3) & ~3;
   }
   const int64_t x_max = (int64_t)max_len + 3;
-  int cs = 1;
-  while (cs < max_cs && (x_max + cs - 1) / cs > kChunkTarget) cs <<= 1;
-  pl.cs = cs;
-  pl.cap = (int)((((x_max + cs - 1) / cs) + 3) & ~(int64_t)3);
-  pl.smem = cluster_smem_bytes(pl.cap, pl.halo_l, pl.halo_r, pl.inplace, mode, 0);
-  pl.fits = pl.smem <= (size_t)kSmemLimit;
+  // The cluster size with the least estimated time: a CTA takes 7 us and another 10 for 8192 positions (32768 positions
+  // in 4 CTAs: 17 us), and two CTAs share an SM where their memory allows; GPCs hold about 0.8 of the
+  // slots' worth of clusters.
+  double best = 1e30;
+  pl.fits = false;
+  for (int cs = max_cs; cs >= 1; cs >>= 1) {
+    const int cap = (int)((((x_max + cs - 1) / cs) + 3) & ~(int64_t)3);
+    const size_t smem = cluster_smem_bytes(cap, pl.halo_l, pl.halo_r, pl.inplace, mode, 0);
+    if (smem > (size_t)kSmemLimit || (cs > 1 && cap < kChunkMin)) continue;
+    const int64_t slots = (smem + (size_t)(5 * (int64_t)budget / 2 + 1024) * 4 <= (size_t)kSmemLimit / 2 ? 2 : 1) * (cs > 2 ? 120 : 140);
+    const double t = (double)((n_units * cs + slots - 1) / slots) * (7.0 + 10.0 * cap / 8192);
+    if (t < best) {
+      best = t;
+      pl.fits = true;
+      pl.cs = cs;
+      pl.cap = cap;
+      pl.smem = smem;
+    }
+  }
+  if (!pl.fits) { pl.cs = 1; pl.cap = 0; pl.smem = 0; }
   // The floor lets through 1.3 (large budgets) to 2.5 times the budget; short units send all of their keys.  Where
   // there is no room for that (budgets of a third of a very long sequence), the radix select does without.
   const int64_t room = ((int64_t)kSmemLimit - (int64_t)pl.smem) / 4;
@@ -960,7 +956,7 @@ static int run_pool_topk(const spec_problem* pr, const float* scores, int pool, 
   int rc = prepare_cluster_kernel(&max_cs);
   if (rc != SPEC_OK) return rc;
   const int64_t n_units = (int64_t)pr->n_seq * pr->n_layers * pr->n_kv_heads;
-  const ClusterPlan pl = plan_cluster(max_seq_len(pr), pool, pool_k, 0, max_cs, std::max(c_max, n_vert));
+  const ClusterPlan pl = plan_cluster(max_seq_len(pr), pool, pool_k, 0, max_cs, std::max(c_max, n_vert), n_units);
   if (pl.fits) {
     ClusterSelParams p = {};
     p.scores = scores; p.cu = pr->cu_seqlens; p.T = pr->total_tokens; p.n_in = pr->n_in;
@@ -995,7 +991,7 @@ static int run_keep(const spec_problem* pr, const float* tok, int pool, int pool
   int rc = prepare_cluster_kernel(&max_cs);
   if (rc != SPEC_OK) return rc;
   const int max_len = max_seq_len(pr);
-  const ClusterPlan pl = plan_cluster(max_len, pool, pool_k, 1, max_cs, c_max);
+  const ClusterPlan pl = plan_cluster(max_len, pool, pool_k, 1, max_cs, c_max, pr->n_seq);
   if (pl.fits) {
     ClusterSelParams p = {};
     p.scores = tok; p.cu = pr->cu_seqlens; p.T = pr->total_tokens; p.n_in = pr->n_in;

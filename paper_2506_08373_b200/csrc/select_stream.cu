@@ -154,7 +154,7 @@ __device__ __forceinline__ void finish_unit(const StreamParams& p, const UnitGeo
     uint32_t T;
     int need_eq;
     if (!failed && n >= tk) {
-      find_threshold(sm, keys, n, floor_key, top, tk, T, need_eq);
+      find_threshold<false>(sm, keys, n, floor_key, top, tk, T, need_eq);
       emit_selected(sm, keys, pos, n, T, need_eq, idx);
     } else {
       __syncthreads();
