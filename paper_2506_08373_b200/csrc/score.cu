@@ -78,7 +78,7 @@ struct ScoreParams {
   long long T;
   int n_in, n_seq, L, Hq, Hkv, G, R, M, M_pad, d;   // M, M_pad: the query rows of this launch, rows [row0, row0 + M) of every unit
   int row0;
-  int causal, n_window;  // causal != 0: window row r sees keys up to position n - n_window + r only
+  int n_window;          // causal kernels: window row r sees keys up to position n - n_window + r only
   int merge_slots;       // threads that share the merging of a unit's statistics when there are fewer rows than threads (0: none do)
   int n_stages, n_chunks, cw_last;   // pass 2: chunks of 128 query rows, the last of cw_last (a multiple of 16)
   int n_full, rem_cols;  // pass 1: blocks of 128 query rows on lanes, and 16..48 remaining rows on columns (0: none)
@@ -450,8 +450,10 @@ __device__ __forceinline__ void rem_block(uint32_t taddr, bool general, uint32_t
 __device__ __forceinline__ float row_const(int row, float negc) {
   return is_poly<kPolyPairs>((row & 31) >> 1) ? (negc + 125.f) * (1.f / 128.f) : negc;
 }
-template <bool MAXRED, int COLS>
-__device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const float* __restrict__ rowc, float2 a2, float a128, float2 (&acc)[2]) {
+// hidden (MASKED): the columns that do not see this thread's key.
+template <bool MAXRED, int COLS, bool MASKED = false>
+__device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const float* __restrict__ rowc, float2 a2, float a128, float2 (&acc)[2],
+                                                uint32_t hidden = 0) {
   const float4* c4 = reinterpret_cast<const float4*>(rowc);
 #pragma unroll
   for (int i = 0; i < COLS / 4; ++i) {
@@ -459,7 +461,11 @@ __device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const f
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const float x0 = __uint_as_float(r[4 * i + 2 * u]), x1 = __uint_as_float(r[4 * i + 2 * u + 1]);
-      const float2 cc = u == 0 ? make_float2(c.x, c.y) : make_float2(c.z, c.w);
+      float2 cc = u == 0 ? make_float2(c.x, c.y) : make_float2(c.z, c.w);
+      if (MASKED) {
+        if ((hidden >> (4 * i + 2 * u)) & 1u) cc.x = -INFINITY;
+        if ((hidden >> (4 * i + 2 * u + 1)) & 1u) cc.y = -INFINITY;
+      }
       const float2 e = is_poly<kPolyPairs>(2 * i + u) ? ex2_poly2<125>(x0, x1, a128, cc) : ex2_mufu2(__ffma2_rn(make_float2(x0, x1), a2, cc));
       if (MAXRED) {
         if (u == 0) acc[0].x = max3(acc[0].x, e.x, e.y);   // one maximum per chain: they are merged at the end
@@ -471,22 +477,19 @@ __device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const f
   }
 }
 
-// The same for a key tile that reaches into the causal window: the probability of query row
-// (row0 + i) for this thread's key (position `key` of a sequence of n) is dropped when the row
-// is window row r < n_window and the key lies after the row's own position n - n_window + r.
-// Plain scalar code: only the last tile or two of a sequence come here.
-template <bool MAXRED>
-__device__ __forceinline__ void prob_accumulate_causal(const uint32_t (&r)[32], const float* __restrict__ rowc, float a,
-                                                       float2 (&acc)[2], int row0, int cols, int R, int n_window, int n, int key) {
-  int rr = row0 % R;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const float negc = is_poly<kPolyPairs>(i >> 1) ? fmaf(rowc[i], 128.f, -125.f) : rowc[i];
-    float pr = ex2(fmaf(__uint_as_float(r[i]), a, negc));
-    if (i >= cols || (rr < n_window && key > max(n - n_window + rr, 0))) pr = 0.f;
-    if (MAXRED) acc[0].x = fmaxf(acc[0].x, pr); else acc[0].x += pr;
-    if (++rr == R) rr = 0;
+// The columns from row0 on (bit i: row0 + i) that may not see key position `key` of a sequence of n: window row
+// r < n_window does not when the key lies after the row's own position n - n_window + r, that is,
+// when r < key - (n - n_window).
+__device__ __forceinline__ uint32_t hidden_columns(int row0, int R, int n_window, int n, int key) {
+  const int lim = key > 0 ? min(max(key - (n - n_window), 0), n_window) : 0;
+  uint32_t hidden = 0;
+  if (lim > 0) {
+    for (int b = -(row0 % R); b < 32; b += R) {
+      const int lo = max(b, 0), hi = min(b + lim, 32);       // columns lo .. hi - 1
+      if (hi > lo) hidden |= (0xffffffffu >> (32 - (hi - lo))) << lo;
+    }
   }
+  return hidden;
 }
 
 // Combines the statistics that pass 1 left for a unit (one partial per warpgroup and CTA that worked
@@ -559,8 +562,9 @@ __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2
 // ------------------------------------------------------------------ the kernel --------
 
 // FLAG: pass 1, whether remaining rows are scored on columns (a variant of its own: the registers that it needs
-// slowed the other one down by 4 to 20 %); pass 2, whether the reduction is the maximum.
-template <int PASS, bool FLAG>
+// slowed the other one down by 4 to 20 %); pass 2, whether the reduction is the maximum.  CAUSAL: the causal window,
+// likewise apart (its masks cost the other kernels 1 to 2 % in registers).
+template <int PASS, bool FLAG, bool CAUSAL>
 __global__ void __launch_bounds__(kThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -771,7 +775,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         for (int t = pair; t < sg.nt && ok; t += 2) {
           const int key0 = (sg.t0 + t) * kTileKeys;                                // first key of the tile
           const int nv = min(kTileKeys, sg.n - key0);                              // valid keys of the tile
-          const bool in_window = p.causal && key0 + kTileKeys > sg.n - p.n_window;    // warp-uniform
+          const bool in_window = CAUSAL && key0 + kTileKeys > sg.n - p.n_window;    // warp-uniform
           const bool plain = nv >= kTileKeys && !in_window;
           if (clears && half == 0 && row_in_tile < nv) out[key0 + row_in_tile] = 0.f;
           for (int mt = ((t >> 1) + half) & 1; mt < n_sub && ok; mt += 2) {
@@ -908,7 +912,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         for (int t = pair; t < sg.nt && ok; t += 2) {
           float2 acc[2] = {splat2(0.f), splat2(0.f)};
           const int key = (sg.t0 + t) * kTileKeys + row_in_tile;
-          const bool in_window = p.causal && (sg.t0 + t + 1) * kTileKeys > sg.n - p.n_window;   // warp-uniform
+          const bool in_window = CAUSAL && (sg.t0 + t + 1) * kTileKeys > sg.n - p.n_window;   // warp-uniform
           bool any = false;
           for (int ch = ((t >> 1) + half) & 1; ch < p.n_chunks; ch += 2) {
             ok = mbar_wait(&t_full[wg], used & 1, abort_flag);
@@ -922,9 +926,16 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             if (in_window) {
 #pragma unroll 1
               for (int c = 0; c < cw; c += 32) {
-                tmem_ld32(my_taddr + c, ra);
-                tmem_wait(ra);
-                prob_accumulate_causal<MAXRED>(ra, rowc + c, p.a, acc, row0 + c, cw - c, p.R, p.n_window, sg.n, key);
+                const uint32_t hidden = hidden_columns(row0 + c, p.R, p.n_window, sg.n, key);
+                if (c + 32 <= cw) {
+                  tmem_ld32(my_taddr + c, ra);
+                  tmem_wait(ra);
+                  prob_accumulate<MAXRED, 32, true>(ra, rowc + c, a2, a128, acc, hidden);
+                } else {
+                  tmem_ld16(my_taddr + c, ra);
+                  tmem_wait(ra);
+                  prob_accumulate<MAXRED, 16, true>(ra, rowc + c, a2, a128, acc, hidden);
+                }
               }
               tc_fence_before();
               arrive_lane0(&t_empty[wg], lane);
@@ -1085,13 +1096,15 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   p.n_in = pr->n_in; p.n_seq = pr->n_seq; p.L = pr->n_layers; p.Hq = pr->n_q_heads; p.Hkv = pr->n_kv_heads;
   p.G = G; p.R = R; p.d = d;
   p.reduce = reduce;
-  p.causal = causal_window;
   p.n_window = pr->n_window;
   p.a = (float)((double)pr->softmax_scale * 1.4426950408889634);
   p.stage_bytes = (uint32_t)kTileKeys * d * 2;
 
   const int n_ctas = wp.score_ctas;
-  auto pass2 = reduce == SPEC_REDUCE_MAX ? score_kernel<2, true> : score_kernel<2, false>;
+  typedef void (*ScoreKernel)(const CUtensorMap, const CUtensorMap, const ScoreParams);
+  static const ScoreKernel kernels[2][2][2] = {             // [pass][flag][causal]
+      {{score_kernel<1, false, false>, score_kernel<1, false, true>}, {score_kernel<1, true, false>, score_kernel<1, true, true>}},
+      {{score_kernel<2, false, false>, score_kernel<2, false, true>}, {score_kernel<2, true, false>, score_kernel<2, true, true>}}};
   // The kernels may use all of an SM's shared memory; the attribute is set once per device (it is per
   // function and context, so setting it per call would race between host threads).
   {
@@ -1100,14 +1113,11 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     SPEC_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(SPEC_ERR_UNSUPPORTED, "device ordinal %d is not supported", dev);
     if (!__atomic_load_n(&set[dev], __ATOMIC_ACQUIRE)) {
-      SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-      SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-      SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-      SPEC_CUDA_OK(cudaFuncSetAttribute(score_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-      // The warpgroups divide the registers that the block was launched with: a build that launches with fewer
-      // would wait for registers that do not exist.
-      const void* fns[4] = {(const void*)score_kernel<1, false>, (const void*)score_kernel<1, true>, (const void*)score_kernel<2, false>, (const void*)score_kernel<2, true>};
-      for (const void* f : fns) {
+      for (int i = 0; i < 8; ++i) {
+        const void* f = (const void*)kernels[i >> 2][(i >> 1) & 1][i & 1];
+        SPEC_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        // The warpgroups divide the registers that the block was launched with: a build that launches with fewer
+        // would wait for registers that do not exist.
         cudaFuncAttributes at;
         SPEC_CUDA_OK(cudaFuncGetAttributes(&at, f));
         if (at.numRegs < kLaunchRegs) return fail(SPEC_ERR_UNSUPPORTED, "the scoring kernel was built with %d registers per thread, %d needed", at.numRegs, kLaunchRegs);
@@ -1150,8 +1160,8 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     p.n_stages = stages;
     int smem = stages * (int)p.stage_bytes + (int)p.q_bytes + small + rem_bytes;
     if (smem < 120 * 1024) smem = 120 * 1024;             // one CTA per SM: each CTA owns the whole TMEM
-    SPEC_CUDA_OK(launch_dependent(p.rem_cols ? score_kernel<1, true> : score_kernel<1, false>, dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
-    SPEC_CUDA_OK(launch_dependent(pass2, dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
+    SPEC_CUDA_OK(launch_dependent(kernels[0][p.rem_cols > 0][causal_window], dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
+    SPEC_CUDA_OK(launch_dependent(kernels[1][reduce == SPEC_REDUCE_MAX][causal_window], dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
   }
   return SPEC_OK;
 }
