@@ -444,11 +444,14 @@ __device__ __forceinline__ void rem_block(uint32_t taddr, bool general, uint32_t
   rem_general<COLS>(taddr, visible, a, lane, ref, m, z);
 }
 
-// Pass 2: probabilities of COLS (16 or 32) query rows for this thread's key, reduced into acc (two packed
-// partial sums, or two packed maxima).  The row constants come in the form that each column's
-// exponential wants.
+// Pass 2: COLS (16 or 32) query rows for this thread's key, reduced into acc.  SUM: two packed partial sums of the
+// probabilities; the row constants come in the form that each column's exponential wants (row_const).
+// MAX: four maxima of the exponents a*s - c_i, for the largest probability is the one with the largest
+// exponent: one exponential per key, at the end, instead of one per logit (16 layers of 32768, 260 rows of
+// head_dim 64: pass 2 284 -> 195 us; 8 layers of 32768, 640 rows of head_dim 128: 330 -> 245 us).
+template <bool MAXRED>
 __device__ __forceinline__ float row_const(int row, float negc) {
-  return is_poly<kPolyPairs>((row & 31) >> 1) ? (negc + 125.f) * (1.f / 128.f) : negc;
+  return !MAXRED && is_poly<kPolyPairs>((row & 31) >> 1) ? (negc + 125.f) * (1.f / 128.f) : negc;
 }
 // hidden (MASKED): the columns that do not see this thread's key.
 template <bool MAXRED, int COLS, bool MASKED = false>
@@ -466,11 +469,12 @@ __device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const f
         if ((hidden >> (4 * i + 2 * u)) & 1u) cc.x = -INFINITY;
         if ((hidden >> (4 * i + 2 * u + 1)) & 1u) cc.y = -INFINITY;
       }
-      const float2 e = is_poly<kPolyPairs>(2 * i + u) ? ex2_poly2<125>(x0, x1, a128, cc) : ex2_mufu2(__ffma2_rn(make_float2(x0, x1), a2, cc));
       if (MAXRED) {
-        if (u == 0) acc[0].x = max3(acc[0].x, e.x, e.y);   // one maximum per chain: they are merged at the end
-        else acc[1].x = max3(acc[1].x, e.x, e.y);
+        const float2 x = __ffma2_rn(make_float2(x0, x1), a2, cc);
+        float& m = i & 1 ? acc[u].y : acc[u].x;            // four chains, merged at the end
+        m = max3(m, x.x, x.y);
       } else {
+        const float2 e = is_poly<kPolyPairs>(2 * i + u) ? ex2_poly2<125>(x0, x1, a128, cc) : ex2_mufu2(__ffma2_rn(make_float2(x0, x1), a2, cc));
         acc[u] = __fadd2_rn(acc[u], e);
       }
     }
@@ -507,6 +511,7 @@ __device__ __forceinline__ void fold_stats(float& m, float& z, float pm, float p
 
 constexpr int kMergeLoads = 16;       // in flight per thread; with 8, one layer of 12K (72 partials per row) spent 8 us here
 
+template <bool MAXRED>
 __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2* __restrict__ part, int n, int et, float scale_log2, float* c_sm, float2* merge_sm) {
   const int Mr = (p.M + 31) & ~31;
   const int slices = p.merge_slots > 0 ? p.merge_slots / Mr : 1;
@@ -550,7 +555,7 @@ __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2
         if (p.row_weight) c -= log2f(p.row_weight[(p.row0 + i) % p.R]) - scale_log2;
         c = -c;
       }
-      c_sm[i] = row_const(i, c);
+      c_sm[i] = row_const<MAXRED>(i, c);
     }
     if (slices > 1) {                                          // the padding rows beyond the slices' reach
       for (int j = Mr + et; j < p.M_pad; j += kEpilogueThreads) c_sm[j] = -INFINITY;
@@ -885,7 +890,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       // Weighted probabilities above 8 would leave the range of the polynomial exponential: with larger weights
       // everything is scaled down by a power of two, and the scores up again as they are written.
       float scale_log2 = 0.f;
-      if (p.row_weight) {
+      if (!MAXRED && p.row_weight) {
         float w = 0.f;
         for (int i = lane; i < p.R; i += 32) w = fmaxf(w, __ldg(p.row_weight + i));
 #pragma unroll
@@ -904,13 +909,13 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const long long u0 = (long long)(sg.l * p.Hkv + sg.h) * it.TT + tp[sg.s];
           const int n_tiles = tp[sg.s + 1] - tp[sg.s];
           const int b0 = (int)(u0 / per_cta), b1 = (int)((u0 + n_tiles - 1) / per_cta);
-          row_constants(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
+          row_constants<MAXRED>(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
                         (b1 - b0 + 1) * kEpilogueWarpgroups, et, scale_log2, c_sm, merge_sm);
         }
         asm volatile("bar.sync 1, 512;" ::: "memory");
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
         for (int t = pair; t < sg.nt && ok; t += 2) {
-          float2 acc[2] = {splat2(0.f), splat2(0.f)};
+          float2 acc[2] = {splat2(MAXRED ? -INFINITY : 0.f), splat2(MAXRED ? -INFINITY : 0.f)};
           const int key = (sg.t0 + t) * kTileKeys + row_in_tile;
           const bool in_window = CAUSAL && (sg.t0 + t + 1) * kTileKeys > sg.n - p.n_window;   // warp-uniform
           bool any = false;
@@ -979,7 +984,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             // The output was zero-filled; the two warpgroups of the pair contribute once per key.
             const float v0 = acc[0].x, v1 = acc[0].y, v2 = acc[1].x, v3 = acc[1].y;
             if (MAXRED) {
-              const float v = fmaxf(fmaxf(v0, v1), fmaxf(v2, v3)) * *scale_sm;
+              const float v = ex2(fmaxf(fmaxf(v0, v1), fmaxf(v2, v3)));
               asm volatile("red.global.max.u32 [%0], %1;" ::"l"(out + key), "r"(__float_as_uint(v)) : "memory");
             } else {
               const float v = ((v0 + v1) + (v2 + v3)) * *scale_sm;
