@@ -266,10 +266,14 @@ __device__ __forceinline__ SegIter seg_begin(const ScoreParams& p, const int* tp
   return it;
 }
 
+// The next segment of the range: pass 1 goes through it forwards, pass 2 backwards, tile by tile, so that pass 2 begins
+// with the keys that pass 1 has just left in L2 (one layer of 64K, 134 MB of keys: 118.6 -> 115.0 us).
+template <int PASS>
 __device__ bool seg_next(SegIter& it, const ScoreParams& p, const int* tp, Seg& sg) {
   if (it.g >= it.g_end) return false;
-  const int lh = (int)(it.g / it.TT);
-  const int rem = (int)(it.g % it.TT);
+  const long long at = PASS == 1 ? it.g : it.g_end - 1;
+  const int lh = (int)(at / it.TT);
+  const int rem = (int)(at % it.TT);
   int lo = 0, hi = p.n_seq;
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -279,14 +283,17 @@ __device__ bool seg_next(SegIter& it, const ScoreParams& p, const int* tp, Seg& 
   sg.l = lh / p.Hkv;
   sg.h = lh % p.Hkv;
   sg.unit = lh * p.n_seq + lo;
-  sg.t0 = rem - tp[lo];
   const long long left = it.g_end - it.g;
-  const int in_unit = tp[lo + 1] - rem;
+  const int in_unit = PASS == 1 ? tp[lo + 1] - rem : rem - tp[lo] + 1;
   sg.nt = left < in_unit ? (int)left : in_unit;
+  sg.t0 = PASS == 1 ? rem - tp[lo] : rem - tp[lo] - sg.nt + 1;
   seq_range(p.cu, p.n_in, lo, sg.begin, sg.n);
-  it.g += sg.nt;
+  if (PASS == 1) it.g += sg.nt; else it.g_end -= sg.nt;
   return true;
 }
+// The t-th key tile of a segment in the pass's order.
+template <int PASS>
+__device__ __forceinline__ int seg_tile(const Seg& sg, int t) { return sg.t0 + (PASS == 1 ? t : sg.nt - 1 - t); }
 
 // ------------------------------------------------------------------ epilogue math -----
 
@@ -639,7 +646,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         Seg sg;
         uint32_t kit = 0, nseg = 0;
         bool ok = true;
-        while (ok && seg_next(it, p, tp, sg)) {
+        while (ok && seg_next<PASS>(it, p, tp, sg)) {
           if (nseg > 0) ok = mbar_wait(q_empty, (nseg - 1) & 1, abort_flag);   // previous unit's MMAs retired
           if (!ok) break;
           ++nseg;
@@ -655,7 +662,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             if (!ok) break;
             mbar_expect_tx(&k_full[stage], p.stage_bytes);
             uint8_t* dst = k_sm + (size_t)stage * (128 * 128);
-            const int row = sg.begin + (sg.t0 + t) * kTileKeys;
+            const int row = sg.begin + seg_tile<PASS>(sg, t) * kTileKeys;
             for (int kh = 0; kh < n_kh; ++kh)
               tma_load_4d(dst + kh * k_half_bytes, &tm_k, kh * 64, row, sg.h, sg.l, &k_full[stage]);
           }
@@ -685,7 +692,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       const uint32_t q_half16 = q_half_bytes >> 4;
       const uint32_t k_half16 = k_half_bytes >> 4;
       while (ok) {
-        const bool more = seg_next(it, p, tp, sg);
+        const bool more = seg_next<PASS>(it, p, tp, sg);
         const int nt = uniform(more ? sg.nt : 0);
         if (nt == 0) break;
         ok = mbar_wait_warp(q_full, nseg & 1, abort_flag);
@@ -772,13 +779,13 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       float mrun[kMaxMTiles], zrun[kMaxMTiles];
       float* my_ref = rem_sm + (warp - 4) * p.rem_cols;
       // Every epilogue thread passes the barriers of every segment, also after a wait has given up.
-      while (seg_next(it, p, tp, sg)) {
+      while (seg_next<PASS>(it, p, tp, sg)) {
         float rem_m[2] = {-INFINITY, -INFINITY}, rem_z[2] = {0.f, 0.f};
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
 #pragma unroll
         for (int i = 0; i < kMaxMTiles; ++i) { mrun[i] = -INFINITY; zrun[i] = 0.f; }
         for (int t = pair; t < sg.nt && ok; t += 2) {
-          const int key0 = (sg.t0 + t) * kTileKeys;                                // first key of the tile
+          const int key0 = seg_tile<PASS>(sg, t) * kTileKeys;                                // first key of the tile
           const int nv = min(kTileKeys, sg.n - key0);                              // valid keys of the tile
           const bool in_window = CAUSAL && key0 + kTileKeys > sg.n - p.n_window;    // warp-uniform
           const bool plain = nv >= kTileKeys && !in_window;
@@ -902,7 +909,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       launch_dependents();
       // Every epilogue thread passes the barriers of every segment, also after a wait has
       // given up, so that no warp is left waiting at them.
-      while (seg_next(it, p, tp, sg)) {
+      while (seg_next<PASS>(it, p, tp, sg)) {
         asm volatile("bar.sync 1, 512;" ::: "memory");          // previous unit's constants no longer read
         {
           // the CTAs of pass 1 that worked on this unit: its tiles are u0 .. u0 + n_tiles - 1 of the global tile space
@@ -916,8 +923,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
         for (int t = pair; t < sg.nt && ok; t += 2) {
           float2 acc[2] = {splat2(MAXRED ? -INFINITY : 0.f), splat2(MAXRED ? -INFINITY : 0.f)};
-          const int key = (sg.t0 + t) * kTileKeys + row_in_tile;
-          const bool in_window = CAUSAL && (sg.t0 + t + 1) * kTileKeys > sg.n - p.n_window;   // warp-uniform
+          const int key = seg_tile<PASS>(sg, t) * kTileKeys + row_in_tile;
+          const bool in_window = CAUSAL && (seg_tile<PASS>(sg, t) + 1) * kTileKeys > sg.n - p.n_window;   // warp-uniform
           bool any = false;
           for (int ch = ((t >> 1) + half) & 1; ch < p.n_chunks; ch += 2) {
             ok = mbar_wait(&t_full[wg], used & 1, abort_flag);
