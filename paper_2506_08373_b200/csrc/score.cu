@@ -239,8 +239,13 @@ struct Seg {
 };
 
 struct SegIter {
-  long long g, g_end, per_cta;
+  long long g, g_end, per_cta, n_tiles;
   int TT;
+  // Whether a unit that ends before tile `end` is the last one that CTA `cta` worked on.
+  __device__ __forceinline__ bool last_segment(int cta, long long end) const {
+    const long long range_end = (cta + 1) * per_cta;
+    return end >= (range_end < n_tiles ? range_end : n_tiles);
+  }
 };
 
 // Tile-count prefix over sequences, tp[0..n_seq].
@@ -261,6 +266,7 @@ __device__ __forceinline__ SegIter seg_begin(const ScoreParams& p, const int* tp
   const long long N = (long long)p.L * p.Hkv * it.TT;
   const long long P = (N + n_ctas - 1) / n_ctas;
   it.per_cta = P;
+  it.n_tiles = N;
   it.g = P * cta;
   it.g_end = it.g + P < N ? it.g + P : N;
   return it;
@@ -503,8 +509,8 @@ __device__ __forceinline__ uint32_t hidden_columns(int row0, int R, int n_window
   return hidden;
 }
 
-// Combines the statistics that pass 1 left for a unit (one partial per warpgroup and CTA that worked
-// on it, `n` of them from `part`, M rows each) into minus the softmax constant of every row, in
+// Combines the statistics that pass 1 left for a unit (`n` partials of M rows each: one from each of the n_last + 1 CTAs
+// that worked on it, at every fourth place from `part`, or four from the last of them) into minus the softmax constant of every row, in
 // shared memory.  Called by all epilogue threads.  Every CTA of pass 2 does this for each of its
 // segments: a unit's partials are read from L2 by the few CTAs that share the unit, which takes
 // about a microsecond, where a kernel of its own between the passes took 4 to 22 (one layer of 64K:
@@ -519,7 +525,7 @@ __device__ __forceinline__ void fold_stats(float& m, float& z, float pm, float p
 constexpr int kMergeLoads = 16;       // in flight per thread; with 8, one layer of 12K (72 partials per row) spent 8 us here
 
 template <bool MAXRED>
-__device__ __forceinline__ void row_constants(const ScoreParams& p, const float2* __restrict__ part, int n, int et, float scale_log2, float* c_sm, float2* merge_sm) {
+__device__ __forceinline__ void row_constants(const ScoreParams& p, const float2* __restrict__ part, int n_last, int n, int et, float scale_log2, float* c_sm, float2* merge_sm) {
   const int Mr = (p.M + 31) & ~31;
   const int slices = p.merge_slots > 0 ? p.merge_slots / Mr : 1;
   for (int i0 = 0; i0 < p.M_pad; i0 += kEpilogueThreads) {
@@ -533,7 +539,7 @@ __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2
 #pragma unroll
         for (int u = 0; u < kMergeLoads; ++u) {
           const int c = c0 + u * slices;
-          v[u] = c < n ? __ldcg(part + (size_t)c * p.M + i) : make_float2(-INFINITY, 0.f);
+          v[u] = c < n ? __ldcg(part + (size_t)(min(c, n_last) * kEpilogueWarpgroups + max(c - n_last, 0)) * p.M + i) : make_float2(-INFINITY, 0.f);
         }
 #pragma unroll
         for (int u = 0; u < kMergeLoads; ++u) mx = fmaxf(mx, v[u].x);
@@ -857,14 +863,18 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             zrun[mt] = z;
           }
         }
+        // The statistics of a CTA's last segment are combined here, in the memory of the key ring, which nobody reads any
+        // more once every warpgroup has seen its last accumulator; those of the segments before it go out per
+        // warpgroup.  In a short call every segment is a last one, and pass 2 has a quarter of the partials
+        // to read (one layer of 12K: 72 -> 21 per row, spec_score 43.4 -> 39.1 us).
+        const bool last = it.g >= it.g_end;
+        float2* part = reinterpret_cast<float2*>(p.partial) + (size_t)(sg.unit + blockIdx.x) * kEpilogueWarpgroups * p.M;
+        float2* mine = (last ? reinterpret_cast<float2*>(k_sm) : part) + (size_t)wg * p.M;
+        if (last) asm volatile("bar.sync 1, 512;" ::: "memory");
         if (ok) {
-          float* dst = p.partial + ((size_t)(sg.unit + blockIdx.x) * kEpilogueWarpgroups + wg) * p.M * 2;
           for (int mt = 0; mt < n_full; ++mt) {
             const int row = mt * 128 + row_in_tile;
-            if (row < p.M) {
-              dst[row * 2 + 0] = mrun[mt];
-              dst[row * 2 + 1] = zrun[mt];
-            }
+            if (row < p.M) mine[row] = make_float2(mrun[mt], zrun[mt]);
           }
         }
         if (REM) {
@@ -881,11 +891,19 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               const int o = (wg * 4 + w) * p.rem_cols + row_in_tile;
               fold_stats(m, z, rem_sm[o], sums[o]);
             }
-            float* dst = p.partial + (((size_t)(sg.unit + blockIdx.x) * kEpilogueWarpgroups + wg) * p.M + row) * 2;
-            dst[0] = m;
-            dst[1] = z;
+            mine[row] = make_float2(m, z);
           }
           asm volatile("bar.sync %0, 128;" ::"r"(2 + wg) : "memory");
+        }
+        if (last) {
+          asm volatile("bar.sync 1, 512;" ::: "memory");
+          const float2* of = reinterpret_cast<const float2*>(k_sm);
+          for (int row = et; row < p.M && ok; row += kEpilogueThreads) {
+            float2 v = of[row];
+#pragma unroll
+            for (int w = 1; w < kEpilogueWarpgroups; ++w) fold_stats(v.x, v.y, of[(size_t)w * p.M + row].x, of[(size_t)w * p.M + row].y);
+            part[row] = v;
+          }
         }
       }
     } else {
@@ -917,7 +935,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const int n_tiles = tp[sg.s + 1] - tp[sg.s];
           const int b0 = (int)(u0 / per_cta), b1 = (int)((u0 + n_tiles - 1) / per_cta);
           row_constants<MAXRED>(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
-                        (b1 - b0 + 1) * kEpilogueWarpgroups, et, scale_log2, c_sm, merge_sm);
+                        b1 - b0, b1 - b0 + (it.last_segment(b1, u0 + n_tiles) ? 1 : kEpilogueWarpgroups), et, scale_log2, c_sm, merge_sm);
         }
         asm volatile("bar.sync 1, 512;" ::: "memory");
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
