@@ -78,6 +78,7 @@ struct ScoreParams {
   long long T;
   int n_in, n_seq, L, Hq, Hkv, G, R, M, M_pad, d;   // M, M_pad: the query rows of this launch, rows [row0, row0 + M) of every unit
   int row0;
+  int pieces;            // CTAs per unit, each of which has a share of that unit only (0: equal shares of the whole tile space)
   int n_window;          // causal kernels: window row r sees keys up to position n - n_window + r only
   int merge_slots;       // threads that share the merging of a unit's statistics when there are fewer rows than threads (0: none do)
   int n_stages, n_chunks, cw_last;   // pass 2: chunks of 128 query rows, the last of cw_last (a multiple of 16)
@@ -264,9 +265,20 @@ __device__ __forceinline__ SegIter seg_begin(const ScoreParams& p, const int* tp
   SegIter it;
   it.TT = tp[p.n_seq];
   const long long N = (long long)p.L * p.Hkv * it.TT;
+  it.n_tiles = N;
+  if (p.pieces > 0) {                                      // every unit cut evenly among as many CTAs of its own
+    const int unit = cta / p.pieces, i = cta - unit * p.pieces;
+    const int base = it.TT / p.pieces, extra = it.TT - base * p.pieces;
+    it.per_cta = 0;
+    it.g = it.g_end = 0;
+    if (unit < p.L * p.Hkv) {
+      it.g = (long long)unit * it.TT + i * base + min(i, extra);
+      it.g_end = it.g + base + (i < extra);
+    }
+    return it;
+  }
   const long long P = (N + n_ctas - 1) / n_ctas;
   it.per_cta = P;
-  it.n_tiles = N;
   it.g = P * cta;
   it.g_end = it.g + P < N ? it.g + P : N;
   return it;
@@ -854,7 +866,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                 if (c * 32 >= nv) break;                                    // warp-uniform
                 tmem_ld32(my_taddr + c * 32, ra);
                 tmem_wait(ra);
-                if (vis - c * 32 > 0) stats_general(ra, min(vis - c * 32, 32), p.a, m, z);
+                if (__all_sync(0xffffffffu, vis - c * 32 >= 32)) stats_update(ra, p.a, m, z);
+                else if (vis - c * 32 > 0) stats_general(ra, min(vis - c * 32, 32), p.a, m, z);
               }
               tc_fence_before();
               arrive_lane0(&t_empty[wg], lane);
@@ -923,20 +936,27 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         scale_log2 = fminf(fmaxf(floorf(log2f(w)) - 1.f, 0.f), 126.f);
       }
       if (et == 0) *scale_sm = exp2f(scale_log2);               // read after the barriers below
-      wait_for_previous_grid();                                 // pass 1: statistics and zeroed scores
-      launch_dependents();
+      bool waited = false;
       // Every epilogue thread passes the barriers of every segment, also after a wait has
       // given up, so that no warp is left waiting at them.
       while (seg_next<PASS>(it, p, tp, sg)) {
-        asm volatile("bar.sync 1, 512;" ::: "memory");          // previous unit's constants no longer read
-        {
-          // the CTAs of pass 1 that worked on this unit: its tiles are u0 .. u0 + n_tiles - 1 of the global tile space
+        // the CTAs of pass 1 that worked on this unit: its tiles are u0 .. u0 + n_tiles - 1 of the global tile space
+        int b0 = sg.unit * p.pieces, b1 = b0 + p.pieces - 1, n_part = p.pieces;
+        if (p.pieces == 0) {
           const long long u0 = (long long)(sg.l * p.Hkv + sg.h) * it.TT + tp[sg.s];
           const int n_tiles = tp[sg.s + 1] - tp[sg.s];
-          const int b0 = (int)(u0 / per_cta), b1 = (int)((u0 + n_tiles - 1) / per_cta);
-          row_constants<MAXRED>(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
-                        b1 - b0, b1 - b0 + (it.last_segment(b1, u0 + n_tiles) ? 1 : kEpilogueWarpgroups), et, scale_log2, c_sm, merge_sm);
+          b0 = (int)(u0 / per_cta);
+          b1 = (int)((u0 + n_tiles - 1) / per_cta);
+          n_part = b1 - b0 + (it.last_segment(b1, u0 + n_tiles) ? 1 : kEpilogueWarpgroups);
         }
+        if (!waited) {
+          waited = true;
+          wait_for_previous_grid();                             // pass 1: statistics and zeroed scores
+          launch_dependents();
+        }
+        asm volatile("bar.sync 1, 512;" ::: "memory");          // previous unit's constants no longer read
+        row_constants<MAXRED>(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
+                              b1 - b0, n_part, et, scale_log2, c_sm, merge_sm);
         asm volatile("bar.sync 1, 512;" ::: "memory");
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
         for (int t = pair; t < sg.nt && ok; t += 2) {
@@ -1017,6 +1037,10 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             }
           }
         }
+      }
+      if (!waited) {                                            // nothing to do: the grid still ends after the one before it
+        wait_for_previous_grid();
+        launch_dependents();
       }
     }
   }
@@ -1154,6 +1178,14 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
       }
       __atomic_store_n(&set[dev], 1, __ATOMIC_RELEASE);
     }
+  }
+  // A CTA whose share spans two units pays for a second set of queries and constants (5 us of a short call), so units
+  // of one length, few to a GPU, are cut each among CTAs of its own, if that costs no CTA more than two tiles.
+  p.pieces = 0;
+  if (!pr->cu_seqlens) {
+    const int64_t units = (int64_t)pr->n_layers * pr->n_kv_heads, tiles_unit = (pr->n_in + kTileKeys - 1) / kTileKeys;
+    const int64_t pieces = std::min(n_ctas / units, tiles_unit);
+    if (pieces >= 2 && (tiles_unit + pieces - 1) / pieces <= (units * tiles_unit + n_ctas - 1) / n_ctas + 2) p.pieces = (int)pieces;
   }
   for (int g = 0; g < n_groups; ++g) {
     p.row0 = g * rows_group;
