@@ -9,8 +9,8 @@
 // gives a floor under the threshold; the keys at or above it, about one and a half to two and a half
 // times the budget, are sent to every CTA as well, and each finds the exact threshold among them by
 // itself (find_threshold).  That takes two cluster barriers; the radix select over distributed
-// histograms that it replaced took four, and added every non-empty bin into all CTAs (32768 token
-// scores, 1024 kept: 25 -> CLUS1 us).  The radix select (11 + 11 + 10 bits) is what remains for units whose
+// histograms that it replaced took four, and added every non-empty bin into all CTAs (keep set of 1024 among 32768 tokens
+// of 16 layers, with the reduction: 29 -> 18 us).  The radix select (11 + 11 + 10 bits) is what remains for units whose
 // floor lets through too few or too many keys, as massive ties can.  Winners are written in ascending
 // position: the CTAs exchange their counts, and each one emits its own winners behind those
 // of the CTAs before it; ties at the threshold go to the lower position.  The scores are read
@@ -259,6 +259,9 @@ __device__ void exchange_counts(const ClusterCtx& c, int a, int b, int& a_before
   }
 }
 
+// MODE 0: index lists, 1: keep set.  Two kernels, because a selection behind a scoring pass finds none of its instructions in
+// the SM's caches: each fetches only what it executes (keep set of 1024 among 8192 tokens there: 19.4 -> 18.4 us).
+template <int MODE>
 __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const ClusterSelParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   ClusterCtx c;
@@ -277,7 +280,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   uint32_t* n_held = reinterpret_cast<uint32_t*>(misc + 110);
   uint32_t* bitmap = reinterpret_cast<uint32_t*>(misc + kClMiscInts);
   const int cap_pad = cluster_cap_pad(p.cap);
-  float* raw = reinterpret_cast<float*>(bitmap + cluster_bitmap_words(p.cap, p.mode));
+  float* raw = reinterpret_cast<float*>(bitmap + cluster_bitmap_words(p.cap, MODE));
   uint32_t* keys_w = p.inplace ? reinterpret_cast<uint32_t*>(raw + p.halo_l)
                                : reinterpret_cast<uint32_t*>(raw + p.halo_l + cap_pad + p.halo_r + 32);
   uint32_t* held = p.inplace ? reinterpret_cast<uint32_t*>(raw + p.halo_l + cap_pad + p.halo_r + 32) : keys_w + cap_pad + 32;
@@ -290,7 +293,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   const uint32_t lt_mask = (1u << lane) - 1u;
   // ---- clear what other CTAs will add to, then let them know this CTA is up
   reinterpret_cast<uint4*>(sm.hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
-  if (p.mode == 1)
+  if (MODE == 1)
     for (int w = tid; w < cluster_bitmap_words(p.cap, 1); w += kSelThreads) bitmap[w] = 0;
   if (tid == 0) {
     *timed_out = 0;
@@ -326,9 +329,9 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   c.j_hi = max(x1 - x0, 0);
 
   // budgets
-  const int n_budgets = p.mode == 0 && p.n_vert > 0 ? 2 : 1;
+  const int n_budgets = MODE == 0 && p.n_vert > 0 ? 2 : 1;
   int take[2];
-  take[0] = p.mode == 0 ? min(p.c_max - forced, e) : min(p.c_max, e);
+  take[0] = MODE == 0 ? min(p.c_max - forced, e) : min(p.c_max, e);
   take[1] = min(p.n_vert, e);
   bool selects = false;
   for (int b = 0; b < n_budgets; ++b) selects = selects || (take[b] > 0 && take[b] < e);
@@ -490,7 +493,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
 
   const int slab = ((CL + kSelThreads - 1) / kSelThreads) * 32;    // local positions per warp in the ordered sweeps
 
-  if (p.mode == 0) {
+  if (MODE == 0) {
     for (int b = 0; b < n_budgets; ++b) {
       int32_t* idx = (b == 0 ? p.idx_out + (int64_t)unit * p.c_max : p.vert_out + (int64_t)unit * p.n_vert);
       int32_t* cnt = b == 0 ? p.count_out : p.vert_count_out;
@@ -660,7 +663,7 @@ __global__ void __launch_bounds__(kSelThreads) pool_topk_generic_kernel(TopkPara
 // Token score: reduction over all layers and KV heads.  HBM-bound: every score is read once.  The eight warps of a
 // CTA share the vectors of 128 tokens, 16 loads in flight per lane; their partial results are
 // combined in warp order, so the result does not depend on timing.  (One thread per token over all
-// vectors left most of the GPU idle: 128 vectors of 32768 tokens 12.4 -> REDUS us.)
+// vectors left most of the GPU idle: 128 vectors of 32768 tokens 13.0 -> 6.2 us.)
 constexpr int kReduceTokens = 128;
 constexpr int kReduceWarps = 8;
 
@@ -880,8 +883,8 @@ static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int
   // The floor lets through 1.3 (large budgets) to 2.5 times the budget; short units send all of their keys.  Where
   // there is no room for that (budgets of a third of a very long sequence), the radix select does without.
   const int64_t room = ((int64_t)kSmemLimit - (int64_t)pl.smem) / 4;
-  const int64_t want = std::min<int64_t>(5 * (int64_t)budget / 2 + 1024, x_max + 1);
-  pl.cand_cap = pl.fits ? (int)(std::min(want, room) & ~(int64_t)3) : 0;
+  const int64_t want = std::min<int64_t>(5 * (int64_t)budget / 2 + 1024, x_max + 1 + 3) & ~(int64_t)3;
+  pl.cand_cap = pl.fits ? (int)std::min(want, room & ~(int64_t)3) : 0;
   if (pl.cand_cap < std::min<int64_t>(want, 3 * (int64_t)budget / 2)) pl.cand_cap = 0;
   pl.smem += (size_t)pl.cand_cap * 4;
   return pl;
@@ -889,18 +892,15 @@ static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int
 
 // One-time function attributes of the cluster kernel on the current device.
 static int prepare_cluster_kernel(int* max_cs_out) {
-  static int state[kMaxDevices] = {0};                     // 0: not set, 8 / 16: largest cluster size usable
+  static int state[kMaxDevices] = {0};                     // 0: not set, else the largest cluster size usable
   int dev = 0;
   SPEC_CUDA_OK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= kMaxDevices) return fail(SPEC_ERR_UNSUPPORTED, "device ordinal %d is not supported", dev);
   int st = __atomic_load_n(&state[dev], __ATOMIC_ACQUIRE);
   if (!st) {
-    SPEC_CUDA_OK(cudaFuncSetAttribute(cluster_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
-    st = 8;
-    if (kClusterUse > 8) {
-      if (cudaFuncSetAttribute(cluster_select_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) st = kClusterUse;
-      else cudaGetLastError();
-    }
+    SPEC_CUDA_OK(cudaFuncSetAttribute(cluster_select_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
+    SPEC_CUDA_OK(cudaFuncSetAttribute(cluster_select_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit));
+    st = kClusterUse;
     __atomic_store_n(&state[dev], st, __ATOMIC_RELEASE);
   }
   *max_cs_out = st;
@@ -923,7 +923,7 @@ static int launch_cluster(const ClusterSelParams& p, int64_t n_units, const Clus
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  SPEC_CUDA_OK(cudaLaunchKernelEx(&cfg, cluster_select_kernel, p));
+  SPEC_CUDA_OK(cudaLaunchKernelEx(&cfg, p.mode == 0 ? cluster_select_kernel<0> : cluster_select_kernel<1>, p));
   return SPEC_OK;
 }
 

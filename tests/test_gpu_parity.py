@@ -144,6 +144,29 @@ def test_score_rows_behind_the_last_full_block(B, W, oracle, rows, d):
                 assert_scores_close(got[l:l + 1, h:h + 1].cpu().numpy(), ref, cu)
 
 
+@pytest.mark.parametrize("heads,n", [(1, 20000), (3, 130), (8, 2304), (8, 2305), (49, 1300), (50, 12800), (74, 385), (75, 385)])
+def test_score_units_cut_among_ctas(B, W, oracle, heads, n):
+    """Few units of one length are cut each among CTAs of its own (148 CTAs, at least two per unit, at most two tiles more
+    than equal shares: all but the sixth and the last pair), others into equal shares of all tiles.  Pieces of one
+    tile, pieces that stay empty and partial last tiles, both reductions, with and without the causal window."""
+    rows, window, d = 16, 9, 128
+    gen = torch.Generator().manual_seed(n)
+    q = torch.randn(1, 1, 2 * heads, rows, d, generator=gen).to(torch.bfloat16).cuda()
+    k = torch.randn(1, heads, n, d, generator=gen).to(torch.bfloat16).cuda()
+    pr = B.make_problem(n_layers=1, n_q_heads=2 * heads, n_kv_heads=heads, head_dim=d, n_lookahead=rows - window, n_window=window,
+                        softmax_scale=d ** -0.5, total_tokens=n, n_in=n, n_seq=1, k=k)
+    ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for reduce, causal in ((0, 0), (0, 1), (1, 0)):
+        got = torch.full((1, heads, n), float("nan"), device="cuda")
+        B.spec_score(pr, q, k, got, ws, reduce=reduce, causal_window=causal, status_word=status)
+        assert status.item() == 0
+        for h in sorted({0, heads // 2, heads - 1}):
+            ref = oracle.spec_score(bits(q[:, :, 2 * h:2 * h + 2]), bits(k[:, h:h + 1]), [0, n], rows - window, window, d ** -0.5,
+                                    mode=reduce, causal_window=bool(causal))
+            assert_scores_close(got[:, h:h + 1].cpu().numpy(), ref, [0, n])
+
+
 @pytest.mark.parametrize("reduce", [0, 1])
 @pytest.mark.parametrize("case", ["large_weights", "rising_logits", "falling_logits", "steep_logits"])
 def test_score_range_of_the_exponentials(B, W, oracle, case, reduce):
@@ -793,6 +816,20 @@ def test_topk_short_units_in_one_cta_and_streamed(B, W, oracle):
     z[:, :, 100:140] = 0.75                                          # a run of ties around the threshold of some units
     run_topk_case(B, W, oracle, z, [0, 3000], 0, 7, 256, 0)
     run_vert_case(B, oracle, z, [0, 1000, 3000], 7, 128, 8, 150)
+
+
+@pytest.mark.parametrize("n,k,c_max,units", [
+    (1013, 5, 100, 1), (1014, 5, 100, 1),                        # one CTA, the first size for two
+    (4080, 9, 4000, 2), (4081, 9, 4000, 2),                      # eight CTAs of the least share, all keys sent
+    (33000, 5, 1000, 3), (33000, 5, 1000, 70),                   # the same units in clusters of eight and of two
+    (150000, 5, 9000, 1), (150000, 5, 9500, 1),                  # the least memory for candidates, and none
+    (75000, 7, 12480, 1), (75000, 7, 12481, 1),                  # the largest budget that is streamed
+    (524285, 7, 700, 1), (524286, 7, 700, 1),                    # one round per sweeping warp, two
+    (1048573, 7, 700, 1), (1048574, 7, 700, 1)])                 # the longest unit that is streamed
+def test_topk_at_the_limits_of_the_selection_kernels(B, W, oracle, n, k, c_max, units):
+    x = (np.random.default_rng(n + units).random((1, units, n)) ** 5).astype(np.float32)
+    x[:, :, n // 2:n // 2 + 60] = x[:, :, :1]                     # a run of equal keys
+    run_topk_case(B, W, oracle, x, [0, n], 0, k, c_max, min(c_max // 2, 33))
 
 
 def test_topk_unit_too_long_for_a_cluster_takes_the_generic_path(B, W, oracle):
