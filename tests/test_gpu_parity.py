@@ -832,6 +832,16 @@ def test_topk_at_the_limits_of_the_selection_kernels(B, W, oracle, n, k, c_max, 
     run_topk_case(B, W, oracle, x, [0, n], 0, k, c_max, min(c_max // 2, 33))
 
 
+@pytest.mark.parametrize("spread", [2.0 ** -4, 2.0 ** -7, 2.0 ** -12])
+def test_topk_scores_that_differ_little(B, W, oracle, spread):
+    """Sampled keys within one or a few bins of the floor's histogram, in all three selections: above the bin's
+    middle, at its edges, and (the narrowest) with fewer distinct values than positions."""
+    rng = np.random.default_rng(5)
+    for n, k, c_max in ((4000, 7, 500), (40000, 7, 3000), (40000, 9, 3000)):
+        x = (1.0 + spread * rng.random((1, 3, n)) ** np.array([0.2, 1.0, 5.0])[None, :, None]).astype(np.float32)
+        run_topk_case(B, W, oracle, x, [0, n], 0, k, c_max, 0)
+
+
 def test_topk_unit_too_long_for_a_cluster_takes_the_generic_path(B, W, oracle):
     rng = np.random.default_rng(41)
     n = 2_000_003
