@@ -6,8 +6,8 @@
 // raw score at or above the floor: a sweep over the scores costs one comparison per score, and
 // pooled values are only ever computed for candidates.  A warp holds 1024 scores in registers (eight
 // float4 per lane), turns them into hit bits, widens the bits by three positions on either side
-// (bit arithmetic on eight nibbles at a time), ranks the candidates in position order with one packed
-// scan and pools them from its registers.
+// (bit arithmetic on eight nibbles at a time), lists the groups of four positions that hold candidates and
+// pools and ranks those, a group to a lane.
 //
 // Long units take three kernels on the caller's stream, chained as programmatic dependents; no CTA
 // ever waits for another:
@@ -38,6 +38,7 @@ namespace spec {
 
 constexpr int kWarpSteps = 8;                    // 128-position steps a warp holds in registers
 constexpr int kWarpSpan = kWarpSteps * 128;
+constexpr int kListSlots = kWarpSpan / 4;         // groups of four positions of a warp
 constexpr int kMaxSamples = 4096;
 constexpr uint32_t kNoSelection = 0xFFFFFFFFu;   // floor value of a unit that keeps everything or nothing
 
@@ -187,13 +188,20 @@ __device__ __forceinline__ float score_at(const UnitGeom& g, int x) {
 __device__ __forceinline__ void load_scores(const UnitGeom& g, int x0, int n_steps, int lane, WarpScores& w) {
   w.x0 = x0;
   w.n_steps = n_steps;
-  const bool inside = x0 >= g.mis && x0 + n_steps * 128 <= g.X;          // warp-uniform
+  if (n_steps == kWarpSteps && x0 - 4 >= g.mis && x0 + kWarpSpan + 4 <= g.X) {    // warp-uniform: full, with neighbours on both sides
+    const float* at = g.src + (x0 - g.mis);
+#pragma unroll
+    for (int k = 0; k < kWarpSteps; ++k) w.v[k] = __ldcg(reinterpret_cast<const float4*>(at) + k * 32 + lane);
+    w.before = __ldcg(at - 3 + min(lane, 2));
+    w.after = __ldcg(at + kWarpSpan + min(lane, 2));
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < kWarpSteps; ++k) {
     w.v[k] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
     if (k < n_steps) {
       const int x = x0 + k * 128 + lane * 4;
-      if (inside || (x >= g.mis && x + 4 <= g.X)) w.v[k] = __ldcg(reinterpret_cast<const float4*>(g.src + (x - g.mis)));
+      if (x >= g.mis && x + 4 <= g.X) w.v[k] = __ldcg(reinterpret_cast<const float4*>(g.src + (x - g.mis)));
       else w.v[k] = make_float4(score_at(g, x), score_at(g, x + 1), score_at(g, x + 2), score_at(g, x + 3));
     }
   }
@@ -201,27 +209,30 @@ __device__ __forceinline__ void load_scores(const UnitGeom& g, int x0, int n_ste
   w.after = lane < 3 ? score_at(g, x0 + n_steps * 128 + lane) : -INFINITY;
 }
 
-// Candidate bits of this lane (bit 4k + u: its position u of step k), the lane's place behind the candidates of
-// lower lanes for each step (packed bytes: even steps, odd steps), and the totals per step likewise.
+// Candidate bits of this lane (bit 4k + u: its position u of step k), and how many the warp has.
 struct WarpCandidates {
-  uint32_t mask, pre_even, pre_odd, tot_even, tot_odd;
+  uint32_t mask;
   int total;
 };
 
+// Sets `bit` if v >= floor_f, in two instructions; written in C++, the bit is selected first and costs a third.
+__device__ __forceinline__ void set_if_reached(uint32_t& bits, float v, float floor_f, uint32_t bit) {
+  asm("{\n.reg .pred p;\nsetp.ge.f32 p, %1, %2;\n@p or.b32 %0, %0, %3;\n}" : "+r"(bits) : "f"(v), "f"(floor_f), "r"(bit));
+}
 __device__ __forceinline__ WarpCandidates find_candidates(const UnitGeom& g, const WarpScores& w, float floor_f, int lane) {
   constexpr uint32_t ones = 0x11111111u;
   uint32_t hit = 0;
 #pragma unroll
   for (int k = 0; k < kWarpSteps; ++k) {
-    if (w.v[k].x >= floor_f) hit |= 1u << (4 * k);
-    if (w.v[k].y >= floor_f) hit |= 2u << (4 * k);
-    if (w.v[k].z >= floor_f) hit |= 4u << (4 * k);
-    if (w.v[k].w >= floor_f) hit |= 8u << (4 * k);
+    set_if_reached(hit, w.v[k].x, floor_f, 1u << (4 * k));
+    set_if_reached(hit, w.v[k].y, floor_f, 2u << (4 * k));
+    set_if_reached(hit, w.v[k].z, floor_f, 4u << (4 * k));
+    set_if_reached(hit, w.v[k].w, floor_f, 8u << (4 * k));
   }
   const uint32_t near_l = __ballot_sync(0xffffffffu, w.before >= floor_f) & 7u;
   const uint32_t near_r = __ballot_sync(0xffffffffu, w.after >= floor_f) & 7u;
   WarpCandidates c;
-  c.mask = c.pre_even = c.pre_odd = c.tot_even = c.tot_odd = 0;
+  c.mask = 0;
   c.total = 0;
   if (!__any_sync(0xffffffffu, hit != 0) && near_l == 0 && near_r == 0) return c;
   // the nibbles to the left and to the right of each of mine: neighbouring lanes, or the neighbouring step
@@ -243,58 +254,69 @@ __device__ __forceinline__ WarpCandidates find_candidates(const UnitGeom& g, con
       c.mask &= ~((ok ^ 0xfu) << (4 * k));
     }
   }
-  // candidates per step, in the nibbles, then one byte each; a step has at most 128
-  uint32_t n4 = c.mask - ((c.mask >> 1) & 0x55555555u);
-  n4 = (n4 & 0x33333333u) + ((n4 >> 2) & 0x33333333u);
-  const uint32_t even = n4 & 0x0f0f0f0fu, odd = (n4 >> 4) & 0x0f0f0f0fu;
-  c.pre_even = even;
-  c.pre_odd = odd;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t a = __shfl_up_sync(0xffffffffu, c.pre_even, o), b = __shfl_up_sync(0xffffffffu, c.pre_odd, o);
-    if (lane >= o) { c.pre_even += a; c.pre_odd += b; }
-  }
-  c.tot_even = __shfl_sync(0xffffffffu, c.pre_even, 31);
-  c.tot_odd = __shfl_sync(0xffffffffu, c.pre_odd, 31);
-  c.pre_even -= even;
-  c.pre_odd -= odd;
-  c.total = (int)__dp4a(c.tot_even, 0x01010101u, __dp4a(c.tot_odd, 0x01010101u, 0u));
+  c.total = (int)__reduce_add_sync(0xffffffffu, (uint32_t)__popc(c.mask));
   return c;
 }
 
-// Calls put(rank, key, position) for every candidate of the warp, rank in position order from `base` on.
-// Every lane walks its own nibbles, most lanes none and few more than one, and reads the twelve scores
-// around each again from L2: a step-by-step walk of the whole warp over its registers (18 shuffles a step)
-// was three times the instructions.
+// Calls put(rank, key, position) for every candidate of the warp, rank in position order from `base` on.  The groups of
+// four positions that hold candidates (a dozen of 256, as a rule) are listed in position order in
+// shared memory; every lane takes one from the list, pools its four positions from the twelve scores around
+// them, read again from L2, and ranks them by a scan over the list.  (The sweep is bound by the instructions that it
+// issues.  With every lane walking its own groups, two to four turns of the loop for the warp, it took 674 per
+// 1024 positions and 35.6 us for 256 units of 131072; with this, a short path for chunks inside a unit and two
+// instructions per score in find_candidates, 530 and 27.4.  Leaving out steps without candidates, or a persistent
+// sweep that copies its chunks ahead into shared memory, was slower.)
 template <class Put>
-__device__ __forceinline__ void pool_candidates(const UnitGeom& g, const WarpScores& w, const WarpCandidates& c, int base, int lane, Put put) {
-  uint32_t left = c.mask;
-  while (left) {
-    const int k = (__ffs((int)left) - 1) >> 2;
-    const uint32_t nib = (left >> (4 * k)) & 15u;
-    left &= ~(15u << (4 * k));
-    const int x0 = w.x0 + k * 128 + lane * 4;
-    float4 pv, cv, nv;
-    if (x0 - 4 >= g.mis && x0 + 8 <= g.X) {
-      const float4* at = reinterpret_cast<const float4*>(g.src + (x0 - g.mis));
-      pv = __ldcg(at - 1); cv = __ldcg(at); nv = __ldcg(at + 1);
-    } else {
-      pv = make_float4(0.f, score_at(g, x0 - 3), score_at(g, x0 - 2), score_at(g, x0 - 1));
-      cv = make_float4(score_at(g, x0), score_at(g, x0 + 1), score_at(g, x0 + 2), score_at(g, x0 + 3));
-      nv = make_float4(score_at(g, x0 + 4), score_at(g, x0 + 5), score_at(g, x0 + 6), 0.f);
-    }
-    // candidates of earlier steps (even steps below k: (k + 1) / 2 of them, odd ones: k / 2), of lower lanes in this one
-    const uint32_t in_even = (uint32_t)((1ull << (8 * ((k + 1) >> 1))) - 1ull), in_odd = (uint32_t)((1ull << (8 * (k >> 1))) - 1ull);
-    int at = base + (int)__dp4a(c.tot_even & in_even, 0x01010101u, __dp4a(c.tot_odd & in_odd, 0x01010101u, 0u)) +
-             (int)(((k & 1 ? c.pre_odd : c.pre_even) >> (8 * (k >> 1))) & 255u);
-    // the four windows share the middle four; neighbouring windows share a pair on either side
-    const float mid = fmax3(cv.x, cv.y, fmaxf(cv.z, cv.w)), l12 = fmaxf(pv.z, pv.w), r78 = fmaxf(nv.x, nv.y);
-    const float v4[4] = {fmax3(mid, pv.y, l12), fmax3(mid, l12, nv.x), fmax3(mid, pv.w, r78), fmax3(mid, r78, nv.z)};
-    const int j0 = x0 - g.mis;
+__device__ __forceinline__ void pool_candidates(const UnitGeom& g, const WarpScores& w, const WarpCandidates& c, int base, int lane, uint16_t* list, Put put) {
+  if (c.total == 0) return;                                // warp-uniform
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  int count = 0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (nib & (1u << u)) { put(at, to_key(v4[u]), j0 + u); ++at; }
+  for (int k = 0; k < kWarpSteps; ++k) {
+    const uint32_t nib = (c.mask >> (4 * k)) & 15u;
+    const uint32_t has = __ballot_sync(0xffffffffu, nib != 0);
+    if (nib) list[count + __popc(has & lt_mask)] = (uint16_t)(nib | ((uint32_t)(k * 32 + lane) << 4));
+    count += __popc(has);
   }
+  __syncwarp();
+#pragma unroll 1
+  for (int i0 = 0; i0 < count; i0 += 32) {
+    const uint32_t entry = i0 + lane < count ? list[i0 + lane] : 0u;
+    const uint32_t nib = entry & 15u;
+    const int x0 = w.x0 + (int)(entry >> 4) * 4;
+    float4 pv, cv, nv;
+    if (nib != 0) {
+      if (x0 - 4 >= g.mis && x0 + 8 <= g.X) {
+        const float4* at = reinterpret_cast<const float4*>(g.src + (x0 - g.mis));
+        pv = __ldcg(at - 1); cv = __ldcg(at); nv = __ldcg(at + 1);
+      } else {
+        pv = make_float4(0.f, score_at(g, x0 - 3), score_at(g, x0 - 2), score_at(g, x0 - 1));
+        cv = make_float4(score_at(g, x0), score_at(g, x0 + 1), score_at(g, x0 + 2), score_at(g, x0 + 3));
+        nv = make_float4(score_at(g, x0 + 4), score_at(g, x0 + 5), score_at(g, x0 + 6), 0.f);
+      }
+    }
+    const int mine = __popc(nib);
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      asm volatile("{\n.reg .pred p;\n.reg .b32 t;\nshfl.sync.up.b32 t|p, %0, %1, 0, 0xffffffff;\n@p add.s32 %0, %0, t;\n}" : "+r"(incl) : "r"(o));
+    }
+    const int at = base + incl - mine;
+    base += __shfl_sync(0xffffffffu, incl, 31);
+    if (nib != 0) {
+      // the four windows share the middle four; neighbouring windows share a pair on either side
+      const float mid = fmax3(cv.x, cv.y, fmaxf(cv.z, cv.w)), l12 = fmaxf(pv.z, pv.w), r78 = fmaxf(nv.x, nv.y);
+      const uint32_t k4[4] = {to_key(fmax3(mid, pv.y, l12)), to_key(fmax3(mid, l12, nv.x)), to_key(fmax3(mid, pv.w, r78)), to_key(fmax3(mid, r78, nv.z))};
+      const int j0 = x0 - g.mis;
+      int to[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) to[u] = at + __popc(nib & ((1u << u) - 1u));
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (nib & (1u << u)) put(to[u], k4[u], j0 + u);
+    }
+  }
+  __syncwarp();                                            // the list is free again
 }
 
 // ---------------------------------------------------------------- 1. the floor -------
@@ -353,14 +375,12 @@ __global__ void __launch_bounds__(kSelThreads) sample_floor_kernel(const StreamP
 
 // ---------------------------------------------------------------- 2. the sweep -------
 
-#ifndef SPEC_SWEEP_CTAS
-#define SPEC_SWEEP_CTAS 8
-#endif
-constexpr int kSweepThreads = 128;
+constexpr int kSweepThreads = 128, kSweepCtas = 8;        // 6 CTAs to an SM: 135.0 us for selection and gather of 256 units of 131072, 8: 133.0, 10: 136.1
 constexpr int kSweepWarps = kSweepThreads / 32;
 
-// One warp per chunk; warps never meet.  No shared memory: a lane's eight 16-byte loads are in flight at once.
-__global__ void __launch_bounds__(kSweepThreads, SPEC_SWEEP_CTAS) stream_sweep_kernel(const StreamParams p) {
+// One warp per chunk; warps never meet.  A lane's eight 16-byte loads are in flight at once.
+__global__ void __launch_bounds__(kSweepThreads, kSweepCtas) stream_sweep_kernel(const StreamParams p) {
+  __shared__ uint16_t lists[kSweepWarps][kListSlots];
   const int lane = threadIdx.x & 31;
   const int chunk_id = blockIdx.x * kSweepWarps + (threadIdx.x >> 5);
   const int row = blockIdx.y, s = blockIdx.z;
@@ -380,7 +400,9 @@ __global__ void __launch_bounds__(kSweepThreads, SPEC_SWEEP_CTAS) stream_sweep_k
   int n = 0;
   for (int r = 0;; ++r) {
     const WarpCandidates c = find_candidates(g, w, floor_f, lane);
-    pool_candidates(g, w, c, n, lane, [&](int at, uint32_t key, int j) { dst[at] = make_uint2(key, (uint32_t)j); });
+    pool_candidates(g, w, c, n, lane, lists[threadIdx.x >> 5], [&](int at, uint32_t key, int j) {
+      *reinterpret_cast<uint2*>(reinterpret_cast<char*>(dst) + (uint32_t)at * 8u) = make_uint2(key, (uint32_t)j);
+    });
     n += c.total;
     const int x = c0 + (r + 1) * kWarpSpan;
     if (r + 1 >= p.rounds || x >= g.X) break;
@@ -520,7 +542,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) unit_select_kernel(const Strea
     const int base = (int)__reduce_add_sync(0xffffffffu, (uint32_t)(lane < warp ? wt : 0));
     failed = n > p.held_cap;
     if (!failed) {
-      pool_candidates(g, w, c, base, lane, [&](int at, uint32_t key, int j) {
+      pool_candidates(g, w, c, base, lane, reinterpret_cast<uint16_t*>(pos + p.held_cap) + warp * kListSlots, [&](int at, uint32_t key, int j) {
         keys[at] = key;
         pos[at] = (uint32_t)j;
         top = max(top, key);
@@ -548,7 +570,7 @@ static int run_unit_topk(const spec_problem* pr, StreamParams p, cudaStream_t st
   if (n_units < 1 || n_units > 0x7fffffff) return SPEC_OK;
   // the floor, from one sample in 16, lets through 1.4 (budget 2048) to 2.5 (256) times the budget
   p.held_cap = (5 * std::max(p.c_max, p.n_vert) / 2 + 1024 + 3) & ~3;
-  const size_t smem = held_bytes(p.held_cap);
+  const size_t smem = held_bytes(p.held_cap) + kSelWarps * kListSlots * sizeof(uint16_t);
   if (smem > (size_t)kSmemLimit - 16 * 1024) return SPEC_OK;
   static int set[64] = {0};
   int dev = 0;
