@@ -31,7 +31,14 @@
 // memory are scored in several launches over groups of rows (ScoreParams::row0), each adding
 // into the same output.
 // The global key-tile space (layer, KV head, sequence, tile) is cut into equal contiguous
-// ranges, one per CTA.
+// ranges, one per CTA; units of one length, few to a GPU, are cut among CTAs of their own.
+//
+// What bounds it: long calls run at the board's power limit, so that their time is the energy of a logit (tensor
+// core, TMEM read, two packed FMA-pipe operations, the exponential), whatever the clock: 32 layers of 131072 keys,
+// 640 rows of head_dim 128, 12.32 -> 11.82 ms for the step in a loop, at 1575 MHz; of 16384 keys, 384 rows, at full
+// clock 0.94 -> 0.885 ms.  Short calls are bound by the way into each pass: one layer of 12345 keys (36 us) waits 3.4 us
+// for its queries and 1.5 for the first accumulators in pass 1, which ends at 18, and in pass 2 from 18 to 23.5 for the
+// last CTA of pass 1, the statistics (2.5 us) and the constants.
 //
 // Every wait on an mbarrier is bounded in time; on expiry the CTA reports SPEC_ERR_TIMEOUT
 // through the status word, lets its copies land, frees its TMEM and returns.
@@ -50,11 +57,8 @@ constexpr int kThreads = 128 + kEpilogueThreads;        // one more warpgroup: T
 constexpr int kLaunchRegs = 96, kIssueRegs = 64, kEpilogueRegs = 104;
 static_assert(128 * kIssueRegs + kEpilogueThreads * kEpilogueRegs <= kThreads * kLaunchRegs, "the warpgroups' shares must fit what the block is launched with");
 // Of the 16 element pairs in a 32-element block, evaluated on the FMA pipes.  Sustained time of 8 layers at 128K
-// (640 rows) for 3, 4, 5, 6 pairs: 3.083, 3.061, 3.057, 3.128 ms.
-#ifndef SPEC_POLY_PAIRS
-#define SPEC_POLY_PAIRS 5
-#endif
-constexpr int kPolyPairs = SPEC_POLY_PAIRS;
+// (640 rows) for 2, 3, 4, 5 pairs: 3.120, 3.068, 3.033, 3.030 ms (6 was 2 % slower than 5).
+constexpr int kPolyPairs = 5;
 // minimax quartic of 2^f on [-1/2, 1/2], from the lowest coefficient
 constexpr float kExpC0 = 0.9999992614f, kExpC1 = 0.6931218147f, kExpC2 = 0.2402474482f, kExpC3 = 0.0559178603f, kExpC4 = 0.0095701019f;
 constexpr int kBufCols = 128;                 // TMEM columns of an accumulator buffer, one per epilogue warpgroup
