@@ -150,12 +150,13 @@ struct ClusterCtx {
   uint32_t* merged;           // [2][kBins]
   int* wsum;
   int* out2;
-  int* r_a;                   // [16] per-rank counts, first kind
-  int* r_b;                   // [16] per-rank counts, second kind
+  int* r_a;                   // [2][kClusterUse] per-rank counts, first kind
+  int* r_b;                   // [2][kClusterUse] per-rank counts, second kind
   const uint32_t* keys;
   int j_lo, j_hi;             // valid local positions
   uint32_t rank, cs;
   int stage;                  // merged-histogram uses so far
+  int exchanges;              // exchange_counts calls so far
 };
 
 // Adds the non-empty bins of the local histogram into merged[stage & 1] of every CTA.
@@ -243,16 +244,21 @@ __device__ void count_winners(const ClusterCtx& c, uint32_t T, int slab, int& ct
 }
 
 // Publishes two counts of this CTA to every CTA of the cluster (slot = my rank); after the
-// barrier returns the sums over the lower ranks and over all ranks.
-__device__ void exchange_counts(const ClusterCtx& c, int a, int b, int& a_before, int& b_before, int& a_total, int& b_total) {
+// barrier returns the sums over the lower ranks and over all ranks.  Calls take two sets of slots in turn, because no
+// cluster barrier has to lie between one call's reads and the next call's stores (find_threshold is local to a CTA).  A CTA
+// stores into this call's slots again only behind the next call's barrier, which every CTA reaches after its reads here.
+__device__ void exchange_counts(ClusterCtx& c, int a, int b, int& a_before, int& b_before, int& a_total, int& b_total) {
+  int* r_a = c.r_a + (c.exchanges & 1) * kClusterUse;
+  int* r_b = c.r_b + (c.exchanges & 1) * kClusterUse;
+  ++c.exchanges;
   if (threadIdx.x < c.cs) {
-    remote_store(in_rank(shared_u32(c.r_a + c.rank), threadIdx.x), a);
-    remote_store(in_rank(shared_u32(c.r_b + c.rank), threadIdx.x), b);
+    remote_store(in_rank(shared_u32(r_a + c.rank), threadIdx.x), a);
+    remote_store(in_rank(shared_u32(r_b + c.rank), threadIdx.x), b);
   }
   cluster_sync_all();
   a_before = b_before = a_total = b_total = 0;
   for (uint32_t r = 0; r < c.cs; ++r) {
-    const int x = c.r_a[r], y = c.r_b[r];
+    const int x = r_a[r], y = r_b[r];
     if (r < c.rank) { a_before += x; b_before += y; }
     a_total += x;
     b_total += y;
@@ -271,6 +277,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   int* misc = reinterpret_cast<int*>(c.merged + 2 * kBins);
   c.wsum = misc;                                           // 32
   c.out2 = misc + 32;                                      // 4
+  static_assert(2 * kClusterUse <= 16, "two sets of counts in 16 words");
   c.r_a = misc + 40;                                       // 16
   c.r_b = misc + 56;                                       // 16
   int* sh_gt = misc + 72;                                  // 16
@@ -288,6 +295,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) cluster_select_kernel(const Cl
   c.rank = cluster_rank();
   c.cs = cluster_size();
   c.stage = 0;
+  c.exchanges = 0;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t lt_mask = (1u << lane) - 1u;

@@ -689,15 +689,16 @@ def test_score_zero_length_prompt_clears_the_output(B, W):
 
 # ------------------------------------------------------------------ widening rows -----
 
-def run_vert_case(B, oracle, scores, cu, k, c_max, forced, n_vert):
-    """spec_pool_topk_vert against two oracle selections on the same pooled scores."""
+def run_vert_case(B, oracle, scores, cu, k, c_max, forced, n_vert, pool=0):
+    """spec_pool_topk_vert against two oracle selections on the same pooled scores.  Nothing behind the last unit's
+    lists may be written."""
     L, H, T = scores.shape
     n_seq = len(cu) - 1
     cu_t = torch.tensor(cu, dtype=torch.int32, device="cuda") if n_seq > 1 else None
     pr = B.make_problem(n_layers=L, n_q_heads=H, n_kv_heads=H, head_dim=128, n_lookahead=1, n_window=0,
                         softmax_scale=1.0, total_tokens=T, n_in=int(max(np.diff(cu))), n_seq=n_seq, cu_seqlens=cu_t)
     s64 = scores.astype(np.float64)
-    o_cache, o_cnt, _, _ = oracle.pool_topk(s64, cu, oracle.POOL_MAX, k, c_max, forced)
+    o_cache, o_cnt, _, _ = oracle.pool_topk(s64, cu, pool, k, c_max, forced)
     # i_vert is the plain top-n_vert of the positions before the forced tail: the oracle gets them as
     # sequences cut at the tail, with the same pooling clipped to that range
     o_vert = np.full((n_seq, L, H, n_vert), -1, dtype=np.int32)
@@ -706,23 +707,22 @@ def run_vert_case(B, oracle, scores, cu, k, c_max, forced, n_vert):
         n = cu[s + 1] - cu[s]
         e = n - min(forced, n)
         if e > 0:
-            oi, oc, _, _ = oracle.pool_topk(s64[:, :, cu[s]:cu[s] + e].copy(), [0, e], oracle.POOL_MAX, k, n_vert, 0)
+            oi, oc, _, _ = oracle.pool_topk(s64[:, :, cu[s]:cu[s] + e].copy(), [0, e], pool, k, n_vert, 0)
             o_vert[s], o_vcnt[s] = oi[0], oc[0]
     ws = torch.empty(max(B.spec_workspace_bytes(pr), 16), dtype=torch.uint8, device="cuda")
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    scores_t = torch.from_numpy(scores).cuda()
+    units = n_seq * L * H
     for workspace in (None, ws):                       # cluster-resident and streaming selection
-        idx = torch.full((n_seq, L, H, c_max), -7, dtype=torch.int32, device="cuda")
-        cnt = torch.full((n_seq, L, H), -7, dtype=torch.int32, device="cuda")
-        vidx = torch.full((n_seq, L, H, n_vert), -7, dtype=torch.int32, device="cuda")
-        vcnt = torch.full((n_seq, L, H), -7, dtype=torch.int32, device="cuda")
-        B.spec_pool_topk_vert(pr, torch.from_numpy(scores).cuda(), B.POOL_MAX, k, c_max, forced, idx, cnt, n_vert, vidx, vcnt,
+        bufs = [torch.full((units * w + 64,), -7, dtype=torch.int32, device="cuda") for w in (c_max, 1, n_vert, 1)]
+        B.spec_pool_topk_vert(pr, scores_t, pool, k, c_max, forced, bufs[0], bufs[1], n_vert, bufs[2], bufs[3],
                               workspace=workspace, status_word=status)
         torch.cuda.synchronize()
         assert status.item() == 0
-        np.testing.assert_array_equal(idx.cpu().numpy(), o_cache)
-        np.testing.assert_array_equal(cnt.cpu().numpy(), o_cnt)
-        np.testing.assert_array_equal(vidx.cpu().numpy(), o_vert)
-        np.testing.assert_array_equal(vcnt.cpu().numpy(), o_vcnt)
+        for buf, want in zip(bufs, (o_cache, o_cnt, o_vert, o_vcnt)):
+            got = buf.cpu().numpy()
+            np.testing.assert_array_equal(got[:want.size].reshape(want.shape), want)
+            assert np.all(got[want.size:] == -7), "written behind the last list"
 
 
 def test_vertical_and_cache_indices_from_one_sweep(B, W, oracle):
@@ -741,6 +741,45 @@ def test_vertical_and_cache_indices_from_one_sweep(B, W, oracle):
     g = Gpu(B, W, w, [0])
     sc = g.score().cpu().numpy()
     run_vert_case(B, oracle, sc, g.cu, w.pool_k, 256, w.n_window, 2048)
+
+
+def cluster_sample_positions(unit, n, cluster, shift):
+    """The positions that a cluster of that size samples for its floor, one in 2^shift of every CTA's share (a unit on a
+    16-byte boundary)."""
+    share = (-(-n // cluster) + 3) & ~3
+    where = []
+    for rank in range(cluster):
+        for q in range(-(-share >> shift)):
+            h = (unit * 0x9E3779B1 & 0xFFFFFFFF) ^ ((rank * 65536 + q) * 0x85EBCA6B & 0xFFFFFFFF)
+            h ^= h >> 15
+            h = h * 0x2C1B3C6D & 0xFFFFFFFF
+            h ^= h >> 12
+            j = (q << shift) + (h & ((1 << shift) - 1))
+            if j < share and rank * share + j < n:
+                where.append(rank * share + j)
+    return np.array(where)
+
+
+@pytest.mark.parametrize("pool,k", [(0, 5), (1, 13)])
+@pytest.mark.parametrize("units", [3, 70])                       # clusters of eight CTAs, and of two
+@pytest.mark.parametrize("scores", ["random", "ties", "crowded_sample"])
+def test_two_budgets_in_a_cluster(B, oracle, pool, k, units, scores):
+    """Two budgets from one cluster, either one the larger, one beyond the sequence, and budgets that need different
+    threshold searches: large keys on sampled positions alone (more than the 610 samples that the floor of 8192 is taken
+    from) raise the floor so far that it serves the smaller budget and sends the larger to the radix select.  Scores on a dyadic grid, so that averages compare as exactly as maxima."""
+    n = 33000
+    rng = np.random.default_rng(units + k)
+    if scores == "ties":
+        x = rng.integers(0, 5, size=(1, units, n)) / 8.0
+    else:
+        x = rng.integers(0, 1 << 17, size=(1, units, n)) / (1 << 18)
+        if scores == "crowded_sample":
+            for u in range(units):
+                at = cluster_sample_positions(u, n, 8 if units == 3 else 2, 4)
+                x[0, u, rng.choice(at, 700, replace=False)] += 16.0
+    x = x.astype(np.float32)
+    for c_max, n_vert, forced in ((256, 8192, 32), (8192, 256, 0), (256, 40000, 16), (40000, 700, 0), (1024, 1024, 0)):
+        run_vert_case(B, oracle, x, [0, n], k, c_max, forced, n_vert, pool=pool)
 
 
 STRUCTURED = {
