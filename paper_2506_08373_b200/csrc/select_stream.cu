@@ -378,7 +378,10 @@ __global__ void __launch_bounds__(kSelThreads) sample_floor_kernel(const StreamP
 constexpr int kSweepThreads = 128, kSweepCtas = 8;        // 6 CTAs to an SM: 135.0 us for selection and gather of 256 units of 131072, 8: 133.0, 10: 136.1
 constexpr int kSweepWarps = kSweepThreads / 32;
 
-// One warp per chunk; warps never meet.  A lane's eight 16-byte loads are in flight at once.
+// One warp per chunk; warps never meet.  A lane's eight 16-byte loads are in flight at once.  The finishing kernel is not let
+// in early: its CTAs would take the first SMs that the sweep leaves, two to each, and run there in each other's way, while
+// other SMs have none (64 units of 131072: 24.3 -> 22.0 us; 64 units of 65536 with all scores tied, where a CTA works for
+// 200 us, 366 -> 272).
 __global__ void __launch_bounds__(kSweepThreads, kSweepCtas) stream_sweep_kernel(const StreamParams p) {
   __shared__ uint16_t lists[kSweepWarps][kListSlots];
   const int lane = threadIdx.x & 31;
@@ -390,7 +393,6 @@ __global__ void __launch_bounds__(kSweepThreads, kSweepCtas) stream_sweep_kernel
   WarpScores w;
   if (c0 < g.X) load_scores(g, c0, min(kWarpSteps, (g.X - c0 + 127) >> 7), lane, w);
   wait_for_previous_grid();                                // the floors are written by the grid before this one
-  launch_dependents();
   if (c0 >= g.X) return;
   int32_t* hd = p.head + ((int64_t)s * (p.H * p.L) + row) * p.head_words;
   const uint32_t floor_key = (uint32_t)__ldcg(hd);
@@ -415,7 +417,9 @@ __global__ void __launch_bounds__(kSweepThreads, kSweepCtas) stream_sweep_kernel
 
 static size_t held_bytes(int held_cap) { return std::max((size_t)held_cap * 8, kGenericBytes); }
 
-// One CTA per unit and budget (a second budget costs a second CTA, not a second turn).
+// One CTA per unit and budget (a second budget costs a second CTA, not a second turn).  The next kernel is not let in early
+// either: the floor CTAs of a selection that follows would crowd on the few SMs with room beside two finishing CTAs, and
+// the sweep behind them waits for the slowest (256 units of 131072, one selection after the other: 70.4 -> 46.9 us each).
 __global__ void __launch_bounds__(kSelThreads, 2) stream_finish_kernel(const StreamParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   __shared__ __align__(16) SelectMem sm;
@@ -425,7 +429,6 @@ __global__ void __launch_bounds__(kSelThreads, 2) stream_finish_kernel(const Str
   reinterpret_cast<uint4*>(sm.hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) sm.top = 0;
   wait_for_previous_grid();                                // the candidates are written by the grid before this one
-  launch_dependents();
   const UnitGeom g = unit_geom(p, unit);
   const int32_t* hd = p.head + (int64_t)unit * p.head_words;
   uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);

@@ -829,6 +829,33 @@ def test_topk_structured_score_vectors_exact_and_not_slow(B, W, oracle):
         assert t <= 3.0 * base + 0.02, "%s takes %.3f ms against %.3f ms for random scores" % (key, t, base)
 
 
+def test_selections_in_a_row_cost_no_more_than_one(B):
+    """The kernels of one selection may start under those of the one before it, which must not slow either down: 20
+    selections of 256 units of 131072 in a row against single ones on an idle GPU with their scores out of L2."""
+    g = torch.Generator(device="cuda").manual_seed(2)
+    x = torch.rand(1, 256, 131072, device="cuda", generator=g) ** 6
+    pr = B.make_problem(n_layers=1, n_q_heads=256, n_kv_heads=256, head_dim=128, n_lookahead=1, n_window=0, softmax_scale=1.0,
+                        total_tokens=131072, n_in=131072)
+    ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+    idx = torch.empty((1, 1, 256, 2048), dtype=torch.int32, device="cuda")
+    other = torch.empty(1 << 26, device="cuda")
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    times = {}
+    for calls in (1, 20):
+        best = float("inf")
+        for _ in range(8):
+            other.zero_()
+            torch.cuda.synchronize()
+            e0.record()
+            for _ in range(calls):
+                B.spec_pool_topk(pr, x, B.POOL_MAX, 7, 2048, 0, idx, None, workspace=ws)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1) / calls)
+        times[calls] = best
+    assert times[20] <= times[1], "a selection takes %.4f ms in a row and %.4f on its own" % (times[20], times[1])
+
+
 def test_topk_short_units_in_one_cta_and_streamed(B, W, oracle):
     """Units of up to 16381 positions are selected by one CTA each (scores, floor sample, candidates and the
     finishing step all in shared memory); many hundreds of such units with a workspace are streamed
