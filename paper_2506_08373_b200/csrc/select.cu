@@ -869,31 +869,51 @@ static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int
   }
   const int64_t x_max = (int64_t)max_len + 3;
   // The cluster size with the least estimated time: a CTA takes 7 us and another 10 for 8192 positions (32768 positions
-  // in 4 CTAs: 17 us), and two CTAs share an SM where their memory allows; GPCs hold about 0.8 of the
-  // slots' worth of clusters.
-  double best = 1e30;
-  pl.fits = false;
-  for (int cs = max_cs; cs >= 1; cs >>= 1) {
-    const int cap = (int)((((x_max + cs - 1) / cs) + 3) & ~(int64_t)3);
-    const size_t smem = cluster_smem_bytes(cap, pl.halo_l, pl.halo_r, pl.inplace, mode, 0);
-    if (smem > (size_t)kSmemLimit || (cs > 1 && cap < kChunkMin)) continue;
-    const int64_t slots = (smem + (size_t)(5 * (int64_t)budget / 2 + 1024) * 4 <= (size_t)kSmemLimit / 2 ? 2 : 1) * (cs > 2 ? 120 : 140);
-    const double t = (double)((n_units * cs + slots - 1) / slots) * (7.0 + 10.0 * cap / 8192);
-    if (t < best) {
-      best = t;
-      pl.fits = true;
-      pl.cs = cs;
-      pl.cap = cap;
-      pl.smem = smem;
+  // in 4 CTAs: 17 us), and two CTAs share an SM where their memory, with `held` bytes for keys, allows; GPCs hold about 0.8
+  // of the slots' worth of clusters.
+  double waves = 0;
+  auto size_cluster = [&](size_t held) {
+    double best = 1e30;
+    pl.fits = false;
+    for (int cs = max_cs; cs >= 1; cs >>= 1) {
+      const int cap = (int)((((x_max + cs - 1) / cs) + 3) & ~(int64_t)3);
+      const size_t smem = cluster_smem_bytes(cap, pl.halo_l, pl.halo_r, pl.inplace, mode, 0);
+      if (smem > (size_t)kSmemLimit || (cs > 1 && cap < kChunkMin)) continue;
+      const int64_t slots = (smem + held <= (size_t)kSmemLimit / 2 ? 2 : 1) * (cs > 2 ? 120 : 140);
+      const double w = (double)((n_units * cs + slots - 1) / slots), t = w * (7.0 + 10.0 * cap / 8192);
+      if (t < best) {
+        best = t;
+        waves = w;
+        pl.fits = true;
+        pl.cs = cs;
+        pl.cap = cap;
+        pl.smem = smem;
+      }
     }
+  };
+  size_cluster((size_t)(5 * (int64_t)budget / 2 + 1024) * 4);
+  if (!pl.fits) {
+    pl.cs = 1; pl.cap = 0; pl.smem = 0; pl.cand_cap = 0;
+    return pl;
   }
-  if (!pl.fits) { pl.cs = 1; pl.cap = 0; pl.smem = 0; }
-  // The floor lets through 1.3 (large budgets) to 2.5 times the budget; short units send all of their keys.  Where
-  // there is no room for that (budgets of a third of a very long sequence), the radix select does without.
+  // The floor lets through 1.3 (large budgets) to 2.5 times the budget; short units send all of their keys.
   const int64_t room = ((int64_t)kSmemLimit - (int64_t)pl.smem) / 4;
   const int64_t want = std::min<int64_t>(5 * (int64_t)budget / 2 + 1024, x_max + 1 + 3) & ~(int64_t)3;
-  pl.cand_cap = pl.fits ? (int)std::min(want, room & ~(int64_t)3) : 0;
-  if (pl.cand_cap < std::min<int64_t>(want, 3 * (int64_t)budget / 2)) pl.cand_cap = 0;
+  pl.cand_cap = (int)std::min(want, room & ~(int64_t)3);
+  // The radix select over the keys where they are instead: where there is no room for those sent (budgets of a third of a
+  // very long sequence); where sending and searching them, 0.4 us for 1000 keys in every CTA, takes longer than the
+  // radix passes' 1.5 us and 0.3 for 1000 positions of a CTA (units of 33000 in clusters of eight, a 24th, an 8th and half of the
+  // positions kept: 14, 16.1 and 33 us by the keys, 16, 15.7 and 15 by the passes); and where the keys' memory keeps
+  // clusters from being on the GPU all at once (256 units of 8000, a third kept: 34.5 against 25.6 us).
+  const double sent = x_max <= want ? (double)x_max : 1.5 * budget;
+  const bool fits_keys = pl.cand_cap >= std::min<int64_t>(want, 3 * (int64_t)budget / 2);
+  if (!fits_keys || 0.4e-3 * sent > 1.5 + 0.3e-3 * pl.cap) pl.cand_cap = 0;
+  if (waves > 1) {
+    const ClusterPlan with_keys = pl;
+    size_cluster(0);
+    if (waves > 1) pl = with_keys;
+    else pl.cand_cap = 0;
+  }
   pl.smem += (size_t)pl.cand_cap * 4;
   return pl;
 }

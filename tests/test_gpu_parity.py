@@ -898,6 +898,52 @@ def test_topk_at_the_limits_of_the_selection_kernels(B, W, oracle, n, k, c_max, 
     run_topk_case(B, W, oracle, x, [0, n], 0, k, c_max, min(c_max // 2, 33))
 
 
+@pytest.mark.parametrize("n,k,c_max,units", [
+    (33000, 5, 4563, 3), (33000, 5, 4565, 3),                    # keys sent to every CTA, radix select over them where they are
+    (60000, 7, 6252, 8), (60000, 7, 20000, 8),
+    (8003, 5, 2400, 140), (8003, 5, 2666, 141),                  # a CTA to a unit: all on the GPU at once with the keys' memory
+    (8003, 5, 2666, 256), (16000, 7, 8000, 256)])                # and only without it
+def test_topk_at_the_limits_of_the_cluster_threshold_searches(B, W, oracle, n, k, c_max, units):
+    x = (np.random.default_rng(n + units).random((1, units, n)) ** 5).astype(np.float32)
+    x[:, :, n // 2:n // 2 + 60] = x[:, :, :1]
+    run_topk_case(B, W, oracle, x, [0, n], 0, k, c_max, 33)
+    if k == 5:
+        run_vert_case(B, oracle, x[:, :8], [0, n], k, 300, 16, c_max)
+
+
+def test_large_budgets_cost_little_more_than_small_ones(B):
+    """Cluster selections and keep sets of half of the positions against a 24th of them."""
+    g = torch.Generator(device="cuda").manual_seed(2)
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+
+    def time_of(call):
+        best = float("inf")
+        for _ in range(6):
+            e0.record()
+            for _ in range(10):
+                call()
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1) / 10)
+        return best
+
+    for units, n in ((1, 33000), (256, 8000), (0, 32768)):       # 0 units: the keep set
+        heads = max(units, 1)
+        x = torch.rand(1, heads, n, device="cuda", generator=g) ** 6
+        pr = B.make_problem(n_layers=1, n_q_heads=heads, n_kv_heads=heads, head_dim=128, n_lookahead=1, n_window=0, softmax_scale=1.0,
+                            total_tokens=n, n_in=n)
+        ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+        out = torch.empty(heads * n, dtype=torch.int32, device="cuda")
+        cnt = torch.empty(heads, dtype=torch.int32, device="cuda")
+        times = []
+        for c_max in (n // 24, n // 2):
+            if units:
+                times.append(time_of(lambda: B.spec_pool_topk(pr, x, B.POOL_MAX, 5, c_max, 0, out, cnt)))
+            else:
+                times.append(time_of(lambda: B.specpc_token_select(pr, x, 0, B.POOL_MAX, 5, c_max, 2, 0, out, n, cnt, ws)))
+        assert times[1] <= 1.7 * times[0], "%d units of %d: %.4f ms for half of the positions, %.4f for a 24th" % (units, n, times[1], times[0])
+
+
 @pytest.mark.parametrize("spread", [2.0 ** -4, 2.0 ** -7, 2.0 ** -12])
 def test_topk_scores_that_differ_little(B, W, oracle, spread):
     """Sampled keys within one or a few bins of the floor's histogram, in all three selections: above the bin's
