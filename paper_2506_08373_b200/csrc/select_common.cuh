@@ -314,10 +314,14 @@ __device__ __forceinline__ bool find_bin(SelectMem& sm, int need, int& bin, int&
 // 64 bins to a factor of two over 32 factors of two, or, if the rank lies deeper than that, by their
 // leading 11 bits.  Scores that differ by a few per cent only (sums over many heads, averages) would crowd into a bin
 // or two: the bin is cut again then, or the floor lets through more keys than there is room for (keep set of 1024
-// among 32768 such tokens: 29.6 -> 23.6 us).  0 when the sample is too small to tell.  `keys`: N samples of this thread, 0 = none.
-// All threads of the CTA call this; the histogram is clear on entry and on return.
+// among 32768 such tokens: 29.6 -> 23.6 us).  0, which all keys reach, when the sample is too small to tell.  `keys`: N samples
+// of this thread, 0 = none.  All threads of the CTA call this; the histogram is clear on entry and on return.
+struct Floor {
+  uint32_t key;
+  int reach;                   // samples at or above it
+};
 template <int N>
-__device__ __forceinline__ uint32_t floor_from_samples(SelectMem& sm, const uint32_t (&keys)[N], int take, int rate_shift) {
+__device__ __forceinline__ Floor floor_from_samples(SelectMem& sm, const uint32_t (&keys)[N], int take, int rate_shift) {
   // about take / 2^rate_shift samples lie above the threshold; the floor is taken four standard deviations further down
   const float m_exp = (float)take / (float)(1 << rate_shift);
   const int rho = (int)(m_exp + 4.f * sqrtf(m_exp) + 8.f);
@@ -332,24 +336,26 @@ __device__ __forceinline__ uint32_t floor_from_samples(SelectMem& sm, const uint
   for (int i = 0; i < N; ++i)
     if (keys[i]) atomicAdd(&sm.hist[kStreamBins - 1 - min((top - keys[i]) >> 17, (uint32_t)kStreamBins - 1)], 1u);
   int bin, above, count;
-  if (!find_bin(sm, rho, bin, above, count)) return 0u;
+  if (!find_bin(sm, rho, bin, above, count)) return {0u, 0x7fffffff};
   if (bin > 0) {
     uint32_t depth = ((uint32_t)(kStreamBins - bin) << 17) - 1u;             // the bin's lower edge
+    int higher = 0;
     if (above + count > rho + (rho >> 2) + 8) {            // the bin holds many more samples than were asked for: it is cut again
       const uint32_t upper = depth >> 17;
 #pragma unroll
       for (int i = 0; i < N; ++i)
         if (keys[i] && (top - keys[i]) >> 17 == upper) atomicAdd(&sm.hist[kStreamBins - 1 - (((top - keys[i]) >> 6) & (kStreamBins - 1))], 1u);
-      find_bin(sm, rho - above, bin, above, count);
+      higher = above;
+      find_bin(sm, rho - higher, bin, above, count);
       depth = (upper << 17) + ((uint32_t)(kStreamBins - bin) << 6) - 1u;
     }
-    return top > depth ? top - depth : 0u;
+    return {top > depth ? top - depth : 0u, higher + above + count};
   }
 #pragma unroll
   for (int i = 0; i < N; ++i)
     if (keys[i]) atomicAdd(&sm.hist[keys[i] >> 21], 1u);
   find_bin(sm, rho, bin, above, count);
-  return (uint32_t)bin << 21;
+  return {(uint32_t)bin << 21, above + count};
 }
 
 // The key T of the need-th largest of keys[0..n), all of them in [lo, hi], and how many elements equal to T

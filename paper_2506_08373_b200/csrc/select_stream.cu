@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(kSelThreads) sample_floor_kernel(const StreamP
       keys[i] = to_key(fmax3(fmax3(v[0], v[1], v[2]), fmax3(v[3], v[4], v[5]), v[6]));   // pooled value of the centre
     }
     __syncthreads();
-    floor_key = floor_from_samples(sm, keys, tk, shift);
+    floor_key = floor_from_samples(sm, keys, tk, shift).key;
   }
   if (tid == 0) {
     if (g.over) report(p.status, SPEC_ERR_BAD_ARG);
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) unit_select_kernel(const Strea
       if (mine && x >= g.mis && x < g.X) samples[k] = to_key(fmax3(fmax3(v.x, v.y, v.z), fmax3(v.w, q0, q1), q2));
     }
     __syncthreads();
-    floor_key = floor_from_samples(sm, samples, g.take[b], kUnitSampleShift);
+    floor_key = floor_from_samples(sm, samples, g.take[b], kUnitSampleShift).key;
     // ---- the candidates
     const WarpCandidates c = find_candidates(g, w, key_to_float(floor_key), lane);
     __syncthreads();                                       // the scan's memory is free; everyone has the sample's largest key

@@ -911,8 +911,9 @@ def test_topk_at_the_limits_of_the_cluster_threshold_searches(B, W, oracle, n, k
         run_vert_case(B, oracle, x[:, :8], [0, n], k, 300, 16, c_max)
 
 
-def test_large_budgets_cost_little_more_than_small_ones(B):
-    """Cluster selections and keep sets of half of the positions against a 24th of them."""
+def test_large_budgets_and_ties_cost_little_more(B):
+    """Cluster selections and keep sets of half of the positions against a 24th of them, and of tied scores, which leave the
+    floor without use, against random ones."""
     g = torch.Generator(device="cuda").manual_seed(2)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
 
@@ -942,6 +943,12 @@ def test_large_budgets_cost_little_more_than_small_ones(B):
             else:
                 times.append(time_of(lambda: B.specpc_token_select(pr, x, 0, B.POOL_MAX, 5, c_max, 2, 0, out, n, cnt, ws)))
         assert times[1] <= 1.7 * times[0], "%d units of %d: %.4f ms for half of the positions, %.4f for a 24th" % (units, n, times[1], times[0])
+    n = 65536
+    pr = B.make_problem(n_layers=1, n_q_heads=1, n_kv_heads=1, head_dim=128, n_lookahead=1, n_window=0, softmax_scale=1.0,
+                        total_tokens=n, n_in=n)
+    x = torch.rand(1, 1, n, device="cuda", generator=g) ** 6
+    times = [time_of(lambda: B.spec_pool_topk(pr, y, B.POOL_MAX, 5, 2048, 0, out, None)) for y in (x, torch.zeros_like(x))]
+    assert times[1] <= 1.6 * times[0], "%.4f ms for tied scores, %.4f for random ones" % (times[1], times[0])
 
 
 @pytest.mark.parametrize("spread", [2.0 ** -4, 2.0 ** -7, 2.0 ** -12])
