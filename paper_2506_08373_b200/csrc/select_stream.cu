@@ -21,9 +21,9 @@
 //      memory once, straight into registers (the loads are issued before the floors are waited for);
 //      candidates go, as (key, position) pairs in position order, to the chunk's own segment of
 //      the unit's candidate array in the workspace.
-//   3. stream_finish_kernel, one CTA per unit and budget: the candidates come into shared memory, the
-//      exact threshold is found (find_threshold), and the winners are written out as they stand,
-//      already in ascending position, ties to the lower position.
+//   3. stream_finish_kernel, one CTA per unit and budget, or per unit where those are many: the
+//      candidates come into shared memory, the exact threshold is found (find_threshold), and the winners
+//      are written out as they stand, already in ascending position, ties to the lower position.
 // Units of up to 16384 positions, a few to an SM, skip the workspace and the three launches:
 // unit_select_kernel holds a unit in the registers of one CTA and does the same steps.
 //
@@ -138,8 +138,8 @@ __device__ __forceinline__ void emit_selected(SelectMem& sm, const uint32_t* key
 constexpr size_t kGenericBytes = (size_t)(kSelWarps * 256 + 2 * kSelWarps + 8) * 4;
 
 // The list of one budget of a unit, given its candidates (or `failed`, or too few of them: the generic
-// selection, in the shared memory at `scratch`).
-__device__ __forceinline__ void finish_unit(const StreamParams& p, const UnitGeom& g, int unit, int b, SelectMem& sm, const uint32_t* keys,
+// selection, in the shared memory at `scratch`, which is the candidates').  False when they are gone.
+__device__ __forceinline__ bool finish_unit(const StreamParams& p, const UnitGeom& g, int unit, int b, SelectMem& sm, const uint32_t* keys,
                                             const uint32_t* pos, int n, bool failed, uint32_t floor_key, uint32_t top, void* scratch) {
   const int tid = threadIdx.x;
   const int width = b == 0 ? p.c_max : p.n_vert;
@@ -168,9 +168,24 @@ __device__ __forceinline__ void finish_unit(const StreamParams& p, const UnitGeo
       key.keys = nullptr;
       radix_select(key, g.e, tk, sc, T, need_eq);
       ordered_emit(key, g.e, T, need_eq, sc, [&](int rank, int j) { idx[rank] = j; });
+      return false;
     }
   }
+  return true;
 }
+// The list of budget b of a unit, or (BOTH) of its two.
+template <bool BOTH>
+__device__ __forceinline__ void finish_budgets(const StreamParams& p, const UnitGeom& g, int unit, int b, SelectMem& sm, const uint32_t* keys,
+                                               const uint32_t* pos, int n, bool failed, uint32_t floor_key, uint32_t top, void* scratch) {
+  if (!BOTH) {
+    finish_unit(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, scratch);
+    return;
+  }
+#pragma unroll 1
+  for (b = 0; b < 2; ++b)
+    if (!finish_unit(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, scratch)) failed = true;
+}
+__device__ __forceinline__ bool cuts(const UnitGeom& g, int b) { return g.take[b] > 0 && g.take[b] < g.e; }
 
 // -------------------------------------------------------- a warp's scores in registers --
 
@@ -417,15 +432,18 @@ __global__ void __launch_bounds__(kSweepThreads, kSweepCtas) stream_sweep_kernel
 
 static size_t held_bytes(int held_cap) { return std::max((size_t)held_cap * 8, kGenericBytes); }
 
-// One CTA per unit and budget (a second budget costs a second CTA, not a second turn).  The next kernel is not let in early
+// One CTA per unit and budget while all of them are on the GPU at once, two to an SM; BOTH: one per unit for its two budgets, which
+// then cost a second threshold and emission but no second copy of the candidates (148 units of 17001, 384 and 400 kept:
+// 15.5 us with two CTAs to a unit, 17.1 with one; 2048 units 137 and 118).  The next kernel is not let in early
 // either: the floor CTAs of a selection that follows would crowd on the few SMs with room beside two finishing CTAs, and
 // the sweep behind them waits for the slowest (256 units of 131072, one selection after the other: 70.4 -> 46.9 us each).
+template <bool BOTH>
 __global__ void __launch_bounds__(kSelThreads, 2) stream_finish_kernel(const StreamParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   __shared__ __align__(16) SelectMem sm;
   __shared__ int chunk_at[kSelThreads], chunk_n[kSelThreads];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int unit = blockIdx.x, b = blockIdx.y;
+  const int unit = blockIdx.x, b = BOTH ? 0 : blockIdx.y;
   reinterpret_cast<uint4*>(sm.hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) sm.top = 0;
   wait_for_previous_grid();                                // the candidates are written by the grid before this one
@@ -433,7 +451,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) stream_finish_kernel(const Str
   const int32_t* hd = p.head + (int64_t)unit * p.head_words;
   uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);
   uint32_t* pos = keys + p.held_cap;
-  const bool selects = g.take[b] > 0 && g.take[b] < g.e;
+  const bool selects = cuts(g, b) || (BOTH && cuts(g, 1));
   int n = 0;
   bool failed = false;
   uint32_t floor_key = 0, top = 0;
@@ -482,7 +500,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) stream_finish_kernel(const Str
     __syncthreads();
     top = sm.top;
   }
-  finish_unit(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, smem_raw);
+  finish_budgets<BOTH>(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, smem_raw);
 }
 
 // --------------------------------------------------- short units: all steps in one CTA --
@@ -490,13 +508,14 @@ __global__ void __launch_bounds__(kSelThreads, 2) stream_finish_kernel(const Str
 constexpr int kUnitSlots = kSelWarps * kWarpSpan;          // 16384
 constexpr int kUnitSampleShift = 4;                        // the floor's sample: one position in 16
 
-// One CTA per unit and budget: the unit's scores in the registers of 16 warps, the floor from a sample of
-// them, the candidates in shared memory.
+// One CTA per unit and budget, or BOTH in one as above (256 units of 16384, 384 and 400 kept: 20.8 us with two CTAs to a unit,
+// 14.7 with one): the unit's scores in the registers of 16 warps, the floor from a sample of them, the candidates in shared memory.
+template <bool BOTH>
 __global__ void __launch_bounds__(kSelThreads, 2) unit_select_kernel(const StreamParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   __shared__ __align__(16) SelectMem sm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int unit = blockIdx.x, b = blockIdx.y;
+  const int unit = blockIdx.x, b = BOTH ? 0 : blockIdx.y;
   reinterpret_cast<uint4*>(sm.hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) sm.top = 0;
   wait_for_previous_grid();
@@ -508,7 +527,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) unit_select_kernel(const Strea
   int n = 0;
   bool failed = false;
   uint32_t floor_key = 0, top = 0;
-  if (g.take[b] > 0 && g.take[b] < g.e) {
+  if (cuts(g, b) || (BOTH && cuts(g, 1))) {
     const int n_steps = (g.X + 127) >> 7;                  // <= kSelWarps * kWarpSteps, checked on the host
     const int per_warp = (n_steps + kSelWarps - 1) / kSelWarps;
     const int s0 = warp * per_warp;
@@ -533,7 +552,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) unit_select_kernel(const Strea
       if (mine && x >= g.mis && x < g.X) samples[k] = to_key(fmax3(fmax3(v.x, v.y, v.z), fmax3(v.w, q0, q1), q2));
     }
     __syncthreads();
-    floor_key = floor_from_samples(sm, samples, g.take[b], kUnitSampleShift).key;
+    floor_key = floor_from_samples(sm, samples, BOTH ? max(g.take[0], g.take[1]) : g.take[b], kUnitSampleShift).key;
     // ---- the candidates
     const WarpCandidates c = find_candidates(g, w, key_to_float(floor_key), lane);
     __syncthreads();                                       // the scan's memory is free; everyone has the sample's largest key
@@ -557,10 +576,13 @@ __global__ void __launch_bounds__(kSelThreads, 2) unit_select_kernel(const Strea
     __syncthreads();
     top = sm.top;
   }
-  finish_unit(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, smem_raw);
+  finish_budgets<BOTH>(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, smem_raw);
 }
 
 // ------------------------------------------------------------------ host side ---------
+
+// Two budgets of a unit in one CTA: where a CTA for each would not all be on the GPU at once.
+static bool both_budgets(const StreamParams& p, int64_t n_units) { return p.n_vert > 0 && n_units > sm_count(); }
 
 // The one-CTA selection of short units.  *done = false: the shapes do not fit it.
 static int run_unit_topk(const spec_problem* pr, StreamParams p, cudaStream_t st, bool* done) {
@@ -580,10 +602,13 @@ static int run_unit_topk(const spec_problem* pr, StreamParams p, cudaStream_t st
   SPEC_CUDA_OK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return SPEC_OK;
   if (!__atomic_load_n(&set[dev], __ATOMIC_ACQUIRE)) {
-    SPEC_CUDA_OK(cudaFuncSetAttribute(unit_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
+    SPEC_CUDA_OK(cudaFuncSetAttribute(unit_select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
+    SPEC_CUDA_OK(cudaFuncSetAttribute(unit_select_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
     __atomic_store_n(&set[dev], 1, __ATOMIC_RELEASE);
   }
-  SPEC_CUDA_OK(launch_dependent(unit_select_kernel, dim3((unsigned)n_units, p.n_vert > 0 ? 2 : 1), kSelThreads, smem, st, p));
+  const bool both = both_budgets(p, n_units);
+  SPEC_CUDA_OK(launch_dependent(both ? unit_select_kernel<true> : unit_select_kernel<false>, dim3((unsigned)n_units, p.n_vert > 0 && !both ? 2 : 1),
+                                kSelThreads, smem, st, p));
   *done = true;
   return SPEC_OK;
 }
@@ -634,13 +659,16 @@ int run_stream_topk(const spec_problem* pr, const float* scores, int c_max, int 
   SPEC_CUDA_OK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return SPEC_OK;
   if (!__atomic_load_n(&set[dev], __ATOMIC_ACQUIRE)) {
-    SPEC_CUDA_OK(cudaFuncSetAttribute(stream_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
+    SPEC_CUDA_OK(cudaFuncSetAttribute(stream_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
+    SPEC_CUDA_OK(cudaFuncSetAttribute(stream_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
     __atomic_store_n(&set[dev], 1, __ATOMIC_RELEASE);
   }
   SPEC_CUDA_OK(launch_dependent(sample_floor_kernel, dim3((unsigned)n_units), kSelThreads, 0, st, p));
   const dim3 sweep_grid((unsigned)((p.chunks_max + kSweepWarps - 1) / kSweepWarps), (unsigned)(pr->n_layers * pr->n_kv_heads), (unsigned)pr->n_seq);
   SPEC_CUDA_OK(launch_dependent(stream_sweep_kernel, sweep_grid, kSweepThreads, 0, st, p));
-  SPEC_CUDA_OK(launch_dependent(stream_finish_kernel, dim3((unsigned)n_units, n_vert > 0 ? 2 : 1), kSelThreads, held_bytes(p.held_cap), st, p));
+  const bool both = both_budgets(p, n_units);
+  SPEC_CUDA_OK(launch_dependent(both ? stream_finish_kernel<true> : stream_finish_kernel<false>, dim3((unsigned)n_units, n_vert > 0 && !both ? 2 : 1),
+                                kSelThreads, held_bytes(p.held_cap), st, p));
   *done = true;
   return SPEC_OK;
 }

@@ -743,6 +743,13 @@ def test_vertical_and_cache_indices_from_one_sweep(B, W, oracle):
     run_vert_case(B, oracle, sc, g.cu, w.pool_k, 256, w.n_window, 2048)
 
 
+def sample_hash(unit, m):
+    h = (unit * 0x9E3779B1 & 0xFFFFFFFF) ^ (m * 0x85EBCA6B & 0xFFFFFFFF)
+    h ^= h >> 15
+    h = h * 0x2C1B3C6D & 0xFFFFFFFF
+    return h ^ h >> 12
+
+
 def cluster_sample_positions(unit, n, cluster, shift):
     """The positions that a cluster of that size samples for its floor, one in 2^shift of every CTA's share (a unit on a
     16-byte boundary)."""
@@ -750,14 +757,28 @@ def cluster_sample_positions(unit, n, cluster, shift):
     where = []
     for rank in range(cluster):
         for q in range(-(-share >> shift)):
-            h = (unit * 0x9E3779B1 & 0xFFFFFFFF) ^ ((rank * 65536 + q) * 0x85EBCA6B & 0xFFFFFFFF)
-            h ^= h >> 15
-            h = h * 0x2C1B3C6D & 0xFFFFFFFF
-            h ^= h >> 12
-            j = (q << shift) + (h & ((1 << shift) - 1))
+            j = (q << shift) + (sample_hash(unit, rank * 65536 + q) & ((1 << shift) - 1))
             if j < share and rank * share + j < n:
                 where.append(rank * share + j)
     return np.array(where)
+
+
+def one_cta_sample_positions(unit, n):
+    """Those of the selection of a unit in one CTA (on a 16-byte boundary): in every step of 128 positions, one lane of four."""
+    steps = -(-n // 128)
+    per_warp = -(-steps // 16)
+    where = [st * 128 + lane * 4 + (3 if st % per_warp & 1 else 0) for st in range(steps) for lane in range(32)
+             if sample_hash(unit, st * 8 + (lane >> 2)) & 3 == lane & 3]
+    return np.array([j for j in where if j < n])
+
+
+def stream_sample_positions(unit, n, shift):
+    """Those of the streaming selection: the middle of one 32-byte sector in 2^shift positions, for unit `unit` of an array
+    of units of n positions."""
+    mis, per = unit * n % 8, 1 << (shift - 3)
+    sectors = (n + mis + 7) >> 3
+    where = [8 * (m * per + sample_hash(unit, m) % min(per, sectors - m * per)) - mis + 3 for m in range(-(-sectors // per))]
+    return np.array([j for j in where if 0 <= j < n])
 
 
 @pytest.mark.parametrize("pool,k", [(0, 5), (1, 13)])
@@ -780,6 +801,24 @@ def test_two_budgets_in_a_cluster(B, oracle, pool, k, units, scores):
     x = x.astype(np.float32)
     for c_max, n_vert, forced in ((256, 8192, 32), (8192, 256, 0), (256, 40000, 16), (40000, 700, 0), (1024, 1024, 0)):
         run_vert_case(B, oracle, x, [0, n], k, c_max, forced, n_vert, pool=pool)
+
+
+@pytest.mark.parametrize("n", [16384, 17001])                    # one CTA to a unit, streamed
+@pytest.mark.parametrize("units", [148, 149])                    # a CTA to each budget, one for both
+@pytest.mark.parametrize("scores", ["random", "ties", "crowded_sample"])
+def test_two_budgets_of_many_units(B, oracle, n, units, scores):
+    """Two budgets of width-7 pooling, with a floor that serves both, neither, or the smaller alone, whichever comes first: the
+    larger then goes through the generic selection, which works in the candidates' memory."""
+    rng = np.random.default_rng(units + n)
+    x = rng.integers(0, 5, size=(1, units, n)) / 8.0 if scores == "ties" else rng.random((1, units, n)) ** 6
+    if scores == "crowded_sample":
+        for u in range(units):
+            at = one_cta_sample_positions(u, n) if n == 16384 else stream_sample_positions(u, n, 6)
+            x[0, u, rng.choice(at, 260 if n == 16384 else 90, replace=False)] += 16.0
+    x = x.astype(np.float32)
+    for c_max, n_vert, forced in ((200, 2700, 0), (2700, 200, 32), (300, 400, 16), (200, 20000, 0), (n, 300, 0)):
+        if max(c_max, n_vert) * 6 <= n or scores == "random":
+            run_vert_case(B, oracle, x, [0, n], 7, c_max, forced, n_vert)
 
 
 STRUCTURED = {
@@ -949,6 +988,16 @@ def test_large_budgets_and_ties_cost_little_more(B):
     x = torch.rand(1, 1, n, device="cuda", generator=g) ** 6
     times = [time_of(lambda: B.spec_pool_topk(pr, y, B.POOL_MAX, 5, 2048, 0, out, None)) for y in (x, torch.zeros_like(x))]
     assert times[1] <= 1.6 * times[0], "%.4f ms for tied scores, %.4f for random ones" % (times[1], times[0])
+    # two budgets of many units share the sweep and the candidates
+    units, n = 2048, 3000
+    pr = B.make_problem(n_layers=1, n_q_heads=units, n_kv_heads=units, head_dim=128, n_lookahead=1, n_window=0, softmax_scale=1.0,
+                        total_tokens=n, n_in=n)
+    ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+    x = torch.rand(1, units, n, device="cuda", generator=g) ** 6
+    out = torch.empty((2, units * 400), dtype=torch.int32, device="cuda")
+    one = time_of(lambda: B.spec_pool_topk(pr, x, B.POOL_MAX, 7, 375, 0, out[0], None, workspace=ws))
+    two = time_of(lambda: B.spec_pool_topk_vert(pr, x, B.POOL_MAX, 7, 375, 0, out[0], None, 300, out[1], None, workspace=ws))
+    assert two <= 1.35 * one, "%.4f ms for two budgets, %.4f for one" % (two, one)
 
 
 @pytest.mark.parametrize("spread", [2.0 ** -4, 2.0 ** -7, 2.0 ** -12])
