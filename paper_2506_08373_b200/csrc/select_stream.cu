@@ -33,6 +33,7 @@
 #include "select_common.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace spec {
 
@@ -177,13 +178,13 @@ __device__ __forceinline__ bool finish_unit(const StreamParams& p, const UnitGeo
 template <bool BOTH>
 __device__ __forceinline__ void finish_budgets(const StreamParams& p, const UnitGeom& g, int unit, int b, SelectMem& sm, const uint32_t* keys,
                                                const uint32_t* pos, int n, bool failed, uint32_t floor_key, uint32_t top, void* scratch) {
-  if (!BOTH) {
-    finish_unit(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, scratch);
-    return;
-  }
+  if constexpr (BOTH) {
 #pragma unroll 1
-  for (b = 0; b < 2; ++b)
-    if (!finish_unit(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, scratch)) failed = true;
+    for (b = 0; b < 2; ++b)
+      if (!finish_unit(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, scratch)) failed = true;
+  } else {
+    finish_unit(p, g, unit, b, sm, keys, pos, n, failed, floor_key, top, scratch);
+  }
 }
 __device__ __forceinline__ bool cuts(const UnitGeom& g, int b) { return g.take[b] > 0 && g.take[b] < g.e; }
 
@@ -336,6 +337,13 @@ __device__ __forceinline__ void pool_candidates(const UnitGeom& g, const WarpSco
 
 // ---------------------------------------------------------------- 1. the floor -------
 
+// One sample per 2^shift positions of a unit (of the eligible ones; extent: with the slots before the first).
+__host__ __device__ inline int sample_shift(int eligible, int extent) {
+  int shift = eligible >= 65536 ? 7 : eligible >= 16384 ? 6 : 5;
+  while (((extent >> shift) + 1) > kMaxSamples) ++shift;
+  return shift;
+}
+
 __global__ void __launch_bounds__(kSelThreads) sample_floor_kernel(const StreamParams p) {
   __shared__ __align__(16) SelectMem sm;
   const int unit = blockIdx.x, tid = threadIdx.x;
@@ -353,8 +361,7 @@ __global__ void __launch_bounds__(kSelThreads) sample_floor_kernel(const StreamP
     // x = position + mis8 puts every multiple of eight on a 32-byte boundary of global memory
     const int mis8 = (int)((reinterpret_cast<uintptr_t>(g.src) >> 2) & 7u);
     const int X = g.e + mis8;
-    int shift = g.e >= 65536 ? 7 : g.e >= 16384 ? 6 : 5;             // one sample per 2^shift positions
-    while (((X >> shift) + 1) > kMaxSamples) ++shift;
+    const int shift = sample_shift(g.e, X);
     const int spg = 1 << (shift - 3);                                // sectors per sample group
     const int n_sectors = (X + 7) >> 3;
     const int n_groups = (n_sectors + spg - 1) / spg;                // <= kMaxSamples
@@ -434,11 +441,13 @@ static size_t held_bytes(int held_cap) { return std::max((size_t)held_cap * 8, k
 
 // One CTA per unit and budget while all of them are on the GPU at once, two to an SM; BOTH: one per unit for its two budgets, which
 // then cost a second threshold and emission but no second copy of the candidates (148 units of 17001, 384 and 400 kept:
-// 15.5 us with two CTAs to a unit, 17.1 with one; 2048 units 137 and 118).  The next kernel is not let in early
+// 15.5 us with two CTAs to a unit, 17.1 with one; 2048 units 137 and 118).  CTAS: three to an SM with 40 registers a thread for
+// units in several waves whose candidates leave the memory (2048 units of 3000, 428 kept: 83 -> 73 us; 256 units of 131072,
+// all there at once, 47.0 -> 48.2).  The next kernel is not let in early
 // either: the floor CTAs of a selection that follows would crowd on the few SMs with room beside two finishing CTAs, and
 // the sweep behind them waits for the slowest (256 units of 131072, one selection after the other: 70.4 -> 46.9 us each).
-template <bool BOTH>
-__global__ void __launch_bounds__(kSelThreads, 2) stream_finish_kernel(const StreamParams p) {
+template <int CTAS, bool BOTH>
+__global__ void __launch_bounds__(kSelThreads, CTAS) stream_finish_kernel(const StreamParams p) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
   __shared__ __align__(16) SelectMem sm;
   __shared__ int chunk_at[kSelThreads], chunk_n[kSelThreads];
@@ -640,35 +649,41 @@ int run_stream_topk(const spec_problem* pr, const float* scores, int c_max, int 
   if (p.rounds * kWarpSpan > kSelChunkMax) return SPEC_OK;
   static_assert(kWarpSpan == kSelChunkMin, "the workspace has a count per kSelChunkMin positions");
   p.chunks_max = (int)(((int64_t)p.max_len + 3 + p.rounds * kWarpSpan - 1) / (p.rounds * kWarpSpan));
-  // The floor lets through about (m + 4 sqrt(m) + 8) * rate candidates (m = budget / rate, rate = 32 to 128
-  // positions per sample), with the spread of as many samples: 1.6 to 3.4 times budgets from 8192 down to 1024.  At
-  // this capacity a unit overflows less than once in 10^6; with 3 * budget + 2048 one unit in 100 did at 128K,
-  // and one generic selection costs more than the other 255 units together.
   const int largest = std::max(c_max, n_vert);
   const int64_t room = ((int64_t)kSmemLimit - 16 * 1024) / 8;
   p.held_cap = (int)(std::min<int64_t>(4 * (int64_t)largest + 4096, room) & ~(int64_t)3);
   if (p.held_cap < 2 * (int64_t)largest + 2048) return SPEC_OK;                 // too large a budget for the finishing CTA
+  // The floor is about the rho-th of the samples, rho = m + 4 sqrt(m) + 8 and m = budget / rate, rate = 32 to 128 positions
+  // per sample; a full bin lets r = 1.25 rho + 8 samples in at most.  With room for rate * (r + 5 sqrt(r) + 12) candidates a
+  // unit overflows less than once in 10^7 (Poisson), and for 2048 of 131072 with 4 * budget + 4096 less than once in 10^5 (with
+  // 3 * budget + 2048 one unit in 100 did, and one generic selection costs more than the other 255 units together).  Memory
+  // beyond that only keeps a second CTA off the SM: 2048 units of 16384, 2730 kept, 214 us with 4 * budget + 4096, 153 so.
+  const int rate = 1 << sample_shift(p.max_len, p.max_len + 7);
+  const double m = (double)largest / rate, r = 1.25 * (m + 4.0 * std::sqrt(m) + 8.0) + 8.0;
+  const int64_t enough = std::min<int64_t>((int64_t)(rate * (r + 5.0 * std::sqrt(r) + 12.0)), p.max_len);
+  p.held_cap = (int)std::min<int64_t>(p.held_cap, (enough + 3) & ~(int64_t)3);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   p.head = reinterpret_cast<int32_t*>(ws + wp.sel_head_off);
   p.head_words = wp.sel_head_words;
   p.cand = reinterpret_cast<uint2*>(ws + wp.sel_cand_off);
   p.row_entries = wp.sel_row_entries;
 
+  typedef void (*FinishKernel)(const StreamParams);
+  static const FinishKernel finish[4] = {stream_finish_kernel<2, false>, stream_finish_kernel<2, true>, stream_finish_kernel<3, false>, stream_finish_kernel<3, true>};
   static int set[64] = {0};
   int dev = 0;
   SPEC_CUDA_OK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return SPEC_OK;
   if (!__atomic_load_n(&set[dev], __ATOMIC_ACQUIRE)) {
-    SPEC_CUDA_OK(cudaFuncSetAttribute(stream_finish_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
-    SPEC_CUDA_OK(cudaFuncSetAttribute(stream_finish_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
+    for (const FinishKernel f : finish) SPEC_CUDA_OK(cudaFuncSetAttribute((const void*)f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit - 16 * 1024));
     __atomic_store_n(&set[dev], 1, __ATOMIC_RELEASE);
   }
   SPEC_CUDA_OK(launch_dependent(sample_floor_kernel, dim3((unsigned)n_units), kSelThreads, 0, st, p));
   const dim3 sweep_grid((unsigned)((p.chunks_max + kSweepWarps - 1) / kSweepWarps), (unsigned)(pr->n_layers * pr->n_kv_heads), (unsigned)pr->n_seq);
   SPEC_CUDA_OK(launch_dependent(stream_sweep_kernel, sweep_grid, kSweepThreads, 0, st, p));
   const bool both = both_budgets(p, n_units);
-  SPEC_CUDA_OK(launch_dependent(both ? stream_finish_kernel<true> : stream_finish_kernel<false>, dim3((unsigned)n_units, n_vert > 0 && !both ? 2 : 1),
-                                kSelThreads, held_bytes(p.held_cap), st, p));
+  const bool three = n_units > 2 * sm_count() && held_bytes(p.held_cap) <= (size_t)(228 * 1024 / 3 - 14 * 1024);   // 13 KB and 1 KB beside them
+  SPEC_CUDA_OK(launch_dependent(finish[2 * three + both], dim3((unsigned)n_units, n_vert > 0 && !both ? 2 : 1), kSelThreads, held_bytes(p.held_cap), st, p));
   *done = true;
   return SPEC_OK;
 }

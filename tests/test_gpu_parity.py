@@ -930,7 +930,9 @@ def test_topk_short_units_in_one_cta_and_streamed(B, W, oracle):
     (150000, 5, 9000, 1), (150000, 5, 9500, 1),                  # the least memory for candidates, and none
     (75000, 7, 12480, 1), (75000, 7, 12481, 1),                  # the largest budget that is streamed
     (524285, 7, 700, 1), (524286, 7, 700, 1),                    # one round per sweeping warp, two
-    (1048573, 7, 700, 1), (1048574, 7, 700, 1)])                 # the longest unit that is streamed
+    (1048573, 7, 700, 1), (1048574, 7, 700, 1),                  # the longest unit that is streamed
+    (16385, 7, 800, 296), (16385, 7, 800, 297),                  # two finishing CTAs to an SM, three
+    (16385, 7, 1450, 297), (16385, 7, 1451, 297)])               # and the largest budget for three
 def test_topk_at_the_limits_of_the_selection_kernels(B, W, oracle, n, k, c_max, units):
     x = (np.random.default_rng(n + units).random((1, units, n)) ** 5).astype(np.float32)
     x[:, :, n // 2:n // 2 + 60] = x[:, :, :1]                     # a run of equal keys
@@ -998,6 +1000,15 @@ def test_large_budgets_and_ties_cost_little_more(B):
     one = time_of(lambda: B.spec_pool_topk(pr, x, B.POOL_MAX, 7, 375, 0, out[0], None, workspace=ws))
     two = time_of(lambda: B.spec_pool_topk_vert(pr, x, B.POOL_MAX, 7, 375, 0, out[0], None, 300, out[1], None, workspace=ws))
     assert two <= 1.35 * one, "%.4f ms for two budgets, %.4f for one" % (two, one)
+    # many units of a large budget: two finishing CTAs to an SM
+    n = 16384
+    pr = B.make_problem(n_layers=1, n_q_heads=units, n_kv_heads=units, head_dim=128, n_lookahead=1, n_window=0, softmax_scale=1.0,
+                        total_tokens=n, n_in=n)
+    ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+    x = torch.rand(1, units, n, device="cuda", generator=g) ** 6
+    out = torch.empty(units * 2730, dtype=torch.int32, device="cuda")
+    times = [time_of(lambda: B.spec_pool_topk(pr, x, B.POOL_MAX, 7, c, 0, out, None, workspace=ws)) for c in (682, 2730)]
+    assert times[1] <= 1.8 * times[0], "%.4f ms for a sixth of the positions, %.4f for a 24th" % (times[1], times[0])
 
 
 @pytest.mark.parametrize("spread", [2.0 ** -4, 2.0 ** -7, 2.0 ** -12])
