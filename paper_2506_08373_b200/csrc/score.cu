@@ -253,7 +253,7 @@ struct Seg {
 
 struct SegIter {
   long long g, g_end, per_cta, n_tiles;
-  int TT;
+  int TT, s;              // s: sequence of the last segment
   // Whether a unit that ends before tile `end` is the last one that CTA `cta` worked on.
   __device__ __forceinline__ bool last_segment(int cta, long long end) const {
     const long long range_end = (cta + 1) * per_cta;
@@ -276,6 +276,7 @@ __device__ void build_tile_prefix(const ScoreParams& p, int* tp) {
 __device__ __forceinline__ SegIter seg_begin(const ScoreParams& p, const int* tp, int n_ctas, int cta) {
   SegIter it;
   it.TT = tp[p.n_seq];
+  it.s = -2;                                               // none
   const long long N = (long long)p.L * p.Hkv * it.TT;
   it.n_tiles = N;
   if (p.pieces > 0) {                                      // every unit cut evenly among as many CTAs of its own
@@ -298,17 +299,22 @@ __device__ __forceinline__ SegIter seg_begin(const ScoreParams& p, const int* tp
 
 // The next segment of the range: pass 1 goes through it forwards, pass 2 backwards, tile by tile, so that pass 2 begins
 // with the keys that pass 1 has just left in L2 (one layer of 64K, 134 MB of keys: 118.6 -> 115.0 us).
-template <int PASS>
+template <int PASS, bool RAGGED>
 __device__ bool seg_next(SegIter& it, const ScoreParams& p, const int* tp, Seg& sg) {
   if (it.g >= it.g_end) return false;
   const long long at = PASS == 1 ? it.g : it.g_end - 1;
   const int lh = (int)(at / it.TT);
   const int rem = (int)(at % it.TT);
-  int lo = 0, hi = p.n_seq;
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (tp[mid] <= rem) lo = mid; else hi = mid;
+  // the sequence that the tile belongs to, the last one with tp[lo] <= rem: as a rule the neighbour of the last segment's
+  int lo = PASS == 1 ? it.s + 1 : it.s - 1, hi = p.n_seq;
+  if (!RAGGED || lo < 0 || lo >= hi || tp[lo] > rem || tp[lo + 1] <= rem) {
+    lo = 0;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (tp[mid] <= rem) lo = mid; else hi = mid;
+    }
   }
+  it.s = lo;
   sg.s = lo;
   sg.l = lh / p.Hkv;
   sg.h = lh % p.Hkv;
@@ -539,7 +545,9 @@ __device__ __forceinline__ uint32_t hidden_columns(int row0, int R, int n_window
 // segments: a unit's partials are read from L2 by the few CTAs that share the unit, which takes
 // about a microsecond, where a kernel of its own between the passes took 4 to 22 (one layer of 64K:
 // 80 partials per row in a serial loop) plus two launch gaps.  When there are fewer rows than half
-// the threads, several threads take a share of a row's partials each and meet in shared memory.
+// the threads and more partials than a thread loads at once, several threads take a share of a row's partials each and
+// meet in shared memory.  Short sequences have a few partials in hundreds of segments per CTA, where the meeting and 16
+// exponentials for four partials cost more than all else (see RAGGED below).
 __device__ __forceinline__ void fold_stats(float& m, float& z, float pm, float pz) {
   const float mn = fmaxf(m, pm);
   if (mn > -INFINITY) z = z * exp2f(m - mn) + pz * exp2f(pm - mn);
@@ -548,22 +556,34 @@ __device__ __forceinline__ void fold_stats(float& m, float& z, float pm, float p
 
 constexpr int kMergeLoads = 16;       // in flight per thread; with 8, one layer of 12K (72 partials per row) spent 8 us here
 
-template <bool MAXRED>
+template <bool MAXRED, bool RAGGED>
 __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2* __restrict__ part, int n_last, int n, int et, float scale_log2, float* c_sm, float2* merge_sm) {
   const int Mr = (p.M + 31) & ~31;
-  const int slices = p.merge_slots > 0 ? p.merge_slots / Mr : 1;
+  const int slices = p.merge_slots > 0 && n > kMergeLoads ? p.merge_slots / Mr : 1;
   for (int i0 = 0; i0 < p.M_pad; i0 += kEpilogueThreads) {
     const int sl = slices > 1 ? et / Mr : 0;
     const int i = slices > 1 ? et - sl * Mr : i0 + et;
     float m = -INFINITY, z = 0.f;
-    if (i < p.M && sl < slices) {
+    auto partial_at = [&](int c) { return __ldcg(part + (size_t)(min(c, n_last) * kEpilogueWarpgroups + max(c - n_last, 0)) * p.M + i); };
+    if (RAGGED && n <= 4) {
+      if (i < p.M) {
+        float2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = u < n ? partial_at(u) : make_float2(-INFINITY, 0.f);
+        m = fmaxf(fmaxf(v[0].x, v[1].x), fmaxf(v[2].x, v[3].x));
+        if (m > -INFINITY) {
+#pragma unroll
+          for (int u = 0; u < 4; ++u) z += v[u].y * exp2f(v[u].x - m);
+        }
+      }
+    } else if (i < p.M && sl < slices) {
       for (int c0 = sl; c0 < n; c0 += kMergeLoads * slices) {
         float2 v[kMergeLoads];
         float mx = m;
 #pragma unroll
         for (int u = 0; u < kMergeLoads; ++u) {
           const int c = c0 + u * slices;
-          v[u] = c < n ? __ldcg(part + (size_t)(min(c, n_last) * kEpilogueWarpgroups + max(c - n_last, 0)) * p.M + i) : make_float2(-INFINITY, 0.f);
+          v[u] = c < n ? partial_at(c) : make_float2(-INFINITY, 0.f);
         }
 #pragma unroll
         for (int u = 0; u < kMergeLoads; ++u) mx = fmaxf(mx, v[u].x);
@@ -605,8 +625,10 @@ __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2
 
 // FLAG: pass 1, whether remaining rows are scored on columns (a variant of its own: the registers that it needs
 // slowed the other one down by 4 to 20 %); pass 2, whether the reduction is the maximum.  CAUSAL: the causal window,
-// likewise apart (its masks cost the other kernels 1 to 2 % in registers).
-template <int PASS, bool FLAG, bool CAUSAL>
+// likewise apart (its masks cost the other kernels 1 to 2 % in registers).  RAGGED: more than one sequence.  What a
+// segment costs beside its tiles counts there (1024 sequences of 100 to 199 keys, 2 layers of 8 heads, 32 rows: 925 us with
+// the code for one sequence, 661 so), and the code for it cost one layer of 12345 keys 0.4 of 52.8 us.
+template <int PASS, bool FLAG, bool CAUSAL, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -677,7 +699,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         const uint64_t policy = evict_first_policy();
         uint32_t kit = 0, nseg = 0;
         bool ok = true;
-        while (ok && seg_next<PASS>(it, p, tp, sg)) {
+        while (ok && seg_next<PASS, RAGGED>(it, p, tp, sg)) {
           if (nseg > 0) ok = mbar_wait(q_empty, (nseg - 1) & 1, abort_flag);   // previous unit's MMAs retired
           if (!ok) break;
           ++nseg;
@@ -723,7 +745,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       const uint32_t q_half16 = q_half_bytes >> 4;
       const uint32_t k_half16 = k_half_bytes >> 4;
       while (ok) {
-        const bool more = seg_next<PASS>(it, p, tp, sg);
+        const bool more = seg_next<PASS, RAGGED>(it, p, tp, sg);
         const int nt = uniform(more ? sg.nt : 0);
         if (nt == 0) break;
         ok = mbar_wait_warp(q_full, nseg & 1, abort_flag);
@@ -810,7 +832,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       float mrun[kMaxMTiles], zrun[kMaxMTiles];
       float* my_ref = rem_sm + (warp - 4) * p.rem_cols;
       // Every epilogue thread passes the barriers of every segment, also after a wait has given up.
-      while (seg_next<PASS>(it, p, tp, sg)) {
+      while (seg_next<PASS, RAGGED>(it, p, tp, sg)) {
         float rem_m[2] = {-INFINITY, -INFINITY}, rem_z[2] = {0.f, 0.f};
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
 #pragma unroll
@@ -952,14 +974,17 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       bool waited = false;
       // Every epilogue thread passes the barriers of every segment, also after a wait has
       // given up, so that no warp is left waiting at them.
-      while (seg_next<PASS>(it, p, tp, sg)) {
+      while (seg_next<PASS, RAGGED>(it, p, tp, sg)) {
         // the CTAs of pass 1 that worked on this unit: its tiles are u0 .. u0 + n_tiles - 1 of the global tile space
         int b0 = sg.unit * p.pieces, b1 = b0 + p.pieces - 1, n_part = p.pieces;
         if (p.pieces == 0) {
           const long long u0 = (long long)(sg.l * p.Hkv + sg.h) * it.TT + tp[sg.s];
           const int n_tiles = tp[sg.s + 1] - tp[sg.s];
-          b0 = (int)(u0 / per_cta);
-          b1 = (int)((u0 + n_tiles - 1) / per_cta);
+          b0 = b1 = (int)blockIdx.x;
+          if (sg.nt < n_tiles) {                                // other CTAs had a part of it, too
+            b0 = (int)(u0 / per_cta);
+            b1 = (int)((u0 + n_tiles - 1) / per_cta);
+          }
           n_part = b1 - b0 + (it.last_segment(b1, u0 + n_tiles) ? 1 : kEpilogueWarpgroups);
         }
         if (!waited) {
@@ -968,7 +993,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           launch_dependents();
         }
         asm volatile("bar.sync 1, 512;" ::: "memory");          // previous unit's constants no longer read
-        row_constants<MAXRED>(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
+        row_constants<MAXRED, RAGGED>(p, reinterpret_cast<const float2*>(p.partial) + (size_t)(sg.unit + b0) * kEpilogueWarpgroups * p.M,
                               b1 - b0, n_part, et, scale_log2, c_sm, merge_sm);
         asm volatile("bar.sync 1, 512;" ::: "memory");
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
@@ -1169,9 +1194,12 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
 
   const int n_ctas = wp.score_ctas;
   typedef void (*ScoreKernel)(const CUtensorMap, const CUtensorMap, const ScoreParams);
-  static const ScoreKernel kernels[2][2][2] = {             // [pass][flag][causal]
-      {{score_kernel<1, false, false>, score_kernel<1, false, true>}, {score_kernel<1, true, false>, score_kernel<1, true, true>}},
-      {{score_kernel<2, false, false>, score_kernel<2, false, true>}, {score_kernel<2, true, false>, score_kernel<2, true, true>}}};
+  static const ScoreKernel kernels[2][2][2][2] = {          // [ragged][pass][flag][causal]
+      {{{score_kernel<1, false, false, false>, score_kernel<1, false, true, false>}, {score_kernel<1, true, false, false>, score_kernel<1, true, true, false>}},
+       {{score_kernel<2, false, false, false>, score_kernel<2, false, true, false>}, {score_kernel<2, true, false, false>, score_kernel<2, true, true, false>}}},
+      {{{score_kernel<1, false, false, true>, score_kernel<1, false, true, true>}, {score_kernel<1, true, false, true>, score_kernel<1, true, true, true>}},
+       {{score_kernel<2, false, false, true>, score_kernel<2, false, true, true>}, {score_kernel<2, true, false, true>, score_kernel<2, true, true, true>}}}};
+  const bool ragged = pr->n_seq > 1;
   // The kernels may use all of an SM's shared memory; the attribute is set once per device (it is per
   // function and context, so setting it per call would race between host threads).
   {
@@ -1180,8 +1208,8 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     SPEC_CUDA_OK(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) return fail(SPEC_ERR_UNSUPPORTED, "device ordinal %d is not supported", dev);
     if (!__atomic_load_n(&set[dev], __ATOMIC_ACQUIRE)) {
-      for (int i = 0; i < 8; ++i) {
-        const void* f = (const void*)kernels[i >> 2][(i >> 1) & 1][i & 1];
+      for (int i = 0; i < 16; ++i) {
+        const void* f = (const void*)kernels[i >> 3][(i >> 2) & 1][(i >> 1) & 1][i & 1];
         SPEC_CUDA_OK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         // The warpgroups divide the registers that the block was launched with: a build that launches with fewer
         // would wait for registers that do not exist.
@@ -1235,8 +1263,8 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     p.n_stages = stages;
     int smem = stages * (int)p.stage_bytes + (int)p.q_bytes + small + rem_bytes;
     if (smem < 120 * 1024) smem = 120 * 1024;             // one CTA per SM: each CTA owns the whole TMEM
-    SPEC_CUDA_OK(launch_dependent(kernels[0][p.rem_cols > 0][causal_window], dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
-    SPEC_CUDA_OK(launch_dependent(kernels[1][reduce == SPEC_REDUCE_MAX][causal_window], dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
+    SPEC_CUDA_OK(launch_dependent(kernels[ragged][0][p.rem_cols > 0][causal_window], dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
+    SPEC_CUDA_OK(launch_dependent(kernels[ragged][1][reduce == SPEC_REDUCE_MAX][causal_window], dim3(n_ctas), kThreads, smem, st, tm_q, tm_k, p));
   }
   return SPEC_OK;
 }

@@ -90,6 +90,59 @@ def test_score_ragged_with_empty_and_tile_edge_lengths(B, W, oracle):
     assert list(ocnt[:, 0, 0]) == [1, 32, 32, 32, 0, 32, 32, 5]
 
 
+@pytest.mark.parametrize("causal", [0, 1])
+@pytest.mark.parametrize("n_seq,longest,rows", [(2, 3000, 8), (1024, 200, 8), (1000, 130, 48)])
+def test_score_many_short_sequences(B, W, oracle, n_seq, longest, rows, causal):
+    """Hundreds of segments to a CTA, most of them whole sequences of one or two tiles, with runs of empty ones."""
+    L, H, G, d, window = 2, 4, 4, 64, 5
+    rng = np.random.default_rng(n_seq + causal)
+    lens = rng.integers(1, longest + 1, n_seq)
+    lens[rng.random(n_seq) < 0.3] = 0
+    lens[-1] = longest
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    gen = torch.Generator().manual_seed(n_seq)
+    q = torch.randn(n_seq, L, H * G, rows, d, generator=gen).to(torch.bfloat16).cuda()
+    k = torch.randn(L, H, cu[-1], d, generator=gen).to(torch.bfloat16).cuda()
+    cu_t = torch.tensor(cu, dtype=torch.int32, device="cuda")
+    pr = B.make_problem(n_layers=L, n_q_heads=H * G, n_kv_heads=H, head_dim=d, n_lookahead=rows - window, n_window=window,
+                        softmax_scale=d ** -0.5, total_tokens=cu[-1], n_in=longest, n_seq=n_seq, cu_seqlens=cu_t, k=k)
+    ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for reduce in (0, 1):
+        got = torch.full((L, H, cu[-1]), float("nan"), device="cuda")
+        B.spec_score(pr, q, k, got, ws, reduce=reduce, causal_window=causal, status_word=status)
+        assert status.item() == 0
+        ref = oracle.spec_score(bits(q), bits(k), cu, rows - window, window, d ** -0.5, mode=reduce, causal_window=bool(causal))
+        assert_scores_close(got.cpu().numpy(), ref, cu)
+
+
+def test_short_sequences_are_scored_at_the_rate_of_tiles(B):
+    """1024 sequences of 100 to 199 keys against one prompt of as many key tiles: queries, constants and bookkeeping per
+    sequence may cost a small multiple of a tile's arithmetic and no more."""
+    L, H, R, d = 2, 8, 32, 64
+    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    times = []
+    for lens in ([100 + i % 100 for i in range(1024)], [128 * sum(-(-(100 + i % 100) // 128) for i in range(1024))]):
+        T, n_seq = sum(lens), len(lens)
+        q = torch.randn(n_seq, L, H, R, d, device="cuda").to(torch.bfloat16)
+        k = torch.randn(L, H, T, d, device="cuda").to(torch.bfloat16)
+        cu = torch.tensor(np.cumsum([0] + lens), dtype=torch.int32, device="cuda") if n_seq > 1 else None
+        pr = B.make_problem(n_layers=L, n_q_heads=H, n_kv_heads=H, head_dim=d, n_lookahead=R, n_window=0, softmax_scale=d ** -0.5,
+                            total_tokens=T, n_in=max(lens), n_seq=n_seq, cu_seqlens=cu, k=k)
+        ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+        out = torch.empty((L, H, T), device="cuda")
+        best = float("inf")
+        for _ in range(6):
+            e0.record()
+            for _ in range(5):
+                B.spec_score(pr, q, k, out, ws)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1) / 5)
+        times.append(best)
+    assert times[0] <= 4.8 * times[1], "%.4f ms for short sequences, %.4f for one prompt" % tuple(times)
+
+
 def test_score_max_reduce_and_row_weights(B, W, oracle):
     w = small(W, n_in=600)
     g = Gpu(B, W, w, [0])
