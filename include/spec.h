@@ -12,8 +12,8 @@
  *     the device's address space, which suits a source that is read sparsely,
  *     such as v in spec_compact_kv).  The library never allocates, frees or
  *     retains them.  Scratch memory is passed in as
- *     `workspace` (size from spec_workspace_bytes); its contents are undefined
- *     on entry and on return.
+ *     `workspace` (size from spec_workspace_bytes, any alignment); its contents
+ *     are undefined on entry and on return.
  *   - Work is enqueued asynchronously on `stream` (a cudaStream_t passed as
  *     void*; NULL = the legacy default stream).  The int32 return value is a
  *     spec_status: argument errors are detected on the host before anything is

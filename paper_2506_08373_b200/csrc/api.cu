@@ -99,7 +99,7 @@ WorkspacePlan plan_workspace(const spec_problem* p) {
   w.sel_cand_off = off;
   w.sel_cand_bytes = (size_t)w.sel_row_entries * (size_t)p->n_layers * p->n_kv_heads * 8;
   off = align_up(off + w.sel_cand_bytes, 256);
-  w.total = off;
+  w.total = off + 16;                                      // for workspace_base
   return w;
 }
 

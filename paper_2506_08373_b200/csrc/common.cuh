@@ -40,6 +40,11 @@ struct WorkspacePlan {
   size_t total;
 };
 SPEC_HIDDEN WorkspacePlan plan_workspace(const spec_problem* p);
+// Where the layout begins: the kernels read and write up to 16 bytes at a time there, and the caller's memory may begin
+// anywhere (plan_workspace counts the bytes in front in).
+SPEC_HIDDEN inline uint8_t* workspace_base(void* workspace) {
+  return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(workspace) + 15) & ~(uintptr_t)15);
+}
 // Streaming selection: every chunk of a sequence owns a segment of the candidate array as long as
 // the chunk itself (at most kSelChunkMax positions, at least kSelChunkMin), so a sequence needs
 // its length plus a partial chunk; the chunks' candidate counts sit in the unit's header.

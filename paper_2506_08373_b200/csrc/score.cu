@@ -1180,7 +1180,7 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   ScoreParams p;
   p.cu = pr->cu_seqlens;
   p.row_weight = row_weight;
-  uint8_t* ws = static_cast<uint8_t*>(workspace);
+  uint8_t* ws = workspace_base(workspace);
   p.partial = reinterpret_cast<float*>(ws + wp.partial_off);
   p.scores = scores_out;
   p.status = status_word;

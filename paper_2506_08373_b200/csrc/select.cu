@@ -1136,7 +1136,7 @@ SPEC_EXPORT int32_t specpc_token_select(const spec_problem* pr, const float* sco
   if (rc != SPEC_OK) return rc;
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  float* tok = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + wp.token_off);
+  float* tok = reinterpret_cast<float*>(workspace_base(workspace) + wp.token_off);
   const int64_t T = pr->total_tokens;
   if (T > 0) {
     SPEC_CUDA_OK(launch_token_reduce(scores, tok, T, pr->n_layers * pr->n_kv_heads, layer_head_reduce, st));

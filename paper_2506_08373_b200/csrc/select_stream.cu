@@ -662,7 +662,7 @@ int run_stream_topk(const spec_problem* pr, const float* scores, int c_max, int 
   const double m = (double)largest / rate, r = 1.25 * (m + 4.0 * std::sqrt(m) + 8.0) + 8.0;
   const int64_t enough = std::min<int64_t>((int64_t)(rate * (r + 5.0 * std::sqrt(r) + 12.0)), p.max_len);
   p.held_cap = (int)std::min<int64_t>(p.held_cap, (enough + 3) & ~(int64_t)3);
-  uint8_t* ws = static_cast<uint8_t*>(workspace);
+  uint8_t* ws = workspace_base(workspace);
   p.head = reinterpret_cast<int32_t*>(ws + wp.sel_head_off);
   p.head_words = wp.sel_head_words;
   p.cand = reinterpret_cast<uint2*>(ws + wp.sel_cand_off);

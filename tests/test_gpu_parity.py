@@ -727,6 +727,41 @@ def test_specpc_paper_settings_from_real_scores(B, W, oracle):
     run_topk_case(B, W, oracle, sc, g.cu, oracle.POOL_MAX, 32, 512, 0)
 
 
+@pytest.mark.parametrize("offset", [1, 4, 8, 12])
+def test_workspace_at_any_alignment(B, W, offset):
+    """A workspace that begins between 16-byte boundaries, of exactly the size asked for, gives what an aligned one does and
+    nothing behind it is written: scoring, streamed and two-budget selection, keep set with both pooling stages."""
+    w = small(W, n_layers=1, n_in=20000, c_max=256)
+    g = Gpu(B, W, w, [0])
+    need = B.spec_workspace_bytes(g.pr)
+
+    def path(ws):
+        scores = torch.full((1, w.n_kv_heads, g.T), float("nan"), device="cuda")
+        B.spec_score(g.pr, g.q, g.k, scores, ws, status_word=g.status)
+        out = [scores]
+        for n_vert in (0, 512):
+            idx = torch.full((w.n_kv_heads, w.c_max), -7, dtype=torch.int32, device="cuda")
+            vidx = torch.full((w.n_kv_heads, 512), -7, dtype=torch.int32, device="cuda")
+            if n_vert:
+                B.spec_pool_topk_vert(g.pr, scores, 0, 7, w.c_max, 0, idx, None, n_vert, vidx, workspace=ws, status_word=g.status)
+            else:
+                B.spec_pool_topk(g.pr, scores, 0, 7, w.c_max, 0, idx, None, workspace=ws, status_word=g.status)
+            out += [idx, vidx]
+        keep = torch.full((1, 300), -7, dtype=torch.int32, device="cuda")
+        n_keep = torch.full((1,), -7, dtype=torch.int32, device="cuda")
+        B.specpc_token_select(g.pr, scores, 0, B.POOL_AVG_THEN_MAX, 8, 300, 8, 0, keep, 300, n_keep, ws, status_word=g.status)
+        return out + [keep, n_keep]
+
+    want = path(g.ws)
+    buf = torch.full((need + 64,), 99, dtype=torch.uint8, device="cuda")
+    got = path(buf[offset:offset + need])
+    torch.cuda.synchronize()
+    assert g.status.item() == 0
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
+    assert torch.all(buf[:offset] == 99) and torch.all(buf[offset + need:] == 99)
+
+
 def test_score_zero_length_prompt_clears_the_output(B, W):
     """n_in = 0 with a non-empty token axis: nothing to score, and the whole output buffer reads as zero."""
     pr = B.make_problem(n_layers=2, n_q_heads=4, n_kv_heads=2, head_dim=64, n_lookahead=2, n_window=2, softmax_scale=0.125,
