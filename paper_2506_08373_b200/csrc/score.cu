@@ -1134,9 +1134,17 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   const int R = pr->n_lookahead + pr->n_window;
   const int G = pr->n_q_heads / pr->n_kv_heads;
   const int M = G * R;
-  // The query rows of a unit stay resident in shared memory; more than fit (G*R*head_dim > 81920) are
-  // scored in several launches over equal groups of rows, whose contributions add up in scores_out.
-  const int rows_max = std::min(81920 / d, kMaxMTiles * 128) / 128 * 128;
+  // The query rows of a unit stay resident in shared memory, in blocks of 128, beside two key stages and what grows with
+  // them and with the number of sequences (from 70 sequences on, 512 instead of 640 rows of head_dim 128); more than fit
+  // are scored in several launches over groups of as many blocks as the largest needs, whose contributions add up in scores_out.
+  const int smem_max = 227 * 1024;
+  auto small_bytes = [&](int rows) {                       // all but queries and keys
+    const int Mr = (rows + 31) & ~31, rows_pad = (rows + 127) / 128 * 128;
+    const int slots = 2 * Mr <= kEpilogueThreads ? kEpilogueThreads / Mr * Mr : 0;
+    return rows_pad * 4 + slots * 8 + (pr->n_seq + 1) * 4 + 8 + kNumBars * 8 + 16;
+  };
+  int rows_max = std::min(81920 / d, kMaxMTiles * 128) / 128 * 128;
+  while (rows_max > 128 && rows_max * d * 2 + 2 * kTileKeys * d * 2 + small_bytes(rows_max) > smem_max) rows_max -= 128;
   const int n_groups = (M + rows_max - 1) / rows_max;
   const int rows_group = ((M + n_groups - 1) / n_groups + 127) / 128 * 128;
   const WorkspacePlan wp = plan_workspace(pr);
@@ -1237,8 +1245,7 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     p.q_bytes = (uint32_t)p.M_pad * d * 2;
     const int Mr = (p.M + 31) & ~31;
     p.merge_slots = 2 * Mr <= kEpilogueThreads ? kEpilogueThreads / Mr * Mr : 0;
-    const int small = p.M_pad * 4 + p.merge_slots * 8 + (pr->n_seq + 1) * 4 + 8 + kNumBars * 8 + 16;
-    const int smem_max = 227 * 1024;
+    const int small = small_bytes(p.M);
     int stages = std::min((smem_max - (int)p.q_bytes - small) / (int)p.stage_bytes, kMaxStages);
     // Up to 48 rows behind the last full block are scored on columns: head_dim 64, 128 units of 32768, 260 rows 0.657 ->
     // 0.580 ms, 132 rows 0.447 -> 0.350.  Not where CTAs have only a few tiles each (the first tile of a segment, which

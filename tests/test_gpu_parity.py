@@ -116,6 +116,29 @@ def test_score_many_short_sequences(B, W, oracle, n_seq, longest, rows, causal):
         assert_scores_close(got.cpu().numpy(), ref, cu)
 
 
+@pytest.mark.parametrize("n_seq,rows", [(69, 160), (70, 160), (1024, 130), (70, 275)])
+def test_score_many_sequences_of_many_rows(B, W, oracle, n_seq, rows):
+    """The tile prefix of the sequences shares memory with the queries: 640 rows of head_dim 128 stay resident at once beside
+    69 sequences and are scored in two groups beside 70; 1100 rows in three groups."""
+    L, G, d = 1, 4, 128
+    lens = [1 + (i * 37) % 150 if i % 5 else 0 for i in range(n_seq)]
+    cu = [0] + [int(x) for x in np.cumsum(lens)]
+    gen = torch.Generator().manual_seed(n_seq)
+    q = torch.randn(n_seq, L, G, rows, d, generator=gen).to(torch.bfloat16).cuda()
+    k = torch.randn(L, 1, cu[-1], d, generator=gen).to(torch.bfloat16).cuda()
+    cu_t = torch.tensor(cu, dtype=torch.int32, device="cuda")
+    pr = B.make_problem(n_layers=L, n_q_heads=G, n_kv_heads=1, head_dim=d, n_lookahead=rows - 7, n_window=7, softmax_scale=d ** -0.5,
+                        total_tokens=cu[-1], n_in=max(lens), n_seq=n_seq, cu_seqlens=cu_t, k=k)
+    ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for reduce in (0, 1):
+        got = torch.full((L, 1, cu[-1]), float("nan"), device="cuda")
+        B.spec_score(pr, q, k, got, ws, reduce=reduce, causal_window=1, status_word=status)
+        assert status.item() == 0
+        ref = oracle.spec_score(bits(q), bits(k), cu, rows - 7, 7, d ** -0.5, mode=reduce, causal_window=True)
+        assert_scores_close(got.cpu().numpy(), ref, cu)
+
+
 def test_short_sequences_are_scored_at_the_rate_of_tiles(B):
     """1024 sequences of 100 to 199 keys against one prompt of as many key tiles: queries, constants and bookkeeping per
     sequence may cost a small multiple of a tile's arithmetic and no more."""
