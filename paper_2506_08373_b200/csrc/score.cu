@@ -1114,6 +1114,21 @@ static EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// The tensor map of a bf16 array.  A driver call, which wants a context on the calling thread; the runtime binds one where it
+// needs it itself, and on a thread whose first call this is it has not yet.
+static CUresult encode_map(EncodeTiledFn encode, CUtensorMap* map, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides,
+                           const cuuint32_t* box) {
+  const cuuint32_t es[4] = {1, 1, 1, 1};
+  auto call = [&]() {
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = call();
+  int dev = 0;
+  if (r == CUDA_ERROR_INVALID_CONTEXT && cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = call();
+  return r;
+}
+
 }  // namespace spec
 
 SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void* k, const float* row_weight,
@@ -1168,20 +1183,14 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     const cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)pr->n_seq * pr->n_layers * pr->n_q_heads * R};
     const cuuint64_t strides[1] = {(cuuint64_t)d * 2};
     const cuuint32_t box[2] = {64, 128};
-    const cuuint32_t es[2] = {1, 1};
-    CUresult r = encode(&tm_q, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(q), dims, strides, box, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = encode_map(encode, &tm_q, q, 2, dims, strides, box);
     if (r != CUDA_SUCCESS) return fail(SPEC_ERR_CUDA, "tensor map for q could not be encoded (CUresult %d)", (int)r);
   }
   {
     const cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)pr->total_tokens, (cuuint64_t)pr->n_kv_heads, (cuuint64_t)pr->n_layers};
     const cuuint64_t strides[3] = {(cuuint64_t)pr->k_stride_token * 2, (cuuint64_t)pr->k_stride_head * 2, (cuuint64_t)pr->k_stride_layer * 2};
     const cuuint32_t box[4] = {64, 128, 1, 1};
-    const cuuint32_t es[4] = {1, 1, 1, 1};
-    CUresult r = encode(&tm_k, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(k), dims, strides, box, es,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = encode_map(encode, &tm_k, k, 4, dims, strides, box);
     if (r != CUDA_SUCCESS) return fail(SPEC_ERR_CUDA, "tensor map for k could not be encoded (CUresult %d)", (int)r);
   }
 

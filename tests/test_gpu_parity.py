@@ -2,6 +2,8 @@
 seeded inputs.  Scores within 2e-3 relative + 1e-6 absolute; index sets identical outside the
 tolerance band around the weakest selected score; index work on given scores and the gather
 bit-exact."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -748,6 +750,46 @@ def test_specpc_paper_settings_from_real_scores(B, W, oracle):
     run_topk_case(B, W, oracle, sc, g.cu, oracle.POOL_AVG, 7, 512, n_window, exact=False)
     run_topk_case(B, W, oracle, sc, g.cu, oracle.POOL_AVG, 64, 512, 0, exact=False)
     run_topk_case(B, W, oracle, sc, g.cu, oracle.POOL_MAX, 32, 512, 0)
+
+
+def test_calls_from_threads_that_never_used_cuda(B, W, oracle):
+    """Every entry point as the first CUDA work of a thread, and several threads at once on streams of their own."""
+    w = small(W, n_in=3000)
+    g = Gpu(B, W, w, [0, 1])
+
+    def path(stream, out, scores=None):
+        try:
+            ws = torch.empty(B.spec_workspace_bytes(g.pr), dtype=torch.uint8, device="cuda") if stream else g.ws
+            with torch.cuda.stream(stream):
+                if scores is None:
+                    scores = torch.full((2, w.n_kv_heads, g.T), float("nan"), device="cuda")
+                B.spec_score(g.pr, g.q, g.k, scores, ws, status_word=g.status)
+                idx = torch.empty((1, 2, w.n_kv_heads, w.c_max), dtype=torch.int32, device="cuda")
+                B.spec_pool_topk(g.pr, scores, 0, 5, w.c_max, 0, idx, None, workspace=ws, status_word=g.status)
+                kept = torch.empty((1, 2, w.n_kv_heads, w.c_max, w.head_dim), dtype=torch.bfloat16, device="cuda")
+                B.spec_compact_kv(g.pr, g.k, None, idx, w.c_max, kept, None, status_word=g.status)
+            torch.cuda.current_stream().synchronize() if stream is None else stream.synchronize()
+            out.append((scores, idx, kept))
+        except Exception as e:                              # a thread's exception would be lost
+            out.append(e)
+
+    buf = torch.full((2, w.n_kv_heads, g.T), float("nan"), device="cuda")
+    torch.cuda.synchronize()
+    want, first, many = [], [], []
+    path(None, want)
+    t = threading.Thread(target=path, args=(None, first, buf))   # its first CUDA call is spec_score's
+    t.start()
+    t.join()
+    threads = [threading.Thread(target=path, args=(torch.cuda.Stream(), many)) for _ in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for got in first + many:
+        assert not isinstance(got, Exception), got
+        for a, b in zip(got, want[0]):
+            assert torch.equal(a, b)
+    assert g.status.item() == 0
 
 
 @pytest.mark.parametrize("offset", [1, 4, 8, 12])
