@@ -64,7 +64,6 @@ constexpr float kExpC0 = 0.9999992614f, kExpC1 = 0.6931218147f, kExpC2 = 0.24024
 constexpr int kBufCols = 128;                 // TMEM columns of an accumulator buffer, one per epilogue warpgroup
 constexpr int kTileKeys = 128;
 constexpr int kMaxStages = 8;
-constexpr int kRemMinTiles = 16;              // key tiles per CTA from which remaining rows are scored on columns
 constexpr int kMaxMTiles = 10;
 constexpr int kNumBars = 2 * kMaxStages + 2 + 8;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
@@ -1256,16 +1255,18 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     p.merge_slots = 2 * Mr <= kEpilogueThreads ? kEpilogueThreads / Mr * Mr : 0;
     const int small = small_bytes(p.M);
     int stages = std::min((smem_max - (int)p.q_bytes - small) / (int)p.stage_bytes, kMaxStages);
-    // Up to 48 rows behind the last full block are scored on columns: head_dim 64, 128 units of 32768, 260 rows 0.657 ->
-    // 0.580 ms, 132 rows 0.447 -> 0.350.  Not where CTAs have only a few tiles each (the first tile of a segment, which
-    // sets the references, takes the general form: 148 rows, 16 units of 9000, 8 tiles per CTA, 0.023 -> 0.028 ms), nor
-    // where the memory for it would leave fewer than three key stages.
+    // Up to 48 rows behind the last full block are scored on columns, from as many key tiles per CTA on as that needs: the first
+    // tile of a segment, which sets the references, takes the general form, and a block of columns costs more the wider it
+    // is.  Blocks of rows against columns (128 units of head_dim 64, us): 8 rows 22.3 and 21.7 at 8 tiles, 58 and 51 at 48;
+    // 136 rows 39.4 and 41.0 at 12, 60 and 58 at 24; 152 rows 62 and 67 at 24, 107 and 104 at 48; 168 rows 107 and 119 at 48,
+    // 212 and 208 at 96.  Not where the memory for it would leave fewer than three key stages.
     p.n_full = p.M_pad / 128;
     p.rem_cols = 0;
     int rem_bytes = 0;
     const int rem_cols = (p.M % 128 + 15) / 16 * 16;
     const int64_t tiles = (int64_t)pr->n_layers * pr->n_kv_heads * ((tokens + kTileKeys - 1) / kTileKeys);
-    if (rem_cols >= 16 && rem_cols <= 48 && tiles >= (int64_t)kRemMinTiles * n_ctas) {
+    const int min_tiles = rem_cols == 16 ? (p.M < 128 ? 0 : 16) : rem_cols == 32 ? 32 : 96;
+    if (rem_cols >= 16 && rem_cols <= 48 && tiles >= (int64_t)min_tiles * n_ctas) {
       const int bytes = 2 * 16 * rem_cols * 4;
       const int left = std::min((smem_max - (int)p.q_bytes - small - bytes) / (int)p.stage_bytes, kMaxStages);
       if (left >= std::min(stages, 3)) {

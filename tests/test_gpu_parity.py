@@ -196,7 +196,7 @@ def test_score_max_reduce_and_row_weights(B, W, oracle):
 @pytest.mark.parametrize("rows", [1, 16, 17, 31, 33, 40, 48, 49])
 @pytest.mark.parametrize("d", [64, 128])
 def test_score_rows_behind_the_last_full_block(B, W, oracle, rows, d):
-    """Row counts whose remainder behind full blocks of 128 is scored on columns (up to 48, given 16 key tiles per CTA) or not
+    """Row counts whose remainder behind full blocks of 128 can be scored on columns (up to 48; at these lengths up to 16) or not
     (49), alone and behind a full block, with tiles that end inside a segment, a causal window that hides the last
     keys, and several sequences.  The first, a middle and the last head of many are compared."""
     L, H = 16, 24                                     # 384 units of 7 tiles on up to 148 CTAs
@@ -220,6 +220,31 @@ def test_score_rows_behind_the_last_full_block(B, W, oracle, rows, d):
                 ref = oracle.spec_score(bits(q[:, l:l + 1, h:h + 1]), bits(k[l:l + 1, h:h + 1]), cu, lookahead - window, window,
                                         d ** -0.5, causal_window=bool(causal))
                 assert_scores_close(got[l:l + 1, h:h + 1].cpu().numpy(), ref, cu)
+
+
+@pytest.mark.parametrize("rows,n", [(1, 130), (16, 300), (16, 860), (17, 1700), (31, 1500), (32, 1700), (33, 4800), (40, 4800), (48, 4800), (48, 4500)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_score_rows_on_columns(B, W, oracle, rows, n, d):
+    """Remaining rows with as many key tiles per CTA as scoring them on columns needs, and one size below for each width: 16
+    columns from 16 tiles on (alone always), 32 from 32, 48 from 96; alone and behind a full block, both reductions."""
+    L, H = 16, 24                                     # 384 units on 148 CTAs
+    window = min(rows, 13)
+    gen = torch.Generator().manual_seed(rows + n)
+    k = torch.randn(L, H, n, d, generator=gen).to(torch.bfloat16).cuda()
+    for lookahead in (rows, 128 + rows):
+        q = torch.randn(1, L, H, lookahead, d, generator=gen).to(torch.bfloat16).cuda()
+        pr = B.make_problem(n_layers=L, n_q_heads=H, n_kv_heads=H, head_dim=d, n_lookahead=lookahead - window, n_window=window,
+                            softmax_scale=d ** -0.5, total_tokens=n, n_in=n, k=k)
+        ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        for reduce, causal in ((0, 0), (1, 1)):
+            got = torch.full((L, H, n), float("nan"), device="cuda")
+            B.spec_score(pr, q, k, got, ws, reduce=reduce, causal_window=causal, status_word=status)
+            assert status.item() == 0
+            for l, h in ((0, 0), (7, 11), (L - 1, H - 1)):
+                ref = oracle.spec_score(bits(q[:, l:l + 1, h:h + 1]), bits(k[l:l + 1, h:h + 1]), [0, n], lookahead - window, window,
+                                        d ** -0.5, mode=reduce, causal_window=bool(causal))
+                assert_scores_close(got[l:l + 1, h:h + 1].cpu().numpy(), ref, [0, n])
 
 
 @pytest.mark.parametrize("heads,n", [(1, 20000), (3, 130), (8, 2304), (8, 2305), (49, 1300), (50, 12800), (74, 385), (75, 385)])
@@ -1049,10 +1074,10 @@ def test_selections_in_a_row_cost_no_more_than_one(B):
 
 
 def test_topk_short_units_in_one_cta_and_streamed(B, W, oracle):
-    """Units of up to 16381 positions are selected by one CTA each (scores, floor sample, candidates and the
-    finishing step all in shared memory); many hundreds of such units with a workspace are streamed
-    instead.  Both against the oracle: sizes at the one-CTA limit, odd offsets of the units in memory,
-    empty and tiny sequences, a forced tail, structured scores, heavy ties, a second budget."""
+    """Units of up to 16381 positions are selected by one CTA each (scores and floor sample in registers, candidates and
+    the finishing step in shared memory), longer ones are streamed.  Both against the oracle: sizes at the one-CTA limit,
+    odd offsets of the units in memory, empty and tiny sequences, a forced tail, structured scores, heavy ties, a second
+    budget."""
     rng = np.random.default_rng(61)
     for n in (16381, 16382, 16384, 9001):                     # 16384 (units on 16-byte boundaries) and 16381 (anywhere) are the longest
         x = (rng.random((1, 2, n)) ** 6).astype(np.float32)
@@ -1069,7 +1094,7 @@ def test_topk_short_units_in_one_cta_and_streamed(B, W, oracle):
         run_vert_case(B, oracle, y, [0, 5000, 12000], 7, 300, 16, 700)
     y = np.zeros((1, 2, 8000), np.float32)                        # every key equal: the generic selection
     run_topk_case(B, W, oracle, y, [0, 8000], 0, 7, 1000, 0)
-    # 640 units of 3000 with a workspace: more units than the one-CTA kernel is given, so they are streamed
+    # many units of 3000, in several waves
     z = (rng.random((40, 16, 3000)) ** 4).astype(np.float32)
     z[:, :, 100:140] = 0.75                                          # a run of ties around the threshold of some units
     run_topk_case(B, W, oracle, z, [0, 3000], 0, 7, 256, 0)
