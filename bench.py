@@ -249,12 +249,11 @@ class State:
             # what the path produces: the index lists and the compacted cache
             self.results = [self.idx, self.cnt, self.k_out, self.v_out]
         # kernels of the library per step: two scoring passes; keep set: reduce + cluster select;
-        # else the selection (sample floor + sweep + finish; one kernel for up to 592 units of up to 16384
-        # positions, and for a budget above a sixth of the sequence) and the gather
+        # else the selection (sample floor + sweep + finish; one kernel for units of up to 16384 positions, and for a
+        # budget above a sixth of the sequence) and the gather
         max_len = w.len_hi if w.n_seq > 1 else w.n_in
-        n_units = w.n_seq * self.L * w.n_kv_heads
         self.select_kernels = ("sample_floor + stream_sweep + stream_finish" if w.c_max * 6 <= max_len and
-                               (max_len + 3 > 16384 + (3 if w.n_seq == 1 else 0) or n_units > 592) else
+                               max_len + 3 > 16384 + (3 if w.n_seq == 1 else 0) else
                                "unit_select" if w.c_max * 6 <= max_len else "cluster_select")
         self.launches_per_step = 2 + ((3 if w.paper_specpc else 2) if self.specpc else
                                       (3 if self.select_kernels.startswith("sample") else 1) + 1)

@@ -24,7 +24,7 @@
 //   3. stream_finish_kernel, one CTA per unit and budget, or per unit where those are many: the
 //      candidates come into shared memory, the exact threshold is found (find_threshold), and the winners
 //      are written out as they stand, already in ascending position, ties to the lower position.
-// Units of up to 16384 positions, a few to an SM, skip the workspace and the three launches:
+// Units of up to 16384 positions skip the workspace and the three launches:
 // unit_select_kernel holds a unit in the registers of one CTA and does the same steps.
 //
 // If the floor was too high or too low (fewer candidates than the budget, or more than the finishing
@@ -602,8 +602,10 @@ static int run_unit_topk(const spec_problem* pr, StreamParams p, cudaStream_t st
   if (p.max_len < 1 || p.max_len + (aligned ? 0 : 3) > kUnitSlots) return SPEC_OK;
   const int64_t n_units = (int64_t)pr->n_seq * pr->n_layers * pr->n_kv_heads;
   if (n_units < 1 || n_units > 0x7fffffff) return SPEC_OK;
-  // the floor, from one sample in 16, lets through 1.4 (budget 2048) to 2.5 (256) times the budget
-  p.held_cap = (5 * std::max(p.c_max, p.n_vert) / 2 + 1024 + 3) & ~3;
+  // The floor, from one sample in 16, lets through 1.4 (budget 2048) to 2.5 (256) times the budget.  Up to 8192 positions there
+  // is room for all of them, so that ties never need the generic selection (2048 units of 3000 of five values 178 -> 68 us);
+  // beyond that the memory would cost more (2048 units of 16384 with room for 12000 94 -> 105 us).
+  p.held_cap = ((p.max_len <= 8192 ? p.max_len : 5 * std::max(p.c_max, p.n_vert) / 2 + 1024) + 3) & ~3;
   const size_t smem = held_bytes(p.held_cap) + kSelWarps * kListSlots * sizeof(uint16_t);
   if (smem > (size_t)kSmemLimit - 16 * 1024) return SPEC_OK;
   static int set[64] = {0};
@@ -633,12 +635,10 @@ int run_stream_topk(const spec_problem* pr, const float* scores, int c_max, int 
   p.max_len = max_seq_len(pr);
   p.idx_out = idx_out; p.count_out = count_out; p.vert_out = vert_out; p.vert_count_out = vert_count_out;
   p.status = status_word;
-  // Short units, a few to an SM: one CTA does all of it.  Many more units than the GPU holds at once
-  // are better streamed (the one-CTA kernel is a chain of latencies, the streaming one is not).
-  if (!workspace || n_units <= 592) {
-    const int rc = run_unit_topk(pr, p, st, done);
-    if (rc != SPEC_OK || *done) return rc;
-  }
+  // Short units: one CTA does all of it, however many they are (256 units of 16384, a 7th kept, 15 us and 24 streamed; 592 of
+  // 5000 19.9 and 31.2; 4096 of 1500, a 40th kept, 100 and 102; 16384 of 300 355 and 354).
+  const int rc = run_unit_topk(pr, p, st, done);
+  if (rc != SPEC_OK || *done) return rc;
   if (!workspace) return SPEC_OK;
   const WorkspacePlan wp = plan_workspace(pr);
   if (workspace_bytes < wp.total) return SPEC_OK;

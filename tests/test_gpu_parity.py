@@ -1117,6 +1117,17 @@ def test_topk_at_the_limits_of_the_selection_kernels(B, W, oracle, n, k, c_max, 
     run_topk_case(B, W, oracle, x, [0, n], 0, k, c_max, min(c_max // 2, 33))
 
 
+@pytest.mark.parametrize("n,c_max", [(8192, 1365), (8193, 1365), (16381, 2730), (16382, 2730)])
+@pytest.mark.parametrize("scores", ["random", "few_values", "tied"])
+def test_many_short_units(B, W, oracle, n, c_max, scores):
+    """600 units in one CTA each, with and without room for all of their positions, and the first length that is streamed."""
+    rng = np.random.default_rng(n)
+    x = {"random": lambda: rng.random((1, 600, n)) ** 6, "few_values": lambda: rng.integers(0, 5, (1, 600, n)) / 8.0,
+         "tied": lambda: np.full((1, 600, n), 0.25)}[scores]().astype(np.float32)
+    x[:, ::2, n - 3:] = 2.0
+    run_topk_case(B, W, oracle, x, [0, n], 0, 7, c_max, 5)
+
+
 @pytest.mark.parametrize("n,k,c_max,units", [
     (33000, 5, 4563, 3), (33000, 5, 4565, 3),                    # keys sent to every CTA, radix select over them where they are
     (60000, 7, 6252, 8), (60000, 7, 20000, 8),
