@@ -82,6 +82,12 @@ SPEC_HIDDEN inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // Token range of sequence s.
 __device__ __forceinline__ void seq_range(const int32_t* cu, int n_in, int s, int& begin, int& n) {
   if (cu) {

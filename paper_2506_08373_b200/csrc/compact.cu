@@ -88,10 +88,7 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(CompactParams 
 
 // ------------------------------------------------------ rows by bulk asynchronous copy ----
 
-#ifndef SPEC_BULK_ROWS
-#define SPEC_BULK_ROWS 16
-#endif
-constexpr int kBulkRows = SPEC_BULK_ROWS;         // destination rows per CTA
+constexpr int kBulkRows = 16;                     // destination rows per CTA
 constexpr int kBulkThreads = kBulkRows < 32 ? 32 : kBulkRows;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -99,8 +96,9 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)
 // A CTA gathers kBulkRows destination rows of one (sequence, layer, KV head) for K and V: one
 // bulk copy per source row into shared memory, all in flight together, then bulk copies out (a
 // contiguous destination takes one per tensor, a paged one takes one per row).  Small CTAs
-// and many of them: 16 rows per CTA measured best (8 to 256 tried).  Bound by the bandwidth: 256 units of 2048 rows of
-// 256 bytes in 0.080 ms alone, 0.089 behind their selection, 6.0 to 6.7 TB/s of 6.54 for a plain copy.
+// and many of them: 16 rows per CTA measured best (8 to 256 tried).  Bound by the memory: 256 units of 2048 rows of 256 bytes,
+// 537 MB read and written, in 0.080 ms alone and 0.089 behind their selection.  That is 6.0 to 6.7 TB/s of these bytes, against
+// 6.5 for a plain copy, but not the rate of the DRAM: part of the rows written is still in L2 at the end.
 template <bool HAS_V>
 __global__ void __launch_bounds__(kBulkThreads) compact_bulk_kernel(CompactParams p, int row_bytes) {
   extern __shared__ __align__(128) uint8_t rows_sm[];      // [K | V][kBulkRows][row_bytes]

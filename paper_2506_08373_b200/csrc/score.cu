@@ -22,7 +22,7 @@
 // another.
 // The exponential is the scarce resource (16 MUFU results per clock per SM against 32 logits per
 // clock from the tensor cores), so a fixed share of the elements is evaluated on the FMA pipes
-// instead (range reduction + quartic polynomial, relative error 2.6e-6), and the surrounding
+// instead (range reduction + quartic polynomial, relative error up to 5.3e-6), and the surrounding
 // arithmetic uses the packed two-lane fp32 instructions to halve its issue slots.  Warpgroups
 // never synchronise inside a unit: pass 1 writes their statistics as separate partials; in
 // pass 2 a key tile belongs to one pair, whose two warpgroups add their per-key sums (over the
@@ -67,10 +67,7 @@ constexpr int kMaxStages = 8;
 constexpr int kMaxMTiles = 10;
 constexpr int kNumBars = 2 * kMaxStages + 2 + 8;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
-#ifndef SPEC_SUSPEND_HINT_NS
-#define SPEC_SUSPEND_HINT_NS 100000
-#endif
-constexpr uint32_t kSuspendHintNs = SPEC_SUSPEND_HINT_NS;
+constexpr uint32_t kSuspendHintNs = 100000;
 
 struct ScoreParams {
   const int32_t* cu;
@@ -86,7 +83,6 @@ struct ScoreParams {
   int merge_slots;       // threads that share the merging of a unit's statistics when there are fewer rows than threads (0: none do)
   int n_stages, n_chunks, cw_last;   // pass 2: chunks of 128 query rows, the last of cw_last (a multiple of 16)
   int n_full, rem_cols;  // pass 1: blocks of 128 query rows on lanes, and 16..48 remaining rows on columns (0: none)
-  int reduce;
   float a;              // softmax_scale * log2(e)
   uint32_t q_bytes, stage_bytes;
 };
@@ -100,9 +96,6 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 }
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 // One arrival for the whole warp, after a warp-wide (.sync.aligned) instruction has completed
 // for all lanes: predicated, no branch.
@@ -334,11 +327,6 @@ __device__ __forceinline__ int seg_tile(const Seg& sg, int t) { return sg.t0 + (
 
 // The packed fp32 instructions (two lanes per instruction) through the float2 intrinsics.
 __device__ __forceinline__ float2 splat2(float v) { return make_float2(v, v); }
-__device__ __forceinline__ float max3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
 
 // 2^x for both lanes on the MUFU unit.
 __device__ __forceinline__ float2 ex2_mufu2(float2 x) {
@@ -347,8 +335,8 @@ __device__ __forceinline__ float2 ex2_mufu2(float2 x) {
 // 2^x for both lanes without the MUFU unit, x = s*a + c held in [-B, 128 - B]: in units of 128,
 // y = (x + B) / 128 is one multiply-add that saturates to [0, 1] for nothing, so that neither end of the
 // range needs a clamp of its own.  Adding 1.5 * 2^16 rounds y to a multiple of 1/128 and leaves
-// n = round(128 y) in the low mantissa bits; 2^f of the rest, |f| <= 1/2, is a quartic (relative
-// error 2.6e-6), and n goes into the exponent field.  a128 = a / 128, c128 = (c + B) / 128.
+// n = round(128 y) in the low mantissa bits; 2^f of the rest, |f| <= 1/2, is a quartic, and n goes into the exponent
+// field.  Relative error: 2.6e-6 of the quartic, and as much of the rounding of y to 2^-25, together up to 5.3e-6.  a128 = a / 128, c128 = (c + B) / 128.
 template <int B>
 __device__ __forceinline__ float2 ex2_poly2(float s0, float s1, float a128, float2 c128) {
   constexpr float k = B == 64 ? 5.421010862427522e-20f : 2.350988701644575e-38f;   // 2^-B
@@ -514,7 +502,7 @@ __device__ __forceinline__ void prob_accumulate(const uint32_t (&r)[32], const f
       if (MAXRED) {
         const float2 x = __ffma2_rn(make_float2(x0, x1), a2, cc);
         float& m = i & 1 ? acc[u].y : acc[u].x;            // four chains, merged at the end
-        m = max3(m, x.x, x.y);
+        m = fmax3(m, x.x, x.y);
       } else {
         const float2 e = is_poly<kPolyPairs>(2 * i + u) ? ex2_poly2<125>(x0, x1, a128, cc) : ex2_mufu2(__ffma2_rn(make_float2(x0, x1), a2, cc));
         acc[u] = __fadd2_rn(acc[u], e);
@@ -1203,7 +1191,6 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   p.T = pr->total_tokens;
   p.n_in = pr->n_in; p.n_seq = pr->n_seq; p.L = pr->n_layers; p.Hq = pr->n_q_heads; p.Hkv = pr->n_kv_heads;
   p.G = G; p.R = R; p.d = d;
-  p.reduce = reduce;
   p.n_window = pr->n_window;
   p.a = (float)((double)pr->softmax_scale * 1.4426950408889634);
   p.stage_bytes = (uint32_t)kTileKeys * d * 2;

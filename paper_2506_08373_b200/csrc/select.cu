@@ -10,7 +10,7 @@
 // times the budget, are sent to every CTA as well, and each finds the exact threshold among them by
 // itself (find_threshold).  That takes two cluster barriers; the radix select over distributed
 // histograms that it replaced took four, and added every non-empty bin into all CTAs (keep set of 1024 among 32768 tokens
-// of 16 layers, with the reduction: 29 -> 18 us).  The radix select (11 + 11 + 10 bits) is what remains for units whose
+// of 16 layers with random scores, with the reduction: 29 -> 18 us).  The radix select (11 + 11 + 10 bits) is what remains for units whose
 // floor lets through too few or too many keys, as massive ties can.  Winners are written in ascending
 // position: the CTAs exchange their counts, and each one emits its own winners behind those
 // of the CTAs before it; ties at the threshold go to the lower position.  The scores are read
@@ -877,7 +877,8 @@ static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int
   const int64_t x_max = (int64_t)max_len + 3;
   // The cluster size with the least estimated time: a CTA takes 7 us and another 10 for 8192 positions (32768 positions
   // in 4 CTAs: 17 us), and two CTAs share an SM where their memory, with `held` bytes for keys, allows; GPCs hold about 0.8
-  // of the slots' worth of clusters.
+  // of the slots' worth of clusters (of 148 SMs 120; of clusters of two or one 140).
+  const int sms = sm_count();
   double waves = 0;
   auto size_cluster = [&](size_t held) {
     double best = 1e30;
@@ -886,7 +887,7 @@ static ClusterPlan plan_cluster(int max_len, int pool, int pool_k, int mode, int
       const int cap = (int)((((x_max + cs - 1) / cs) + 3) & ~(int64_t)3);
       const size_t smem = cluster_smem_bytes(cap, pl.halo_l, pl.halo_r, pl.inplace, mode, 0);
       if (smem > (size_t)kSmemLimit || (cs > 1 && cap < kChunkMin)) continue;
-      const int64_t slots = (smem + held <= (size_t)kSmemLimit / 2 ? 2 : 1) * (cs > 2 ? 120 : 140);
+      const int64_t slots = (smem + held <= (size_t)kSmemLimit / 2 ? 2 : 1) * (cs > 2 ? sms * 13 / 16 : sms * 19 / 20);
       const double w = (double)((n_units * cs + slots - 1) / slots), t = w * (7.0 + 10.0 * cap / 8192);
       if (t < best) {
         best = t;

@@ -18,12 +18,6 @@ __device__ __forceinline__ uint32_t to_key(float v) {
   return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);   // negative: all bits flipped; else: sign bit set
 }
 
-__device__ __forceinline__ float fmax3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-
 // Block-wide exclusive scan of one int per thread; total returned to every thread.
 // wsum: kSelWarps ints of shared memory that no thread touches again before the CTA's next
 // synchronisation after this call.  One __syncthreads.
@@ -314,7 +308,7 @@ __device__ __forceinline__ bool find_bin(SelectMem& sm, int need, int& bin, int&
 // 64 bins to a factor of two over 32 factors of two, or, if the rank lies deeper than that, by their
 // leading 11 bits.  Scores that differ by a few per cent only (sums over many heads, averages) would crowd into a bin
 // or two: the bin is cut again then, or the floor lets through more keys than there is room for (keep set of 1024
-// among 32768 such tokens: 29.6 -> 23.6 us).  0, which all keys reach, when the sample is too small to tell.  `keys`: N samples
+// among 32768 tokens whose scores are such sums: 29.6 -> 23.6 us).  0, which all keys reach, when the sample is too small to tell.  `keys`: N samples
 // of this thread, 0 = none.  All threads of the CTA call this; the histogram is clear on entry and on return.
 struct Floor {
   uint32_t key;
