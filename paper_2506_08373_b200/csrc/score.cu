@@ -612,9 +612,10 @@ __device__ __forceinline__ void row_constants(const ScoreParams& p, const float2
 
 // FLAG: pass 1, whether remaining rows are scored on columns (a variant of its own: the registers that it needs
 // slowed the other one down by 4 to 20 %); pass 2, whether the reduction is the maximum.  CAUSAL: the causal window,
-// likewise apart (its masks cost the other kernels 1 to 2 % in registers).  RAGGED: more than one sequence.  What a
-// segment costs beside its tiles counts there (1024 sequences of 100 to 199 keys, 2 layers of 8 heads, 32 rows: 925 us with
-// the code for one sequence, 661 so), and the code for it cost one layer of 12345 keys 0.4 of 52.8 us.
+// likewise apart (its masks cost the other kernels 1 to 2 % in registers).  RAGGED: many sequences,
+// dozens of segments to a CTA.  What a segment costs beside its tiles counts there (1024 sequences of 100 to 199 keys, 2
+// layers of 8 heads, 32 rows: 925 us with the other kernels, 661 so; 128 sequences of 1000, 28 units to a CTA, 405 and 396),
+// and the code for it cost one layer of 12345 keys 0.4 of 52.8 us, one of two sequences 1 of 27.
 template <int PASS, bool FLAG, bool CAUSAL, bool RAGGED>
 __global__ void __launch_bounds__(kThreads, 1)
 score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const ScoreParams p) {
@@ -1202,7 +1203,7 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
        {{score_kernel<2, false, false, false>, score_kernel<2, false, true, false>}, {score_kernel<2, true, false, false>, score_kernel<2, true, true, false>}}},
       {{{score_kernel<1, false, false, true>, score_kernel<1, false, true, true>}, {score_kernel<1, true, false, true>, score_kernel<1, true, true, true>}},
        {{score_kernel<2, false, false, true>, score_kernel<2, false, true, true>}, {score_kernel<2, true, false, true>, score_kernel<2, true, true, true>}}}};
-  const bool ragged = pr->n_seq > 1;
+  const bool ragged = pr->n_seq > 1 && (int64_t)pr->n_seq * pr->n_layers * pr->n_kv_heads > 16 * (int64_t)n_ctas;
   // The kernels may use all of an SM's shared memory; the attribute is set once per device (it is per
   // function and context, so setting it per call would race between host threads).
   {

@@ -602,10 +602,12 @@ static int run_unit_topk(const spec_problem* pr, StreamParams p, cudaStream_t st
   if (p.max_len < 1 || p.max_len + (aligned ? 0 : 3) > kUnitSlots) return SPEC_OK;
   const int64_t n_units = (int64_t)pr->n_seq * pr->n_layers * pr->n_kv_heads;
   if (n_units < 1 || n_units > 0x7fffffff) return SPEC_OK;
-  // The floor, from one sample in 16, lets through 1.4 (budget 2048) to 2.5 (256) times the budget.  Up to 8192 positions there
-  // is room for all of them, so that ties never need the generic selection (2048 units of 3000 of five values 178 -> 68 us);
-  // beyond that the memory would cost more (2048 units of 16384 with room for 12000 94 -> 105 us).
-  p.held_cap = ((p.max_len <= 8192 ? p.max_len : 5 * std::max(p.c_max, p.n_vert) / 2 + 1024) + 3) & ~3;
+  // The floor, from one sample in 16, lets through 1.4 (budget 2048) to 2.5 (256) times the budget.  For units in several waves
+  // of up to 8192 positions there is room for all of them, so that ties never need the generic selection (2048 units of 3000 of
+  // five values 178 -> 68 us).  Not for longer units, where it costs more (2048 units of 16384 with room for 12000 94 -> 105 us),
+  // nor for fewer, where a kernel that follows starts later beside that memory (64 units of 4164 with their gather 14.0 -> 15.8).
+  const bool room_for_all = n_units > 2 * sm_count() && p.max_len <= 8192;
+  p.held_cap = ((room_for_all ? p.max_len : std::min(5 * std::max(p.c_max, p.n_vert) / 2 + 1024, p.max_len)) + 3) & ~3;
   const size_t smem = held_bytes(p.held_cap) + kSelWarps * kListSlots * sizeof(uint16_t);
   if (smem > (size_t)kSmemLimit - 16 * 1024) return SPEC_OK;
   static int set[64] = {0};
