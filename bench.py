@@ -43,12 +43,12 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 NCU_TRAFFIC = {
     # workload index -> {kernel group: (bytes per layer, source files, hash of those sources)}
     # profiles/score_kernel_c2.md (2 layers) and profiles/select_and_gather_c2.md (8 layers)
-    2: {"score": ((539.571456e6 + 7.040512e6 + 549.027584e6 + 6.06592e6) / 2, ["score.cu"], "7453c361d88711cb"),
-        "select": ((8.41728e6 + 33.594368e6 + 0.002816e6 + 3.77088e6) / 8, ["select_stream.cu", "select_common.cuh"], "eca10b0a19f6b12e"),
-        "gather": ((67.691008e6 + 14.267136e6) / 8, ["compact.cu"], "3fd4843278130ca6")},
+    2: {"score": ((539.575552e6 + 6.23744e6 + 549.031168e6 + 3.440896e6) / 2, ["score.cu"], "66cfeb62d8fa04e5"),
+        "select": ((8.41728e6 + 33.594112e6 + 0.001792e6 + 3.770624e6) / 8, ["select_stream.cu", "select_common.cuh"], "06b0153d0faabae6"),
+        "gather": ((67.678976e6 + 14.346752e6) / 8, ["compact.cu"], "94d32f5d239a0cb5")},
     # profiles/select_and_gather_c2.md, the capture of all 32 layers of workload 1 (unit_select_kernel, compact_bulk_kernel)
-    1: {"select": ((16.8512e6 + 0.00256e6) / 32, ["select_stream.cu", "select_common.cuh"], "eca10b0a19f6b12e"),
-        "gather": ((135.296e6 + 76.041984e6) / 32, ["compact.cu"], "3fd4843278130ca6")},
+    1: {"select": ((16.851456e6 + 0.003328e6) / 32, ["select_stream.cu", "select_common.cuh"], "06b0153d0faabae6"),
+        "gather": ((135.31648e6 + 75.32928e6) / 32, ["compact.cu"], "94d32f5d239a0cb5")},
 }
 
 
