@@ -15,7 +15,7 @@
 // 128 x 128 logits: 128 query rows x the 128 keys of a tile in pass 1, the 128 keys of a tile x
 // a chunk of 128 query rows in pass 2.  Key tiles alternate between the two pairs of
 // warpgroups (each pair has its own issuing warp); within a pair the items of a tile
-// alternate between its two warpgroups, which start alternately from tile to tile.  A
+// alternate between its two warpgroups, which start alternately from tile to tile where that evens out their work.  A
 // warpgroup drains an item whole, four 32-column loads with the arithmetic in between (two
 // blocks in registers: the other roles give up registers for that), and hands the buffer back
 // after the last load, so the four warps that share an SM sub-partition run out of step with one
@@ -83,6 +83,7 @@ struct ScoreParams {
   int merge_slots;       // threads that share the merging of a unit's statistics when there are fewer rows than threads (0: none do)
   int n_stages, n_chunks, cw_last;   // pass 2: chunks of 128 query rows, the last of cw_last (a multiple of 16)
   int n_full, rem_cols;  // pass 1: blocks of 128 query rows on lanes, and 16..48 remaining rows on columns (0: none)
+  int turn;             // 1: the warpgroups of a pair begin a tile in turn, 0: the first always does
   float a;              // softmax_scale * log2(e)
   uint32_t q_bytes, stage_bytes;
 };
@@ -742,7 +743,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         tc_fence_after();
         // A key tile belongs to the pair with the parity of its index in the segment; within the
         // pair, sub-item `sub` (a block of 128 query rows) of the pair's k-th tile goes to the
-        // warpgroup (sub + k) & 1, whose private 128-column buffer receives it.
+        // warpgroup (sub + k * turn) & 1, whose private 128-column buffer receives it.
         for (int t = 0; t < nt && ok; ++t) {
           ok = mbar_wait_warp(&k_full[stage], k_par, abort_flag);
           if (!ok) break;
@@ -750,7 +751,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const uint32_t k_lo = k_lo0 + stage * ((128 * 128) >> 4);
           if ((t & 1) == strm) {
             for (int sub = 0; sub < n_sub; ++sub) {
-              const int h = (sub + (t >> 1)) & 1;
+              const int h = (sub + (t >> 1) * p.turn) & 1;
               const int buf = strm * 2 + h;
               ok = mbar_wait_warp(&t_empty[buf], ((h ? uses1 : uses0) & 1) ^ 1, abort_flag);
               if (!ok) break;
@@ -831,7 +832,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const bool in_window = CAUSAL && key0 + kTileKeys > sg.n - p.n_window;    // warp-uniform
           const bool plain = nv >= kTileKeys && !in_window;
           if (clears && half == 0 && row_in_tile < nv) out[key0 + row_in_tile] = 0.f;
-          for (int mt = ((t >> 1) + half) & 1; mt < n_sub && ok; mt += 2) {
+          for (int mt = ((t >> 1) * p.turn + half) & 1; mt < n_sub && ok; mt += 2) {
             ok = mbar_wait(&t_full[wg], used & 1, abort_flag);
             if (!ok) break;
             ++used;
@@ -990,7 +991,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const int key = seg_tile<PASS>(sg, t) * kTileKeys + row_in_tile;
           const bool in_window = CAUSAL && (seg_tile<PASS>(sg, t) + 1) * kTileKeys > sg.n - p.n_window;   // warp-uniform
           bool any = false;
-          for (int ch = ((t >> 1) + half) & 1; ch < p.n_chunks; ch += 2) {
+          for (int ch = ((t >> 1) * p.turn + half) & 1; ch < p.n_chunks; ch += 2) {
             ok = mbar_wait(&t_full[wg], used & 1, abort_flag);
             if (!ok) break;
             ++used;
@@ -1249,6 +1250,10 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     // 136 rows 39.4 and 41.0 at 12, 60 and 58 at 24; 152 rows 62 and 67 at 24, 107 and 104 at 48; 168 rows 107 and 119 at 48,
     // 212 and 208 at 96.  Not where the memory for it would leave fewer than three key stages.
     p.n_full = p.M_pad / 128;
+    // An odd number of items to a tile, or a short last one, evens out over the tiles when the warpgroups begin in turn. With an even
+    // number of equal items that gives a warpgroup two items in a row, for which its one buffer makes it wait: 8 layers of
+    // 32768, head_dim 128, 256 rows 309 -> 296 us, 512 rows 549 -> 527 (of head_dim 64 477 -> 470).
+    p.turn = p.M % 128 != 0 || p.n_full % 2 != 0;
     p.rem_cols = 0;
     int rem_bytes = 0;
     const int rem_cols = (p.M % 128 + 15) / 16 * 16;

@@ -247,6 +247,33 @@ def test_score_rows_on_columns(B, W, oracle, rows, n, d):
                 assert_scores_close(got[l:l + 1, h:h + 1].cpu().numpy(), ref, [0, n])
 
 
+@pytest.mark.parametrize("d,rows", [(128, 128), (128, 192), (128, 256), (128, 384), (128, 448), (128, 512), (128, 640),
+                                    (64, 256), (64, 512), (64, 896), (64, 1024), (64, 1280)])
+def test_score_row_blocks(B, W, oracle, d, rows):
+    """Every number of row blocks to a key tile, even and odd, full and with a short last one, and with it every number of key
+    stages from two to eight (two to five at head_dim 128), over enough tiles per CTA that the stages go round several times; calls in a row."""
+    L, H, n, window = 1, 37, 7600, 9                  # 60 tiles to a unit, 15 to a CTA, shares that span units
+    gen = torch.Generator().manual_seed(rows + d)
+    q = torch.randn(1, L, H, rows, d, generator=gen).to(torch.bfloat16).cuda()
+    k = torch.randn(L, H, n, d, generator=gen).to(torch.bfloat16).cuda()
+    pr = B.make_problem(n_layers=L, n_q_heads=H, n_kv_heads=H, head_dim=d, n_lookahead=rows - window, n_window=window,
+                        softmax_scale=d ** -0.5, total_tokens=n, n_in=n, k=k)
+    ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for reduce, causal in ((0, 0), (1, 0), (0, 1)):
+        first = torch.full((L, H, n), float("nan"), device="cuda")
+        B.spec_score(pr, q, k, first, ws, reduce=reduce, causal_window=causal, status_word=status)
+        for h in (0, 18, 36):
+            ref = oracle.spec_score(bits(q[:, :, h:h + 1]), bits(k[:, h:h + 1]), [0, n], rows - window, window, d ** -0.5, mode=reduce,
+                                    causal_window=bool(causal))
+            assert_scores_close(first[:, h:h + 1].cpu().numpy(), ref, [0, n])
+        for _ in range(20):
+            again = torch.full_like(first, float("nan"))
+            B.spec_score(pr, q, k, again, ws, reduce=reduce, causal_window=causal, status_word=status)
+            assert torch.equal(first, again)
+    assert status.item() == 0
+
+
 @pytest.mark.parametrize("heads,n", [(1, 20000), (3, 130), (8, 2304), (8, 2305), (49, 1300), (50, 12800), (74, 385), (75, 385)])
 def test_score_units_cut_among_ctas(B, W, oracle, heads, n):
     """Few units of one length are cut each among CTAs of its own (148 CTAs, at least two per unit, at most two tiles more
