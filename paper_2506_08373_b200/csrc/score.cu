@@ -65,7 +65,7 @@ constexpr int kBufCols = 128;                 // TMEM columns of an accumulator 
 constexpr int kTileKeys = 128;
 constexpr int kMaxStages = 8;
 constexpr int kMaxMTiles = 10;
-constexpr int kNumBars = 2 * kMaxStages + 2 + 8;
+constexpr int kNumBars = 2 * kMaxStages + 2 + 4;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 constexpr uint32_t kSuspendHintNs = 100000;
 
@@ -98,12 +98,13 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }
-// One arrival for the whole warp, after a warp-wide (.sync.aligned) instruction has completed
-// for all lanes: predicated, no branch.
-__device__ __forceinline__ void arrive_lane0(uint64_t* bar, int lane) {
-  asm volatile("{\n.reg .pred p;\nsetp.eq.s32 p, %1, 0;\n@p mbarrier.arrive.shared::cta.b64 _, [%0];\n}"
-               ::"r"(smem_u32(bar)), "r"(lane) : "memory");
-}
+// A buffer's return from its warpgroup to the warp that issues into it: a named barrier, on which the four epilogue warps
+// arrive and the issuing warp waits.  An mbarrier's arrivals and tests stand in one queue with the exponentials, and the issuing
+// warp saw a buffer's return some 900 cycles late; where pass 2 has no exponentials (MAX), that is the time of its items: 8
+// layers of 32768, 260 rows of head_dim 64, 251 -> 234 us; with exponentials 471 -> 467 (512 rows).
+constexpr int kReturnBarrier = 6, kReturnThreads = 128 + 32;
+__device__ __forceinline__ void return_arrive(int buf) { asm volatile("bar.arrive %0, %1;" ::"r"(kReturnBarrier + buf), "n"(kReturnThreads) : "memory"); }
+__device__ __forceinline__ void return_sync(int buf) { asm volatile("bar.sync %0, %1;" ::"r"(kReturnBarrier + buf), "n"(kReturnThreads) : "memory"); }
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -637,7 +638,6 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   uint64_t* q_full = bars + 2 * kMaxStages;
   uint64_t* q_empty = q_full + 1;
   uint64_t* t_full = q_full + 2;
-  uint64_t* t_empty = t_full + 4;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kNumBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* scale_sm = reinterpret_cast<float*>(tmem_slot + 2);
@@ -651,11 +651,15 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_q) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
   }
+  // Every wait tells two phases of a key stage apart by their parity. With an even number of stages, a stage has tiles of one pair
+  // only, whose issuing warp sees all of its phases; with an odd one its tiles are of both pairs in turn, and both warps wait for
+  // every tile and hand it back.
+  const bool both_take = (p.n_stages & 1) != 0;
   if (tid == 32) {
-    for (int i = 0; i < kMaxStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 2); }
+    for (int i = 0; i < kMaxStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 1 + both_take); }
     mbar_init(q_full, 1);
     mbar_init(q_empty, 2);
-    for (int i = 0; i < 4; ++i) { mbar_init(&t_full[i], 1); mbar_init(&t_empty[i], 4); }
+    for (int i = 0; i < 4; ++i) mbar_init(&t_full[i], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -713,8 +717,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     } else if (warp <= 2) {
       // ------------------------------------------------ MMA issuers -----
       // Two issuing warps, one per warpgroup pair: warp s feeds the buffers of that pair's two
-      // warpgroups.  Both wait for every key tile and commit to its "empty" barrier, whether or not
-      // they used it, so that every phase of those barriers sees exactly two arrivals.
+      // warpgroups, and hands the pair's key tiles back.
       // The whole warp runs the loops, and one elected lane issues: in converged code the descriptors stay in
       // the uniform registers that tcgen05.mma reads them from.  Issued from a branch that one lane had
       // taken, the eight instructions of an item took 1400 cycles among the epilogue warps (512 on the
@@ -723,9 +726,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       const int strm = warp - 1;
       SegIter it = seg_begin(p, tp, gridDim.x, blockIdx.x);
       Seg sg;
-      uint32_t nseg = 0, uses0 = 0, uses1 = 0;                 // segments; items issued into each of my pair's two buffers
-      int stage = 0;
-      uint32_t k_par = 0;
+      uint32_t nseg = 0, kit = 0;                              // segments, key tiles of the segments before
+      bool in_use[2] = {false, false};                         // my pair's two buffers: an item has been issued into them
       bool ok = true;
       const uint32_t idesc_full = make_idesc(128);
       const uint32_t idesc_last = make_idesc(PASS == 2 ? p.cw_last : REM ? p.rem_cols : 128);
@@ -733,29 +735,31 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       const uint32_t q_lo0 = desc_lo(smem_u32(q_sm)), k_lo0 = desc_lo(smem_u32(k_sm));
       const uint32_t q_half16 = q_half_bytes >> 4;
       const uint32_t k_half16 = k_half_bytes >> 4;
-      while (ok) {
+      const int t_first = both_take ? 0 : strm, t_step = both_take ? 1 : 2;
+      // Every item passes its buffer's barrier, also after a wait has given up, so that no warp is left waiting there.
+      for (;;) {
         const bool more = seg_next<PASS, RAGGED>(it, p, tp, sg);
         const int nt = uniform(more ? sg.nt : 0);
         if (nt == 0) break;
-        ok = mbar_wait_warp(q_full, nseg & 1, abort_flag);
-        if (!ok) break;
+        ok = ok && mbar_wait_warp(q_full, nseg & 1, abort_flag);
         ++nseg;
         tc_fence_after();
         // A key tile belongs to the pair with the parity of its index in the segment; within the
         // pair, sub-item `sub` (a block of 128 query rows) of the pair's k-th tile goes to the
         // warpgroup (sub + k * turn) & 1, whose private 128-column buffer receives it.
-        for (int t = 0; t < nt && ok; ++t) {
-          ok = mbar_wait_warp(&k_full[stage], k_par, abort_flag);
-          if (!ok) break;
+        int stage = (int)((kit + t_first) % p.n_stages);
+        uint32_t k_par = ((kit + t_first) / p.n_stages) & 1;
+        kit += nt;
+        for (int t = t_first; t < nt; t += t_step) {
+          ok = ok && mbar_wait_warp(&k_full[stage], k_par, abort_flag);
           tc_fence_after();
           const uint32_t k_lo = k_lo0 + stage * ((128 * 128) >> 4);
           if ((t & 1) == strm) {
             for (int sub = 0; sub < n_sub; ++sub) {
               const int h = (sub + (t >> 1) * p.turn) & 1;
               const int buf = strm * 2 + h;
-              ok = mbar_wait_warp(&t_empty[buf], ((h ? uses1 : uses0) & 1) ^ 1, abort_flag);
-              if (!ok) break;
-              if (h) ++uses1; else ++uses0;
+              if (h ? in_use[1] : in_use[0]) return_sync(buf);
+              if (h) in_use[1] = true; else in_use[0] = true;
               tc_fence_after();
               const uint32_t d_tmem = tmem_base + buf * BUFCOLS;
               const uint32_t q_lo = q_lo0 + sub * ((128 * 128) >> 4);
@@ -763,7 +767,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               const bool rows_on_lanes = PASS == 1 && (!REM || sub < p.n_full);
               const uint32_t a_lo = rows_on_lanes ? q_lo : k_lo, a_half16 = rows_on_lanes ? q_half16 : k_half16;
               const uint32_t b_lo = rows_on_lanes ? k_lo : q_lo, b_half16 = rows_on_lanes ? k_half16 : q_half16;
-              if (elect_one()) {
+              if (ok && elect_one()) {
 #pragma unroll
                 for (int kh = 0; kh < 2; ++kh) {
                   if (kh < n_kh) {
@@ -778,13 +782,16 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               __syncwarp();
             }
           }
-          if (ok && elect_one()) tc_commit(&k_empty[stage]);      // arrives once my MMAs on this stage (if any) retire
+          if (ok && elect_one()) tc_commit(&k_empty[stage]);        // arrives once my MMAs on this stage (if any) retire
           __syncwarp();
-          if (++stage == p.n_stages) { stage = 0; k_par ^= 1; }
+          stage += t_step;
+          if (stage >= p.n_stages) { stage -= p.n_stages; k_par ^= 1; }
         }
         if (ok && elect_one()) tc_commit(q_empty);
         __syncwarp();
       }
+      if (in_use[0]) return_sync(strm * 2);                      // of the last items
+      if (in_use[1]) return_sync(strm * 2 + 1);
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpilogueRegs));
@@ -826,15 +833,15 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
 #pragma unroll
         for (int i = 0; i < kMaxMTiles; ++i) { mrun[i] = -INFINITY; zrun[i] = 0.f; }
-        for (int t = pair; t < sg.nt && ok; t += 2) {
+        for (int t = pair; t < sg.nt; t += 2) {
           const int key0 = seg_tile<PASS>(sg, t) * kTileKeys;                                // first key of the tile
           const int nv = min(kTileKeys, sg.n - key0);                              // valid keys of the tile
           const bool in_window = CAUSAL && key0 + kTileKeys > sg.n - p.n_window;    // warp-uniform
           const bool plain = nv >= kTileKeys && !in_window;
           if (clears && half == 0 && row_in_tile < nv) out[key0 + row_in_tile] = 0.f;
-          for (int mt = ((t >> 1) * p.turn + half) & 1; mt < n_sub && ok; mt += 2) {
-            ok = mbar_wait(&t_full[wg], used & 1, abort_flag);
-            if (!ok) break;
+          for (int mt = ((t >> 1) * p.turn + half) & 1; mt < n_sub; mt += 2) {
+            ok = ok && mbar_wait(&t_full[wg], used & 1, abort_flag);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_sync(wg); continue; }
             ++used;
             tc_fence_after();
             if (REM && mt == n_full) {
@@ -856,8 +863,9 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               if (cols >= 32) rem_block<32>(my_taddr, general, seen, p.a, lane, my_ref, rem_m[0], rem_z[0]);
               else rem_block<16>(my_taddr, general, seen, p.a, lane, my_ref, rem_m[0], rem_z[0]);
               if (cols > 32) rem_block<16>(my_taddr + 32, general, seen1, p.a, lane, my_ref + 32, rem_m[1], rem_z[1]);
+              __syncwarp();
               tc_fence_before();
-              arrive_lane0(&t_empty[wg], lane);
+              return_arrive(wg);
               continue;
             }
             float m = mrun[mt], z = zrun[mt];
@@ -876,7 +884,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               tmem_wait(ra);
               tmem_wait(rb);
               tc_fence_before();
-              arrive_lane0(&t_empty[wg], lane);
+              return_arrive(wg);
               stats_update(ra, p.a, m, z);
               stats_update(rb, p.a, m, z);
             } else {
@@ -893,8 +901,9 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                 if (__all_sync(0xffffffffu, vis - c * 32 >= 32)) stats_update(ra, p.a, m, z);
                 else if (vis - c * 32 > 0) stats_general(ra, min(vis - c * 32, 32), p.a, m, z);
               }
+              __syncwarp();
               tc_fence_before();
-              arrive_lane0(&t_empty[wg], lane);
+              return_arrive(wg);
             }
             mrun[mt] = m;
             zrun[mt] = z;
@@ -986,14 +995,14 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                               b1 - b0, n_part, et, scale_log2, c_sm, merge_sm);
         asm volatile("bar.sync 1, 512;" ::: "memory");
         float* out = p.scores + ((long long)sg.l * p.Hkv + sg.h) * p.T + sg.begin;
-        for (int t = pair; t < sg.nt && ok; t += 2) {
+        for (int t = pair; t < sg.nt; t += 2) {
           float2 acc[2] = {splat2(MAXRED ? -INFINITY : 0.f), splat2(MAXRED ? -INFINITY : 0.f)};
           const int key = seg_tile<PASS>(sg, t) * kTileKeys + row_in_tile;
           const bool in_window = CAUSAL && (seg_tile<PASS>(sg, t) + 1) * kTileKeys > sg.n - p.n_window;   // warp-uniform
           bool any = false;
           for (int ch = ((t >> 1) * p.turn + half) & 1; ch < p.n_chunks; ch += 2) {
-            ok = mbar_wait(&t_full[wg], used & 1, abort_flag);
-            if (!ok) break;
+            ok = ok && mbar_wait(&t_full[wg], used & 1, abort_flag);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_sync(wg); continue; }
             ++used;
             any = true;
             tc_fence_after();
@@ -1014,8 +1023,9 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                   prob_accumulate<MAXRED, 16, true>(ra, rowc + c, a2, a128, acc, hidden);
                 }
               }
+              __syncwarp();
               tc_fence_before();
-              arrive_lane0(&t_empty[wg], lane);
+              return_arrive(wg);
               continue;
             }
             if (cw == 128) {                                    // look-ahead as in pass 1
@@ -1030,7 +1040,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               tmem_wait(ra);
               tmem_wait(rb);
               tc_fence_before();
-              arrive_lane0(&t_empty[wg], lane);
+              return_arrive(wg);
               prob_accumulate<MAXRED, 32>(ra, rowc + 64, a2, a128, acc);
               prob_accumulate<MAXRED, 32>(rb, rowc + 96, a2, a128, acc);
             } else {
@@ -1039,20 +1049,19 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               if (cw & 16) {
                 tmem_ld16(my_taddr + n32 * 32, rb);
                 tmem_wait(rb);
-                if (n32 == 0) { tc_fence_before(); arrive_lane0(&t_empty[wg], lane); }
+                if (n32 == 0) { tc_fence_before(); return_arrive(wg); }
                 prob_accumulate<MAXRED, 16>(rb, rowc + n32 * 32, a2, a128, acc);
               }
 #pragma unroll 1
               for (int c = 0; c < n32; ++c) {
                 tmem_ld32(my_taddr + c * 32, ra);
                 tmem_wait(ra);
-                if (c == n32 - 1) { tc_fence_before(); arrive_lane0(&t_empty[wg], lane); }
+                if (c == n32 - 1) { tc_fence_before(); return_arrive(wg); }
                 prob_accumulate<MAXRED, 32>(ra, rowc + c * 32, a2, a128, acc);
               }
             }
           }
-          if (!ok) break;
-          if (any && key < sg.n) {
+          if (ok && any && key < sg.n) {
             // The output was zero-filled; the two warpgroups of the pair contribute once per key.
             const float v0 = acc[0].x, v1 = acc[0].y, v2 = acc[1].x, v3 = acc[1].y;
             if (MAXRED) {
