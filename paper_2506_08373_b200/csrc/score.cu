@@ -103,10 +103,8 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 // warp saw a buffer's return some 900 cycles late; where pass 2 has no exponentials (MAX), that is the time of its items: 8
 // layers of 32768, 260 rows of head_dim 64, 251 -> 234 us; with exponentials 471 -> 467 (512 rows).
 constexpr int kReturnBarrier = 6, kReturnThreads = 128 + 32;
-template <int THREADS = kReturnThreads>
-__device__ __forceinline__ void return_arrive(int buf) { asm volatile("bar.arrive %0, %1;" ::"r"(kReturnBarrier + buf), "n"(THREADS) : "memory"); }
-template <int THREADS = kReturnThreads>
-__device__ __forceinline__ void return_sync(int buf) { asm volatile("bar.sync %0, %1;" ::"r"(kReturnBarrier + buf), "n"(THREADS) : "memory"); }
+__device__ __forceinline__ void return_arrive(int buf) { asm volatile("bar.arrive %0, %1;" ::"r"(kReturnBarrier + buf), "n"(kReturnThreads) : "memory"); }
+__device__ __forceinline__ void return_sync(int buf) { asm volatile("bar.sync %0, %1;" ::"r"(kReturnBarrier + buf), "n"(kReturnThreads) : "memory"); }
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -626,7 +624,6 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   extern __shared__ __align__(1024) uint8_t smem[];
   constexpr int BUFCOLS = kBufCols;
   constexpr bool REM = PASS == 1 && FLAG, MAXRED = PASS == 2 && FLAG;
-  constexpr bool OWN = MAXRED;             // the warpgroups issue their own MMAs
 
   const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   uint8_t* k_sm = smem;
@@ -659,9 +656,9 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   // every tile and hand it back.
   const bool both_take = (p.n_stages & 1) != 0;
   if (tid == 32) {
-    for (int i = 0; i < kMaxStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], (OWN ? 2 : 1) * (1 + both_take)); }
+    for (int i = 0; i < kMaxStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 1 + both_take); }
     mbar_init(q_full, 1);
-    mbar_init(q_empty, OWN ? 4 : 2);
+    mbar_init(q_empty, 2);
     for (int i = 0; i < 4; ++i) mbar_init(&t_full[i], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -717,7 +714,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           }
         }
       }
-    } else if (!OWN && warp <= 2) {
+    } else if (warp <= 2) {
       // ------------------------------------------------ MMA issuers -----
       // Two issuing warps, one per warpgroup pair: warp s feeds the buffers of that pair's two
       // warpgroups, and hands the pair's key tiles back.
@@ -973,67 +970,6 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       }
       if (et == 0) *scale_sm = exp2f(scale_log2);               // read after the barriers below
       bool waited = false;
-      // OWN: one warp of the warpgroup, in another sub-partition for each, issues the warpgroup's next item as soon as all four have
-      // read the last one.  The state of that warp: the next item's tile and chunk (-1: the tile not waited for yet) and the stage.
-      const bool issues = OWN && quarter == wg;
-      const int t_first = both_take ? 0 : pair, t_step = both_take ? 1 : 2;
-      uint32_t nseg = 0, kit = 0, k_par = 0;
-      int it_t = 0, it_ch = -1, stage = 0;
-      bool q_done = false;
-      const uint32_t q_half16 = q_half_bytes >> 4, k_half16 = k_half_bytes >> 4;
-      const uint32_t q_lo0 = desc_lo(smem_u32(q_sm)), k_lo0 = desc_lo(smem_u32(k_sm));
-      const uint32_t idesc_full = make_idesc(128), idesc_last = make_idesc(p.cw_last);
-      auto issue_next = [&](int nt) {
-        for (;;) {
-          if (it_t >= nt) {
-            if (!q_done && ok && elect_one()) tc_commit(q_empty);
-            __syncwarp();
-            q_done = true;
-            return;
-          }
-          if (it_ch < 0) {
-            ok = ok && mbar_wait_warp(&k_full[stage], k_par, abort_flag);
-            it_ch = (it_t & 1) == pair ? ((it_t >> 1) * p.turn + half) & 1 : p.n_chunks;
-          }
-          const bool hit = it_ch < p.n_chunks;
-          if (hit) {
-            tc_fence_after();
-            const uint32_t k_lo = k_lo0 + stage * ((128 * 128) >> 4), q_lo = q_lo0 + it_ch * ((128 * 128) >> 4);
-            const uint32_t idesc = it_ch == p.n_chunks - 1 ? idesc_last : idesc_full;
-            if (ok && elect_one()) {
-#pragma unroll
-              for (int kh = 0; kh < 2; ++kh) {
-                if (kh < n_kh) {
-#pragma unroll
-                  for (int ks = 0; ks < 4; ++ks)
-                    tc_mma(tmem_base + wg * BUFCOLS, desc_at(k_lo + kh * k_half16 + ks * 2), desc_at(q_lo + kh * q_half16 + ks * 2), idesc, (kh | ks) != 0);
-                }
-              }
-              tc_commit(&t_full[wg]);
-            }
-            __syncwarp();
-            it_ch += 2;
-          }
-          if (it_ch >= p.n_chunks) {
-            it_t += t_step;
-            it_ch = -1;
-            q_done = hit && it_t >= nt;
-            if (ok && elect_one()) {
-              tc_commit(&k_empty[stage]);
-              if (q_done) tc_commit(q_empty);
-            }
-            __syncwarp();
-            stage += t_step;
-            if (stage >= p.n_stages) { stage -= p.n_stages; k_par ^= 1; }
-          }
-          if (hit) return;
-        }
-      };
-      auto hand_back = [&](int nt) {
-        if (!OWN) return_arrive(wg);
-        else if (issues) { return_sync<128>(wg); issue_next(nt); }
-        else return_arrive<128>(wg);
-      };
       // Every epilogue thread passes the barriers of every segment, also after a wait has
       // given up, so that no warp is left waiting at them.
       while (seg_next<PASS, RAGGED>(it, p, tp, sg)) {
@@ -1048,17 +984,6 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             b1 = (int)((u0 + n_tiles - 1) / per_cta);
           }
           n_part = b1 - b0 + (it.last_segment(b1, u0 + n_tiles) ? 1 : kEpilogueWarpgroups);
-        }
-        if (issues) {                                           // the segment's first item
-          ok = ok && mbar_wait_warp(q_full, nseg & 1, abort_flag);
-          it_t = t_first;
-          it_ch = -1;
-          q_done = false;
-          stage = (int)((kit + t_first) % p.n_stages);
-          k_par = ((kit + t_first) / p.n_stages) & 1;
-          ++nseg;
-          kit += sg.nt;
-          issue_next(sg.nt);
         }
         if (!waited) {
           waited = true;
@@ -1077,11 +1002,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           bool any = false;
           for (int ch = ((t >> 1) * p.turn + half) & 1; ch < p.n_chunks; ch += 2) {
             ok = ok && mbar_wait(&t_full[wg], used & 1, abort_flag);
-            if (!__all_sync(0xffffffffu, ok)) {
-              ok = false;
-              return_sync<OWN ? 128 : kReturnThreads>(wg);
-              continue;
-            }
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_sync(wg); continue; }
             ++used;
             any = true;
             tc_fence_after();
@@ -1104,7 +1025,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               }
               __syncwarp();
               tc_fence_before();
-              hand_back(sg.nt);
+              return_arrive(wg);
               continue;
             }
             if (cw == 128) {                                    // look-ahead as in pass 1
@@ -1119,20 +1040,24 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               tmem_wait(ra);
               tmem_wait(rb);
               tc_fence_before();
-              hand_back(sg.nt);
+              return_arrive(wg);
               prob_accumulate<MAXRED, 32>(ra, rowc + 64, a2, a128, acc);
               prob_accumulate<MAXRED, 32>(rb, rowc + 96, a2, a128, acc);
             } else {
               // a last chunk of 16 to 112 rows, the odd half block first
               const int n32 = cw >> 5;
+              if (cw & 16) {
+                tmem_ld16(my_taddr + n32 * 32, rb);
+                tmem_wait(rb);
+                if (n32 == 0) { tc_fence_before(); return_arrive(wg); }
+                prob_accumulate<MAXRED, 16>(rb, rowc + n32 * 32, a2, a128, acc);
+              }
 #pragma unroll 1
-              for (int c = cw & 16 ? -1 : 0; c < n32; ++c) {
-                const int col = c < 0 ? n32 * 32 : c * 32;
-                if (c < 0) tmem_ld16(my_taddr + col, ra); else tmem_ld32(my_taddr + col, ra);
+              for (int c = 0; c < n32; ++c) {
+                tmem_ld32(my_taddr + c * 32, ra);
                 tmem_wait(ra);
-                if (c == n32 - 1) { tc_fence_before(); hand_back(sg.nt); }
-                if (c < 0) prob_accumulate<MAXRED, 16>(ra, rowc + col, a2, a128, acc);
-                else prob_accumulate<MAXRED, 32>(ra, rowc + col, a2, a128, acc);
+                if (c == n32 - 1) { tc_fence_before(); return_arrive(wg); }
+                prob_accumulate<MAXRED, 32>(ra, rowc + c * 32, a2, a128, acc);
               }
             }
           }
