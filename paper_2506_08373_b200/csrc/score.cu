@@ -152,6 +152,17 @@ __device__ __forceinline__ bool elect_one() {
   asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(e));
   return e != 0;
 }
+// An epilogue warp that has given up has no item to wait for, but its share in every later return is still counted on.  The barrier
+// tells no phase from the next: an arrival before the issuing warp (last of the five, perhaps: it may be waiting for keys) has
+// taken the return before would count as that one's fifth, and every phase from then on lack an arrival, for good.  So the
+// issuing warp publishes, per buffer, how many returns it has taken, and a warp that has given up passes the next one only when that
+// is as many as the warp has made.  Every wait of the issuing warp's own ends in bounded time, so this one does; the limit is a form.
+__device__ __forceinline__ void return_given_up(int buf, uint32_t returned, const volatile uint8_t* taken) {
+#pragma unroll 1
+  for (int it = 0; taken[buf] != (uint8_t)returned && it < (1 << 26); ++it) __nanosleep(500);
+  __syncwarp();
+  return_sync(buf);
+}
 __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
@@ -641,6 +652,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kNumBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* scale_sm = reinterpret_cast<float*>(tmem_slot + 2);
+  volatile uint8_t* taken = reinterpret_cast<volatile uint8_t*>(tmem_slot + 3);   // per buffer, modulo 256: returns that its issuing warp has taken
 
   if ((smem_u32(smem) & 1023u) != 0) {      // the swizzled tiles need 1024-byte alignment
     if (tid == 0) report(p.status, SPEC_ERR_ALIGNMENT);
@@ -648,6 +660,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   }
   if (tid == 0) {
     *abort_flag = 0;
+    tmem_slot[3] = 0;
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_q) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
   }
@@ -727,7 +740,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       SegIter it = seg_begin(p, tp, gridDim.x, blockIdx.x);
       Seg sg;
       uint32_t nseg = 0, kit = 0;                              // segments, key tiles of the segments before
-      bool in_use[2] = {false, false};                         // my pair's two buffers: an item has been issued into them
+      uint32_t uses[2] = {0, 0};                               // items issued into my pair's two buffers
       bool ok = true;
       const uint32_t idesc_full = make_idesc(128);
       const uint32_t idesc_last = make_idesc(PASS == 2 ? p.cw_last : REM ? p.rem_cols : 128);
@@ -736,7 +749,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       const uint32_t q_half16 = q_half_bytes >> 4;
       const uint32_t k_half16 = k_half_bytes >> 4;
       const int t_first = both_take ? 0 : strm, t_step = both_take ? 1 : 2;
-      // Every item passes its buffer's barrier, also after a wait has given up, so that no warp is left waiting there.
+      // Every item passes its buffer's barrier, also after a wait has given up, so that no warp is left waiting there (return_given_up).
       for (;;) {
         const bool more = seg_next<PASS, RAGGED>(it, p, tp, sg);
         const int nt = uniform(more ? sg.nt : 0);
@@ -758,8 +771,12 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             for (int sub = 0; sub < n_sub; ++sub) {
               const int h = (sub + (t >> 1) * p.turn) & 1;
               const int buf = strm * 2 + h;
-              if (h ? in_use[1] : in_use[0]) return_sync(buf);
-              if (h) in_use[1] = true; else in_use[0] = true;
+              const uint32_t use = h ? uses[1] : uses[0];
+              if (use > 0) {
+                return_sync(buf);
+                if (lane == 0) taken[buf] = (uint8_t)use;
+              }
+              if (h) ++uses[1]; else ++uses[0];
               tc_fence_after();
               const uint32_t d_tmem = tmem_base + buf * BUFCOLS;
               const uint32_t q_lo = q_lo0 + sub * ((128 * 128) >> 4);
@@ -790,8 +807,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         if (ok && elect_one()) tc_commit(q_empty);
         __syncwarp();
       }
-      if (in_use[0]) return_sync(strm * 2);                      // of the last items
-      if (in_use[1]) return_sync(strm * 2 + 1);
+      if (uses[0] > 0) return_sync(strm * 2);                    // of the last items
+      if (uses[1] > 0) return_sync(strm * 2 + 1);
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpilogueRegs));
@@ -841,7 +858,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           if (clears && half == 0 && row_in_tile < nv) out[key0 + row_in_tile] = 0.f;
           for (int mt = ((t >> 1) * p.turn + half) & 1; mt < n_sub; mt += 2) {
             ok = ok && mbar_wait(&t_full[wg], used & 1, abort_flag);
-            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_sync(wg); continue; }
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_given_up(wg, used++, taken); continue; }
             ++used;
             tc_fence_after();
             if (REM && mt == n_full) {
@@ -1002,7 +1019,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           bool any = false;
           for (int ch = ((t >> 1) * p.turn + half) & 1; ch < p.n_chunks; ch += 2) {
             ok = ok && mbar_wait(&t_full[wg], used & 1, abort_flag);
-            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_sync(wg); continue; }
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_given_up(wg, used++, taken); continue; }
             ++used;
             any = true;
             tc_fence_after();
