@@ -250,9 +250,10 @@ def test_score_rows_on_columns(B, W, oracle, rows, n, d):
 @pytest.mark.parametrize("d,rows", [(128, 128), (128, 192), (128, 256), (128, 384), (128, 448), (128, 512), (128, 640),
                                     (64, 256), (64, 512), (64, 896), (64, 1024), (64, 1280)])
 def test_score_row_blocks(B, W, oracle, d, rows):
-    """Every number of row blocks to a key tile, even and odd, full and with a short last one, and with it every number of key
-    stages from two to eight (two to five at head_dim 128), over enough tiles per CTA that the stages go round several times; calls in a row."""
-    L, H, n, window = 1, 37, 7600, 9                  # 60 tiles to a unit, 15 to a CTA, shares that span units
+    """Numbers of row blocks to a key tile, even and odd, full and with a short last one, and with them two to five, six and eight key
+    stages, over enough tiles per CTA that the stages go round several times; calls in a row.  A CTA has one segment
+    (test_score_row_blocks_over_segments has several)."""
+    L, H, n, window = 1, 37, 7600, 9                  # 60 tiles to a unit, which four CTAs share evenly
     gen = torch.Generator().manual_seed(rows + d)
     q = torch.randn(1, L, H, rows, d, generator=gen).to(torch.bfloat16).cuda()
     k = torch.randn(L, H, n, d, generator=gen).to(torch.bfloat16).cuda()
@@ -270,6 +271,42 @@ def test_score_row_blocks(B, W, oracle, d, rows):
         for _ in range(20):
             again = torch.full_like(first, float("nan"))
             B.spec_score(pr, q, k, again, ws, reduce=reduce, causal_window=causal, status_word=status)
+            assert torch.equal(first, again)
+    assert status.item() == 0
+
+
+# Query rows to a unit with which every number of key stages occurs (test_library_cpu.py reckons them): two to eight.
+ROW_BLOCKS = [(128, 128), (128, 192), (128, 256), (128, 300), (128, 384), (128, 448), (128, 512), (128, 640),
+              (64, 100), (64, 256), (64, 512), (64, 700), (64, 768), (64, 896), (64, 1024), (64, 1280)]
+SEGMENT_LENS = [641, 129, 1000, 1, 385, 0, 300]
+
+
+@pytest.mark.parametrize("d,rows", ROW_BLOCKS)
+@pytest.mark.parametrize("heads,lens", [(75, [2650]), (593, [375]), (40, SEGMENT_LENS), (400, SEGMENT_LENS)])
+def test_score_row_blocks_over_segments(B, W, oracle, d, rows, heads, lens):
+    """CTAs with several segments each, of odd and even numbers of tiles, so that a segment begins at any stage of the ring and with
+    either pair's: units of 21 tiles in shares of 11, of 3 in shares of 13, and of 1 to 8 in shares of 7 and of 65 (the kernels for many short sequences).  All heads, all four kinds of call, and
+    calls in a row."""
+    n_seq, T, window, base = len(lens), sum(lens), 9, 5
+    gen = torch.Generator().manual_seed(rows + d)
+    q = torch.randn(n_seq, 1, base, rows, d, generator=gen).to(torch.bfloat16)
+    k = torch.randn(1, base, T, d, generator=gen).to(torch.bfloat16)
+    cu = [0] + list(np.cumsum(lens))
+    which = torch.arange(heads) % base
+    qs, ks = q.cuda()[:, :, which.cuda()], k.cuda()[:, which.cuda()]
+    cu_t = torch.tensor(cu, dtype=torch.int32, device="cuda") if n_seq > 1 else None
+    pr = B.make_problem(n_layers=1, n_q_heads=heads, n_kv_heads=heads, head_dim=d, n_lookahead=rows - window, n_window=window,
+                        softmax_scale=d ** -0.5, total_tokens=T, n_in=max(lens), n_seq=n_seq, cu_seqlens=cu_t, k=ks)
+    ws = torch.empty(B.spec_workspace_bytes(pr), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for reduce, causal in ((0, 0), (1, 0), (0, 1), (1, 1)):
+        first = torch.full((1, heads, T), float("nan"), device="cuda")
+        B.spec_score(pr, qs, ks, first, ws, reduce=reduce, causal_window=causal, status_word=status)
+        ref = oracle.spec_score(bits(q), bits(k), cu, rows - window, window, d ** -0.5, mode=reduce, causal_window=bool(causal))
+        assert_scores_close(first.cpu().numpy(), ref[:, which.numpy()], cu)
+        for _ in range(5):
+            again = torch.full_like(first, float("nan"))
+            B.spec_score(pr, qs, ks, again, ws, reduce=reduce, causal_window=causal, status_word=status)
             assert torch.equal(first, again)
     assert status.item() == 0
 

@@ -101,3 +101,21 @@ def test_missing_library_fails_loudly(B, monkeypatch):
     monkeypatch.setattr(build, "LIB_PATH", "/nonexistent/libspec.so")
     with pytest.raises(RuntimeError, match="no fallback"):
         binding.lib()
+
+
+def test_every_number_of_key_stages_is_tested_on_the_gpu():
+    """The scoring's key ring has as many stages as fit beside the queries and the small arrays, and an odd number of them takes
+    other waits than an even one: the rows that the GPU test scores give every number from two to the most that there are."""
+    from test_gpu_parity import ROW_BLOCKS
+    with open(os.path.join(ROOT, "paper_2506_08373_b200", "csrc", "score.cu")) as f:
+        src = f.read()
+    most = int(re.search(r"kMaxStages = (\d+);", src).group(1))
+    bars = eval(re.search(r"kNumBars = ([^;]+);", src).group(1), {"kMaxStages": most})
+    threads, smem = 512, 227 * 1024                    # of the epilogue; per CTA
+    seen = set()
+    for d, rows in ROW_BLOCKS:
+        padded, to_32 = (rows + 127) // 128 * 128, (rows + 31) // 32 * 32
+        slots = threads // to_32 * to_32 if 2 * to_32 <= threads else 0
+        small = padded * 4 + slots * 8 + 2 * 4 + 8 + bars * 8 + 16
+        seen.add(min(most, (smem - padded * d * 2 - small) // (128 * d * 2)))
+    assert seen == set(range(2, most + 1))
