@@ -122,7 +122,7 @@ const char* spec_last_error(void);
  *  scores_out  [n_layers, n_kv_heads, T] fp32; the whole buffer is overwritten (tokens that no
  *              sequence covers are set to 0)
  * Query rows: up to M*head_dim = 81920 (M <= 640 at head_dim 128, 1280 at 64; M <= 512 at head_dim
- * 128 with 70 sequences or more) are scored in one sweep over the keys and the result is
+ * 128 with 78 sequences or more) are scored in one sweep over the keys and the result is
  * bit-reproducible from run to run; a larger M (a long lookahead, a wide GQA group) is scored in
  * ceil(M / that many) sweeps over groups of rows, a multiple of 128 each but the last,
  * whose contributions are added in scores_out (SUM then rounds in an order that may differ between

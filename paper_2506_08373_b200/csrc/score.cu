@@ -1165,7 +1165,7 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
   const int G = pr->n_q_heads / pr->n_kv_heads;
   const int M = G * R;
   // The query rows of a unit stay resident in shared memory, in blocks of 128, beside two key stages and what grows with
-  // them and with the number of sequences (from 70 sequences on, 512 instead of 640 rows of head_dim 128); more than fit
+  // them and with the number of sequences (from 78 sequences on, 512 instead of 640 rows of head_dim 128); more than fit
   // are scored in several launches over groups of as many blocks as the largest needs, whose contributions add up in scores_out.
   const int smem_max = 227 * 1024;
   auto small_bytes = [&](int rows) {                       // all but queries and keys

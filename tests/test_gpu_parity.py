@@ -118,10 +118,10 @@ def test_score_many_short_sequences(B, W, oracle, n_seq, longest, rows, causal):
         assert_scores_close(got.cpu().numpy(), ref, cu)
 
 
-@pytest.mark.parametrize("n_seq,rows", [(69, 160), (70, 160), (1024, 130), (70, 275)])
+@pytest.mark.parametrize("n_seq,rows", [(69, 160), (70, 160), (77, 160), (78, 160), (1024, 130), (70, 275), (78, 275)])
 def test_score_many_sequences_of_many_rows(B, W, oracle, n_seq, rows):
     """The tile prefix of the sequences shares memory with the queries: 640 rows of head_dim 128 stay resident at once beside
-    69 sequences and are scored in two groups beside 70; 1100 rows in three groups."""
+    77 sequences and are scored in two groups beside 78; 1100 rows in two groups beside 70, in three beside 78."""
     L, G, d = 1, 4, 128
     lens = [1 + (i * 37) % 150 if i % 5 else 0 for i in range(n_seq)]
     cu = [0] + [int(x) for x in np.cumsum(lens)]
