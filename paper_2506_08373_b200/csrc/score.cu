@@ -40,8 +40,8 @@
 // for its queries and 1.5 for the first accumulators in pass 1, which ends at 18, and in pass 2 from 18 to 23.5 for the
 // last CTA of pass 1, the statistics (2.5 us) and the constants.
 //
-// Every wait on an mbarrier is bounded in time; on expiry the CTA reports SPEC_ERR_TIMEOUT
-// through the status word, lets its copies land, frees its TMEM and returns.
+// Every wait on an mbarrier is bounded in time; on expiry the CTA passes the named barriers that are left, without the
+// items (return_given_up), reports SPEC_ERR_TIMEOUT through the status word, lets its copies land, frees its TMEM and returns.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -100,8 +100,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 }
 // A buffer's return from its warpgroup to the warp that issues into it: a named barrier, on which the four epilogue warps
 // arrive and the issuing warp waits.  An mbarrier's arrivals and tests stand in one queue with the exponentials, and the issuing
-// warp saw a buffer's return some 900 cycles late; where pass 2 has no exponentials (MAX), that is the time of its items: 8
-// layers of 32768, 260 rows of head_dim 64, 251 -> 234 us; with exponentials 471 -> 467 (512 rows).
+// warp saw a buffer's return some 900 cycles late; where pass 2 has no exponentials (MAX), that is the time of its items.  With it,
+// and with issuing warps that see their own pair's key tiles only, 8 layers of 16384, 260 rows of head_dim 64: MAX 137.2 -> 128.5 us,
+// SUM 158.7 -> 155.0; 384 rows of head_dim 128: 187.9 -> 184.4 and 210.2 -> 209.2.
 constexpr int kReturnBarrier = 6, kReturnThreads = 128 + 32;
 __device__ __forceinline__ void return_arrive(int buf) { asm volatile("bar.arrive %0, %1;" ::"r"(kReturnBarrier + buf), "n"(kReturnThreads) : "memory"); }
 __device__ __forceinline__ void return_sync(int buf) { asm volatile("bar.sync %0, %1;" ::"r"(kReturnBarrier + buf), "n"(kReturnThreads) : "memory"); }
@@ -664,8 +665,11 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_q) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
   }
-  // Every wait tells two phases of a key stage apart by their parity. With an even number of stages, a stage has tiles of one pair
-  // only, whose issuing warp sees all of its phases; with an odd one its tiles are of both pairs in turn, and both warps wait for
+  // Every wait tells two phases of a key stage apart by their parity, so that a phase may be waited for only once the one before it
+  // has completed.  With an even number of stages, a stage has tiles of one pair only within a segment, whose issuing warp takes
+  // them all.  From one segment to the next pairs and stages may change places (a segment of an odd number of tiles); there
+  // the producer's wait for q_empty keeps the phases apart: q_full of a segment is armed when both issuing warps have taken and
+  // handed back all their tiles of the segment before.  With an odd number of stages, a stage has tiles of both pairs in turn, and both warps wait for
   // every tile and hand it back.
   const bool both_take = (p.n_stages & 1) != 0;
   if (tid == 32) {
@@ -706,7 +710,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         uint32_t kit = 0, nseg = 0;
         bool ok = true;
         while (ok && seg_next<PASS, RAGGED>(it, p, tp, sg)) {
-          if (nseg > 0) ok = mbar_wait(q_empty, (nseg - 1) & 1, abort_flag);   // previous unit's MMAs retired
+          if (nseg > 0) ok = mbar_wait(q_empty, (nseg - 1) & 1, abort_flag);   // previous segment's MMAs retired, its key stages' phases complete (both_take)
           if (!ok) break;
           ++nseg;
           mbar_expect_tx(q_full, p.q_bytes);
@@ -1278,7 +1282,10 @@ SPEC_EXPORT int32_t spec_score(const spec_problem* pr, const void* q, const void
     p.n_full = p.M_pad / 128;
     // An odd number of items to a tile, or a short last one, evens out over the tiles when the warpgroups begin in turn. With an even
     // number of equal items that gives a warpgroup two items in a row, for which its one buffer makes it wait: 8 layers of
-    // 32768, head_dim 128, 256 rows 309 -> 296 us, 512 rows 549 -> 527 (of head_dim 64 477 -> 470).
+    // 32768, SUM, in turns and without: head_dim 128, 256 rows 308 and 295 us, 512 rows 546 and 527 (of head_dim 64 475 and 472); odd
+    // numbers: 128 rows 181 and 199, 352 rows 399 and 412, 640 rows 651 and 657.  The line lies at full blocks.  An even number with a
+    // short last one is left in turns, although many of these do better without: 160 rows 238 and 235, 192 rows 281 and 272,
+    // 240 rows 314 and 288, 496 rows 545 and 521; of head_dim 64, 160 rows 193 and 199, 192 rows 229 and 232, 240 rows 252 and 249.
     p.turn = p.M % 128 != 0 || p.n_full % 2 != 0;
     p.rem_cols = 0;
     int rem_bytes = 0;
