@@ -41,7 +41,7 @@
 // last CTA of pass 1, the statistics (2.5 us) and the constants.
 //
 // Every wait on an mbarrier is bounded in time; on expiry the CTA passes the named barriers that are left, without the
-// items (return_given_up), reports SPEC_ERR_TIMEOUT through the status word, lets its copies land, frees its TMEM and returns.
+// items (kReturnBarrier), reports SPEC_ERR_TIMEOUT through the status word, lets its copies land, frees its TMEM and returns.
 #include <cuda.h>
 
 #include "common.cuh"
@@ -103,9 +103,15 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
 // warp saw a buffer's return some 900 cycles late; where pass 2 has no exponentials (MAX), that is the time of its items.  With it,
 // and with issuing warps that see their own pair's key tiles only, 8 layers of 16384, 260 rows of head_dim 64: MAX 137.2 -> 128.5 us,
 // SUM 158.7 -> 155.0; 384 rows of head_dim 128: 187.9 -> 184.4 and 210.2 -> 209.2.
+// A buffer has two such barriers, which its returns take in turn; the parity of their number is also that of the item's phase.  A
+// barrier counts arrivals and does not know whose they are: an epilogue warp that has given up waiting for items goes on to
+// the next return at once, and with one barrier, where the issuing warp has not taken the one before yet (it may be waiting
+// for keys), that would count as its fifth arrival, and every phase from then on lack one, for good.  It waits at that next
+// return, so it is never further ahead.
 constexpr int kReturnBarrier = 6, kReturnThreads = 128 + 32;
-__device__ __forceinline__ void return_arrive(int buf) { asm volatile("bar.arrive %0, %1;" ::"r"(kReturnBarrier + buf), "n"(kReturnThreads) : "memory"); }
-__device__ __forceinline__ void return_sync(int buf) { asm volatile("bar.sync %0, %1;" ::"r"(kReturnBarrier + buf), "n"(kReturnThreads) : "memory"); }
+static_assert(kReturnBarrier % 2 == 0 && kReturnBarrier + 2 * kEpilogueWarpgroups <= 16, "the low bit is the parity, and a CTA has sixteen barriers");
+__device__ __forceinline__ void return_arrive(uint32_t ret) { asm volatile("bar.arrive %0, %1;" ::"r"(ret), "n"(kReturnThreads) : "memory"); }
+__device__ __forceinline__ void return_sync(uint32_t ret) { asm volatile("bar.sync %0, %1;" ::"r"(ret), "n"(kReturnThreads) : "memory"); }
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -133,36 +139,28 @@ __device__ __forceinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity, v
 }
 
 // The common case, a phase that has already completed, costs one non-blocking test inline.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
       : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
-  if (ok) return true;
-  return mbar_wait_slow(bar, parity, abort_flag);
+  return ok != 0;
 }
-
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return mbar_test(bar, parity) || mbar_wait_slow(bar, parity, abort_flag);
+}
 // The same for a whole warp: every lane gets the same answer, and the branches that depend on it do not
-// diverge as far as the compiler can see.
+// diverge as far as the compiler can see.  The vote on the test comes before the slow path, not behind both: 16 layers of
+// 32768, 512 rows of head_dim 64, 917 -> 893 us, pass 1 with rows on columns without spills.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+  if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag));
 }
 // True in exactly one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t e;
   asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(e));
   return e != 0;
-}
-// An epilogue warp that has given up has no item to wait for, but its share in every later return is still counted on.  The barrier
-// tells no phase from the next: an arrival before the issuing warp (last of the five, perhaps: it may be waiting for keys) has
-// taken the return before would count as that one's fifth, and every phase from then on lack an arrival, for good.  So the
-// issuing warp publishes, per buffer, how many returns it has taken, and a warp that has given up passes the next one only when that
-// is as many as the warp has made.  Every wait of the issuing warp's own ends in bounded time, so this one does; the limit is a form.
-__device__ __forceinline__ void return_given_up(int buf, uint32_t returned, const volatile uint8_t* taken) {
-#pragma unroll 1
-  for (int it = 0; taken[buf] != (uint8_t)returned && it < (1 << 26); ++it) __nanosleep(500);
-  __syncwarp();
-  return_sync(buf);
 }
 __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
@@ -653,7 +651,6 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kNumBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   float* scale_sm = reinterpret_cast<float*>(tmem_slot + 2);
-  volatile uint8_t* taken = reinterpret_cast<volatile uint8_t*>(tmem_slot + 3);   // per buffer, modulo 256: returns that its issuing warp has taken
 
   if ((smem_u32(smem) & 1023u) != 0) {      // the swizzled tiles need 1024-byte alignment
     if (tid == 0) report(p.status, SPEC_ERR_ALIGNMENT);
@@ -661,7 +658,6 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   }
   if (tid == 0) {
     *abort_flag = 0;
-    tmem_slot[3] = 0;
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_q) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tm_k) : "memory");
   }
@@ -744,7 +740,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       SegIter it = seg_begin(p, tp, gridDim.x, blockIdx.x);
       Seg sg;
       uint32_t nseg = 0, kit = 0;                              // segments, key tiles of the segments before
-      uint32_t uses[2] = {0, 0};                               // items issued into my pair's two buffers
+      uint32_t ret[2] = {0, 0};                                // my pair's two buffers: the barrier of the next return (0: no item issued yet)
       bool ok = true;
       const uint32_t idesc_full = make_idesc(128);
       const uint32_t idesc_last = make_idesc(PASS == 2 ? p.cw_last : REM ? p.rem_cols : 128);
@@ -753,7 +749,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       const uint32_t q_half16 = q_half_bytes >> 4;
       const uint32_t k_half16 = k_half_bytes >> 4;
       const int t_first = both_take ? 0 : strm, t_step = both_take ? 1 : 2;
-      // Every item passes its buffer's barrier, also after a wait has given up, so that no warp is left waiting there (return_given_up).
+      // Every item passes its buffer's barrier, also after a wait has given up, so that no warp is left waiting there (kReturnBarrier).
       for (;;) {
         const bool more = seg_next<PASS, RAGGED>(it, p, tp, sg);
         const int nt = uniform(more ? sg.nt : 0);
@@ -775,12 +771,10 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
             for (int sub = 0; sub < n_sub; ++sub) {
               const int h = (sub + (t >> 1) * p.turn) & 1;
               const int buf = strm * 2 + h;
-              const uint32_t use = h ? uses[1] : uses[0];
-              if (use > 0) {
-                return_sync(buf);
-                if (lane == 0) taken[buf] = (uint8_t)use;
-              }
-              if (h) ++uses[1]; else ++uses[0];
+              const uint32_t back = h ? ret[1] : ret[0];
+              if (back) return_sync(back);
+              const uint32_t next = back ? back ^ 1 : kReturnBarrier + 2 * buf;
+              if (h) ret[1] = next; else ret[0] = next;
               tc_fence_after();
               const uint32_t d_tmem = tmem_base + buf * BUFCOLS;
               const uint32_t q_lo = q_lo0 + sub * ((128 * 128) >> 4);
@@ -811,8 +805,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         if (ok && elect_one()) tc_commit(q_empty);
         __syncwarp();
       }
-      if (uses[0] > 0) return_sync(strm * 2);                    // of the last items
-      if (uses[1] > 0) return_sync(strm * 2 + 1);
+      if (ret[0]) return_sync(ret[0]);                           // of the last items
+      if (ret[1]) return_sync(ret[1]);
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kEpilogueRegs));
@@ -828,7 +822,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     Seg sg;
     bool ok = true;
     uint32_t ra[32], rb[32];
-    uint32_t used = 0;                                       // items drained from my warpgroup's buffer
+    uint32_t ret = kReturnBarrier + 2 * wg;                  // the barrier of my buffer's next return, whose parity is that of its next item
     const uint32_t my_taddr = lane_base + wg * BUFCOLS;
     if (PASS == 1) {
       // Work item = 128 query rows (on lanes) x the 128 keys of a tile, all of it mine.
@@ -861,9 +855,9 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const bool plain = nv >= kTileKeys && !in_window;
           if (clears && half == 0 && row_in_tile < nv) out[key0 + row_in_tile] = 0.f;
           for (int mt = ((t >> 1) * p.turn + half) & 1; mt < n_sub; mt += 2) {
-            ok = ok && mbar_wait(&t_full[wg], used & 1, abort_flag);
-            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_given_up(wg, used++, taken); continue; }
-            ++used;
+            ok = ok && mbar_wait_warp(&t_full[wg], ret & 1, abort_flag);
+            if (!ok) { return_sync(ret); ret ^= 1; continue; }
+            ret ^= 1;                                           // the item's own is now ret ^ 1
             tc_fence_after();
             if (REM && mt == n_full) {
               // the remaining rows, on columns; this lane's key is key0 + row_in_tile
@@ -886,7 +880,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               if (cols > 32) rem_block<16>(my_taddr + 32, general, seen1, p.a, lane, my_ref + 32, rem_m[1], rem_z[1]);
               __syncwarp();
               tc_fence_before();
-              return_arrive(wg);
+              return_arrive(ret ^ 1);
               continue;
             }
             float m = mrun[mt], z = zrun[mt];
@@ -905,7 +899,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               tmem_wait(ra);
               tmem_wait(rb);
               tc_fence_before();
-              return_arrive(wg);
+              return_arrive(ret ^ 1);
               stats_update(ra, p.a, m, z);
               stats_update(rb, p.a, m, z);
             } else {
@@ -924,7 +918,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               }
               __syncwarp();
               tc_fence_before();
-              return_arrive(wg);
+              return_arrive(ret ^ 1);
             }
             mrun[mt] = m;
             zrun[mt] = z;
@@ -1022,9 +1016,10 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const bool in_window = CAUSAL && (seg_tile<PASS>(sg, t) + 1) * kTileKeys > sg.n - p.n_window;   // warp-uniform
           bool any = false;
           for (int ch = ((t >> 1) * p.turn + half) & 1; ch < p.n_chunks; ch += 2) {
-            ok = ok && mbar_wait(&t_full[wg], used & 1, abort_flag);
-            if (!__all_sync(0xffffffffu, ok)) { ok = false; return_given_up(wg, used++, taken); continue; }
-            ++used;
+            // causal: the vote behind both, without which these kernels spill (one layer of 12345 keys 34.9 and 34.6 us)
+            ok = ok && (CAUSAL ? __all_sync(0xffffffffu, mbar_wait(&t_full[wg], ret & 1, abort_flag)) : mbar_wait_warp(&t_full[wg], ret & 1, abort_flag));
+            if (!ok) { return_sync(ret); ret ^= 1; continue; }
+            ret ^= 1;                                           // the item's own is now ret ^ 1
             any = true;
             tc_fence_after();
             const int cw = ch == p.n_chunks - 1 ? p.cw_last : 128;            // my columns
@@ -1046,7 +1041,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               }
               __syncwarp();
               tc_fence_before();
-              return_arrive(wg);
+              return_arrive(ret ^ 1);
               continue;
             }
             if (cw == 128) {                                    // look-ahead as in pass 1
@@ -1061,7 +1056,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               tmem_wait(ra);
               tmem_wait(rb);
               tc_fence_before();
-              return_arrive(wg);
+              return_arrive(ret ^ 1);
               prob_accumulate<MAXRED, 32>(ra, rowc + 64, a2, a128, acc);
               prob_accumulate<MAXRED, 32>(rb, rowc + 96, a2, a128, acc);
             } else {
@@ -1070,14 +1065,14 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
               if (cw & 16) {
                 tmem_ld16(my_taddr + n32 * 32, rb);
                 tmem_wait(rb);
-                if (n32 == 0) { tc_fence_before(); return_arrive(wg); }
+                if (n32 == 0) { tc_fence_before(); return_arrive(ret ^ 1); }
                 prob_accumulate<MAXRED, 16>(rb, rowc + n32 * 32, a2, a128, acc);
               }
 #pragma unroll 1
               for (int c = 0; c < n32; ++c) {
                 tmem_ld32(my_taddr + c * 32, ra);
                 tmem_wait(ra);
-                if (c == n32 - 1) { tc_fence_before(); return_arrive(wg); }
+                if (c == n32 - 1) { tc_fence_before(); return_arrive(ret ^ 1); }
                 prob_accumulate<MAXRED, 32>(ra, rowc + c * 32, a2, a128, acc);
               }
             }
