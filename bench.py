@@ -43,7 +43,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 NCU_TRAFFIC = {
     # workload index -> {kernel group: (bytes per layer, source files, hash of those sources)}
     # profiles/score_kernel_c2.md (2 layers) and profiles/select_and_gather_c2.md (8 layers)
-    2: {"score": ((539.575552e6 + 6.23744e6 + 549.031168e6 + 3.440896e6) / 2, ["score.cu"], "66cfeb62d8fa04e5"),
+    2: {"score": ((539.58016e6 + 7.712512e6 + 549.016832e6 + 6.012416e6) / 2, ["score.cu"], "8e4479e268f0bdea"),
         "select": ((8.41728e6 + 33.594112e6 + 0.001792e6 + 3.770624e6) / 8, ["select_stream.cu", "select_common.cuh"], "06b0153d0faabae6"),
         "gather": ((67.678976e6 + 14.346752e6) / 8, ["compact.cu"], "94d32f5d239a0cb5")},
     # profiles/select_and_gather_c2.md, the capture of all 32 layers of workload 1 (unit_select_kernel, compact_bulk_kernel)

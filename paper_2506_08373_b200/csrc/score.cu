@@ -35,8 +35,8 @@
 //
 // What bounds it: long calls run at the board's power limit, so that their time is the energy of a logit (tensor
 // core, TMEM read, two packed FMA-pipe operations, the exponential), whatever the clock: 32 layers of 131072 keys,
-// 640 rows of head_dim 128, 12.32 -> 11.82 ms for the step in a loop, at 1575 MHz; of 16384 keys, 384 rows, at full
-// clock 0.94 -> 0.885 ms.  Short calls are bound by the way into each pass: one layer of 12345 keys (36 us) waits 3.4 us
+// 640 rows of head_dim 128, 12.32 -> 11.41 ms for the step in a loop, at 1582 MHz; of 16384 keys, 384 rows, at full
+// clock 0.94 -> 0.865 ms.  Short calls are bound by the way into each pass: one layer of 12345 keys (36 us) waits 3.4 us
 // for its queries and 1.5 for the first accumulators in pass 1, which ends at 18, and in pass 2 from 18 to 23.5 for the
 // last CTA of pass 1, the statistics (2.5 us) and the constants.
 //
@@ -151,7 +151,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
 }
 // The same for a whole warp: every lane gets the same answer, and the branches that depend on it do not
 // diverge as far as the compiler can see.  The vote on the test comes before the slow path, not behind both: 16 layers of
-// 32768, 512 rows of head_dim 64, 917 -> 893 us, pass 1 with rows on columns without spills.
+// 32768, 512 rows of head_dim 64, 917 -> 900 us.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
   return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag));
